@@ -466,7 +466,7 @@ struct Warp3X {
 // dropped from its earlier values); stored rounded to nearest, the new
 // remainder is kept in c0.
 template <typename C, bool kExact = false>
-__device__ __forceinline__ void node3(const C *__restrict__ src, C *__restrict__ dst,
+__device__ __forceinline__ void node3(const C *src, C *dst,
                                       const Const3<C> &k, const int64_t p, const uint32_t fl,
                                       const uint32_t lb, Warp3<C> &sh, const int lane,
                                       float *c0 = nullptr, const uint32_t rs = 0u,
@@ -483,6 +483,7 @@ __device__ __forceinline__ void node3(const C *__restrict__ src, C *__restrict__
     const int zw[3] = {c.z + 1 < k.nz ? c.z + 1 : 0, c.z, c.z > 0 ? c.z - 1 : k.nz - 1};
     const int64_t sx = k.nx, sxy = static_cast<int64_t>(k.nx) * k.ny;
     const int64_t tail = 19 * N + lb;
+    lbm::dev::chain_wait();
 #pragma unroll
     for (int q = 0; q < Q; q++) {
       const int64_t nb = q * N + zw[cvel3(q, 2) + 1] * sxy + yw[cvel3(q, 1) + 1] * sx +
@@ -580,7 +581,7 @@ __device__ __forceinline__ void node3(const C *__restrict__ src, C *__restrict__
 // measured 2 to 4 % slower).
 template <typename C, bool kExact = false>
 __global__ void __launch_bounds__(kThreads3, kExact ? 6 : (sizeof(C) == 4 ? 8 : 2))
-step3_kernel(const C *__restrict__ src, C *__restrict__ dst, const uint32_t *__restrict__ flags,
+step3_kernel(const C *src, C *dst, const uint32_t *__restrict__ flags,
              const uint32_t *__restrict__ lbase, const Link3<C> *__restrict__ links,
              const uint2 *__restrict__ fluid, const __grid_constant__ Const3<C> k, int64_t n_fluid,
              const lbm::LinkCoefDF *__restrict__ links_df = nullptr, float *carry = nullptr,
@@ -1164,17 +1165,18 @@ int lbm3d_step(lbm3d_t *h, int64_t n) {
         if (h->exact) {
           Const3<C> kx = h->kc.get(tag);
           kx.sr_seed = lbm::dev::step_seed(h->steps);
-          step3_kernel<C, true><<<blocks, kThreads3, 0, h->stream>>>(
-              static_cast<const C *>(h->f[src]), static_cast<C *>(h->f[dst]), h->flags, h->lbase,
+          return lbm::launch_chained(
+              step3_kernel<C, true>, blocks, kThreads3, h->stream, static_cast<const C *>(h->f[src]),
+              static_cast<C *>(h->f[dst]), h->flags, h->lbase,
               static_cast<const Link3<C> *>(h->links), h->fluid, kx, h->n_fluid, h->links_df,
               h->carry, h->kc.x);
-          return cudaGetLastError();
         }
       }
-      step3_kernel<C><<<blocks, kThreads3, 0, h->stream>>>(
-          static_cast<const C *>(h->f[src]), static_cast<C *>(h->f[dst]), h->flags, h->lbase,
-          static_cast<const Link3<C> *>(h->links), h->fluid, h->kc.get(tag), h->n_fluid);
-      return cudaGetLastError();
+      return lbm::launch_chained(
+          step3_kernel<C, false>, blocks, kThreads3, h->stream, static_cast<const C *>(h->f[src]),
+          static_cast<C *>(h->f[dst]), h->flags, h->lbase, static_cast<const Link3<C> *>(h->links),
+          h->fluid, h->kc.get(tag), h->n_fluid, static_cast<const lbm::LinkCoefDF *>(nullptr),
+          static_cast<float *>(nullptr), Const3<D2>());
     });
     if (e != cudaSuccess) return fail3(h, LBM_ECUDA, std::string("step: ") + cudaGetErrorString(e));
     h->cur = dst;

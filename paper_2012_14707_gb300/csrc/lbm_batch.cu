@@ -92,13 +92,13 @@ constexpr int kChunk = 256;  // node-arena alignment of every case (>= any CTA w
 // cases with moving walls (k.exact) are left to batch_exact_kernel.
 template <typename T, typename C, int THREADS>
 __global__ void __launch_bounds__(THREADS, PullOcc<T>::min_blocks * kPullThreads / THREADS)
-batch_step_kernel(const T *__restrict__ src, T *__restrict__ dst,
+batch_step_kernel(const T *src, T *dst,
                   const uint2 *__restrict__ node, const int2 *__restrict__ grp,
                   const int32_t *__restrict__ ccase, const int32_t *__restrict__ rowstart,
                   const uint32_t *__restrict__ jbslot, const LinkCoef<C> *__restrict__ links,
-                  const BatchCase<C> *__restrict__ cases, const int32_t *__restrict__ active,
+                  const BatchCase<C> *__restrict__ cases, const int32_t *active,
                   const int32_t *__restrict__ work, const uint32_t n_blocks,
-                  const uint32_t pf_dist, const int64_t *__restrict__ counter, const uint32_t j,
+                  const uint32_t pf_dist, const int64_t *counter, const uint32_t j,
                   const PullGeom *__restrict__ geoms) {
   static_assert(kChunk % THREADS == 0, "a CTA stays inside one chunk");
   constexpr uint32_t kPer = kChunk / THREADS;  // CTAs per chunk
@@ -128,7 +128,6 @@ batch_step_kernel(const T *__restrict__ src, T *__restrict__ dst,
   }
   const int32_t chunk = work[blockIdx.x / kPer];
   const int c = ccase[chunk];
-  if (!active[c]) return;
   const BatchCase<C> &bc = cases[c];
   const uint32_t i = static_cast<uint32_t>(chunk) * kChunk + (blockIdx.x % kPer) * THREADS +
                      threadIdx.x - static_cast<uint32_t>(bc.node_off);
@@ -138,10 +137,9 @@ batch_step_kernel(const T *__restrict__ src, T *__restrict__ dst,
   // the case's geometry from the device table (a local copy would be
   // spilled at this kernel's register budget)
   const PullGeom &g = geoms[c];
-  uint32_t seed = 0;
-  if constexpr (kStochastic<T>) seed = step_seed(*counter + j);
   step_node_pull<T, C, false, THREADS / 32>(src + bc.f_off, dst + bc.f_off, g,
-                                            links + bc.link_off, bc.k, i, seed);
+                                            links + bc.link_off, bc.k, i,
+                                            StepGate{j, active + c, counter});
 }
 
 // 16-bit batches: the paired step of the single-case kernel
@@ -150,29 +148,28 @@ batch_step_kernel(const T *__restrict__ src, T *__restrict__ dst,
 // divides kChunk); the step seed is the batch step kernel's.
 template <typename T, int THREADS>
 __global__ void __launch_bounds__(THREADS, PairOcc::min_blocks * kPairThreads / THREADS)
-batch_pair_kernel(const T *__restrict__ src, T *__restrict__ dst, const uint2 *__restrict__ node,
+batch_pair_kernel(const T *src, T *dst, const uint2 *__restrict__ node,
                   const int2 *__restrict__ grp, const int32_t *__restrict__ ccase,
                   const int32_t *__restrict__ rowstart, const uint32_t *__restrict__ jbslot,
                   const LinkCoef<float> *__restrict__ links,
-                  const BatchCase<float> *__restrict__ cases, const int32_t *__restrict__ active,
-                  const int32_t *__restrict__ work, const int64_t *__restrict__ counter,
+                  const BatchCase<float> *__restrict__ cases, const int32_t *active,
+                  const int32_t *__restrict__ work, const int64_t *counter,
                   const uint32_t j, const PullGeom *__restrict__ geoms) {
   static_assert(kChunk % (2 * THREADS) == 0, "a CTA stays inside one chunk");
   constexpr uint32_t kPer = kChunk / (2 * THREADS);  // CTAs per chunk
   const int32_t chunk = work[blockIdx.x / kPer];
   const int c = ccase[chunk];
-  if (!active[c]) return;
   const BatchCase<float> &bc = cases[c];
   const uint32_t i0 = static_cast<uint32_t>(chunk) * kChunk + (blockIdx.x % kPer) * 2 * THREADS +
                       2 * threadIdx.x - static_cast<uint32_t>(bc.node_off);
   if (i0 >= static_cast<uint32_t>(bc.n_fluid)) return;
   const PullGeom &g = geoms[c];
-  const uint32_t seed = step_seed(*counter + j);
+  const StepGate gate{j, active + c, counter};
   if (i0 + 1u < static_cast<uint32_t>(bc.n_fluid))
-    step_pair_pull<T>(src + bc.f_off, dst + bc.f_off, g, links + bc.link_off, bc.k, i0, seed);
+    step_pair_pull<T>(src + bc.f_off, dst + bc.f_off, g, links + bc.link_off, bc.k, i0, gate);
   else
     step_node_pull<T, float, false>(src + bc.f_off, dst + bc.f_off, g, links + bc.link_off, bc.k,
-                                    i0, seed);
+                                    i0, gate);
 }
 
 // The exact-mass cases of an FP32 batch (moving walls; see collide and
@@ -180,14 +177,13 @@ batch_pair_kernel(const T *__restrict__ src, T *__restrict__ dst, const uint2 *_
 // `chunks` (the chunks of those cases); the same register budget per thread
 // (64) as the single-case exact kernel.
 __global__ void __launch_bounds__(kChunk, 4)
-batch_exact_kernel(const float *__restrict__ src, float *__restrict__ dst,
+batch_exact_kernel(const float *src, float *dst,
                    const int32_t *__restrict__ ccase, const LinkCoef<float> *__restrict__ links,
-                   const BatchCase<float> *__restrict__ cases, const int32_t *__restrict__ active,
-                   const int32_t *__restrict__ chunks, const int64_t *__restrict__ counter,
+                   const BatchCase<float> *__restrict__ cases, const int32_t *active,
+                   const int32_t *__restrict__ chunks, const int64_t *counter,
                    const uint32_t j, const PullGeom *__restrict__ geoms) {
   const int32_t ch = chunks[blockIdx.x];
   const int c = ccase[ch];
-  if (!active[c]) return;
   const BatchCase<float> &bc = cases[c];
   const uint32_t i = static_cast<uint32_t>(ch) * kChunk + threadIdx.x -
                      static_cast<uint32_t>(bc.node_off);
@@ -195,7 +191,7 @@ batch_exact_kernel(const float *__restrict__ src, float *__restrict__ dst,
   // the case's geometry and constants from device tables (not copied into
   // this thread's local memory to be passed to the out-of-line step)
   step_node_exact(src + bc.f_off, dst + bc.f_off, geoms[c], links + bc.link_off, bc.k, i,
-                  step_seed(*counter + j));
+                  StepGate{j, active + c, counter});
 }
 
 // One CTA per case: residual of the case (FP64 sums in a fixed order); a
@@ -310,32 +306,33 @@ cudaError_t launch_batch_step(const T *src, T *dst, const uint2 *node, const int
   if constexpr (kStochastic<T>) {
     if constexpr (THREADS <= kChunk / 2) {
       if (n_work > 0)
-        batch_pair_kernel<T, THREADS><<<static_cast<unsigned>(n_work) * (kChunk / (2 * THREADS)),
-                                        THREADS, 0, s>>>(
-            src, dst, node, grp, ccase, rowstart, jbslot,
-            static_cast<const LinkCoef<float> *>(links),
-            static_cast<const BatchCase<float> *>(cases), active, work, counter, j, geoms);
-      return cudaGetLastError();
+        return launch_chained(batch_pair_kernel<T, THREADS>,
+                              static_cast<unsigned>(n_work) * (kChunk / (2 * THREADS)), THREADS, s,
+                              src, dst, node, grp, ccase, rowstart, jbslot,
+                              static_cast<const LinkCoef<float> *>(links),
+                              static_cast<const BatchCase<float> *>(cases), active, work, counter,
+                              j, geoms);
+      return cudaSuccess;
     } else {
       return cudaErrorInvalidValue;  // 16-bit batches use widths 64 and 128
     }
   }
   const int64_t blocks = static_cast<int64_t>(n_work) * (kChunk / THREADS);
+  cudaError_t e = cudaSuccess;
   if (blocks > 0)
-    batch_step_kernel<T, C, THREADS><<<static_cast<unsigned>(blocks), THREADS, 0, s>>>(
-        src, dst, node, grp, ccase, rowstart, jbslot, static_cast<const LinkCoef<C> *>(links),
-        static_cast<const BatchCase<C> *>(cases), active, work, static_cast<uint32_t>(blocks),
-        pf_dist, counter, j, geoms);
+    e = launch_chained(batch_step_kernel<T, C, THREADS>, static_cast<unsigned>(blocks), THREADS, s,
+                       src, dst, node, grp, ccase, rowstart, jbslot,
+                       static_cast<const LinkCoef<C> *>(links),
+                       static_cast<const BatchCase<C> *>(cases), active, work,
+                       static_cast<uint32_t>(blocks), pf_dist, counter, j, geoms);
   if constexpr (std::is_same<T, float>::value) {
-    if (n_exact_chunks > 0) {
-      cudaError_t e = cudaGetLastError();
-      if (e != cudaSuccess) return e;
-      batch_exact_kernel<<<static_cast<unsigned>(n_exact_chunks), kChunk, 0, s>>>(
-          src, dst, ccase, static_cast<const LinkCoef<float> *>(links),
-          static_cast<const BatchCase<float> *>(cases), active, exact_chunks, counter, j, geoms);
-    }
+    if (e == cudaSuccess && n_exact_chunks > 0)
+      e = launch_chained(batch_exact_kernel, static_cast<unsigned>(n_exact_chunks), kChunk, s, src,
+                         dst, ccase, static_cast<const LinkCoef<float> *>(links),
+                         static_cast<const BatchCase<float> *>(cases), active, exact_chunks,
+                         counter, j, geoms);
   }
-  return cudaGetLastError();
+  return e;
 }
 
 // CTAs of batch_step_kernel<T, C, THREADS> resident at once on the current device.

@@ -11,6 +11,18 @@
 namespace lbm {
 namespace dev {
 
+// In a chain of dependent launches (launch_chained): waits until the
+// kernels before this one in the stream are complete and their stores
+// visible, then lets the next launch of the chain start.  Everything a step
+// writes (lattices, carries) is touched after it; node words, group
+// records, link tables and parameters, which no step writes, may be read
+// before it.  The step kernels' src, dst, active and counter pointers are
+// not __restrict__: a load through a const __restrict__ pointer counts as
+// constant for the whole kernel and might be taken before the wait.
+__device__ __forceinline__ void chain_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
 
 // Storage of a deviation d as T and its arithmetic type C.  FP32, FP64 and
 // BF16 (which keeps FP32's exponent range) store d itself; FP16 stores
@@ -450,8 +462,7 @@ constexpr uint32_t kOpp2 = 0x65872143u;
 __device__ __forceinline__ int vel_x2(int j) { return static_cast<int>((kVelX2 >> (2 * j)) & 3u) - 1; }
 __device__ __forceinline__ int vel_y2(int j) { return static_cast<int>((kVelY2 >> (2 * j)) & 3u) - 1; }
 __device__ __forceinline__ int opp2(int j) { return static_cast<int>((kOpp2 >> (4 * (j - 1))) & 15u); }
-__device__ __forceinline__ void link_epilogue_exact(const float *__restrict__ src,
-                                                    float *__restrict__ dst, const PullGeom &g,
+__device__ __forceinline__ void link_epilogue_exact(const float *src, float *dst, const PullGeom &g,
                                                     const uint32_t fl, const uint32_t li,
                                                     const Collided<float, float> &c_,
                                                     const StepConst<float> &k,
@@ -559,7 +570,7 @@ __device__ __forceinline__ void link_epilogue_exact(const float *__restrict__ sr
 // the node's word rs and the direction).  The exact-mass variant (kExact,
 // FP32 storage) runs link_epilogue_exact instead.
 template <typename T, typename C, bool kExact = false>
-__device__ __forceinline__ void link_epilogue_pull(const T *__restrict__ src, T *__restrict__ dst,
+__device__ __forceinline__ void link_epilogue_pull(const T *src, T *dst,
                                                    const PullGeom &g, const uint32_t fl,
                                                    const uint32_t li,
                                                    const LinkCoef<C> *__restrict__ links,
@@ -623,7 +634,7 @@ __device__ __forceinline__ void link_epilogue_pull(const T *__restrict__ src, T 
 // storage the same way.  The lanes of nodes below g.n_fluid take part (a
 // prefix of the warp: lane i mod 32 runs node i).  kWarps: warps per CTA.
 template <typename T, typename C, int kWarps>
-__device__ __forceinline__ void node_links_warp(const T *__restrict__ src, T *__restrict__ dst,
+__device__ __forceinline__ void node_links_warp(const T *src, T *dst,
                                                 const PullGeom &g, const uint32_t fl,
                                                 const uint32_t li,
                                                 const LinkCoef<C> *__restrict__ links,
@@ -702,17 +713,33 @@ __device__ __forceinline__ uint32_t node_random(const uint32_t seed, const uint3
     return 0u;
 }
 
+// What a node's step asks after its predecessors are complete: whether its
+// case still runs, and the step's seed of random bits.  A single case
+// always runs and its launch holds the seed; a batched case reads its
+// active flag (which the residual pass clears) and the batch's step counter.
+struct StepGate {
+  uint32_t seed_ = 0;
+  const int32_t *active = nullptr;
+  const int64_t *counter = nullptr;  // then the seed is that of step *counter + seed_
+  __device__ __forceinline__ bool open() const {
+    chain_wait();
+    return !active || *active != 0;
+  }
+  __device__ __forceinline__ uint32_t seed() const {
+    return counter ? step_seed(*counter + seed_) : seed_;
+  }
+};
+
 // One time step for fluid node i of a lattice in the pull layout
 // (pull_slots): gather f(x, t) (streaming, Sec. 2), collide (collide),
 // store f'(x, t) in the node's own slots of dst, then the link epilogue.
-// Used by the single-case and the batched step kernels alike; seed is the
-// step's seed of random bits (step_seed of the case's step count).
+// Used by the single-case and the batched step kernels alike.
 template <typename T, typename C, bool kExact = false, int kWarps = 0>
-__device__ __forceinline__ void step_node_pull(const T *__restrict__ src, T *__restrict__ dst,
+__device__ __forceinline__ void step_node_pull(const T *src, T *dst,
                                                const PullGeom &g,
                                                const LinkCoef<C> *__restrict__ links,
                                                const StepConst<C> &k, const uint32_t i,
-                                               const uint32_t seed) {
+                                               const StepGate &gate) {
   const uint32_t P = g.plane;
   const uint2 nw = g.node[i];
   const int2 gr = g.grp[i / kGroup];
@@ -720,6 +747,7 @@ __device__ __forceinline__ void step_node_pull(const T *__restrict__ src, T *__r
   {
     uint32_t s[9];
     pull_slots(nw, gr, i, P, g.n_fluid, g.ny, g.periodic_y, g.rowstart, s);
+    if (!gate.open()) return;
 #pragma unroll
     for (int q = 0; q < 9; q++)
       d[q] = Stor<T>::kScaled ? Stor<T>::ld_raw(src[s[q]]) : Stor<T>::ld(src[s[q]], k.inv_sc);
@@ -732,7 +760,7 @@ __device__ __forceinline__ void step_node_pull(const T *__restrict__ src, T *__r
       asm volatile("prefetch.global.L1 [%0];" ::"l"(g.jbslot + gr.y + node_loff(nw)));
     }
   }
-  const uint32_t rs = node_random<T, kExact>(seed, i);
+  const uint32_t rs = node_random<T, kExact>(gate.seed(), i);
   Collided<T, C> c;
   if constexpr (kExact) {
     float c0 = g.carry0[i];
@@ -831,7 +859,7 @@ __device__ __forceinline__ float link_value_rt(const LinkCoef<float> &c, const i
 // warp; a lone last node runs the one-node step instead).
 constexpr int kPairMaxWarps = 4;  // CTAs of up to 128 threads
 template <typename T>
-__device__ __forceinline__ void pair_links_warp(const T *__restrict__ src, T *__restrict__ dst,
+__device__ __forceinline__ void pair_links_warp(const T *src, T *dst,
                                                 const PullGeom &g,
                                                 const LinkCoef<float> *__restrict__ links,
                                                 const StepConst<float> &k, const uint32_t i0,
@@ -894,11 +922,11 @@ __device__ __forceinline__ void pair_links_warp(const T *__restrict__ src, T *__
 }
 
 template <typename T>
-__device__ __forceinline__ void step_pair_pull(const T *__restrict__ src, T *__restrict__ dst,
+__device__ __forceinline__ void step_pair_pull(const T *src, T *dst,
                                                const PullGeom &g,
                                                const LinkCoef<float> *__restrict__ links,
                                                const StepConst<float> &k, const uint32_t i0,
-                                               const uint32_t seed) {
+                                               const StepGate &gate) {
   static_assert(kStochastic<T>, "the paired step is the 16-bit storage step");
   const uint32_t P = g.plane;
   const uint4 nw2 = *reinterpret_cast<const uint4 *>(g.node + i0);
@@ -913,6 +941,7 @@ __device__ __forceinline__ void step_pair_pull(const T *__restrict__ src, T *__r
     uint32_t s0[9], s1[9];
     pull_slots(nw0, gr, i0, P, g.n_fluid, g.ny, g.periodic_y, g.rowstart, s0);
     pull_slots(nw1, gr, i0 + 1u, P, g.n_fluid, g.ny, g.periodic_y, g.rowstart, s1);
+    if (!gate.open()) return;
 #pragma unroll
     for (int q = 0; q < 9; q++)
       d[q] = F2(make_float2(Stor<T>::ld_raw(src[s0[q]]), Stor<T>::ld_raw(src[s1[q]])));
@@ -929,7 +958,7 @@ __device__ __forceinline__ void step_pair_pull(const T *__restrict__ src, T *__r
   F2 ch[9], drho, rho, ux, uy, uu;
   collision_change<kS, false>(d, k, ch, drho, rho, ux, uy, uu);
   // random words of the pair
-  const uint32_t h0 = fmix32(i0 ^ seed), h1 = fmix32(h0 + 0x9E3779B9u),
+  const uint32_t h0 = fmix32(i0 ^ gate.seed()), h1 = fmix32(h0 + 0x9E3779B9u),
                  h2 = fmix32(h0 + 0x3C6EF372u);
   const uint32_t rb[9] = {h0,
                           h1,
@@ -971,12 +1000,12 @@ __device__ __forceinline__ void step_pair_pull(const T *__restrict__ src, T *__r
 // not inlined: the single-case and the batched kernels then run bitwise the
 // same compiled arithmetic (inlined into kernels with different register
 // budgets, the compiler may fuse multiplies and adds differently).
-static __device__ __noinline__ void step_node_exact(const float *__restrict__ src, float *__restrict__ dst,
+static __device__ __noinline__ void step_node_exact(const float *src, float *dst,
                                              const PullGeom &g,
                                              const LinkCoef<float> *__restrict__ links,
                                              const StepConst<float> &k, const uint32_t i,
-                                             const uint32_t seed) {
-  step_node_pull<float, float, true>(src, dst, g, links, k, i, seed);
+                                             const StepGate &gate) {
+  step_node_pull<float, float, true>(src, dst, g, links, k, i, gate);
 }
 
 // Eq. FluidMacr from deviations: returns rho - 1 (kept exact for the mass sum).

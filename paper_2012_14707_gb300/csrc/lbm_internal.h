@@ -354,6 +354,25 @@ void parallel_for(int64_t n, F &&f, int64_t min_per_thread = 1 << 14) {
   for (auto &t : th) t.join();
 }
 
+// Launches kernel f(args...) of a chain of dependent steps in stream s with
+// programmatic stream serialisation: the next kernel of the chain may start
+// its CTAs, and read what no step writes, while this one's last CTAs still
+// run; it waits at dev::chain_wait() for this one's results.
+template <typename... P, typename... A>
+cudaError_t launch_chained(void (*f)(P...), unsigned blocks, unsigned threads, cudaStream_t s,
+                           A &&...args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3(threads);
+  cfg.stream = s;
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, f, P(args)...);
+}
+
 // Validation and layout of one case (lbm_api.cu).
 int build_host_case(const lbm_domain_t *dom, const uint8_t *solid, size_t n_links,
                     const int32_t *link_x, const int32_t *link_y, const int32_t *link_dir,

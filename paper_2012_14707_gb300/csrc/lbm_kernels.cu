@@ -42,7 +42,7 @@ using namespace dev;
 // see collide and link_epilogue_pull), with 64 registers per thread.
 template <typename T, typename C, bool kExact>
 __global__ void __launch_bounds__(kPullThreads, kExact ? 8 : PullOcc<T>::min_blocks)
-step_kernel_pull(const T *__restrict__ src, T *__restrict__ dst, __grid_constant__ const PullGeom g,
+step_kernel_pull(const T *src, T *dst, __grid_constant__ const PullGeom g,
                  const uint32_t n_fluid, const LinkCoef<C> *__restrict__ links,
                  __grid_constant__ const StepConst<C> k) {
   {
@@ -70,9 +70,9 @@ step_kernel_pull(const T *__restrict__ src, T *__restrict__ dst, __grid_constant
   const uint32_t i = blockIdx.x * kPullThreads + threadIdx.x;
   if (i >= n_fluid) return;
   if constexpr (kExact)
-    step_node_exact(src, dst, g, links, k, i, k.sr_seed);
+    step_node_exact(src, dst, g, links, k, i, StepGate{k.sr_seed});
   else
-    step_node_pull<T, C, false, kPullThreads / 32>(src, dst, g, links, k, i, k.sr_seed);
+    step_node_pull<T, C, false, kPullThreads / 32>(src, dst, g, links, k, i, StepGate{k.sr_seed});
 }
 
 // One time step of a single case in 16-bit storage: thread t of CTA b runs
@@ -82,7 +82,7 @@ step_kernel_pull(const T *__restrict__ src, T *__restrict__ dst, __grid_constant
 // step_kernel_pull.
 template <typename T>
 __global__ void __launch_bounds__(kPairThreads, PairOcc::min_blocks)
-step_kernel_pair(const T *__restrict__ src, T *__restrict__ dst, const PullGeom g,
+step_kernel_pair(const T *src, T *dst, const PullGeom g,
                  const uint32_t n_fluid, const LinkCoef<float> *__restrict__ links,
                  const StepConst<float> k) {
   constexpr uint32_t kNodes = 2 * kPairThreads;  // per CTA
@@ -112,9 +112,9 @@ step_kernel_pair(const T *__restrict__ src, T *__restrict__ dst, const PullGeom 
   const uint32_t i0 = 2u * (blockIdx.x * kPairThreads + threadIdx.x);
   if (i0 >= n_fluid) return;
   if (i0 + 1u < n_fluid)
-    step_pair_pull<T>(src, dst, g, links, k, i0, k.sr_seed);
+    step_pair_pull<T>(src, dst, g, links, k, i0, StepGate{k.sr_seed});
   else
-    step_node_pull<T, float, false>(src, dst, g, links, k, i0, k.sr_seed);
+    step_node_pull<T, float, false>(src, dst, g, links, k, i0, StepGate{k.sr_seed});
 }
 
 // Mass deviation of one node, sum_i d_i, to FP64 accuracy.  FP64 storage:
@@ -453,23 +453,22 @@ cudaError_t launch_step_pull(const T *src, T *dst, const PullGeom &g, int64_t n_
   if (n_fluid <= 0) return cudaSuccess;
   if constexpr (kStochastic<T>) {
     const int64_t pairs = (n_fluid + 1) / 2;
-    step_kernel_pair<T><<<static_cast<unsigned>((pairs + kPairThreads - 1) / kPairThreads),
-                          kPairThreads, 0, s>>>(src, dst, g, static_cast<uint32_t>(n_fluid), links,
-                                                k);
+    return launch_chained(step_kernel_pair<T>,
+                          static_cast<unsigned>((pairs + kPairThreads - 1) / kPairThreads),
+                          kPairThreads, s, src, dst, g, static_cast<uint32_t>(n_fluid), links, k);
   } else {
     const int64_t blocks = (n_fluid + kPullThreads - 1) / kPullThreads;
     if constexpr (std::is_same<T, float>::value) {
       if (k.exact) {
         if (!g.links64 || !g.carry || !g.carry0) return cudaErrorInvalidValue;
-        step_kernel_pull<T, C, true><<<static_cast<unsigned>(blocks), kPullThreads, 0, s>>>(
-            src, dst, g, static_cast<uint32_t>(n_fluid), links, k);
-        return cudaGetLastError();
+        return launch_chained(step_kernel_pull<T, C, true>, static_cast<unsigned>(blocks),
+                              kPullThreads, s, src, dst, g, static_cast<uint32_t>(n_fluid), links,
+                              k);
       }
     }
-    step_kernel_pull<T, C, false><<<static_cast<unsigned>(blocks), kPullThreads, 0, s>>>(
-        src, dst, g, static_cast<uint32_t>(n_fluid), links, k);
+    return launch_chained(step_kernel_pull<T, C, false>, static_cast<unsigned>(blocks),
+                          kPullThreads, s, src, dst, g, static_cast<uint32_t>(n_fluid), links, k);
   }
-  return cudaGetLastError();
 }
 
 template <typename T>
