@@ -10,7 +10,7 @@
 // product is accumulated in FP32; master weights, weight gradients and Adam
 // moments are FP32.
 //
-// Kernels:
+// FP32 mode, on CUDA cores:
 //   conv_fwd<KS>    y = act(conv(x, w) + b), KS = 3 (zero padding) or 1;
 //                   a CTA computes a 16x16 pixel tile x 16 output channels,
 //                   staging an input tile (with halo) and the weights of a
@@ -22,6 +22,10 @@
 //                   CTA reduces a pixel chunk for a 16x16 (c, o) tile and
 //                   adds it into FP32 dW; db by a column sum.
 //   pool / upsample / concat / MSE / Adam: elementwise or simple reductions.
+// BF16 mode: the convolutions of lbm_net_tc.cu on the tensor cores, which
+// read the decoder's upsampled-and-concatenated input from its two sources
+// and apply the ReLU's backward mask as they store, and elementwise passes
+// of 8 channels per thread (below).
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
@@ -34,6 +38,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/lbm.h"
+#include "lbm_net_tc.h"
 
 namespace lbm {
 namespace net {
@@ -45,19 +50,11 @@ template <>
 __device__ __forceinline__ float to_f<float>(float v) {
   return v;
 }
-template <>
-__device__ __forceinline__ float to_f<__nv_bfloat16>(__nv_bfloat16 v) {
-  return __bfloat162float(v);
-}
 template <typename A>
 __device__ __forceinline__ A from_f(float v);
 template <>
 __device__ __forceinline__ float from_f<float>(float v) {
   return v;
-}
-template <>
-__device__ __forceinline__ __nv_bfloat16 from_f<__nv_bfloat16>(float v) {
-  return __float2bfloat16_rn(v);
 }
 
 constexpr int TP = 16;  // pixel tile edge
@@ -181,593 +178,6 @@ conv_bwd_weight(const A *__restrict__ x, int xs, const A *__restrict__ gz, int N
     for (int d = 0; d < KS * KS; d++)
       atomicAdd(&dw[(static_cast<int64_t>(d) * Ci + c0 + c) * Co + o0 + o], acc[d]);
     if (c == 0 && c0 == 0 && db) atomicAdd(&db[o0 + o], bacc);
-  }
-}
-
-// ---------------------------------------------------------------------------
-// Tensor-core convolution (BF16 storage): an implicit GEMM on tcgen05.
-//   D[p][o] = sum_{d, c} X[p + d - HALO][c] * Wk[o][d][c]      (M = pixels,
-//   N = output channels, K = taps x input channels)
-// A CTA owns 128 pixels x NT output channels (NT <= 128, a multiple of 16);
-// D lives in tensor memory (FP32, NT columns).  K runs tap by tap in chunks
-// of up to 64 channels: the 128 threads gather one pixel row each of A (the
-// shifted input, zero outside the image) and one row each of B (packed
-// weights, K-major), store both in shared memory in the canonical K-major
-// layout without swizzle (8-row x 16-byte core matrices, core matrices
-// along K 128 B apart, 8-row groups 1024 B apart), and one thread issues
-// the MMAs (M = 128, N = NT, K = 16 each) and commits them to an mbarrier.
-// Two stages: the gather of chunk k + 1 overlaps the MMAs of chunk k.  Every
-// wait is bounded; a wait that runs out sets *err and the CTA stops issuing.
-// The epilogue reads D back with tcgen05.ld (warp w owns lanes 32w..32w+31 =
-// pixels 32w..), adds the bias, applies ReLU and stores BF16.
-
-__device__ __forceinline__ uint32_t smem_addr(const void *p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_addr(bar)), "r"(count)
-               : "memory");
-}
-
-// Waits for the phase with parity `phase` of *bar; false if it did not come
-// within `limit` polls (test_wait: each poll returns at once, so the bound
-// is a bound in time).
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t phase, int limit) {
-  for (int it = 0; it < limit; it++) {
-    uint32_t done;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-        " selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(done)
-        : "r"(smem_addr(bar)), "r"(phase)
-        : "memory");
-    if (done) return true;
-  }
-  return false;
-}
-
-// Shared-memory matrix descriptor (K-major, no swizzle): start address,
-// leading byte offset (between core matrices along K), stride byte offset
-// (between 8-row groups), all in 16-byte units; bit 46 = descriptor version
-// of this architecture; layout type 0 = no swizzle.
-__device__ __forceinline__ uint64_t umma_desc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
-  return static_cast<uint64_t>((addr >> 4) & 0x3FFFu) |
-         (static_cast<uint64_t>((lbo >> 4) & 0x3FFFu) << 16) |
-         (static_cast<uint64_t>((sbo >> 4) & 0x3FFFu) << 32) | (1ull << 46);
-}
-
-// Instruction descriptor, kind::f16: D = F32, A = B = BF16, both K-major,
-// shape M x N.
-__host__ __device__ constexpr uint32_t umma_idesc_bf16(int M, int N) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | (static_cast<uint32_t>(N >> 3) << 17) |
-         (static_cast<uint32_t>(M >> 4) << 24);
-}
-
-constexpr int kTcM = 128;        // pixels per CTA (MMA M)
-constexpr int kTcKC = 64;        // channels per K chunk
-constexpr int kTcNMax = 128;     // output channels per CTA (MMA N)
-constexpr int kTcStageBytes = kTcM * kTcKC * 2;  // one operand, one stage: 16 KB
-constexpr int kTcSmem = 4 * kTcStageBytes + 1024;  // A and B, two stages, + alignment
-constexpr int kTcWaitLimit = 1 << 24;
-
-// Wk[o][d][c] (BF16, K-major, Co rows padded to Cop, Ci padded to Cip with
-// zeros) from the FP32 parameters w[d][c][o].  flip: the adjoint
-// convolution's weights (taps reversed, channels swapped): Wk[c][d][o] =
-// w[KS2 - 1 - d][c][o], i.e. a layer with Ci and Co exchanged.
-__global__ void pack_wk(const float *__restrict__ w, __nv_bfloat16 *__restrict__ wk, int KS2,
-                        int Ci, int Co, int flip, int Cop, int Cip) {
-  // output layer: Ci' = flip ? Co : Ci, Co' = flip ? Ci : Co
-  const int64_t n = static_cast<int64_t>(Cop) * KS2 * Cip;
-  for (int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; e < n;
-       e += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const int c2 = static_cast<int>(e % Cip);
-    const int d = static_cast<int>((e / Cip) % KS2);
-    const int o2 = static_cast<int>(e / (static_cast<int64_t>(Cip) * KS2));
-    float v = 0.f;
-    if (!flip) {
-      if (o2 < Co && c2 < Ci) v = w[(static_cast<int64_t>(d) * Ci + c2) * Co + o2];
-    } else {
-      // o2 = original input channel, c2 = original output channel
-      if (o2 < Ci && c2 < Co) v = w[(static_cast<int64_t>(KS2 - 1 - d) * Ci + o2) * Co + c2];
-    }
-    wk[e] = __float2bfloat16_rn(v);
-  }
-}
-
-template <int KS>
-__global__ void __launch_bounds__(kTcM)
-conv_fwd_tc(const __nv_bfloat16 *__restrict__ x, int xs, const __nv_bfloat16 *__restrict__ wk,
-            int Cip, const float *__restrict__ b, __nv_bfloat16 *__restrict__ y, int ys, int N,
-            int H, int W, int Ci, int Co, int NT, int relu, int vec, int *__restrict__ err) {
-  constexpr int HALO = KS / 2;
-  constexpr int KS2 = KS * KS;
-  extern __shared__ unsigned char tc_smem_raw[];
-  unsigned char *smem = reinterpret_cast<unsigned char *>(
-      (reinterpret_cast<uintptr_t>(tc_smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  __shared__ uint64_t mbar[2];
-  __shared__ uint32_t tmem_slot;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int64_t npix = static_cast<int64_t>(N) * H * W;
-  const int64_t p = static_cast<int64_t>(blockIdx.x) * kTcM + tid;  // this thread's pixel (A row)
-  const int o0 = blockIdx.y * NT;
-  int pn = 0, pi = 0, pj = 0;
-  if (p < npix) {
-    pn = static_cast<int>(p / (static_cast<int64_t>(H) * W));
-    const int r = static_cast<int>(p - static_cast<int64_t>(pn) * H * W);
-    pi = r / W;
-    pj = r - pi * W;
-  }
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
-                     smem_addr(&tmem_slot)),
-                 "r"(kTcNMax)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
-  }
-  if (tid == 0) {
-    mbar_init(&mbar[0], 1);
-    mbar_init(&mbar[1], 1);
-    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-  const uint32_t tmem = tmem_slot;
-  const uint32_t idesc = umma_idesc_bf16(kTcM, NT);
-  const int nck = (Cip + kTcKC - 1) / kTcKC;  // channel chunks per tap
-  const int iters = KS2 * nck;
-  uint32_t phase[2] = {0u, 0u};
-  bool ok = true;
-  for (int it = 0; it < iters; it++) {
-    const int st = it & 1;
-    if (it >= 2) {  // the MMAs that read this stage two chunks ago are done
-      const bool got = mbar_wait(&mbar[st], phase[st], kTcWaitLimit);
-      if (__syncthreads_or(!got)) {  // one decision for the whole CTA
-        ok = false;
-        if (tid == 0) atomicExch(err, 1);
-        break;
-      }
-      phase[st] ^= 1u;
-    }
-    const int d = it / nck, c0 = (it % nck) * kTcKC;
-    const int kc = min(kTcKC, Cip - c0);  // multiple of 16
-    unsigned char *sa = smem + st * 2 * kTcStageBytes;
-    unsigned char *sb = sa + kTcStageBytes;
-    // A row `tid`: input pixel (pi + dy - HALO, pj + dx - HALO), channels c0 .. c0 + kc
-    {
-      const int ii = pi + d / KS - HALO, jj = pj + d % KS - HALO;
-      const bool in = p < npix && ii >= 0 && ii < H && jj >= 0 && jj < W;
-      const __nv_bfloat16 *src = x + ((static_cast<int64_t>(pn) * H + ii) * W + jj) * xs;
-      unsigned char *row = sa + (tid >> 3) * 1024 + (tid & 7) * 16;
-      for (int q = 0; q < kc / 8; q++) {
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        const int c = c0 + q * 8;
-        if (in && c < Ci) {
-          if (vec) {
-            v = *reinterpret_cast<const uint4 *>(src + c);
-          } else {
-            __nv_bfloat16 t8[8];
-#pragma unroll
-            for (int e = 0; e < 8; e++) t8[e] = (c + e < Ci) ? src[c + e] : __float2bfloat16_rn(0.f);
-            v = *reinterpret_cast<const uint4 *>(t8);
-          }
-        }
-        *reinterpret_cast<uint4 *>(row + q * 128) = v;
-      }
-    }
-    // B row `tid` (< NT): output channel o0 + tid, tap d, channels c0 .. c0 + kc
-    if (tid < NT) {
-      const __nv_bfloat16 *src = wk + (static_cast<int64_t>(o0 + tid) * KS2 + d) * Cip + c0;
-      unsigned char *row = sb + (tid >> 3) * 1024 + (tid & 7) * 16;
-      for (int q = 0; q < kc / 8; q++)
-        *reinterpret_cast<uint4 *>(row + q * 128) = *reinterpret_cast<const uint4 *>(src + q * 8);
-    }
-    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-    __syncthreads();
-    if (tid == 0) {
-      asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-      const uint32_t a0 = smem_addr(sa), b0 = smem_addr(sb);
-      for (int k = 0; k < kc / 16; k++) {
-        const uint64_t ad = umma_desc(a0 + k * 256, 128, 1024);
-        const uint64_t bd = umma_desc(b0 + k * 256, 128, 1024);
-        const uint32_t acc = (it > 0 || k > 0) ? 1u : 0u;
-        asm volatile(
-            "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-            " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-            "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
-            : "memory");
-      }
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
-                       smem_addr(&mbar[st]))
-                   : "memory");
-    }
-  }
-  // all MMAs done: the last commit covers every earlier MMA of the issuing thread
-  if (ok && iters > 0) {
-    const int st = (iters - 1) & 1;
-    const bool got = mbar_wait(&mbar[st], phase[st], kTcWaitLimit);
-    if (__syncthreads_or(!got)) {
-      ok = false;
-      if (tid == 0) atomicExch(err, 1);
-    }
-  }
-  asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-  // tcgen05.ld is warp-collective (.sync.aligned): every lane loads, in
-  // converged code, also lanes past the last pixel; only the stores are
-  // predicated.  `ok` is uniform over the CTA.
-  if (ok) {
-    __syncwarp();
-    __nv_bfloat16 *yp = y + (p < npix ? p : 0) * ys;
-    for (int c = 0; c < NT; c += 8) {
-      uint32_t r[8];
-      asm volatile(
-          "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n"
-          : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-            "=r"(r[7])
-          : "r"(tmem + (static_cast<uint32_t>(warp * 32) << 16) + c));
-      asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-      if (p < npix) {
-#pragma unroll
-        for (int e = 0; e < 8; e++) {
-          const int o = o0 + c + e;
-          if (o < Co) {
-            float v = __uint_as_float(r[e]) + (b ? b[o] : 0.f);
-            if (relu) v = fmaxf(v, 0.f);
-            yp[o] = __float2bfloat16_rn(v);
-          }
-        }
-      }
-    }
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-  __syncthreads();
-  if (warp == 0) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem),
-                 "r"(kTcNMax)
-                 : "memory");
-  }
-  (void)lane;
-}
-
-// The same convolution with its operands copied asynchronously (cp.async,
-// 16 bytes per copy, zero-filled outside the image) through a ring of
-// kTcAsyncStages stages: the copies of the next kTcAsyncStages - 1 chunks
-// are in flight while the tensor cores work on the current one, instead of
-// each chunk's gather waiting out its own memory latency.  Needs 16-byte
-// aligned channel rows (input channels and their stride multiples of 8).
-constexpr int kTcAsyncStages = 3;
-constexpr int kTcAsyncSmem = kTcAsyncStages * 2 * kTcStageBytes + 1024;
-
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, uint32_t src_bytes) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src),
-               "r"(src_bytes)
-               : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() {
-  asm volatile("cp.async.commit_group;\n" ::: "memory");
-}
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
-}
-
-template <int KS>
-__global__ void __launch_bounds__(kTcM)
-conv_fwd_tc_async(const __nv_bfloat16 *__restrict__ x, int xs,
-                  const __nv_bfloat16 *__restrict__ wk, int Cip, const float *__restrict__ b,
-                  __nv_bfloat16 *__restrict__ y, int ys, int N, int H, int W, int Ci, int Co,
-                  int NT, int relu, int *__restrict__ err) {
-  constexpr int HALO = KS / 2;
-  constexpr int KS2 = KS * KS;
-  constexpr int S = kTcAsyncStages;
-  extern __shared__ unsigned char tc_smem_raw[];
-  unsigned char *smem = reinterpret_cast<unsigned char *>(
-      (reinterpret_cast<uintptr_t>(tc_smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  __shared__ uint64_t mbar[S];
-  __shared__ uint32_t tmem_slot;
-  const int tid = threadIdx.x, warp = tid >> 5;
-  const int64_t npix = static_cast<int64_t>(N) * H * W;
-  const int64_t p = static_cast<int64_t>(blockIdx.x) * kTcM + tid;  // this thread's pixel (A row)
-  const int o0 = blockIdx.y * NT;
-  int pn = 0, pi = 0, pj = 0;
-  if (p < npix) {
-    pn = static_cast<int>(p / (static_cast<int64_t>(H) * W));
-    const int r = static_cast<int>(p - static_cast<int64_t>(pn) * H * W);
-    pi = r / W;
-    pj = r - pi * W;
-  }
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
-                     smem_addr(&tmem_slot)),
-                 "r"(kTcNMax)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
-  }
-  if (tid == 0) {
-    for (int s = 0; s < S; s++) mbar_init(&mbar[s], 1);
-    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-  const uint32_t tmem = tmem_slot;
-  const uint32_t idesc = umma_idesc_bf16(kTcM, NT);
-  const int nck = (Cip + kTcKC - 1) / kTcKC;  // channel chunks per tap
-  const int iters = KS2 * nck;
-  // copies of chunk `it` into its stage: A row `tid` (input pixel shifted by
-  // the tap, zero outside the image) and B row `tid` (< NT: output channel
-  // o0 + tid of the packed weights)
-  auto load = [&](int it) {
-    const int st = it % S;
-    const int d = it / nck, c0 = (it % nck) * kTcKC;
-    const int kc = min(kTcKC, Cip - c0);
-    const uint32_t sa = smem_addr(smem + st * 2 * kTcStageBytes);
-    const uint32_t sb = sa + kTcStageBytes;
-    const uint32_t row = (tid >> 3) * 1024 + (tid & 7) * 16;
-    const int ii = pi + d / KS - HALO, jj = pj + d % KS - HALO;
-    const bool in = p < npix && ii >= 0 && ii < H && jj >= 0 && jj < W;
-    const __nv_bfloat16 *src =
-        in ? x + ((static_cast<int64_t>(pn) * H + ii) * W + jj) * xs : x;
-    for (int q = 0; q < kc / 8; q++) {
-      const int c = c0 + q * 8;
-      const bool v = in && c < Ci;
-      cp_async16(sa + row + q * 128, v ? src + c : x, v ? 16u : 0u);
-    }
-    if (tid < NT) {
-      const __nv_bfloat16 *ws = wk + (static_cast<int64_t>(o0 + tid) * KS2 + d) * Cip + c0;
-      for (int q = 0; q < kc / 8; q++) cp_async16(sb + row + q * 128, ws + q * 8, 16u);
-    }
-  };
-  for (int s = 0; s < S - 1; s++) {
-    if (s < iters) load(s);
-    cp_async_commit();
-  }
-  bool ok = true;
-  for (int it = 0; it < iters; it++) {
-    const int st = it % S;
-    const int nxt = it + S - 1;
-    if (nxt < iters) {
-      // stage nxt % S was last read by the MMAs of chunk it - 1
-      if (it >= 1) {
-        const bool got = mbar_wait(&mbar[(it - 1) % S], ((it - 1) / S) & 1, kTcWaitLimit);
-        if (__syncthreads_or(!got)) {  // one decision for the whole CTA
-          ok = false;
-          if (tid == 0) atomicExch(err, 1);
-          break;
-        }
-      }
-      load(nxt);
-    }
-    cp_async_commit();
-    cp_async_wait<S - 1>();  // this thread's copies of chunk `it` have landed
-    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-    __syncthreads();
-    if (tid == 0) {
-      asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-      const int c0 = (it % nck) * kTcKC;
-      const int kc = min(kTcKC, Cip - c0);
-      const uint32_t a0 = smem_addr(smem + st * 2 * kTcStageBytes), b0 = a0 + kTcStageBytes;
-      for (int k = 0; k < kc / 16; k++) {
-        const uint64_t ad = umma_desc(a0 + k * 256, 128, 1024);
-        const uint64_t bd = umma_desc(b0 + k * 256, 128, 1024);
-        const uint32_t acc = (it > 0 || k > 0) ? 1u : 0u;
-        asm volatile(
-            "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-            " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-            "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
-            : "memory");
-      }
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
-                       smem_addr(&mbar[st]))
-                   : "memory");
-    }
-  }
-  cp_async_wait<0>();  // no copy left in flight, whatever happened above
-  // all MMAs done: the last commit covers every earlier MMA of the issuing thread
-  if (ok && iters > 0) {
-    const int last = iters - 1;
-    const bool got = mbar_wait(&mbar[last % S], (last / S) & 1, kTcWaitLimit);
-    if (__syncthreads_or(!got)) {
-      ok = false;
-      if (tid == 0) atomicExch(err, 1);
-    }
-  }
-  asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-  if (ok) {
-    __syncwarp();
-    __nv_bfloat16 *yp = y + (p < npix ? p : 0) * ys;
-    for (int c = 0; c < NT; c += 8) {
-      uint32_t r[8];
-      asm volatile(
-          "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n"
-          : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-            "=r"(r[7])
-          : "r"(tmem + (static_cast<uint32_t>(warp * 32) << 16) + c));
-      asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-      if (p < npix) {
-#pragma unroll
-        for (int e = 0; e < 8; e++) {
-          const int o = o0 + c + e;
-          if (o < Co) {
-            float v = __uint_as_float(r[e]) + (b ? b[o] : 0.f);
-            if (relu) v = fmaxf(v, 0.f);
-            yp[o] = __float2bfloat16_rn(v);
-          }
-        }
-      }
-    }
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-  __syncthreads();
-  if (warp == 0) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem),
-                 "r"(kTcNMax)
-                 : "memory");
-  }
-}
-
-// Weight gradient on the tensor cores:
-//   dW[d][c][o] = sum_p X[p + d - HALO][c] gz[p][o]     db[o] = sum_p gz[p][o]
-// as D[m][n] = sum_k A[m][k] B[n][k] with m = d * Ci + c (M = 128 per CTA),
-// n = o (N = NT), k = pixel (K, split over blockIdx.z: kper pixels each).
-// Chunks of 32 pixels are staged K-major: thread t gathers row t of A (tap
-// and channel of m, 32 consecutive pixels shifted by the tap) and row t of
-// B (channel o0 + t of gz); 8 pixels of one row are one 16-byte core-matrix
-// row.  The partial D of the CTA is added into dW with atomics.
-constexpr int kWgKC = 32;                             // pixels per K chunk
-constexpr int kWgStage = kTcM * kWgKC * 2;            // one operand, one stage: 8 KB
-constexpr int kWgSmem = 4 * kWgStage + 1024;
-
-template <int KS>
-__global__ void __launch_bounds__(kTcM)
-conv_wgrad_tc(const __nv_bfloat16 *__restrict__ x, int xs, const __nv_bfloat16 *__restrict__ gz,
-              int gs, int N, int H, int W, int Ci, int Co, int NT, int kper,
-              float *__restrict__ dw, float *__restrict__ db, int *__restrict__ err) {
-  constexpr int HALO = KS / 2;
-  constexpr int KS2 = KS * KS;
-  extern __shared__ unsigned char tc_smem_raw[];
-  unsigned char *smem = reinterpret_cast<unsigned char *>(
-      (reinterpret_cast<uintptr_t>(tc_smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  __shared__ uint64_t mbar[2];
-  __shared__ uint32_t tmem_slot;
-  const int tid = threadIdx.x, warp = tid >> 5;
-  const int64_t npix = static_cast<int64_t>(N) * H * W;
-  const int m0 = blockIdx.x * kTcM, o0 = blockIdx.y * NT;
-  const int64_t pstart = static_cast<int64_t>(blockIdx.z) * kper;
-  const int64_t pend = min(npix, pstart + kper);
-  const int nch = pend > pstart ? static_cast<int>((pend - pstart + kWgKC - 1) / kWgKC) : 0;
-  // this thread's A row: tap d and channel c of m = m0 + tid
-  const int m = m0 + tid;
-  const bool mrow = m < KS2 * Ci;
-  const int d = mrow ? m / Ci : 0, c = mrow ? m - (m / Ci) * Ci : 0;
-  const int sy = d / KS - HALO, sx = d % KS - HALO;
-  const bool nrow = tid < NT && o0 + tid < Co;
-  float bsum = 0.f;
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
-                     smem_addr(&tmem_slot)),
-                 "r"(kTcNMax)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
-  }
-  if (tid == 0) {
-    mbar_init(&mbar[0], 1);
-    mbar_init(&mbar[1], 1);
-    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-  const uint32_t tmem = tmem_slot;
-  const uint32_t idesc = umma_idesc_bf16(kTcM, NT);
-  uint32_t phase[2] = {0u, 0u};
-  bool ok = true;
-  for (int it = 0; it < nch; it++) {
-    const int st = it & 1;
-    if (it >= 2) {
-      const bool got = mbar_wait(&mbar[st], phase[st], kTcWaitLimit);
-      if (__syncthreads_or(!got)) {
-        ok = false;
-        if (tid == 0) atomicExch(err, 1);
-        break;
-      }
-      phase[st] ^= 1u;
-    }
-    const int64_t p0 = pstart + static_cast<int64_t>(it) * kWgKC;
-    unsigned char *sa = smem + st * 2 * kWgStage;
-    unsigned char *sb = sa + kWgStage;
-    // pixel p0 as (image, row, column); advanced one pixel at a time
-    int pn = static_cast<int>(p0 / (static_cast<int64_t>(H) * W));
-    int rem = static_cast<int>(p0 - static_cast<int64_t>(pn) * H * W);
-    int pi = rem / W, pj = rem - (rem / W) * W;
-    for (int k8 = 0; k8 < kWgKC / 8; k8++) {
-      __align__(16) __nv_bfloat16 va[8], vb[8];
-#pragma unroll
-      for (int e = 0; e < 8; e++) {
-        const int64_t p = p0 + k8 * 8 + e;
-        float a = 0.f, bb = 0.f;
-        if (p < pend) {
-          const int ii = pi + sy, jj = pj + sx;
-          if (mrow && ii >= 0 && ii < H && jj >= 0 && jj < W)
-            a = __bfloat162float(x[((static_cast<int64_t>(pn) * H + ii) * W + jj) * xs + c]);
-          if (nrow) {
-            bb = __bfloat162float(gz[p * gs + o0 + tid]);
-            bsum += bb;
-          }
-        }
-        va[e] = __float2bfloat16_rn(a);
-        vb[e] = __float2bfloat16_rn(bb);
-        if (++pj == W) {
-          pj = 0;
-          if (++pi == H) {
-            pi = 0;
-            ++pn;
-          }
-        }
-      }
-      *reinterpret_cast<uint4 *>(sa + (tid >> 3) * 512 + k8 * 128 + (tid & 7) * 16) =
-          *reinterpret_cast<const uint4 *>(va);
-      if (tid < NT)
-        *reinterpret_cast<uint4 *>(sb + (tid >> 3) * 512 + k8 * 128 + (tid & 7) * 16) =
-            *reinterpret_cast<const uint4 *>(vb);
-    }
-    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-    __syncthreads();
-    if (tid == 0) {
-      asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-      const uint32_t a0 = smem_addr(sa), b0 = smem_addr(sb);
-      for (int k = 0; k < kWgKC / 16; k++) {
-        const uint64_t ad = umma_desc(a0 + k * 256, 128, 512);
-        const uint64_t bd = umma_desc(b0 + k * 256, 128, 512);
-        const uint32_t acc = (it > 0 || k > 0) ? 1u : 0u;
-        asm volatile(
-            "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-            " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-            "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
-            : "memory");
-      }
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
-                       smem_addr(&mbar[st]))
-                   : "memory");
-    }
-  }
-  if (ok && nch > 0) {
-    const int st = (nch - 1) & 1;
-    const bool got = mbar_wait(&mbar[st], phase[st], kTcWaitLimit);
-    if (__syncthreads_or(!got)) {
-      ok = false;
-      if (tid == 0) atomicExch(err, 1);
-    }
-  }
-  asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-  if (ok && nch > 0) {  // uniform: every lane takes part in the warp-collective loads
-    __syncwarp();
-    const int mr = m0 + warp * 32 + (tid & 31);  // the TMEM lane this thread reads = row of D
-    for (int cc = 0; cc < NT; cc += 8) {
-      uint32_t r[8];
-      asm volatile(
-          "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n"
-          : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-            "=r"(r[7])
-          : "r"(tmem + (static_cast<uint32_t>(warp * 32) << 16) + cc));
-      asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-      if (mr < KS2 * Ci) {
-#pragma unroll
-        for (int e = 0; e < 8; e++) {
-          const int o = o0 + cc + e;
-          if (o < Co) atomicAdd(&dw[static_cast<int64_t>(mr) * Co + o], __uint_as_float(r[e]));
-        }
-      }
-    }
-  }
-  if (ok && db && blockIdx.x == 0 && nrow) atomicAdd(&db[o0 + tid], bsum);
-  asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-  __syncthreads();
-  if (warp == 0) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem),
-                 "r"(kTcNMax)
-                 : "memory");
   }
 }
 
@@ -908,6 +318,157 @@ __global__ void mse_kernel(const A *__restrict__ y, const float *__restrict__ t,
   if ((threadIdx.x & 31) == 0) atomicAdd(loss, s);
 }
 
+// --- BF16 mode: 8 channels (16 bytes) per thread, channel strides padded to
+// 8 (lbm_net_tc.h), the padding zero; n8 = channel groups per pixel.  These
+// passes run at memory speed; each does in one read and one write what a
+// chain of elementwise passes would.
+
+__device__ __forceinline__ void unpack8(uint4 v, float (&f)[8]) {
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+  for (int e = 0; e < 4; e++) {
+    f[2 * e] = __uint_as_float(w[e] << 16);
+    f[2 * e + 1] = __uint_as_float(w[e] & 0xFFFF0000u);
+  }
+}
+__device__ __forceinline__ uint4 pack8(const float (&f)[8]) {
+  uint32_t w[4];
+#pragma unroll
+  for (int e = 0; e < 4; e++) {
+    const __nv_bfloat162 b = __floats2bfloat162_rn(f[2 * e], f[2 * e + 1]);
+    w[e] = *reinterpret_cast<const uint32_t *>(&b);
+  }
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+__device__ __forceinline__ const uint4 *as8(const __nv_bfloat16 *p) {
+  return reinterpret_cast<const uint4 *>(p);
+}
+__device__ __forceinline__ uint4 *as8(__nv_bfloat16 *p) { return reinterpret_cast<uint4 *>(p); }
+// v where the ReLU output h is positive, else 0
+__device__ __forceinline__ uint4 relu_gate8(uint4 v, uint4 h) {
+  float f[8], g[8];
+  unpack8(v, f);
+  unpack8(h, g);
+#pragma unroll
+  for (int e = 0; e < 8; e++)
+    if (!(g[e] > 0.f)) f[e] = 0.f;
+  return pack8(f);
+}
+
+// d[pixel][8 n8] = s[pixel][c], zero beyond c
+__global__ void __launch_bounds__(256) to_storage8(const float *__restrict__ s, int c,
+                                                   __nv_bfloat16 *__restrict__ d, int n8,
+                                                   int64_t npix) {
+  const int64_t t = blockIdx.x * 256ll + threadIdx.x;
+  if (t >= npix * n8) return;
+  const int64_t p = t / n8;
+  const int c0 = static_cast<int>(t - p * n8) * 8;
+  float f[8];
+#pragma unroll
+  for (int e = 0; e < 8; e++) f[e] = c0 + e < c ? s[p * c + c0 + e] : 0.f;
+  as8(d)[t] = pack8(f);
+}
+
+// 2x2 average pooling; H, W: output size
+__global__ void __launch_bounds__(256) pool2_fwd8(const __nv_bfloat16 *__restrict__ x,
+                                                  __nv_bfloat16 *__restrict__ y, int n8, int H,
+                                                  int W, uint32_t n) {
+  const uint32_t t = blockIdx.x * 256u + threadIdx.x;
+  if (t >= n) return;
+  const uint32_t c = t % n8, p = t / n8, j = p % W, r = p / W;  // r = image * H + row
+  const uint4 *src = as8(x) + (static_cast<int64_t>(2 * r) * 2 * W + 2 * j) * n8 + c;
+  const int64_t row = static_cast<int64_t>(2 * W) * n8;
+  const uint4 v[4] = {src[0], src[n8], src[row], src[row + n8]};
+  float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+  for (int k = 0; k < 4; k++) {
+    float f[8];
+    unpack8(v[k], f);
+#pragma unroll
+    for (int e = 0; e < 8; e++) s[e] += f[e];
+  }
+#pragma unroll
+  for (int e = 0; e < 8; e++) s[e] *= 0.25f;
+  as8(y)[t] = pack8(s);
+}
+
+// Backward of the 2x upsampling and of the ReLU below it: gx = sum of gy's
+// first 8 n8 channels (stride 8 g8) over each 2x2 block, 0 where h <= 0;
+// H, W: size of gx
+__global__ void __launch_bounds__(256) up2_bwd8(const __nv_bfloat16 *__restrict__ gy, int g8,
+                                                const __nv_bfloat16 *__restrict__ h,
+                                                __nv_bfloat16 *__restrict__ gx, int n8, int H,
+                                                int W, uint32_t n) {
+  const uint32_t t = blockIdx.x * 256u + threadIdx.x;
+  if (t >= n) return;
+  const uint32_t c = t % n8, p = t / n8, j = p % W, r = p / W;
+  const uint4 *src = as8(gy) + (static_cast<int64_t>(2 * r) * 2 * W + 2 * j) * g8 + c;
+  const int64_t row = static_cast<int64_t>(2 * W) * g8;
+  const uint4 v[4] = {src[0], src[g8], src[row], src[row + g8]};
+  float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+  for (int k = 0; k < 4; k++) {
+    float f[8];
+    unpack8(v[k], f);
+#pragma unroll
+    for (int e = 0; e < 8; e++) s[e] += f[e];
+  }
+  as8(gx)[t] = relu_gate8(pack8(s), as8(h)[t]);
+}
+
+// Gradient of an encoder level's output: the skip connection's (channels
+// from group g0 of gskip, stride 8 g8) plus the pooled path's (gpool / 4
+// over each 2x2 block), 0 where h <= 0; H, W: size of the level
+__global__ void __launch_bounds__(256) pool2_bwd8(const __nv_bfloat16 *__restrict__ gpool,
+                                                  const __nv_bfloat16 *__restrict__ gskip, int g8,
+                                                  int g0, const __nv_bfloat16 *__restrict__ h,
+                                                  __nv_bfloat16 *__restrict__ gx, int n8, int H,
+                                                  int W, uint32_t n) {
+  const uint32_t t = blockIdx.x * 256u + threadIdx.x;
+  if (t >= n) return;
+  const uint32_t c = t % n8, p = t / n8, j = p % W, r = p / W;
+  const uint4 a = as8(gpool)[(static_cast<int64_t>(r / 2) * (W / 2) + j / 2) * n8 + c];
+  const uint4 b = as8(gskip)[static_cast<int64_t>(p) * g8 + g0 + c];
+  float f[8], g[8];
+  unpack8(a, f);
+  unpack8(b, g);
+#pragma unroll
+  for (int e = 0; e < 8; e++) f[e] = fmaf(0.25f, f[e], g[e]);
+  as8(gx)[t] = relu_gate8(pack8(f), as8(h)[t]);
+}
+
+// Squared error and its gradient gy = 2 (y - t) / n, per pixel; y, gy with
+// 8 n8 channels stored, c real ones.  One atomic per CTA.
+__global__ void __launch_bounds__(256) mse8(const __nv_bfloat16 *__restrict__ y,
+                                            const float *__restrict__ t,
+                                            __nv_bfloat16 *__restrict__ gy, int c, int n8,
+                                            int64_t npix, double *__restrict__ loss) {
+  double s = 0.0;
+  const float n = static_cast<float>(npix * c);
+  for (int64_t q = blockIdx.x * 256ll + threadIdx.x; q < npix * n8;
+       q += static_cast<int64_t>(gridDim.x) * 256) {
+    const int64_t p = q / n8;
+    const int c0 = static_cast<int>(q - p * n8) * 8;
+    float f[8];
+    unpack8(as8(y)[q], f);
+#pragma unroll
+    for (int e = 0; e < 8; e++) {
+      const float d = c0 + e < c ? f[e] - t[p * c + c0 + e] : 0.f;
+      s += static_cast<double>(d) * d;
+      f[e] = 2.f * d / n;
+    }
+    as8(gy)[q] = pack8(f);
+  }
+  __shared__ double sh[8];
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; w++) s += sh[w];
+    atomicAdd(loss, s);
+  }
+}
+
 __global__ void adam_kernel(float *__restrict__ p, const float *__restrict__ g, float *__restrict__ m,
                             float *__restrict__ v, int64_t n, float lr, float b1, float b2, float eps,
                             float c1, float c2) {
@@ -953,15 +514,28 @@ struct lbm_net {
   std::vector<Layer> layers;
   int64_t n_params = 0;
   float *params = nullptr, *grads = nullptr, *m = nullptr, *v = nullptr;
-  void *wq = nullptr;   // weights in the storage type
-  void *wt = nullptr;   // flipped weights (largest layer), storage type
-  void *wk = nullptr;   // packed K-major BF16 weights of the tensor-core path (largest layer)
-  int *d_err = nullptr; // set by a tensor-core kernel whose bounded wait ran out
+  float *wt = nullptr;  // FP32 mode: flipped weights (largest layer)
+  // BF16 mode: every layer's packed weights and their adjoint's, packed from
+  // the FP32 parameters when these have changed (stale); the jobs that pack
+  // them (device); the weight gradient's scratch
+  __nv_bfloat16 *wk = nullptr;
+  std::vector<int64_t> wk_off[2];
+  lbm::net::PackJob *jobs = nullptr;
+  int n_jobs = 0;
+  int64_t max_job = 0;
+  bool stale = true;
+  float *partials = nullptr;
+  int sms = 1;
+  // what a call reads back: the loss (a sum), and a flag that a tensor-core
+  // kernel sets when one of its bounded waits runs out; device and pinned host
+  struct Status {
+    double loss;
+    int err, pad;
+  } *status = nullptr, *h_status = nullptr;
   // activations: per level encoder outputs (skip), decoder concat inputs,
   // temporaries; all storage type, sized for max_batch
   std::vector<void *> bufs;
   std::vector<int64_t> buf_elems;
-  double *loss = nullptr;
   int64_t adam_t = 0;
   std::string err;
 };
@@ -974,7 +548,8 @@ size_t asize(int precision) { return precision == LBM_FP32 ? 4 : 2; }
 //   x_in                       input, c_in channels
 //   e[l]a_out, e[l]b_out       encoder outputs per level (b is the skip)
 //   pool[l]                    pooled input of level l (l >= 1)
-//   cat[l]                     decoder input of level l: [up, skip]
+//   cat[l]                     decoder input of level l: [up, skip] (BF16 mode
+//                              stores only its gradient)
 //   d[l]a_out, d[l]b_out
 //   y                          head output
 // Gradients use a second set of the same shapes.
@@ -990,12 +565,14 @@ Plan make_plan(const lbm_net_t *n) {
     p.elems.push_back(e);
     return static_cast<int>(p.elems.size()) - 1;
   };
+  // channels as stored (BF16 mode pads each source to a multiple of 8)
+  auto st = [&](int c) { return n->precision == LBM_FP32 ? c : lbm::net::pad8(c); };
   const int64_t HW = static_cast<int64_t>(n->H) * n->W;
-  p.x_in = add(HW * n->c_in);
+  p.x_in = add(HW * st(n->c_in));
   for (int l = 0; l < n->levels; l++) {
     const int64_t hw = HW >> (2 * l);
-    const int ch = n->base << l;
-    p.pool.push_back(l > 0 ? add(hw * (n->base << (l - 1))) : -1);
+    const int ch = st(n->base << l);
+    p.pool.push_back(l > 0 ? add(hw * st(n->base << (l - 1))) : -1);
     p.ea.push_back(add(hw * ch));
     p.eb.push_back(add(hw * ch));
   }
@@ -1004,18 +581,13 @@ Plan make_plan(const lbm_net_t *n) {
   p.db.assign(n->levels, -1);
   for (int l = n->levels - 2; l >= 0; l--) {
     const int64_t hw = HW >> (2 * l);
-    const int ch = n->base << l;
-    p.cat[l] = add(hw * (ch * 2 + ch));
+    const int ch = st(n->base << l);
+    p.cat[l] = add(hw * (st(n->base << (l + 1)) + ch));
     p.da[l] = add(hw * ch);
     p.db[l] = add(hw * ch);
   }
-  p.y = add(HW * n->c_out);
+  p.y = add(HW * st(n->c_out));
   return p;
-}
-
-bool tc_timed_out(lbm_net_t *n) {
-  int v = 0;
-  return cudaMemcpy(&v, n->d_err, sizeof(int), cudaMemcpyDeviceToHost) == cudaSuccess && v != 0;
 }
 
 int nfail(lbm_net_t *n, int code, const std::string &m) {
@@ -1024,108 +596,45 @@ int nfail(lbm_net_t *n, int code, const std::string &m) {
   return code;
 }
 
-// Output-channel tile of the tensor-core convolution and the padded sizes
-// of its packed weights.
-void tc_shape(int Ci, int Co, int *NT, int *Cop, int *Cip) {
-  *NT = std::min(lbm::net::kTcNMax, (Co + 15) / 16 * 16);
-  *Cop = (Co + *NT - 1) / *NT * *NT;
-  *Cip = (Ci + 15) / 16 * 16;
+// FP32 mode: y = act(conv(x, w) + b) with Ci inputs and Co outputs (weights
+// [tap][ci][co]).
+void launch_conv(lbm_net_t *n, const float *x, int xs, const float *w, const float *b, float *y,
+                 int ys, int N, int H, int W, int Ci, int Co, int ks, int relu) {
+  using namespace lbm::net;
+  dim3 grid(((W + TP - 1) / TP) * ((H + TP - 1) / TP), (Co + TC - 1) / TC, N);
+  if (ks == 3)
+    conv_fwd<float, 3><<<grid, TP * TP, 0, n->stream>>>(x, xs, w, b, y, ys, H, W, Ci, Co, relu);
+  else
+    conv_fwd<float, 1><<<grid, TP * TP, 0, n->stream>>>(x, xs, w, b, y, ys, H, W, Ci, Co, relu);
 }
 
-// y = act(conv(x, w) + b) with Ci inputs and Co outputs.  FP32 storage: the
-// CUDA-core kernel on w (layout [tap][ci][co]).  BF16 storage: the tensor-core
-// kernel on weights packed from the FP32 parameters wsrc of layer (lci, lco),
-// flipped for the adjoint convolution of the backward pass.
-template <typename A>
-void launch_conv(lbm_net_t *n, const A *x, int xs, const A *w, const float *b, A *y, int ys,
-                 int N, int H, int W, int Ci, int Co, int ks, int relu, const float *wsrc, int flip,
-                 int lci, int lco) {
+void launch_wgrad(const lbm_net_t *n, const float *x, int xs, const float *gz, int N, int H, int W,
+                  int Ci, int Co, int ks, float *dw, float *db) {
   using namespace lbm::net;
-  if constexpr (std::is_same<A, __nv_bfloat16>::value) {
-    (void)w;
-    int NT, Cop, Cip;
-    tc_shape(Ci, Co, &NT, &Cop, &Cip);
-    __nv_bfloat16 *wk = static_cast<__nv_bfloat16 *>(n->wk);
-    pack_wk<<<grid1(static_cast<int64_t>(Cop) * ks * ks * Cip), 256, 0, n->stream>>>(
-        wsrc, wk, ks * ks, lci, lco, flip, Cop, Cip);
-    const int64_t npix = static_cast<int64_t>(N) * H * W;
-    dim3 grid(static_cast<unsigned>((npix + kTcM - 1) / kTcM), Cop / NT);
-    const bool vec = xs % 8 == 0 && Ci % 8 == 0 && reinterpret_cast<uintptr_t>(x) % 16 == 0;
-    if (vec && ks == 3)
-      conv_fwd_tc_async<3><<<grid, kTcM, kTcAsyncSmem, n->stream>>>(
-          x, xs, wk, Cip, b, y, ys, N, H, W, Ci, Co, NT, relu, n->d_err);
-    else if (vec)
-      conv_fwd_tc_async<1><<<grid, kTcM, kTcAsyncSmem, n->stream>>>(
-          x, xs, wk, Cip, b, y, ys, N, H, W, Ci, Co, NT, relu, n->d_err);
-    else if (ks == 3)
-      conv_fwd_tc<3><<<grid, kTcM, kTcSmem, n->stream>>>(x, xs, wk, Cip, b, y, ys, N, H, W, Ci, Co,
-                                                         NT, relu, vec, n->d_err);
-    else
-      conv_fwd_tc<1><<<grid, kTcM, kTcSmem, n->stream>>>(x, xs, wk, Cip, b, y, ys, N, H, W, Ci, Co,
-                                                         NT, relu, vec, n->d_err);
-  } else {
-    (void)wsrc;
-    (void)flip;
-    (void)lci;
-    (void)lco;
-    dim3 grid(((W + TP - 1) / TP) * ((H + TP - 1) / TP), (Co + TC - 1) / TC, N);
-    if (ks == 3)
-      conv_fwd<A, 3><<<grid, TP * TP, 0, n->stream>>>(x, xs, w, b, y, ys, H, W, Ci, Co, relu);
-    else
-      conv_fwd<A, 1><<<grid, TP * TP, 0, n->stream>>>(x, xs, w, b, y, ys, H, W, Ci, Co, relu);
-  }
-}
-
-template <typename A>
-void launch_wgrad(const lbm_net_t *n, const A *x, int xs, const A *gz, int N, int H, int W, int Ci,
-                  int Co, int ks, float *dw, float *db) {
-  using namespace lbm::net;
-  if constexpr (std::is_same<A, __nv_bfloat16>::value) {
-    // tensor cores: M tiles over (tap, channel), N tiles over output
-    // channels, the pixels split so that the grid fills the GPU a few times
-    const int64_t npix = static_cast<int64_t>(N) * H * W;
-    const int NT = std::min(kTcNMax, (Co + 15) / 16 * 16);
-    const int mt = (ks * ks * Ci + kTcM - 1) / kTcM, nt = (Co + NT - 1) / NT;
-    const int64_t want = std::max<int64_t>(1, 1824 / (mt * nt));
-    int64_t kper = (npix + want - 1) / want;
-    kper = std::max<int64_t>(kWgKC * 4, (kper + kWgKC - 1) / kWgKC * kWgKC);
-    const unsigned ks_split = static_cast<unsigned>((npix + kper - 1) / kper);
-    dim3 grid(mt, nt, ks_split);
-    if (ks == 3)
-      conv_wgrad_tc<3><<<grid, kTcM, kWgSmem, n->stream>>>(x, xs, gz, Co, N, H, W, Ci, Co, NT,
-                                                           static_cast<int>(kper), dw, db, n->d_err);
-    else
-      conv_wgrad_tc<1><<<grid, kTcM, kWgSmem, n->stream>>>(x, xs, gz, Co, N, H, W, Ci, Co, NT,
-                                                           static_cast<int>(kper), dw, db, n->d_err);
-    return;
-  }
   const int64_t npix = static_cast<int64_t>(N) * H * W;
   const int chunks = static_cast<int>(std::min<int64_t>(1024, (npix + 255) / 256));
   const int per = static_cast<int>((npix + chunks - 1) / chunks);
   dim3 grid(((Ci + TC - 1) / TC) * ((Co + TC - 1) / TC), chunks);
   if (ks == 3)
-    conv_bwd_weight<A, 3><<<grid, 256, 0, n->stream>>>(x, xs, gz, N, H, W, Ci, Co, per, dw, db);
+    conv_bwd_weight<float, 3><<<grid, 256, 0, n->stream>>>(x, xs, gz, N, H, W, Ci, Co, per, dw, db);
   else
-    conv_bwd_weight<A, 1><<<grid, 256, 0, n->stream>>>(x, xs, gz, N, H, W, Ci, Co, per, dw, db);
+    conv_bwd_weight<float, 1><<<grid, 256, 0, n->stream>>>(x, xs, gz, N, H, W, Ci, Co, per, dw, db);
 }
 
-// forward (and, if t != nullptr, loss + backward into n->grads)
-template <typename A>
-cudaError_t run(lbm_net_t *n, const float *x_in, int N, const float *t, float *y_out, double *loss) {
+// FP32 mode: forward (and, if t != nullptr, loss + backward into n->grads)
+cudaError_t run_fp32(lbm_net_t *n, const float *x_in, int N, const float *t, float *y_out) {
   using namespace lbm::net;
+  using A = float;
   Plan p = make_plan(n);
   const int L = n->levels;
-  A *wq = static_cast<A *>(n->wq);
   auto buf = [&](int i) { return static_cast<A *>(n->bufs[i]); };
   auto gbuf = [&](int i) { return static_cast<A *>(n->bufs[p.elems.size() + i]); };
   const int64_t HW = static_cast<int64_t>(n->H) * n->W;
   cudaStream_t s = n->stream;
   to_storage<A><<<grid1(HW * N * n->c_in), 256, 0, s>>>(x_in, buf(p.x_in), HW * N * n->c_in);
-  to_storage<A><<<grid1(n->n_params), 256, 0, s>>>(n->params, wq, n->n_params);
   int li = 0;
-  auto W_of = [&](int k) { return wq + n->layers[k].w_off; };
+  auto W_of = [&](int k) { return n->params + n->layers[k].w_off; };
   auto B_of = [&](int k) { return n->params + n->layers[k].b_off; };
-  auto P_of = [&](int k) { return n->params + n->layers[k].w_off; };
   // encoder
   const A *h = buf(p.x_in);
   int hc = n->c_in;
@@ -1136,11 +645,9 @@ cudaError_t run(lbm_net_t *n, const float *x_in, int N, const float *t, float *y
                                                                                   H * 2, Wd * 2, hc);
       h = buf(p.pool[l]);
     }
-    launch_conv<A>(n, h, hc, W_of(li), B_of(li), buf(p.ea[l]), ch, N, H, Wd, hc, ch, 3, 1, P_of(li),
-                   0, hc, ch);
+    launch_conv(n, h, hc, W_of(li), B_of(li), buf(p.ea[l]), ch, N, H, Wd, hc, ch, 3, 1);
     li++;
-    launch_conv<A>(n, buf(p.ea[l]), ch, W_of(li), B_of(li), buf(p.eb[l]), ch, N, H, Wd, ch, ch, 3, 1,
-                   P_of(li), 0, ch, ch);
+    launch_conv(n, buf(p.ea[l]), ch, W_of(li), B_of(li), buf(p.eb[l]), ch, N, H, Wd, ch, ch, 3, 1);
     li++;
     h = buf(p.eb[l]);
     hc = ch;
@@ -1153,38 +660,33 @@ cudaError_t run(lbm_net_t *n, const float *x_in, int N, const float *t, float *y
     up2_fwd<A><<<grid1(static_cast<int64_t>(N) * H * Wd * cu), 256, 0, s>>>(h, cat, ct, N, H, Wd, cu);
     copy_channels<A><<<grid1(static_cast<int64_t>(N) * H * Wd * ch), 256, 0, s>>>(
         buf(p.eb[l]), ch, cat + cu, ct, ch, static_cast<int64_t>(N) * H * Wd, 0);
-    launch_conv<A>(n, cat, ct, W_of(li), B_of(li), buf(p.da[l]), ch, N, H, Wd, ct, ch, 3, 1, P_of(li),
-                   0, ct, ch);
+    launch_conv(n, cat, ct, W_of(li), B_of(li), buf(p.da[l]), ch, N, H, Wd, ct, ch, 3, 1);
     li++;
-    launch_conv<A>(n, buf(p.da[l]), ch, W_of(li), B_of(li), buf(p.db[l]), ch, N, H, Wd, ch, ch, 3, 1,
-                   P_of(li), 0, ch, ch);
+    launch_conv(n, buf(p.da[l]), ch, W_of(li), B_of(li), buf(p.db[l]), ch, N, H, Wd, ch, ch, 3, 1);
     li++;
     h = buf(p.db[l]);
     hc = ch;
   }
   const int head = li;
-  launch_conv<A>(n, h, hc, W_of(head), B_of(head), buf(p.y), n->c_out, N, n->H, n->W, hc, n->c_out, 1,
-                 0, P_of(head), 0, hc, n->c_out);
+  launch_conv(n, h, hc, W_of(head), B_of(head), buf(p.y), n->c_out, N, n->H, n->W, hc, n->c_out, 1,
+                 0);
   if (y_out)
     to_float<A><<<grid1(HW * N * n->c_out), 256, 0, s>>>(buf(p.y), n->c_out, y_out, n->c_out, HW * N);
   if (!t) return cudaGetLastError();
 
   // loss and backward
-  cudaMemsetAsync(n->loss, 0, sizeof(double), s);
   mse_kernel<A><<<grid1(HW * N * n->c_out), 256, 0, s>>>(buf(p.y), t, gbuf(p.y), HW * N * n->c_out,
-                                                        n->loss);
+                                                        &n->status->loss);
   cudaMemsetAsync(n->grads, 0, n->n_params * sizeof(float), s);
-  A *wt = static_cast<A *>(n->wt);
+  A *wt = n->wt;
   auto conv_back = [&](int k, const A *x, int xs, A *gz, A *gx, int gxs, int H, int Wd, bool need_gx) {
     const Layer &ly = n->layers[k];
-    launch_wgrad<A>(n, x, xs, gz, N, H, Wd, ly.ci, ly.co, ly.ks, n->grads + ly.w_off,
+    launch_wgrad(n, x, xs, gz, N, H, Wd, ly.ci, ly.co, ly.ks, n->grads + ly.w_off,
                     n->grads + ly.b_off);
     if (need_gx) {
-      if constexpr (!std::is_same<A, __nv_bfloat16>::value)
-        flip_weights<A><<<grid1(static_cast<int64_t>(ly.ks * ly.ks) * ly.ci * ly.co), 256, 0, s>>>(
-            n->params + ly.w_off, wt, ly.ks * ly.ks, ly.ci, ly.co);
-      launch_conv<A>(n, gz, ly.co, wt, nullptr, gx, gxs, N, H, Wd, ly.co, ly.ci, ly.ks, 0,
-                     n->params + ly.w_off, 1, ly.ci, ly.co);
+      flip_weights<A><<<grid1(static_cast<int64_t>(ly.ks * ly.ks) * ly.ci * ly.co), 256, 0, s>>>(
+          n->params + ly.w_off, wt, ly.ks * ly.ks, ly.ci, ly.co);
+      launch_conv(n, gz, ly.co, wt, nullptr, gx, gxs, N, H, Wd, ly.co, ly.ci, ly.ks, 0);
     }
   };
   // head
@@ -1233,12 +735,163 @@ cudaError_t run(lbm_net_t *n, const float *x_in, int N, const float *t, float *y
       pool2_bwd<A><<<grid1(static_cast<int64_t>(N) * H * 2 * Wd * 2 * cin), 256, 0, s>>>(
           gbuf(p.pool[l]), gbuf(p.eb[l - 1]), cin, N, H * 2, Wd * 2, cin, 1);
   }
-  if (loss) {
-    cudaMemcpyAsync(loss, n->loss, sizeof(double), cudaMemcpyDeviceToHost, s);
-    cudaStreamSynchronize(s);
-    *loss /= static_cast<double>(HW * N * n->c_out);
-  }
   return cudaGetLastError();
+}
+
+// BF16 mode: the same on the tensor cores (lbm_net_tc.cu).  Activations have
+// padded channel strides; the decoder's concatenated input is read from its
+// two sources, and every stored gradient is already masked by its ReLU.
+cudaError_t run_bf16(lbm_net_t *n, const float *x_in, int N, const float *t, float *y_out) {
+  using namespace lbm::net;
+  using B16 = __nv_bfloat16;
+  const Plan p = make_plan(n);
+  const int L = n->levels;
+  const int64_t HW = static_cast<int64_t>(n->H) * n->W;
+  cudaStream_t s = n->stream;
+  cudaError_t e = cudaSuccess;
+  auto buf = [&](int i) { return static_cast<B16 *>(n->bufs[i]); };
+  auto gbuf = [&](int i) { return static_cast<B16 *>(n->bufs[p.elems.size() + i]); };
+  auto blocks = [](int64_t k) { return static_cast<unsigned>((k + 255) / 256); };
+  if (n->stale) {
+    e = launch_pack(n->jobs, n->n_jobs, n->max_job, s);
+    if (e != cudaSuccess) return e;
+    n->stale = false;
+  }
+  auto conv = [&](int k, ConvInput in, int H, int W, int relu, B16 *y, float *yf) {
+    if (e != cudaSuccess) return;
+    const Layer &ly = n->layers[k];
+    ConvCall c;
+    c.in = in;
+    c.ks = ly.ks;
+    c.N = N;
+    c.H = H;
+    c.W = W;
+    c.co = ly.co;
+    c.wk = n->wk + n->wk_off[0][k];
+    c.bias = n->params + ly.b_off;
+    c.relu = relu;
+    c.y = y;
+    c.yf = yf;
+    e = launch_conv_tc(c, n->sms, &n->status->err, s);
+  };
+  auto single = [](const B16 *x, int c) {
+    ConvInput in;
+    in.xa = x;
+    in.ca = c;
+    return in;
+  };
+  const int n8x = pad8(n->c_in) / 8;
+  to_storage8<<<blocks(HW * N * n8x), 256, 0, s>>>(x_in, n->c_in, buf(p.x_in), n8x, HW * N);
+  // encoder
+  for (int l = 0; l < L; l++) {
+    const int H = n->H >> l, W = n->W >> l, ch = n->base << l;
+    ConvInput in = single(buf(p.x_in), n->c_in);
+    if (l > 0) {
+      const int cb = n->base << (l - 1), n8 = pad8(cb) / 8;
+      const int64_t k = static_cast<int64_t>(N) * H * W * n8;
+      pool2_fwd8<<<blocks(k), 256, 0, s>>>(buf(p.eb[l - 1]), buf(p.pool[l]), n8, H, W,
+                                           static_cast<uint32_t>(k));
+      in = single(buf(p.pool[l]), cb);
+    }
+    conv(2 * l, in, H, W, 1, buf(p.ea[l]), nullptr);
+    conv(2 * l + 1, single(buf(p.ea[l]), ch), H, W, 1, buf(p.eb[l]), nullptr);
+  }
+  // the decoder's input at level l: the level below upsampled, then the skip
+  auto below = [&](int l) { return l + 1 <= L - 2 ? p.db[l + 1] : p.eb[L - 1]; };
+  auto cat_in = [&](int l) {
+    ConvInput in = single(buf(below(l)), n->base << (l + 1));
+    in.up = 1;
+    in.xb = buf(p.eb[l]);
+    in.cb = n->base << l;
+    return in;
+  };
+  int li = 2 * L;
+  for (int l = L - 2; l >= 0; l--) {
+    const int H = n->H >> l, W = n->W >> l, ch = n->base << l;
+    conv(li++, cat_in(l), H, W, 1, buf(p.da[l]), nullptr);
+    conv(li++, single(buf(p.da[l]), ch), H, W, 1, buf(p.db[l]), nullptr);
+  }
+  const int head = li;
+  const int top = L > 1 ? p.db[0] : p.eb[0];
+  conv(head, single(buf(top), n->base), n->H, n->W, 0, buf(p.y), y_out);
+  if (e != cudaSuccess || !t) return e != cudaSuccess ? e : cudaGetLastError();
+
+  // loss and backward
+  const int n8y = pad8(n->c_out) / 8;
+  mse8<<<std::min<unsigned>(blocks(HW * N * n8y), 4u * n->sms), 256, 0, s>>>(
+      buf(p.y), t, gbuf(p.y), n->c_out, n8y, HW * N, &n->status->loss);
+  // gradients of layer k from its input and its (masked) output gradient gz;
+  // gx: the input's gradient, 0 where mask <= 0 (may be null)
+  auto back = [&](int k, const ConvInput &in, const B16 *gz, B16 *gx, const B16 *mask, int H,
+                  int W) {
+    if (e != cudaSuccess) return;
+    const Layer &ly = n->layers[k];
+    e = launch_wgrad_tc(in, ly.ks, gz, ly.co, N, H, W, n->partials, n->grads + ly.w_off, n->sms,
+                        &n->status->err, s);
+    if (e != cudaSuccess || !gx) return;
+    ConvCall c;
+    c.in = single(gz, ly.co);
+    c.ks = ly.ks;
+    c.N = N;
+    c.H = H;
+    c.W = W;
+    c.co = in.padded();
+    c.wk = n->wk + n->wk_off[1][k];
+    c.mask = mask;
+    c.y = gx;
+    e = launch_conv_tc(c, n->sms, &n->status->err, s);
+  };
+  back(head, single(buf(top), n->base), gbuf(p.y), gbuf(top), buf(top), n->H, n->W);
+  for (int l = 0; l <= L - 2; l++) {
+    const int H = n->H >> l, W = n->W >> l, ch = n->base << l;
+    const int kb = head - 1 - 2 * l, ka = kb - 1;
+    back(kb, single(buf(p.da[l]), ch), gbuf(p.db[l]), gbuf(p.da[l]), buf(p.da[l]), H, W);
+    const ConvInput in = cat_in(l);
+    back(ka, in, gbuf(p.da[l]), gbuf(p.cat[l]), nullptr, H, W);
+    const int n8 = pad8(in.ca) / 8;
+    const int64_t k = static_cast<int64_t>(N) * (H / 2) * (W / 2) * n8;
+    if (e == cudaSuccess)
+      up2_bwd8<<<blocks(k), 256, 0, s>>>(gbuf(p.cat[l]), in.padded() / 8, buf(below(l)),
+                                         gbuf(below(l)), n8, H / 2, W / 2,
+                                         static_cast<uint32_t>(k));
+  }
+  for (int l = L - 1; l >= 0; l--) {
+    const int H = n->H >> l, W = n->W >> l, ch = n->base << l;
+    if (l < L - 1) {  // the deepest level's gradient came from up2_bwd8
+      const ConvInput in = cat_in(l);
+      const int n8 = pad8(ch) / 8;
+      const int64_t k = static_cast<int64_t>(N) * H * W * n8;
+      if (e == cudaSuccess)
+        pool2_bwd8<<<blocks(k), 256, 0, s>>>(gbuf(p.pool[l + 1]), gbuf(p.cat[l]), in.padded() / 8,
+                                             pad8(in.ca) / 8, buf(p.eb[l]), gbuf(p.eb[l]), n8, H,
+                                             W, static_cast<uint32_t>(k));
+    }
+    back(2 * l + 1, single(buf(p.ea[l]), ch), gbuf(p.eb[l]), gbuf(p.ea[l]), buf(p.ea[l]), H, W);
+    if (l > 0)
+      back(2 * l, single(buf(p.pool[l]), n->base << (l - 1)), gbuf(p.ea[l]), gbuf(p.pool[l]),
+           nullptr, H, W);
+    else
+      back(0, single(buf(p.x_in), n->c_in), gbuf(p.ea[0]), nullptr, nullptr, H, W);
+  }
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+// One pass and its status (loss, bounded waits) read back; synchronises.
+int run(lbm_net_t *n, const float *x, int N, const float *t, float *y, double *loss) {
+  cudaError_t e = cudaMemsetAsync(n->status, 0, sizeof(*n->status), n->stream);
+  if (e == cudaSuccess)
+    e = n->precision == LBM_FP32 ? run_fp32(n, x, N, t, y) : run_bf16(n, x, N, t, y);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(n->h_status, n->status, sizeof(*n->status), cudaMemcpyDeviceToHost,
+                        n->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(n->stream);
+  if (e != cudaSuccess) return nfail(n, LBM_ECUDA, cudaGetErrorString(e));
+  if (n->h_status->err)
+    return nfail(n, LBM_ETIMEOUT, "a tensor-core convolution's bounded wait ran out");
+  if (loss)
+    *loss = n->h_status->loss /
+            static_cast<double>(static_cast<int64_t>(n->H) * n->W * N * n->c_out);
+  return LBM_OK;
 }
 
 }  // namespace
@@ -1295,44 +948,56 @@ int lbm_net_create(int32_t base, int32_t levels, int32_t c_in, int32_t c_out, in
   cudaError_t e = cudaSuccess;
   for (float **ptr : {&n->params, &n->grads, &n->m, &n->v})
     if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(ptr), off * sizeof(float));
-  if (e == cudaSuccess) e = cudaMalloc(&n->wq, off * as);
-  if (e == cudaSuccess) e = cudaMalloc(&n->wt, max_w * as);
-  {
-    int64_t max_wk = 1;
-    for (const Layer &ly : n->layers)
-      for (int fl = 0; fl < 2; fl++) {
-        int NT, Cop, Cip;
-        tc_shape(fl ? ly.co : ly.ci, fl ? ly.ci : ly.co, &NT, &Cop, &Cip);
-        max_wk = std::max<int64_t>(max_wk, static_cast<int64_t>(Cop) * ly.ks * ly.ks * Cip);
+  int dev = 0;
+  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n->sms, cudaDevAttrMultiProcessorCount, dev);
+  if (precision == LBM_FP32) {
+    if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&n->wt), max_w * sizeof(float));
+  } else {
+    // packed weights of every layer and of its adjoint (the first layer's
+    // adjoint is never needed), and the largest weight-gradient scratch
+    std::vector<lbm::net::PackJob> jobs;
+    int64_t wk = 0, scratch = 1;
+    for (size_t k = 0; k < n->layers.size(); k++) {
+      const Layer &ly = n->layers[k];
+      const int dec = static_cast<int>(k) - 2 * levels;  // >= 0: decoder layers, then the head
+      const bool cat = k + 1 < n->layers.size() && dec >= 0 && dec % 2 == 0;
+      const int cb = cat ? ly.co : 0, ca = ly.ci - cb;
+      const int padded = lbm::net::pad8(ca) + lbm::net::pad8(cb);
+      const int lev = dec < 0 ? static_cast<int>(k) / 2
+                              : std::max(0, levels - 2 - dec / 2);  // the head: level 0
+      scratch = std::max(scratch, lbm::net::wgrad_scratch(ly.ks, ly.ci, padded, ly.co, max_batch,
+                                                          H >> lev, W >> lev, n->sms));
+      for (int flip = 0; flip < 2; flip++) {
+        const int64_t el = flip ? lbm::net::packed_elems(ly.ks, lbm::net::pad8(ly.co), padded)
+                                : lbm::net::packed_elems(ly.ks, padded, ly.co);
+        n->wk_off[flip].push_back(wk);
+        if (flip && k == 0) continue;
+        jobs.push_back({n->params + ly.w_off, reinterpret_cast<__nv_bfloat16 *>(wk), ly.ks, ca, cb,
+                        ly.co, flip, el});
+        n->max_job = std::max(n->max_job, el);
+        wk += (el + 63) / 64 * 64;
       }
-    if (e == cudaSuccess) e = cudaMalloc(&n->wk, max_wk * 2);
+    }
+    n->n_jobs = static_cast<int>(jobs.size());
+    if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&n->wk), wk * 2);
+    if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&n->partials), scratch * 4);
+    for (auto &j : jobs) j.out = n->wk + reinterpret_cast<intptr_t>(j.out);
+    if (e == cudaSuccess)
+      e = cudaMalloc(reinterpret_cast<void **>(&n->jobs), jobs.size() * sizeof(jobs[0]));
+    if (e == cudaSuccess)
+      e = cudaMemcpy(n->jobs, jobs.data(), jobs.size() * sizeof(jobs[0]), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = lbm::net::setup_tc();
   }
-  if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&n->d_err), sizeof(int));
-  if (e == cudaSuccess) e = cudaMemset(n->d_err, 0, sizeof(int));
-  if (e == cudaSuccess) {
-    e = cudaFuncSetAttribute(lbm::net::conv_fwd_tc<3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             lbm::net::kTcSmem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(lbm::net::conv_fwd_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               lbm::net::kTcSmem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(lbm::net::conv_fwd_tc_async<3>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, lbm::net::kTcAsyncSmem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(lbm::net::conv_fwd_tc_async<1>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, lbm::net::kTcAsyncSmem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(lbm::net::conv_wgrad_tc<3>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, lbm::net::kWgSmem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(lbm::net::conv_wgrad_tc<1>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, lbm::net::kWgSmem);
-  }
-  if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&n->loss), sizeof(double));
+  if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&n->status), sizeof(*n->status));
+  if (e == cudaSuccess)
+    e = cudaMallocHost(reinterpret_cast<void **>(&n->h_status), sizeof(*n->h_status));
   for (int g = 0; g < 2 && e == cudaSuccess; g++)
     for (size_t i = 0; i < p.elems.size() && e == cudaSuccess; i++) {
       void *b = nullptr;
-      e = cudaMalloc(&b, p.elems[i] * max_batch * as);
+      // (BF16 mode reads the decoder's inputs from their sources)
+      const bool cat = std::find(p.cat.begin(), p.cat.end(), static_cast<int>(i)) != p.cat.end();
+      if (g == 1 || !cat || precision == LBM_FP32) e = cudaMalloc(&b, p.elems[i] * max_batch * as);
       n->bufs.push_back(b);
     }
   if (e == cudaSuccess) e = cudaMemset(n->m, 0, off * sizeof(float));
@@ -1373,6 +1038,7 @@ int lbm_net_set_params(lbm_net_t *n, const float *params, int64_t count) {
   cudaError_t e = cudaMemcpy(n->params, params, count * sizeof(float), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemset(n->m, 0, count * sizeof(float));
   if (e == cudaSuccess) e = cudaMemset(n->v, 0, count * sizeof(float));
+  n->stale = true;
   n->adam_t = 0;
   return e == cudaSuccess ? LBM_OK : nfail(n, LBM_ECUDA, cudaGetErrorString(e));
 }
@@ -1386,27 +1052,19 @@ int lbm_net_get_params(const lbm_net_t *n, float *params, int64_t count) {
 
 int lbm_net_forward(lbm_net_t *n, const float *x, int32_t batch, float *y) {
   if (!n || !x || !y || batch < 1 || batch > n->max_batch) return nfail(n, LBM_EINVAL, "bad batch");
-  cudaError_t e = n->precision == LBM_FP32
-                      ? run<float>(n, x, batch, nullptr, y, nullptr)
-                      : run<__nv_bfloat16>(n, x, batch, nullptr, y, nullptr);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(n->stream);
-  if (e == cudaSuccess && tc_timed_out(n))
-    return nfail(n, LBM_ETIMEOUT, "a tensor-core convolution's bounded wait ran out");
-  return e == cudaSuccess ? LBM_OK : nfail(n, LBM_ECUDA, cudaGetErrorString(e));
+  return run(n, x, batch, nullptr, y, nullptr);
 }
 
 int lbm_net_gradients(lbm_net_t *n, const float *x, const float *t, int32_t batch, float *grads,
                       double *loss) {
   if (!n || !x || !t || batch < 1 || batch > n->max_batch) return nfail(n, LBM_EINVAL, "bad batch");
   double l = 0.0;
-  cudaError_t e = n->precision == LBM_FP32 ? run<float>(n, x, batch, t, nullptr, &l)
-                                           : run<__nv_bfloat16>(n, x, batch, t, nullptr, &l);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(n->stream);
-  if (e == cudaSuccess && tc_timed_out(n))
-    return nfail(n, LBM_ETIMEOUT, "a tensor-core convolution's bounded wait ran out");
-  if (e == cudaSuccess && grads)
-    e = cudaMemcpy(grads, n->grads, n->n_params * sizeof(float), cudaMemcpyDeviceToHost);
+  const int rc = run(n, x, batch, t, nullptr, &l);
+  if (rc != LBM_OK) return rc;
   if (loss) *loss = l;
+  if (!grads) return LBM_OK;
+  const cudaError_t e =
+      cudaMemcpy(grads, n->grads, n->n_params * sizeof(float), cudaMemcpyDeviceToHost);
   return e == cudaSuccess ? LBM_OK : nfail(n, LBM_ECUDA, cudaGetErrorString(e));
 }
 
@@ -1415,6 +1073,7 @@ int lbm_net_train_step(lbm_net_t *n, const float *x, const float *t, int32_t bat
   int rc = lbm_net_gradients(n, x, t, batch, nullptr, loss);
   if (rc) return rc;
   n->adam_t++;
+  n->stale = true;
   const float b1 = 0.9f, b2 = 0.999f;
   const float c1 = 1.f - std::pow(b1, static_cast<float>(n->adam_t));
   const float c2 = 1.f - std::pow(b2, static_cast<float>(n->adam_t));
@@ -1428,9 +1087,11 @@ void lbm_net_destroy(lbm_net_t *n) {
   if (!n) return;
   cudaStreamSynchronize(n->stream);
   for (void *p : {static_cast<void *>(n->params), static_cast<void *>(n->grads),
-                  static_cast<void *>(n->m), static_cast<void *>(n->v), n->wq, n->wt, n->wk,
-                  static_cast<void *>(n->d_err), static_cast<void *>(n->loss)})
+                  static_cast<void *>(n->m), static_cast<void *>(n->v), static_cast<void *>(n->wt),
+                  static_cast<void *>(n->wk), static_cast<void *>(n->jobs),
+                  static_cast<void *>(n->partials), static_cast<void *>(n->status)})
     if (p) cudaFree(p);
+  if (n->h_status) cudaFreeHost(n->h_status);
   for (void *b : n->bufs)
     if (b) cudaFree(b);
   delete n;
