@@ -1166,14 +1166,14 @@ int lbm3d_step(lbm3d_t *h, int64_t n) {
           Const3<C> kx = h->kc.get(tag);
           kx.sr_seed = lbm::dev::step_seed(h->steps);
           return lbm::launch_chained(
-              step3_kernel<C, true>, blocks, kThreads3, h->stream, static_cast<const C *>(h->f[src]),
+              step3_kernel<C, true>, dim3(blocks), kThreads3, 0, h->stream, static_cast<const C *>(h->f[src]),
               static_cast<C *>(h->f[dst]), h->flags, h->lbase,
               static_cast<const Link3<C> *>(h->links), h->fluid, kx, h->n_fluid, h->links_df,
               h->carry, h->kc.x);
         }
       }
       return lbm::launch_chained(
-          step3_kernel<C, false>, blocks, kThreads3, h->stream, static_cast<const C *>(h->f[src]),
+          step3_kernel<C, false>, dim3(blocks), kThreads3, 0, h->stream, static_cast<const C *>(h->f[src]),
           static_cast<C *>(h->f[dst]), h->flags, h->lbase, static_cast<const Link3<C> *>(h->links),
           h->fluid, h->kc.get(tag), h->n_fluid, static_cast<const lbm::LinkCoefDF *>(nullptr),
           static_cast<float *>(nullptr), Const3<D2>());

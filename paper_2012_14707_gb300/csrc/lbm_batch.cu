@@ -307,8 +307,8 @@ cudaError_t launch_batch_step(const T *src, T *dst, const uint2 *node, const int
     if constexpr (THREADS <= kChunk / 2) {
       if (n_work > 0)
         return launch_chained(batch_pair_kernel<T, THREADS>,
-                              static_cast<unsigned>(n_work) * (kChunk / (2 * THREADS)), THREADS, s,
-                              src, dst, node, grp, ccase, rowstart, jbslot,
+                              dim3(static_cast<unsigned>(n_work) * (kChunk / (2 * THREADS))),
+                              THREADS, 0, s, src, dst, node, grp, ccase, rowstart, jbslot,
                               static_cast<const LinkCoef<float> *>(links),
                               static_cast<const BatchCase<float> *>(cases), active, work, counter,
                               j, geoms);
@@ -320,14 +320,14 @@ cudaError_t launch_batch_step(const T *src, T *dst, const uint2 *node, const int
   const int64_t blocks = static_cast<int64_t>(n_work) * (kChunk / THREADS);
   cudaError_t e = cudaSuccess;
   if (blocks > 0)
-    e = launch_chained(batch_step_kernel<T, C, THREADS>, static_cast<unsigned>(blocks), THREADS, s,
+    e = launch_chained(batch_step_kernel<T, C, THREADS>, dim3(static_cast<unsigned>(blocks)), THREADS, 0, s,
                        src, dst, node, grp, ccase, rowstart, jbslot,
                        static_cast<const LinkCoef<C> *>(links),
                        static_cast<const BatchCase<C> *>(cases), active, work,
                        static_cast<uint32_t>(blocks), pf_dist, counter, j, geoms);
   if constexpr (std::is_same<T, float>::value) {
     if (e == cudaSuccess && n_exact_chunks > 0)
-      e = launch_chained(batch_exact_kernel, static_cast<unsigned>(n_exact_chunks), kChunk, s, src,
+      e = launch_chained(batch_exact_kernel, dim3(static_cast<unsigned>(n_exact_chunks)), kChunk, 0, s, src,
                          dst, ccase, static_cast<const LinkCoef<float> *>(links),
                          static_cast<const BatchCase<float> *>(cases), active, exact_chunks,
                          counter, j, geoms);

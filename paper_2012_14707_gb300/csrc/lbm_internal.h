@@ -359,11 +359,12 @@ void parallel_for(int64_t n, F &&f, int64_t min_per_thread = 1 << 14) {
 // its CTAs, and read what no step writes, while this one's last CTAs still
 // run; it waits at dev::chain_wait() for this one's results.
 template <typename... P, typename... A>
-cudaError_t launch_chained(void (*f)(P...), unsigned blocks, unsigned threads, cudaStream_t s,
-                           A &&...args) {
+cudaError_t launch_chained(void (*f)(P...), dim3 grid, unsigned threads, size_t smem,
+                           cudaStream_t s, A &&...args) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(blocks);
+  cfg.gridDim = grid;
   cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute at = {};
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;

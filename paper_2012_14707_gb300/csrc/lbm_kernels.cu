@@ -454,20 +454,20 @@ cudaError_t launch_step_pull(const T *src, T *dst, const PullGeom &g, int64_t n_
   if constexpr (kStochastic<T>) {
     const int64_t pairs = (n_fluid + 1) / 2;
     return launch_chained(step_kernel_pair<T>,
-                          static_cast<unsigned>((pairs + kPairThreads - 1) / kPairThreads),
-                          kPairThreads, s, src, dst, g, static_cast<uint32_t>(n_fluid), links, k);
+                          dim3(static_cast<unsigned>((pairs + kPairThreads - 1) / kPairThreads)),
+                          kPairThreads, 0, s, src, dst, g, static_cast<uint32_t>(n_fluid), links, k);
   } else {
     const int64_t blocks = (n_fluid + kPullThreads - 1) / kPullThreads;
     if constexpr (std::is_same<T, float>::value) {
       if (k.exact) {
         if (!g.links64 || !g.carry || !g.carry0) return cudaErrorInvalidValue;
-        return launch_chained(step_kernel_pull<T, C, true>, static_cast<unsigned>(blocks),
-                              kPullThreads, s, src, dst, g, static_cast<uint32_t>(n_fluid), links,
+        return launch_chained(step_kernel_pull<T, C, true>, dim3(static_cast<unsigned>(blocks)),
+                              kPullThreads, 0, s, src, dst, g, static_cast<uint32_t>(n_fluid), links,
                               k);
       }
     }
-    return launch_chained(step_kernel_pull<T, C, false>, static_cast<unsigned>(blocks),
-                          kPullThreads, s, src, dst, g, static_cast<uint32_t>(n_fluid), links, k);
+    return launch_chained(step_kernel_pull<T, C, false>, dim3(static_cast<unsigned>(blocks)),
+                          kPullThreads, 0, s, src, dst, g, static_cast<uint32_t>(n_fluid), links, k);
   }
 }
 

@@ -38,6 +38,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/lbm.h"
+#include "lbm_internal.h"
 #include "lbm_net_tc.h"
 
 namespace lbm {
@@ -323,6 +324,12 @@ __global__ void mse_kernel(const A *__restrict__ y, const float *__restrict__ t,
 // passes run at memory speed; each does in one read and one write what a
 // chain of elementwise passes would.
 
+// (launched as a chain with the convolutions: lbm_net_tc.cu, chain_wait)
+__device__ __forceinline__ void chain_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 __device__ __forceinline__ void unpack8(uint4 v, float (&f)[8]) {
   const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
@@ -370,9 +377,10 @@ __global__ void __launch_bounds__(256) to_storage8(const float *__restrict__ s, 
 }
 
 // 2x2 average pooling; H, W: output size
-__global__ void __launch_bounds__(256) pool2_fwd8(const __nv_bfloat16 *__restrict__ x,
-                                                  __nv_bfloat16 *__restrict__ y, int n8, int H,
+__global__ void __launch_bounds__(256) pool2_fwd8(const __nv_bfloat16 *x,
+                                                  __nv_bfloat16 *y, int n8, int H,
                                                   int W, uint32_t n) {
+  chain_wait();
   const uint32_t t = blockIdx.x * 256u + threadIdx.x;
   if (t >= n) return;
   const uint32_t c = t % n8, p = t / n8, j = p % W, r = p / W;  // r = image * H + row
@@ -395,10 +403,11 @@ __global__ void __launch_bounds__(256) pool2_fwd8(const __nv_bfloat16 *__restric
 // Backward of the 2x upsampling and of the ReLU below it: gx = sum of gy's
 // first 8 n8 channels (stride 8 g8) over each 2x2 block, 0 where h <= 0;
 // H, W: size of gx
-__global__ void __launch_bounds__(256) up2_bwd8(const __nv_bfloat16 *__restrict__ gy, int g8,
-                                                const __nv_bfloat16 *__restrict__ h,
-                                                __nv_bfloat16 *__restrict__ gx, int n8, int H,
+__global__ void __launch_bounds__(256) up2_bwd8(const __nv_bfloat16 *gy, int g8,
+                                                const __nv_bfloat16 *h,
+                                                __nv_bfloat16 *gx, int n8, int H,
                                                 int W, uint32_t n) {
+  chain_wait();
   const uint32_t t = blockIdx.x * 256u + threadIdx.x;
   if (t >= n) return;
   const uint32_t c = t % n8, p = t / n8, j = p % W, r = p / W;
@@ -419,11 +428,12 @@ __global__ void __launch_bounds__(256) up2_bwd8(const __nv_bfloat16 *__restrict_
 // Gradient of an encoder level's output: the skip connection's (channels
 // from group g0 of gskip, stride 8 g8) plus the pooled path's (gpool / 4
 // over each 2x2 block), 0 where h <= 0; H, W: size of the level
-__global__ void __launch_bounds__(256) pool2_bwd8(const __nv_bfloat16 *__restrict__ gpool,
-                                                  const __nv_bfloat16 *__restrict__ gskip, int g8,
-                                                  int g0, const __nv_bfloat16 *__restrict__ h,
-                                                  __nv_bfloat16 *__restrict__ gx, int n8, int H,
+__global__ void __launch_bounds__(256) pool2_bwd8(const __nv_bfloat16 *gpool,
+                                                  const __nv_bfloat16 *gskip, int g8,
+                                                  int g0, const __nv_bfloat16 *h,
+                                                  __nv_bfloat16 *gx, int n8, int H,
                                                   int W, uint32_t n) {
+  chain_wait();
   const uint32_t t = blockIdx.x * 256u + threadIdx.x;
   if (t >= n) return;
   const uint32_t c = t % n8, p = t / n8, j = p % W, r = p / W;
@@ -439,10 +449,11 @@ __global__ void __launch_bounds__(256) pool2_bwd8(const __nv_bfloat16 *__restric
 
 // Squared error and its gradient gy = 2 (y - t) / n, per pixel; y, gy with
 // 8 n8 channels stored, c real ones.  One atomic per CTA.
-__global__ void __launch_bounds__(256) mse8(const __nv_bfloat16 *__restrict__ y,
-                                            const float *__restrict__ t,
-                                            __nv_bfloat16 *__restrict__ gy, int c, int n8,
-                                            int64_t npix, double *__restrict__ loss) {
+__global__ void __launch_bounds__(256) mse8(const __nv_bfloat16 *y,
+                                            const float *t,
+                                            __nv_bfloat16 *gy, int c, int n8,
+                                            int64_t npix, double *loss) {
+  chain_wait();
   double s = 0.0;
   const float n = static_cast<float>(npix * c);
   for (int64_t q = blockIdx.x * 256ll + threadIdx.x; q < npix * n8;
@@ -453,9 +464,13 @@ __global__ void __launch_bounds__(256) mse8(const __nv_bfloat16 *__restrict__ y,
     unpack8(as8(y)[q], f);
 #pragma unroll
     for (int e = 0; e < 8; e++) {
-      const float d = c0 + e < c ? f[e] - t[p * c + c0 + e] : 0.f;
-      s += static_cast<double>(d) * d;
-      f[e] = 2.f * d / n;
+      if (c0 + e < c) {
+        const float d = f[e] - t[p * c + c0 + e];
+        s += static_cast<double>(d) * d;
+        f[e] = 2.f * d / n;
+      } else {
+        f[e] = 0.f;
+      }
     }
     as8(gy)[q] = pack8(f);
   }
@@ -789,8 +804,9 @@ cudaError_t run_bf16(lbm_net_t *n, const float *x_in, int N, const float *t, flo
     if (l > 0) {
       const int cb = n->base << (l - 1), n8 = pad8(cb) / 8;
       const int64_t k = static_cast<int64_t>(N) * H * W * n8;
-      pool2_fwd8<<<blocks(k), 256, 0, s>>>(buf(p.eb[l - 1]), buf(p.pool[l]), n8, H, W,
-                                           static_cast<uint32_t>(k));
+      if (e == cudaSuccess)
+        e = lbm::launch_chained(pool2_fwd8, dim3(blocks(k)), 256, 0, s, buf(p.eb[l - 1]),
+                                buf(p.pool[l]), n8, H, W, static_cast<uint32_t>(k));
       in = single(buf(p.pool[l]), cb);
     }
     conv(2 * l, in, H, W, 1, buf(p.ea[l]), nullptr);
@@ -818,8 +834,8 @@ cudaError_t run_bf16(lbm_net_t *n, const float *x_in, int N, const float *t, flo
 
   // loss and backward
   const int n8y = pad8(n->c_out) / 8;
-  mse8<<<std::min<unsigned>(blocks(HW * N * n8y), 4u * n->sms), 256, 0, s>>>(
-      buf(p.y), t, gbuf(p.y), n->c_out, n8y, HW * N, &n->status->loss);
+  e = lbm::launch_chained(mse8, dim3(std::min<unsigned>(blocks(HW * N * n8y), 4u * n->sms)), 256, 0,
+                          s, buf(p.y), t, gbuf(p.y), n->c_out, n8y, HW * N, &n->status->loss);
   // gradients of layer k from its input and its (masked) output gradient gz;
   // gx: the input's gradient, 0 where mask <= 0 (may be null)
   auto back = [&](int k, const ConvInput &in, const B16 *gz, B16 *gx, const B16 *mask, int H,
@@ -851,9 +867,9 @@ cudaError_t run_bf16(lbm_net_t *n, const float *x_in, int N, const float *t, flo
     const int n8 = pad8(in.ca) / 8;
     const int64_t k = static_cast<int64_t>(N) * (H / 2) * (W / 2) * n8;
     if (e == cudaSuccess)
-      up2_bwd8<<<blocks(k), 256, 0, s>>>(gbuf(p.cat[l]), in.padded() / 8, buf(below(l)),
-                                         gbuf(below(l)), n8, H / 2, W / 2,
-                                         static_cast<uint32_t>(k));
+      e = lbm::launch_chained(up2_bwd8, dim3(blocks(k)), 256, 0, s, gbuf(p.cat[l]),
+                              in.padded() / 8, buf(below(l)), gbuf(below(l)), n8, H / 2, W / 2,
+                              static_cast<uint32_t>(k));
   }
   for (int l = L - 1; l >= 0; l--) {
     const int H = n->H >> l, W = n->W >> l, ch = n->base << l;
@@ -862,9 +878,9 @@ cudaError_t run_bf16(lbm_net_t *n, const float *x_in, int N, const float *t, flo
       const int n8 = pad8(ch) / 8;
       const int64_t k = static_cast<int64_t>(N) * H * W * n8;
       if (e == cudaSuccess)
-        pool2_bwd8<<<blocks(k), 256, 0, s>>>(gbuf(p.pool[l + 1]), gbuf(p.cat[l]), in.padded() / 8,
-                                             pad8(in.ca) / 8, buf(p.eb[l]), gbuf(p.eb[l]), n8, H,
-                                             W, static_cast<uint32_t>(k));
+        e = lbm::launch_chained(pool2_bwd8, dim3(blocks(k)), 256, 0, s, gbuf(p.pool[l + 1]),
+                                gbuf(p.cat[l]), in.padded() / 8, pad8(in.ca) / 8, buf(p.eb[l]),
+                                gbuf(p.eb[l]), n8, H, W, static_cast<uint32_t>(k));
     }
     back(2 * l + 1, single(buf(p.ea[l]), ch), gbuf(p.eb[l]), gbuf(p.ea[l]), buf(p.ea[l]), H, W);
     if (l > 0)

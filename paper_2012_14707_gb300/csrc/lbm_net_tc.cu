@@ -19,7 +19,9 @@
 // give up in turn after waiting for the copies they started.
 #include <algorithm>
 #include <cstdint>
+#include <type_traits>
 
+#include "lbm_internal.h"
 #include "lbm_net_tc.h"
 
 namespace lbm {
@@ -41,21 +43,24 @@ __device__ __forceinline__ void mbar_expect(uint64_t *bar, uint32_t bytes) {
                "r"(bytes)
                : "memory");
 }
-constexpr int kWaitLimit = 1 << 24;  // polls: a fraction of a second
 // Waits for the phase with parity `phase`; false if it did not come within
-// kWaitLimit polls (test_wait: each poll returns at once) or the CTA gave up.
+// kWaitLimit tries or the CTA gave up.  try_wait suspends the warp (for up to
+// about the hint, a microsecond): warps polling with test_wait took so many
+// issue slots that the roles with work to do ran several times slower (a
+// 32-channel 256x256 layer 90 us).
+constexpr int kWaitLimit = 1 << 20;
 __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t phase, volatile int *gave_up) {
   const uint32_t a = smem_addr(bar);
   for (int it = 0; it < kWaitLimit; it++) {
     uint32_t done;
     asm volatile(
-        "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n"
         " selp.u32 %0, 1, 0, p;\n}\n"
         : "=r"(done)
-        : "r"(a), "r"(phase)
+        : "r"(a), "r"(phase), "r"(1000u)
         : "memory");
     if (done) return true;
-    if ((it & 1023) == 1023 && *gave_up) return false;
+    if ((it & 63) == 63 && *gave_up) return false;
   }
   return false;
 }
@@ -64,28 +69,47 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t phase, volatil
 // K-major operand: lbo between core matrices along K, sbo between groups of
 // 8 rows.  MN-major operand: sbo between core matrices along M (N), lbo
 // between groups of 8 along K.  Bit 46: descriptor version.
-__device__ __forceinline__ uint64_t umma_desc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
-  return static_cast<uint64_t>((addr >> 4) & 0x3FFFu) |
-         (static_cast<uint64_t>((lbo >> 4) & 0x3FFFu) << 16) |
-         (static_cast<uint64_t>((sbo >> 4) & 0x3FFFu) << 32) | (1ull << 46);
+// The low word holds the address and lbo, so a descriptor further on in the
+// same tile is the low word plus the distance / 16: one addition per MMA
+// (the issuing thread is alone; 64-bit descriptor arithmetic cost it 150 to
+// 240 cycles an MMA, several times what the MMA takes).
+__device__ __forceinline__ uint32_t desc_lo(uint32_t addr, uint32_t lbo) {
+  return ((addr >> 4) & 0x3FFFu) | (((lbo >> 4) & 0x3FFFu) << 16);
+}
+__device__ __forceinline__ uint32_t desc_hi(uint32_t sbo) {
+  return ((sbo >> 4) & 0x3FFFu) | (1u << 14);
 }
 // kind::f16, D = FP32, A = B = BF16, M = 128; mn: both operands MN-major
 __host__ __device__ constexpr uint32_t umma_idesc(int N, bool mn) {
   return (1u << 4) | (1u << 7) | (1u << 10) | (mn ? (1u << 15) | (1u << 16) : 0u) |
          (static_cast<uint32_t>(N >> 3) << 17) | (static_cast<uint32_t>(128 >> 4) << 24);
 }
-__device__ __forceinline__ void mma_bf16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc,
-                                         bool accumulate) {
+// The MMA warp runs its loops with all lanes, and one lane (leader != 0)
+// issues: descriptors and loop counters are then warp-uniform, as the
+// instruction takes them.
+__device__ __forceinline__ uint32_t elect_leader() {
+  uint32_t l;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xFFFFFFFF;\n selp.u32 %0, 1, 0, p;\n}\n"
+               : "=r"(l));
+  return l;
+}
+__device__ __forceinline__ void mma_bf16(uint32_t leader, uint32_t d, uint32_t alo, uint32_t ahi,
+                                         uint32_t blo, uint32_t bhi, uint32_t idesc,
+                                         uint32_t accumulate) {
   asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
-      "l"(a), "l"(b), "r"(idesc), "r"(accumulate ? 1u : 0u)
+      "{\n .reg .pred p, q;\n .reg .b64 a, b;\n setp.ne.b32 p, %6, 0;\n setp.ne.b32 q, %7, 0;\n"
+      " mov.b64 a, {%1, %2};\n mov.b64 b, {%3, %4};\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n}\n" ::"r"(d),
+      "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc), "r"(accumulate), "r"(leader)
       : "memory");
 }
-__device__ __forceinline__ void mma_commit(uint64_t *bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
-                   smem_addr(bar))
-               : "memory");
+__device__ __forceinline__ void mma_commit(uint32_t leader, uint64_t *bar) {
+  asm volatile(
+      "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
+      " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(
+          smem_addr(bar)),
+      "r"(leader)
+      : "memory");
 }
 __device__ __forceinline__ void tmem_alloc(uint32_t *slot, uint32_t cols) {
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
@@ -122,12 +146,22 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, bool v
                "r"(valid ? 16u : 0u)
                : "memory");
 }
-__device__ __forceinline__ void cp_async_commit() {
-  asm volatile("cp.async.commit_group;\n" ::: "memory");
+// Arrives at *bar (one of its expected arrivals) once this thread's copies so
+// far have landed; the thread goes on at once.
+__device__ __forceinline__ void cp_async_arrive(uint64_t *bar) {
+  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];\n" ::"r"(smem_addr(bar))
+               : "memory");
 }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
+__device__ __forceinline__ void cp_async_wait_all() {
+  asm volatile("cp.async.wait_all;\n" ::: "memory");
+}
+// Waits until the kernels before this one in the stream are complete, then
+// lets the next one start its CTAs as this one's finish (launch_chained).
+// Packed weights and biases, which no kernel of a pass writes, may be read
+// before it.
+__device__ __forceinline__ void chain_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 __device__ __forceinline__ void fence_async_proxy() {
   asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
@@ -148,16 +182,6 @@ struct InputDev {
   int n8a, n8;       // slabs of xa, of both
   int up;
 };
-// The 8 channels of slab c8 of pixel (n, i, j) of an H x W image.
-__device__ __forceinline__ const __nv_bfloat16 *input_at(const InputDev &x, int n, int i, int j,
-                                                         int H, int W, int c8) {
-  if (c8 < x.n8a) {
-    const int Ha = H >> x.up, Wa = W >> x.up;
-    return x.xa + (static_cast<int64_t>((n * Ha + (i >> x.up)) * Wa + (j >> x.up)) * x.sa + c8 * 8);
-  }
-  return x.xb + (static_cast<int64_t>((n * H + i) * W + j) * x.sb + (c8 - x.n8a) * 8);
-}
-
 // ---------------------------------------------------------------------------
 // Forward and backward-data convolution
 // ---------------------------------------------------------------------------
@@ -168,11 +192,12 @@ __device__ __forceinline__ const __nv_bfloat16 *input_at(const InputDev &x, int 
 // and walks over image tiles of MT x (8 x 16) pixels.  Roles: one lane copies
 // packed weights (bulk copies; all of them once where they fit beside the
 // image tiles, else through a ring, tap by tap in chunks of 64 channels),
-// four warps copy image tiles (cp.async, zero outside the image), one lane
-// issues the MMAs (M = 128 pixels, N = NT, K = 16), four warps read the
+// eight warps copy image tiles (cp.async, zero outside the image), one lane
+// issues the MMAs (M = 128 pixels, N = NT, K = 16), eight warps read the
 // accumulators back, of which there are two sets, so that a tile's epilogue
 // overlaps the next tile's MMAs.
-constexpr int kConvThreads = 320;
+constexpr int kLoadThreads = 256;
+constexpr int kConvThreads = 320 + kLoadThreads;
 constexpr int kMaxStagesB = 54;   // 9 taps x 6 chunks of 64: every weight block resident
 constexpr int kMaxStagesA = 3;
 constexpr int kSmemMax = 232448 - 2048;  // dynamic shared memory a CTA may use (static below)
@@ -183,7 +208,7 @@ struct ConvDev {
   // ... in `parts` parts of p8 slabs, as many as shared memory takes at once;
   // one part: a tile is copied once for all taps; more: again for every tap
   int parts, p8, unit_taps;
-  uint32_t magic, magic_last;  // 2^32 / slabs + 1 of a part and of the last one
+  int lanes_log2;         // threads of the image copy that share a pixel
   const __nv_bfloat16 *wk;
   const float *bias;
   const __nv_bfloat16 *mask;
@@ -213,9 +238,11 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_halo_tc(const __grid_con
   __shared__ uint64_t full_a[kMaxStagesA], empty_a[kMaxStagesA];
   __shared__ uint64_t full_b[kMaxStagesB], empty_b[kMaxStagesB];
   __shared__ uint64_t full_d[2], empty_d[2], drained;
+  __shared__ __align__(16) float bias[128];
   __shared__ uint32_t tmem_slot;
   __shared__ int gave_up;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xFFFFFFFFu, static_cast<int>(threadIdx.x >> 5), 0);
+  const int lane = threadIdx.x & 31;
   const uint32_t a_bytes = static_cast<uint32_t>(a.p8) * S::kSlab;
   const uint32_t b_bytes = static_cast<uint32_t>(a.NT) * 128u;  // 64 channels
   const uint32_t base_a = smem_addr(dyn);
@@ -223,7 +250,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_halo_tc(const __grid_con
   const uint32_t stride_a = (a_bytes + 127u) & ~127u;
   if (threadIdx.x == 0) {
     for (int i = 0; i < a.stages_a; i++) {
-      mbar_init(&full_a[i], 128);
+      mbar_init(&full_a[i], kLoadThreads);
       mbar_init(&empty_a[i], 1);
     }
     for (int i = 0; i < a.stages_b; i++) {
@@ -232,18 +259,23 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_halo_tc(const __grid_con
     }
     for (int i = 0; i < 2; i++) {
       mbar_init(&full_d[i], 1);
-      mbar_init(&empty_d[i], 128);
+      mbar_init(&empty_d[i], 256);
     }
     mbar_init(&drained, 1);
     gave_up = 0;
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
+  if (threadIdx.x >= 64 && threadIdx.x < 64 + a.NT) {
+    const int o = blockIdx.y * a.NT + threadIdx.x - 64;
+    bias[threadIdx.x - 64] = a.bias && o < a.co ? a.bias[o] : 0.f;
+  }
   if (warp == 1) tmem_alloc(&tmem_slot, a.tmem_cols);
   fence_before();
   __syncthreads();
   fence_after();
-  const uint32_t tmem = tmem_slot;
+  const uint32_t tmem = __shfl_sync(0xFFFFFFFFu, tmem_slot, 0);
 
+  if (warp != 0) chain_wait();
   if (warp == 0) {
     // weights
     if (lane == 0) {
@@ -288,87 +320,127 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_halo_tc(const __grid_con
     }
   } else if (warp == 1) {
     // MMAs
-    if (lane == 0) {
-      const uint32_t idesc = umma_idesc(a.NT, false);
-      const uint32_t lbo_b = static_cast<uint32_t>(a.NT) * 16u;
-      int sa = 0, sb = 0, it = 0;
-      uint32_t pa = 0, pb = 0;
-      bool ok = true;
-      for (int t = blockIdx.x; ok && t < a.tiles; t += gridDim.x, it++) {
-        const int acc = it & 1;
-        if (it >= 2 && !mbar_wait(&empty_d[acc], ((it >> 1) & 1) ^ 1u, &gave_up)) {
-          ok = false;
-          break;
-        }
-        const uint32_t d0 = tmem + static_cast<uint32_t>(acc * MT * a.NT);
-        if (a.resident) {
-          sb = 0;
-          pb = 0;
-        }
-        bool first = true;
-        const int units = a.parts * (KS * KS / a.unit_taps);
-        for (int u = 0; ok && u < units; u++) {
-          if (!mbar_wait(&full_a[sa], pa, &gave_up)) {
-            ok = false;
-            break;
-          }
-          fence_after();
-          const uint32_t ta = base_a + sa * stride_a;
-          const int t0 = u / a.parts * a.unit_taps, p = u % a.parts;
-          const int k8 = min(a.p8, a.k8 - p * a.p8), chunks = (k8 + 7) / 8;
-          for (int tap = t0; ok && tap < t0 + a.unit_taps; tap++) {
-            const uint32_t shift = static_cast<uint32_t>((tap / KS) * S::kWp + (tap % KS)) * 16u;
-            for (int ch = 0; ch < chunks; ch++) {
-              if (!mbar_wait(&full_b[sb], pb, &gave_up)) {
-                ok = false;
-                break;
-              }
-              fence_after();
-              const int k16 = min(8, k8 - ch * 8) / 2;
-              const uint32_t tb = base_b + sb * b_bytes;
-              for (int k = 0; k < k16; k++) {
-                const uint64_t bd = umma_desc(tb + k * 2 * lbo_b, lbo_b, 128u);
-#pragma unroll
-                for (int m = 0; m < MT; m++) {
-                  const uint64_t ad = umma_desc(
-                      ta + static_cast<uint32_t>(ch * 8 + 2 * k) * S::kSlab + shift + m * 128u,
-                      S::kSlab, S::kWp * 16u);
-                  mma_bf16(d0 + m * a.NT, ad, bd, idesc, !first);
-                }
-                first = false;
-              }
-              if (!a.resident) mma_commit(&empty_b[sb]);
-              if (++sb == a.stages_b) {
-                sb = 0;
-                pb ^= 1u;
-              }
+    const uint32_t leader = elect_leader();
+    const uint32_t idesc = umma_idesc(a.NT, false);
+    const uint32_t lbo_b = static_cast<uint32_t>(a.NT) * 16u;
+    const uint32_t ahi = desc_hi(S::kWp * 16u), bhi = desc_hi(128u);
+    constexpr uint32_t kStepA = 2 * S::kSlab / 16;  // 16 channels on
+    const uint32_t step_b = 2 * lbo_b / 16;
+    int sa = 0, sb = 0, it = 0;
+    uint32_t pa = 0, pb = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; ok && t < a.tiles; t += gridDim.x, it++) {
+      const int acc = it & 1;
+      if (it >= 2 && !mbar_wait(&empty_d[acc], ((it >> 1) & 1) ^ 1u, &gave_up)) {
+        ok = false;
+        break;
+      }
+      const uint32_t d0 = tmem + static_cast<uint32_t>(acc * MT * a.NT);
+      const bool wait_b = !a.resident || it == 0;  // resident weights land once
+      if (a.resident) {
+        sb = 0;
+        pb = 0;
+      }
+      uint32_t accumulate = 0;
+      // the MMAs of one tap of a tile in shared memory
+      auto do_tap = [&](uint32_t alo, int k8) {
+#pragma unroll 1
+        for (int c8 = 0; c8 < k8; c8 += 8) {
+          if (wait_b) {
+            if (!mbar_wait(&full_b[sb], pb, &gave_up)) {
+              ok = false;
+              return;
             }
+            fence_after();
           }
-          if (!ok) break;
-          mma_commit(&empty_a[sa]);
-          if (++sa == a.stages_a) {
-            sa = 0;
-            pa ^= 1u;
+          uint32_t blo = desc_lo(base_b + sb * b_bytes, lbo_b);
+          const int k16 = min(4, (k8 - c8) >> 1);
+#pragma unroll 1
+          for (int k = 0; k < k16; k++) {
+#pragma unroll
+            for (int m = 0; m < MT; m++)
+              mma_bf16(leader, d0 + m * a.NT, alo + m * 8u, ahi, blo, bhi, idesc, accumulate);
+            accumulate = 1;
+            alo += kStepA;
+            blo += step_b;
+          }
+          if (!a.resident) mma_commit(leader, &empty_b[sb]);
+          if (++sb == a.stages_b) {
+            sb = 0;
+            pb ^= 1u;
           }
         }
-        if (ok) mma_commit(&full_d[acc]);
+      };
+      auto next_tile = [&](uint32_t *ta) {
+        if (!mbar_wait(&full_a[sa], pa, &gave_up)) {
+          ok = false;
+          return;
+        }
+        fence_async_proxy();  // the landed copies, for the MMAs
+        fence_after();
+        *ta = desc_lo(base_a + sa * stride_a, S::kSlab);
+      };
+      auto free_tile = [&]() {
+        mma_commit(leader, &empty_a[sa]);
+        if (++sa == a.stages_a) {
+          sa = 0;
+          pa ^= 1u;
+        }
+      };
+      uint32_t ta = 0;
+      if (a.parts == 1) {
+        next_tile(&ta);
+        if (!ok) break;
+        // (rolled: nine copies of the body would miss the instruction cache)
+        int dx = 0;
+#pragma unroll 1
+        for (int tap = 0; tap < KS * KS; tap++) {
+          do_tap(ta, a.k8);
+          if (!ok) break;
+          ta++;
+          if (++dx == KS) {
+            dx = 0;
+            ta += S::kWp - KS;
+          }
+        }
+        if (!ok) break;
+        free_tile();
+      } else {
+        for (int tap = 0; ok && tap < KS * KS; tap++)
+          for (int p = 0; ok && p < a.parts; p++) {
+            next_tile(&ta);
+            if (!ok) break;
+            do_tap(ta + (tap / KS) * S::kWp + (tap % KS), min(a.p8, a.k8 - p * a.p8));
+            if (ok) free_tile();
+          }
+        if (!ok) break;
       }
-      if (!ok) {
-        gave_up = 1;
-        atomicExch(a.err, 1);
-        int never = 0;
-        mma_commit(&drained);  // the MMAs in flight end before the memory is given back
-        mbar_wait(&drained, 0, &never);
-      }
+      mma_commit(leader, &full_d[acc]);
     }
-  } else if (warp < 6) {
-    // epilogue: lane = pixel of the tile's row group, 16 output channels at a time
-    const int q = warp & 3;
+    if (!ok) {
+      gave_up = 1;
+      if (lane == 0) atomicExch(a.err, 1);
+      int never = 0;
+      mma_commit(leader, &drained);  // the MMAs in flight end before the memory is given back
+      mbar_wait(&drained, 0, &never);
+    }
+  } else if (warp < 10) {
+    // epilogue: lane = pixel of a block; the two groups of four warps take a
+    // pixel block each (MT = 2) or alternate channel groups (MT = 1); 16
+    // output channels at a time
+    const int q = warp & 3, grp = (warp - 2) >> 2;
     const int row = q * 32 + lane, py = row >> 3, px = row & 7;
+    const int m = MT == 2 ? grp : 0;
+    const int c_first = MT == 2 ? 0 : grp * 16, c_step = MT == 2 ? 16 : 32;
     const int o0 = blockIdx.y * a.NT;
     int it = 0;
     for (int t = blockIdx.x; t < a.tiles; t += gridDim.x, it++) {
       const int acc = it & 1;
+      const int n = t / (a.tiles_x * a.tiles_y), r = t - n * (a.tiles_x * a.tiles_y);
+      const int ty = r / a.tiles_x, tx = r - ty * a.tiles_x;
+      const int i = ty * S::kH + py, j = tx * S::kW + m * 8 + px;
+      const bool in = i < a.H && j < a.W;
+      const int64_t pix = in ? static_cast<int64_t>((n * a.H + i) * a.W + j) : 0;
       if (!mbar_wait(&full_d[acc], (it >> 1) & 1, &gave_up)) {
         gave_up = 1;
         atomicExch(a.err, 1);
@@ -376,49 +448,58 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_halo_tc(const __grid_con
       }
       __syncwarp();
       fence_after();
-      const int n = t / (a.tiles_x * a.tiles_y), r = t - n * (a.tiles_x * a.tiles_y);
-      const int ty = r / a.tiles_x, tx = r - ty * a.tiles_x;
-      const int i = ty * S::kH + py;
+      const uint32_t col = tmem + (static_cast<uint32_t>(q * 32) << 16) +
+                           static_cast<uint32_t>((acc * MT + m) * a.NT);
+      for (int c = c_first; c < a.NT; c += c_step) {
+        const int o = o0 + c;
+        const bool st0 = in && o < a.cos, st1 = in && o + 8 < a.cos;
+        uint4 mk[2];
+        if (a.mask) {
+          const uint4 *mp = reinterpret_cast<const uint4 *>(a.mask + pix * a.cos + o);
+          if (st0) mk[0] = mp[0];
+          if (st1) mk[1] = mp[1];
+        }
+        uint32_t v[16];
+        tmem_ld16(col + c, v);
+        tmem_wait_ld();
+        // channels beyond the layer's have zero weights and bias: zeros
+        float f[16];
 #pragma unroll
-      for (int m = 0; m < MT; m++) {
-        const int j = tx * S::kW + m * 8 + px;
-        const bool in = i < a.H && j < a.W;
-        const int64_t pix = in ? static_cast<int64_t>((n * a.H + i) * a.W + j) : 0;
-        for (int c = 0; c < a.NT; c += 16) {
-          uint32_t v[16];
-          tmem_ld16(tmem + (static_cast<uint32_t>(q * 32) << 16) +
-                        static_cast<uint32_t>((acc * MT + m) * a.NT + c),
-                    v);
-          tmem_wait_ld();
+        for (int e = 0; e < 16; e += 4) {
+          const float4 b4 = *reinterpret_cast<const float4 *>(&bias[c + e]);
+          f[e] = __uint_as_float(v[e]) + b4.x;
+          f[e + 1] = __uint_as_float(v[e + 1]) + b4.y;
+          f[e + 2] = __uint_as_float(v[e + 2]) + b4.z;
+          f[e + 3] = __uint_as_float(v[e + 3]) + b4.w;
+        }
+        if (a.relu) {
 #pragma unroll
-          for (int h = 0; h < 2; h++) {
-            const int o = o0 + c + 8 * h;
-            if (!in || o >= a.cos) continue;
-            uint4 mk = make_uint4(0x3F803F80u, 0x3F803F80u, 0x3F803F80u, 0x3F803F80u);
-            if (a.mask) mk = *reinterpret_cast<const uint4 *>(a.mask + pix * a.cos + o);
-            const uint32_t mw[4] = {mk.x, mk.y, mk.z, mk.w};
-            uint32_t out[4];
+          for (int e = 0; e < 16; e++) f[e] = fmaxf(f[e], 0.f);
+        }
+        uint32_t w[8];
 #pragma unroll
-            for (int e = 0; e < 8; e += 2) {
-              __nv_bfloat16 w[2];
+        for (int e = 0; e < 8; e++) {
+          const __nv_bfloat162 b2 = __floats2bfloat162_rn(f[2 * e], f[2 * e + 1]);
+          w[e] = *reinterpret_cast<const uint32_t *>(&b2);
+        }
+        if (a.mask) {
+          const uint32_t g[8] = {mk[0].x, mk[0].y, mk[0].z, mk[0].w,
+                                 mk[1].x, mk[1].y, mk[1].z, mk[1].w};
 #pragma unroll
-              for (int s = 0; s < 2; s++) {
-                float f = __uint_as_float(v[8 * h + e + s]);
-                const bool real = o + e + s < a.co;
-                if (a.bias && real) f += a.bias[o + e + s];
-                if (a.relu) f = fmaxf(f, 0.f);
-                const __nv_bfloat16 mm = __ushort_as_bfloat16(
-                    static_cast<unsigned short>(s ? mw[e / 2] >> 16 : mw[e / 2] & 0xFFFFu));
-                if (!real || !(__bfloat162float(mm) > 0.f)) f = 0.f;
-                w[s] = __float2bfloat16_rn(f);
-                if (a.yf && real) a.yf[pix * a.co + o + e + s] = __bfloat162float(w[s]);
-              }
-              out[e / 2] = static_cast<uint32_t>(__bfloat16_as_ushort(w[0])) |
-                           (static_cast<uint32_t>(__bfloat16_as_ushort(w[1])) << 16);
-            }
-            *reinterpret_cast<uint4 *>(a.y + pix * a.cos + o) =
-                make_uint4(out[0], out[1], out[2], out[3]);
+          for (int e = 0; e < 8; e++) {
+            if (!(__uint_as_float(g[e] << 16) > 0.f)) w[e] &= 0xFFFF0000u;
+            if (!(__uint_as_float(g[e] & 0xFFFF0000u) > 0.f)) w[e] &= 0xFFFFu;
           }
+        }
+        uint4 *yp = reinterpret_cast<uint4 *>(a.y + pix * a.cos + o);
+        if (st0) yp[0] = make_uint4(w[0], w[1], w[2], w[3]);
+        if (st1) yp[1] = make_uint4(w[4], w[5], w[6], w[7]);
+        if (a.yf && in) {
+#pragma unroll
+          for (int e = 0; e < 16; e++)
+            if (o + e < a.co)
+              a.yf[pix * a.co + o + e] =
+                  __uint_as_float(e & 1 ? w[e / 2] & 0xFFFF0000u : w[e / 2] << 16);
         }
       }
       fence_before();
@@ -426,7 +507,15 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_halo_tc(const __grid_con
     }
   } else {
     // image tiles
-    const int tid = threadIdx.x - 192;
+    // lane groups of `lanes` threads copy neighbouring slabs of a pixel (the
+    // power of two that divides a part's slabs), then the slabs `lanes` on;
+    // a thread's pixels are `pstep` apart, so its coordinates advance by
+    // additions
+    const int tid = threadIdx.x - 320;
+    const int lanes = 1 << a.lanes_log2, g8 = tid & (lanes - 1);
+    const int pix0 = tid >> a.lanes_log2, pstep = kLoadThreads >> a.lanes_log2;
+    const int dy = pstep / S::kWp, dx = pstep - dy * S::kWp;
+    const int y0 = pix0 / S::kWp, x0 = pix0 - y0 * S::kWp;
     int sa = 0, it = 0;
     uint32_t pa = 0;
     bool ok = true;
@@ -441,41 +530,67 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_halo_tc(const __grid_con
           ok = false;
           break;
         }
-        const uint32_t dst = base_a + sa * stride_a;
         const int k8 = min(a.p8, a.k8 - p * a.p8);
-        const uint32_t magic = p + 1 < a.parts ? a.magic : a.magic_last;
-        for (int e = tid; e < S::kPix * k8; e += 128) {
-          const int pix = static_cast<int>(__umulhi(static_cast<uint32_t>(e), magic));
-          const int s8 = e - pix * k8, c8 = p * a.p8 + s8;
-          const int y = pix / S::kWp, x = pix - y * S::kWp;
-          const int i = i0 + y, j = j0 + x;
-          const bool in = i >= 0 && i < a.H && j >= 0 && j < a.W && c8 < a.x.n8;
-          cp_async16(dst + s8 * S::kSlab + pix * 16,
-                     in ? input_at(a.x, n, i, j, a.H, a.W, c8) : a.x.xa, in);
+        // (a copy instruction whose 16-byte pieces scatter over slabs takes about
+        // 36 cycles whatever the order of the arithmetic: batches of pixels were
+        // no faster)
+        constexpr int kBatch = 1;
+        int y = y0, x = x0;
+        uint32_t dst = base_a + sa * stride_a + pix0 * 16 + g8 * S::kSlab;
+        const int Wa = a.W >> a.x.up, rows = n * (a.H >> a.x.up);
+        const int first = (n * a.H + i0) * a.W + j0, c0 = p * a.p8 + g8;
+        const bool plain = !a.x.up && a.x.n8 == a.x.n8a;  // one source at full resolution
+        for (int pix = pix0; pix < S::kPix; pix += kBatch * pstep) {
+          const __nv_bfloat16 *pa8[kBatch], *pb8[kBatch];
+          bool in[kBatch];
+#pragma unroll
+          for (int q = 0; q < kBatch; q++) {
+            const int i = i0 + y, j = j0 + x;
+            in[q] = static_cast<unsigned>(i) < static_cast<unsigned>(a.H) &&
+                    static_cast<unsigned>(j) < static_cast<unsigned>(a.W);
+            const int here = first + y * a.W + x;
+            pa8[q] = a.x.xa;
+            pb8[q] = a.x.xa;
+            if (in[q]) {
+              pa8[q] += static_cast<int64_t>(
+                            plain ? here : (rows + (i >> a.x.up)) * Wa + (j >> a.x.up)) *
+                            a.x.sa +
+                        c0 * 8;
+              if (!plain)
+                pb8[q] = a.x.xb + static_cast<int64_t>(here) * a.x.sb + (c0 - a.x.n8a) * 8;
+            }
+            y += dy;
+            x += dx;
+            if (x >= S::kWp) {
+              x -= S::kWp;
+              y++;
+            }
+          }
+          uint32_t d = dst;
+          for (int s8 = 0; s8 + g8 < k8; s8 += lanes) {
+            const bool slab = c0 + s8 < a.x.n8, from_a = c0 + s8 < a.x.n8a;
+#pragma unroll
+            for (int q = 0; q < kBatch; q++) {
+              const bool valid = in[q] && slab;
+              if (pix + q * pstep < S::kPix)
+                cp_async16(d + q * pstep * 16,
+                           valid ? (from_a ? pa8[q] : pb8[q]) + s8 * 8 : a.x.xa, valid);
+            }
+            d += lanes * S::kSlab;
+          }
+          dst += kBatch * pstep * 16;
         }
-        cp_async_commit();
-        if (a.stages_a == 1) {
-          cp_async_wait<0>();
-          fence_async_proxy();
-          mbar_arrive(&full_a[sa]);
-        } else if (it > 0) {  // the copies before these have landed
-          cp_async_wait<1>();
-          fence_async_proxy();
-          mbar_arrive(&full_a[sa ? sa - 1 : a.stages_a - 1]);
-        }
+        cp_async_arrive(&full_a[sa]);
         if (++sa == a.stages_a) {
           sa = 0;
           pa ^= 1u;
         }
       }
     }
-    cp_async_wait<0>();
+    cp_async_wait_all();
     if (!ok) {
       gave_up = 1;
       atomicExch(a.err, 1);
-    } else if (a.stages_a > 1 && it > 0) {
-      fence_async_proxy();
-      mbar_arrive(&full_a[sa ? sa - 1 : a.stages_a - 1]);
     }
   }
   __syncwarp();
@@ -499,7 +614,8 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_halo_tc(const __grid_con
 // kRep (few input channels): M = 3 x channels, the three horizontal taps of
 // a row at once -- the tile is stored three times, shifted, and one
 // accumulator per vertical tap remains.
-constexpr int kWgThreads = 160;
+constexpr int kWgLoaders = 256;  // of which the first 128 also read the sums back
+constexpr int kWgThreads = kWgLoaders + 32;
 constexpr int kWgStages = 3;
 
 struct WgradDev {
@@ -510,6 +626,7 @@ struct WgradDev {
   int m_blocks, groups, group_taps;
   int tiles_x, tiles_y, tiles, splits;
   int stages;
+  int lanes_x, lanes_g;           // log2 of the threads that share a pixel's copies
   uint32_t tmem_cols;
   float *partials;
   int64_t len;                    // KS^2 ci co + co
@@ -533,7 +650,8 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc(const __grid_constant_
   __shared__ uint64_t full[kWgStages], empty[kWgStages], done;
   __shared__ uint32_t tmem_slot;
   __shared__ int gave_up;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x;
+  const int warp = __shfl_sync(0xFFFFFFFFu, static_cast<int>(threadIdx.x >> 5), 0);
+  const int lane = threadIdx.x & 31, tid = threadIdx.x;
   const int n8g = a.NT / 8;
   const uint32_t stage_bytes = (S::kBytesX + n8g * S::kSlabG + 127u) & ~127u;
   const uint32_t ones = smem_addr(dyn), base = ones + 4096u;
@@ -551,7 +669,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc(const __grid_constant_
   const int t1 = static_cast<int>(static_cast<int64_t>(a.tiles) * (blockIdx.y + 1) / a.splits);
   if (tid == 0) {
     for (int i = 0; i < kWgStages; i++) {
-      mbar_init(&full[i], 128);
+      mbar_init(&full[i], kWgLoaders);
       mbar_init(&empty[i], 1);
     }
     mbar_init(&done, 1);
@@ -562,64 +680,80 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc(const __grid_constant_
     *reinterpret_cast<uint4 *>(dyn + e * 16) =
         make_uint4(0x3F803F80u, 0x3F803F80u, 0x3F803F80u, 0x3F803F80u);
   fence_async_proxy();
-  if (warp == 4) tmem_alloc(&tmem_slot, a.tmem_cols);
+  if (warp == 8) tmem_alloc(&tmem_slot, a.tmem_cols);
   fence_before();
   __syncthreads();
   fence_after();
-  const uint32_t tmem = tmem_slot;
+  const uint32_t tmem = __shfl_sync(0xFFFFFFFFu, tmem_slot, 0);
 
-  if (warp == 4) {
-    if (lane == 0) {
-      const uint32_t idesc = umma_idesc(a.NT, true);
-      bool ok = true;
-      int st = 0;
-      uint32_t ph = 0;
-      for (int t = t0; t < t1; t++) {
-        if (!mbar_wait(&full[st], ph, &gave_up)) {
-          ok = false;
-          break;
-        }
-        fence_after();
-        const uint32_t sx = base + st * stage_bytes, sg = sx + S::kBytesX;
+  chain_wait();
+  if (warp == 8) {
+    const uint32_t leader = elect_leader();
+    const uint32_t idesc = umma_idesc(a.NT, true);
+    const uint32_t ahi = desc_hi(S::kSlabX), bhi = desc_hi(S::kSlabG);
+    const uint32_t ones_lo = desc_lo(ones, 128u), ones_hi = desc_hi(256u);
+    const uint32_t bias_d = tmem + a.group_taps * a.NT;
+    bool ok = true;
+    int st = 0;
+    uint32_t ph = 0, acc = 0;
+    for (int t = t0; t < t1; t++) {
+      if (!mbar_wait(&full[st], ph, &gave_up)) {
+        ok = false;
+        break;
+      }
+      fence_async_proxy();  // the landed copies, for the MMAs
+      fence_after();
+      const uint32_t sx = base + st * stage_bytes;
+      // 16 pixels (two rows of the tile) per MMA
+      uint32_t xlo = desc_lo(sx, S::kWp * 16u);
+      uint32_t glo = desc_lo(sx + S::kBytesX, 128u);
 #pragma unroll 1
-        for (int k = 0; k < 8; k++) {  // 16 pixels: two rows of the tile
-          const uint64_t bd = umma_desc(sg + k * 256u, 128u, S::kSlabG);
-          const bool acc = t > t0 || k > 0;
-          for (int j = 0; j < ntap; j++) {
-            const int tap = tap0 + j;
-            const int dy = kRep ? tap : tap / KS, dx = kRep ? 0 : tap % KS;
-            const uint64_t ad = umma_desc(
-                sx + static_cast<uint32_t>((dy + 2 * k) * S::kWp + dx) * 16u, S::kWp * 16u,
-                S::kSlabX);
-            mma_bf16(tmem + j * a.NT, ad, bd, idesc, acc);
-          }
-          if (with_bias)
-            mma_bf16(tmem + a.group_taps * a.NT, umma_desc(ones, 128u, 256u), bd, idesc, acc);
+      for (int k = 0; k < 8; k++) {
+        // taps tap0 .. tap0 + ntap - 1 (vertical taps where kRep)
+#pragma unroll
+        for (int tap = 0; tap < (kRep ? KS : KS * KS); tap++) {
+          const int j = tap - tap0;
+          if (j >= 0 && j < ntap)
+            mma_bf16(leader, tmem + j * a.NT,
+                     xlo + (kRep ? tap * S::kWp : (tap / KS) * S::kWp + tap % KS), ahi, glo, bhi,
+                     idesc, acc);
         }
-        mma_commit(&empty[st]);
-        if (++st == a.stages) {
-          st = 0;
-          ph ^= 1u;
-        }
+        if (with_bias) mma_bf16(leader, bias_d, ones_lo, ones_hi, glo, bhi, idesc, acc);
+        acc = 1;
+        xlo += 2 * S::kWp;
+        glo += 16;
       }
-      mma_commit(&done);
-      if (!ok) {
-        gave_up = 1;
-        atomicExch(a.err, 1);
-        int never = 0;
-        mbar_wait(&done, 0, &never);
+      mma_commit(leader, &empty[st]);
+      if (++st == a.stages) {
+        st = 0;
+        ph ^= 1u;
       }
+    }
+    mma_commit(leader, &done);
+    if (!ok) {
+      gave_up = 1;
+      if (lane == 0) atomicExch(a.err, 1);
+      int never = 0;
+      mbar_wait(&done, 0, &never);
     }
     __syncwarp();
   } else {
     // loads: this block's input slabs, then the gradient's
     const int n8x = min(16, a.x.n8 - mb * 16);
-    const int units = kRep ? S::kHp * (8 + 2 * S::kHalo) * n8x : S::kPixX * n8x;
+    constexpr int kPix = S::kHp * (8 + 2 * S::kHalo);
     constexpr int rowp = 8 + 2 * S::kHalo;
-    // quotients by n8x and n8v (n8x may be 1: its reciprocal does not fit 32 bits)
-    const uint32_t mx = n8x > 1 ? 0xFFFFFFFFu / static_cast<uint32_t>(n8x) + 1u : 0u;
     const int n8v = min(n8g, (a.cos - o0) / 8);
-    const uint32_t mv = n8v > 1 ? 0xFFFFFFFFu / static_cast<uint32_t>(n8v) + 1u : 0u;
+    // as in conv_halo_tc: `lanes` threads share a pixel
+    const int lx = 1 << a.lanes_x, gx8 = tid & (lx - 1), px0 = tid >> a.lanes_x,
+              pxs = kWgLoaders >> a.lanes_x;
+    const int ly = 1 << a.lanes_g, gg8 = tid & (ly - 1), pg0 = tid >> a.lanes_g,
+              pgs = kWgLoaders >> a.lanes_g;
+    const int dyx = pxs / rowp, dxx = pxs - dyx * rowp;
+    const int yx0 = px0 / rowp, xx0 = px0 - yx0 * rowp;
+    // this block's slabs of the first source, and which sources it reads
+    const int n8xa = a.x.n8a - mb * 16;
+    const bool use_a = n8xa > 0, use_b = n8xa < n8x;
+    const uint32_t rep_stride = static_cast<uint32_t>(n8x) * S::kSlabX;
     bool ok = true;
     int st = 0, it = 0;
     uint32_t ph = 0;
@@ -631,53 +765,80 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc(const __grid_constant_
       const int n = t / (a.tiles_x * a.tiles_y), r = t - n * (a.tiles_x * a.tiles_y);
       const int ty = r / a.tiles_x, tx = r - ty * a.tiles_x;
       const uint32_t sx = base + st * stage_bytes, sg = sx + S::kBytesX;
-      for (int e = tid; e < units; e += 128) {
-        const int pix = n8x > 1 ? static_cast<int>(__umulhi(e, mx)) : e, c8 = e - pix * n8x;
-        const int y = pix / rowp, x = pix - y * rowp;
-        const int i = ty * 16 + y - S::kHalo, j = tx * 8 + x - S::kHalo;
-        const bool in = i >= 0 && i < a.H && j >= 0 && j < a.W;
-        const __nv_bfloat16 *src =
-            in ? input_at(a.x, n, i, j, a.H, a.W, mb * 16 + c8) : a.x.xa;
-        if constexpr (kRep) {
+      const int i0 = ty * 16 - S::kHalo, j0 = tx * 8 - S::kHalo;
+      const int first = (n * a.H + i0) * a.W + j0, rows = n * (a.H >> a.x.up);
+      constexpr int kBatch = kRep ? 1 : 4;  // pixels whose addresses are formed together
+      int y = yx0, x = xx0;
+      for (int pix = px0; pix < kPix; pix += kBatch * pxs) {
+        const __nv_bfloat16 *pa8[kBatch], *pb8[kBatch];
+        bool in[kBatch];
+        int at[kBatch], xq[kBatch];
 #pragma unroll
-          for (int dx = 0; dx < KS; dx++)
-            if (x >= dx && x < dx + 8)
-              cp_async16(sx + (dx * n8x + c8) * S::kSlabX + (y * 8 + x - dx) * 16, src, in);
-        } else {
-          cp_async16(sx + c8 * S::kSlabX + pix * 16, src, in);
+        for (int q = 0; q < kBatch; q++) {
+          in[q] = static_cast<unsigned>(i0 + y) < static_cast<unsigned>(a.H) &&
+                  static_cast<unsigned>(j0 + x) < static_cast<unsigned>(a.W);
+          pa8[q] = a.x.xa;
+          pb8[q] = a.x.xa;
+          const int here = first + y * a.W + x;
+          if (in[q]) {
+            if (use_a)
+              pa8[q] += static_cast<int64_t>(a.x.up ? (rows + ((i0 + y) >> 1)) * (a.W >> 1) +
+                                                          ((j0 + x) >> 1)
+                                                    : here) *
+                            a.x.sa +
+                        mb * 128;
+            if (use_b)
+              pb8[q] = a.x.xb + static_cast<int64_t>(here) * a.x.sb + (mb * 16 - a.x.n8a) * 8;
+          }
+          at[q] = kRep ? (y * 8 + x) * 16 : (pix + q * pxs) * 16;
+          xq[q] = x;
+          y += dyx;
+          x += dxx;
+          if (x >= rowp) {
+            x -= rowp;
+            y++;
+          }
+        }
+        for (int s8 = gx8; s8 < n8x; s8 += lx) {
+#pragma unroll
+          for (int q = 0; q < kBatch; q++) {
+            if (pix + q * pxs >= kPix) continue;
+            const __nv_bfloat16 *src = in[q] ? (s8 < n8xa ? pa8[q] : pb8[q]) + s8 * 8 : a.x.xa;
+            const uint32_t d = sx + s8 * S::kSlabX + at[q];
+            if constexpr (kRep) {
+#pragma unroll
+              for (int dx = 0; dx < KS; dx++)
+                if (static_cast<unsigned>(xq[q] - dx) < 8u)
+                  cp_async16(d + dx * rep_stride - dx * 16, src, in[q]);
+            } else {
+              cp_async16(d, src, in[q]);
+            }
+          }
         }
       }
-      for (int e = tid; e < 128 * n8v; e += 128) {
-        const int pix = n8v > 1 ? static_cast<int>(__umulhi(e, mv)) : e, c8 = e - pix * n8v;
+#pragma unroll 4
+      for (int pix = pg0; pix < 128; pix += pgs) {
         const int i = ty * 16 + (pix >> 3), j = tx * 8 + (pix & 7);
         const bool in = i < a.H && j < a.W;
-        cp_async16(sg + c8 * S::kSlabG + pix * 16,
-                   in ? a.gz + static_cast<int64_t>((n * a.H + i) * a.W + j) * a.cos + o0 + c8 * 8
-                      : a.gz,
-                   in);
+        const __nv_bfloat16 *src =
+            in ? a.gz + static_cast<int64_t>((n * a.H + i) * a.W + j) * a.cos + o0 : a.gz;
+        for (int s8 = gg8; s8 < n8v; s8 += ly)
+          cp_async16(sg + s8 * S::kSlabG + pix * 16, in ? src + s8 * 8 : a.gz, in);
       }
-      cp_async_commit();
-      if (it > 0) {
-        cp_async_wait<1>();
-        fence_async_proxy();
-        mbar_arrive(&full[st ? st - 1 : a.stages - 1]);
-      }
+      cp_async_arrive(&full[st]);
       if (++st == a.stages) {
         st = 0;
         ph ^= 1u;
       }
     }
-    cp_async_wait<0>();
+    cp_async_wait_all();
     if (!ok) {
       gave_up = 1;
       atomicExch(a.err, 1);
-    } else if (it > 0) {
-      fence_async_proxy();
-      mbar_arrive(&full[st ? st - 1 : a.stages - 1]);
     }
     // the sums of this split: lane = input channel (and horizontal tap)
-    const bool have = ok && mbar_wait(&done, 0, &gave_up);
-    if (!have) {
+    const bool have = ok && warp < 4 && mbar_wait(&done, 0, &gave_up);
+    if (!have && warp < 4) {
       gave_up = 1;
       atomicExch(a.err, 1);
     }
@@ -733,17 +894,34 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc(const __grid_constant_
   fence_before();
   __syncthreads();
   fence_after();
-  if (warp == 4) tmem_dealloc(tmem, a.tmem_cols);
+  if (warp == 8) tmem_dealloc(tmem, a.tmem_cols);
 }
 
-__global__ void __launch_bounds__(256) wgrad_reduce(const float *__restrict__ p, int splits,
-                                                    int64_t len, float *__restrict__ out) {
-  const int64_t e = static_cast<int64_t>(blockIdx.x) * 256 + threadIdx.x;
-  if (e >= len) return;
+// Sums the splits in a fixed order: group g of a CTA's G groups of threads
+// adds splits g, g + G, ... of its 256 / G outputs, then the groups' sums are
+// added in turn.  Many splits of few outputs need the groups to fill the GPU
+// (152 splits of 9 k outputs: 14 us with one group, 7 with eight), few splits
+// of many outputs lose by them (12 of 590 k: 10 against 24 us).
+template <int G>
+__global__ void __launch_bounds__(256) wgrad_reduce(const float *p, int splits, int64_t len,
+                                                    float *out) {
+  constexpr int kOut = 256 / G;
+  __shared__ float sh[G][kOut];
+  chain_wait();
+  const int g = threadIdx.x / kOut, o = threadIdx.x % kOut;
+  const int64_t e = static_cast<int64_t>(blockIdx.x) * kOut + o;
   float s = 0.f;
-#pragma unroll 8
-  for (int k = 0; k < splits; k++) s += p[k * len + e];
-  out[e] = s;
+  if (e < len) {
+#pragma unroll 4
+    for (int k = g; k < splits; k += G) s += p[k * len + e];
+  }
+  if constexpr (G > 1) {
+    sh[g][o] = s;
+    __syncthreads();
+    if (g == 0)
+      for (int k = 1; k < G; k++) s += sh[k][o];
+  }
+  if (g == 0 && e < len) out[e] = s;
 }
 
 // Packed weights: [output tile][tap][chunk of 64 channels][slab][output][8].
@@ -814,8 +992,9 @@ cudaError_t conv_launch(ConvDev d, int sms, cudaStream_t s) {
   d.parts = d.k8 <= fit ? 1 : (d.k8 + fit - 1) / fit;
   d.p8 = d.parts == 1 ? d.k8 : fit;
   const int last = d.k8 - (d.parts - 1) * d.p8;
-  d.magic = static_cast<uint32_t>((uint64_t(1) << 32) / d.p8 + 1);
-  d.magic_last = static_cast<uint32_t>((uint64_t(1) << 32) / last + 1);
+  d.lanes_log2 = 1;  // both are even
+  while (d.lanes_log2 < 5 && (d.p8 >> d.lanes_log2) % 2 == 0 && (last >> d.lanes_log2) % 2 == 0)
+    d.lanes_log2++;
   const int sa_bytes = (d.p8 * static_cast<int>(S::kSlab) + 127) / 128 * 128;
   d.unit_taps = d.parts == 1 ? KS * KS : 1;
   const int blocks =
@@ -830,11 +1009,11 @@ cudaError_t conv_launch(ConvDev d, int sms, cudaStream_t s) {
                           : std::min({blocks, 8, (kSmemMax - d.stages_a * sa_bytes) / b_bytes});
   if (d.stages_b < 1) return cudaErrorInvalidValue;
   d.tmem_cols = pow2_cols(2 * MT * d.NT);
-  // more than half of an SM's shared memory: one CTA per SM, so that its
-  // tensor memory is the CTA's alone
-  const int smem = std::max(d.stages_a * sa_bytes + d.stages_b * b_bytes, 120 * 1024);
-  conv_halo_tc<KS, MT><<<dim3(gx, n_blocks), kConvThreads, smem, s>>>(d);
-  return cudaGetLastError();
+  // where the CTA takes more than half of tensor memory: more than half of
+  // shared memory too, so that no other CTA waits beside it
+  const int smem = std::max(d.stages_a * sa_bytes + d.stages_b * b_bytes,
+                            d.tmem_cols > 256 ? 120 * 1024 : 0);
+  return launch_chained(conv_halo_tc<KS, MT>, dim3(gx, n_blocks), kConvThreads, smem, s, d);
 }
 
 struct WgPlan {
@@ -848,7 +1027,7 @@ void wg_smem(WgPlan *p) {
   using S = WgShape<KS, kRep>;
   const int stage = (static_cast<int>(S::kBytesX + p->NT / 8 * S::kSlabG) + 127) / 128 * 128;
   p->stages = std::min(kWgStages, (kSmemMax - 4096) / stage);
-  p->smem = std::max(4096 + p->stages * stage, 120 * 1024);
+  p->smem = std::max(4096 + p->stages * stage, p->cols > 256 ? 120 * 1024 : 0);
 }
 WgPlan wg_plan(int ks, int ci_padded, int co, int N, int H, int W, int sms) {
   WgPlan p;
@@ -958,19 +1137,32 @@ cudaError_t launch_wgrad_tc(const ConvInput &in, int ks, const __nv_bfloat16 *gz
   d.splits = p.splits;
   d.stages = p.stages;
   d.tmem_cols = p.cols;
+  // as many threads as a block has slabs, at most 16, as a power of two
+  auto log2_floor = [](int v) {
+    int l = 0;
+    while (l < 4 && (2 << l) <= v) l++;
+    return l;
+  };
+  d.lanes_x = log2_floor(std::min(16, in.padded() / 8));
+  d.lanes_g = log2_floor(std::min(p.NT, d.cos) / 8);
   d.partials = partials;
   d.len = static_cast<int64_t>(ks) * ks * d.ci * co + co;
   d.err = err;
   if (p.stages < 2) return cudaErrorInvalidValue;
   const dim3 grid(p.n_blocks * p.m_blocks * p.groups, p.splits);
-  if (ks == 3 && p.rep) wgrad_tc<3, true><<<grid, kWgThreads, p.smem, s>>>(d);
-  else if (ks == 3) wgrad_tc<3, false><<<grid, kWgThreads, p.smem, s>>>(d);
-  else wgrad_tc<1, false><<<grid, kWgThreads, p.smem, s>>>(d);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = ks != 3 ? launch_chained(wgrad_tc<1, false>, grid, kWgThreads, p.smem, s, d)
+                  : p.rep ? launch_chained(wgrad_tc<3, true>, grid, kWgThreads, p.smem, s, d)
+                          : launch_chained(wgrad_tc<3, false>, grid, kWgThreads, p.smem, s, d);
   if (e != cudaSuccess) return e;
-  wgrad_reduce<<<static_cast<unsigned>((d.len + 255) / 256), 256, 0, s>>>(partials, p.splits, d.len,
-                                                                           dw);
-  return cudaGetLastError();
+  auto reduce = [&](auto groups) {
+    constexpr int G = decltype(groups)::value;
+    return launch_chained(wgrad_reduce<G>,
+                          dim3(static_cast<unsigned>((d.len + 256 / G - 1) / (256 / G))), 256, 0, s,
+                          static_cast<const float *>(partials), p.splits, d.len, dw);
+  };
+  if (p.splits >= 64) return reduce(std::integral_constant<int, 8>());
+  if (p.splits >= 32) return reduce(std::integral_constant<int, 2>());
+  return reduce(std::integral_constant<int, 1>());
 }
 
 }  // namespace net
