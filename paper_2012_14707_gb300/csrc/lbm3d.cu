@@ -40,6 +40,11 @@ namespace lbm3 {
 
 constexpr int Q = 19;
 constexpr uint32_t kSolid3 = 0xFFFFFFFFu;
+// an entry of the fluid-node list: the node's index, and its flag word (bits
+// 1..18) with the node's first link, counted from its group of 32 entries'
+// first, in the bits above
+constexpr uint32_t kFlags3 = (1u << 19) - 1u;
+constexpr int kRank3 = 19;
 constexpr int kThreads3 = 128;
 constexpr int kResBlocks3 = 2048;
 constexpr int kResThreads3 = 256;
@@ -100,7 +105,7 @@ __host__ __device__ constexpr int rep3(int p) {
   return t[p];
 }
 
-constexpr int norm3(int r) {
+__host__ __device__ constexpr int norm3(int r) {
   int s = 0;
   for (int q = 0; q < Q; q++) s += m3(r, q) * m3(r, q);
   return s;
@@ -152,6 +157,24 @@ const Lattice &lattice() {
   return L;
 }
 
+// p / d for 0 <= p < 2^31 by a multiplication (Granlund and Montgomery
+// 1994): m = ceil(2^(31 + l) / d) with 2^l >= d, the quotient the product's
+// bits from 31 + l up; m = 0 stands for d = 1.
+struct DivBy3 {
+  uint32_t m = 0, shift = 0;
+  DivBy3() = default;
+  explicit DivBy3(uint32_t d) {
+    uint32_t l = 0;
+    while ((uint64_t(1) << l) < d) l++;
+    if (l == 0) return;
+    m = static_cast<uint32_t>(((uint64_t(1) << (31 + l)) + d - 1) / d);
+    shift = l - 1;
+  }
+  __device__ __forceinline__ uint32_t operator()(uint32_t p) const {
+    return m ? __umulhi(p, m) >> shift : p;
+  }
+};
+
 // Kernel constants of one case (passed by value): the relaxation rates
 // s_k and forcing weights 1 - s_k/2 of the 19 moments, each divided by
 // |M_k|^2 (the scale of M^-1 = M^T diag(1/|M_k|^2)).
@@ -160,6 +183,7 @@ struct Const3 {
   C s_scaled[Q], f_scaled[Q];
   C ax, ay, az;
   int32_t nx, ny, nz, px, py, pz;
+  DivBy3 by_nx, by_ny;
   int32_t diffuse_mode;
   int64_t plane;    // N
   int64_t n_links;  // the exact-mass variant: where the per-node carries start
@@ -184,10 +208,9 @@ struct Coord3 {
 };
 template <typename C>
 __device__ __forceinline__ Coord3 coord3(const Const3<C> &k, int64_t p) {
-  const unsigned u = static_cast<unsigned>(p), row = u / static_cast<unsigned>(k.nx);
+  const unsigned u = static_cast<unsigned>(p), row = k.by_nx(u), z = k.by_ny(row);
   return Coord3{static_cast<int>(u - row * static_cast<unsigned>(k.nx)),
-                static_cast<int>(row % static_cast<unsigned>(k.ny)),
-                static_cast<int>(row / static_cast<unsigned>(k.ny))};
+                static_cast<int>(row - z * static_cast<unsigned>(k.ny)), static_cast<int>(z)};
 }
 
 // Slot of f_q(x, t) for node p (pull layout): the neighbour x - c_q's own
@@ -244,49 +267,77 @@ struct Warp3 {
   C v[kLinkVals3][33];
 };
 
-// Double-FP32 numbers (about 48 significant bits from FP32 operations) with
-// the arithmetic operators, so that the exact-mass variant's moments
-// (exact_moments3) read as the FP32 code does and mac3 serves them too.
-// This GPU runs FP64 at a small fraction of its FP32 rate; the operations
-// are those of lbm::dev::DF.  Its own namespace keeps its fma out of the
-// ordinary lookup of float and double code (argument-dependent lookup finds
-// it for D2).
-namespace df {
-struct D2 {
-  float h, l;
-  D2() = default;
-  __host__ __device__ constexpr D2(float hi, float lo) : h(hi), l(lo) {}
-  __host__ __device__ explicit constexpr D2(double x)
-      : h(static_cast<float>(x)), l(static_cast<float>(x - static_cast<double>(static_cast<float>(x)))) {}
-};
-__device__ __forceinline__ lbm::dev::DF dv(D2 a) { return lbm::dev::DF{a.h, a.l}; }
-__device__ __forceinline__ D2 d2(lbm::dev::DF a) { return D2(a.h, a.l); }
-__device__ __forceinline__ D2 operator+(D2 a, D2 b) { return d2(lbm::dev::df_add(dv(a), dv(b))); }
-__device__ __forceinline__ D2 operator-(D2 a, D2 b) {
-  return d2(lbm::dev::df_add(dv(a), lbm::dev::DF{-b.h, -b.l}));
-}
-__device__ __forceinline__ D2 operator*(D2 a, D2 b) { return d2(lbm::dev::df_mul(dv(a), dv(b))); }
-__device__ __forceinline__ D2 operator/(D2 a, D2 b) { return d2(lbm::dev::df_div(dv(a), dv(b))); }
-__device__ __forceinline__ D2 &operator+=(D2 &a, D2 b) { return a = a + b; }
-__device__ __forceinline__ D2 fma(D2 a, D2 b, D2 c) { return a * b + c; }
-}  // namespace df
-using df::D2;
-
 // lattice weight of direction q in the arithmetic type A
 template <typename A>
 __device__ __forceinline__ A wq3(int q) {
   return w3<A>(q);
 }
-template <>
-__device__ __forceinline__ D2 wq3<D2>(int q) {
-  return D2(q == 0 ? 1.0 / 3.0 : (q < 7 ? 1.0 / 18.0 : 1.0 / 36.0));
+
+// The second half of the collision: from d - d_eq as pair sums (NS) and
+// differences (NA) plus the rest direction's (n0), rho, u and the body force
+// a, the change ch[q] = f'_q - f_q (ch[0] = 0):
+// m' - m = -s (m - m_eq) + (1 - s/2) M Fbar, scaled by 1/|M_k|^2.  M Fbar
+// has a closed form (F = rho a; the moments of Eq. LBEforce): e 38 u.F, eps
+// -11 u.F, j F, q -2/3 F, 3p_xx 2 (3 u_x F_x - u.F), p_ww 2 (u_y F_y -
+// u_z F_z), the fourth-order ones -1/2 of these, p_ab u_a F_b + u_b F_a, m 0.
+// rho does not change and j changes by F exactly, for any s_j, since rho u =
+// j + F/2: taken as such.  (Formed from d - d_eq like the other rows, j came
+// out as F plus rho u times the rounding of the equilibrium's weights, 1e-8
+// every step.)
+template <typename A>
+__device__ __forceinline__ void transform3(const A n0, const A (&NS)[kPairs3],
+                                           const A (&NA)[kPairs3], const A rho, const A (&u)[3],
+                                           const Const3<A> &k, A (&ch)[Q]) {
+  const A F[3] = {rho * k.ax, rho * k.ay, rho * k.az};
+  const A uF[3] = {u[0] * F[0], u[1] * F[1], u[2] * F[2]};
+  const A uf = uF[0] + uF[1] + uF[2];
+  const A pxx = A(2) * (A(3) * uF[0] - uf), pww = A(2) * (uF[1] - uF[2]);
+  const A b[Q] = {A(0), A(38) * uf, A(-11) * uf,
+                  A(0), A(-2.0 / 3.0) * F[0], A(0), A(-2.0 / 3.0) * F[1],
+                  A(0), A(-2.0 / 3.0) * F[2],
+                  pxx, A(-0.5) * pxx, pww, A(-0.5) * pww,
+                  u[0] * F[1] + u[1] * F[0], u[1] * F[2] + u[2] * F[1], u[0] * F[2] + u[2] * F[0],
+                  A(0), A(0), A(0)};
+  A dm[Q];
+#pragma unroll
+  for (int r = 1; r < Q; r++) {
+    if (r == 3 || r == 5 || r == 7) {
+      dm[r] = A(1.0 / norm3(3)) * F[(r - 3) / 2];
+      continue;
+    }
+    A a = A(0);
+    if (!odd_row3(r)) a = mac3(a, m3(r, 0), n0);
+#pragma unroll
+    for (int pp = 0; pp < kPairs3; pp++) a = mac3(a, m3(r, rep3(pp)), odd_row3(r) ? NA[pp] : NS[pp]);
+    dm[r] = r >= 16 ? -k.s_scaled[r] * a : k.f_scaled[r] * b[r] - k.s_scaled[r] * a;
+  }
+  // f' - f = M^T dm: even rows give the same change to q and opp q, odd
+  // rows opposite ones
+  ch[0] = A(0);
+#pragma unroll
+  for (int pp = 0; pp < kPairs3; pp++) {
+    const int q = rep3(pp), qb = opp3(q);
+    A ev = A(0), od = A(0);
+#pragma unroll
+    for (int r = 1; r < Q; r++) {
+      if (odd_row3(r)) od = mac3(od, m3(r, q), dm[r]);
+      else ev = mac3(ev, m3(r, q), dm[r]);
+    }
+    ch[q] = ev + od;
+    ch[qb] = ev - od;
+  }
 }
 
+// v / r by r's reciprocal and one correction from the exact remainder (the
+// correctly rounded quotient, but for rare last-place ties): three divisions
+// by the same density cost one.
+__device__ __forceinline__ float recip3(float r) { return __frcp_rn(r); }
+__device__ __forceinline__ double recip3(double r) { return 1.0 / r; }
 template <typename A>
-__device__ __forceinline__ void transform3(const A n0, const A F0, const A (&NS)[kPairs3],
-                                           const A (&NA)[kPairs3], const A (&FS)[kPairs3],
-                                           const A (&FA)[kPairs3], const Const3<A> &k,
-                                           A (&ch)[Q]);
+__device__ __forceinline__ A quotient3(A v, A r, A inv) {
+  const A q = v * inv;
+  return fma(fma(-q, r, v), inv, q);
+}
 
 // The collision change f' - f of one node from its deviations d (Eq.
 // FluidMacr, Eq. LBEequi, Eq. LBEforce, Eq. MomentPost through M^-1), in
@@ -313,69 +364,30 @@ __device__ __forceinline__ void collide3(const A (&d)[Q], const Const3<A> &k, A 
 #pragma unroll
     for (int pp = 0; pp < kPairs3; pp++) j[a] = mac3(j[a], cvel3(rep3(pp), a), D[pp]);
   rho = A(1) + drho;
-  u[0] = (j[0] + A(0.5) * rho * k.ax) / rho;
-  u[1] = (j[1] + A(0.5) * rho * k.ay) / rho;
-  u[2] = (j[2] + A(0.5) * rho * k.az) / rho;
+  const A inv = recip3(rho), half = A(0.5) * rho;
+  u[0] = quotient3(fma(half, k.ax, j[0]), rho, inv);
+  u[1] = quotient3(fma(half, k.ay, j[1]), rho, inv);
+  u[2] = quotient3(fma(half, k.az, j[2]), rho, inv);
   const A ux = u[0], uy = u[1], uz = u[2];
-  const A uu = ux * ux + uy * uy + uz * uz, ua = ux * k.ax + uy * k.ay + uz * k.az;
-  // d - d_eq (Eq. LBEequi) and Fbar (Eq. LBEforce), as pair sums (S) and
-  // differences (A); the rest direction alone
-  A NS[kPairs3], NA[kPairs3], FS[kPairs3], FA[kPairs3];
-  const A n0 = d[0] - wq3<A>(0) * (drho - A(1.5) * rho * uu);
-  const A F0 = A(-3) * wq3<A>(0) * rho * ua;
+  const A uu = ux * ux + uy * uy + uz * uz;
+  // d - d_eq (Eq. LBEequi), as pair sums and differences; the rest
+  // direction alone.  Per pair of weight w: the sum's 2 w (rho - 1 + rho (9/2
+  // (c.u)^2 - 3/2 u.u)), the difference's 6 w rho c.u.  (The sum's terms
+  // common to all pairs are not formed once and shared: their one rounding
+  // would lean the same way in every pair, and the velocity error of the
+  // sphere pack tripled.)
+  A NS[kPairs3], NA[kPairs3];
+  const A uu15 = A(-1.5) * uu;
+  const A n0 = d[0] - wq3<A>(0) * fma(rho, uu15, drho);
+  const A ga = A(1.0 / 3) * rho, gd = A(0.5) * ga;     // 6 w rho
 #pragma unroll
   for (int pp = 0; pp < kPairs3; pp++) {
     const int q = rep3(pp);
     const A cu = mac3(mac3(mac3(A(0), cvel3(q, 0), ux), cvel3(q, 1), uy), cvel3(q, 2), uz);
-    const A ca = mac3(mac3(mac3(A(0), cvel3(q, 0), k.ax), cvel3(q, 1), k.ay), cvel3(q, 2), k.az);
-    const A wr = wq3<A>(q) * rho;
-    NS[pp] = S[pp] - A(2) * wq3<A>(q) * (drho + rho * (A(4.5) * cu * cu - A(1.5) * uu));
-    NA[pp] = D[pp] - A(6) * wr * cu;
-    FS[pp] = A(2) * wr * (A(9) * cu * ca - A(3) * ua);
-    FA[pp] = A(6) * wr * ca;
+    NS[pp] = fma(A(-2) * wq3<A>(q), fma(rho, fma(A(4.5) * cu, cu, uu15), drho), S[pp]);
+    NA[pp] = fma(-(q < 7 ? ga : gd), cu, D[pp]);
   }
-  transform3<A>(n0, F0, NS, NA, FS, FA, k, ch);
-}
-
-// The second half of the collision: from d - d_eq and Fbar as pair sums
-// (NS, FS) and differences (NA, FA) plus the rest direction's (n0, F0), the
-// change ch[q] = f'_q - f_q (ch[0] = 0).
-template <typename A>
-__device__ __forceinline__ void transform3(const A n0, const A F0, const A (&NS)[kPairs3],
-                                           const A (&NA)[kPairs3], const A (&FS)[kPairs3],
-                                           const A (&FA)[kPairs3], const Const3<A> &k,
-                                           A (&ch)[Q]) {
-  // m' - m = -s (m - m_eq) + (1 - s/2) M Fbar, scaled by 1/|M_k|^2
-  A dm[Q];
-#pragma unroll
-  for (int r = 0; r < Q; r++) {
-    A a = A(0), b = A(0);
-    if (!odd_row3(r)) {
-      a = mac3(a, m3(r, 0), n0);
-      b = mac3(b, m3(r, 0), F0);
-    }
-#pragma unroll
-    for (int pp = 0; pp < kPairs3; pp++) {
-      a = mac3(a, m3(r, rep3(pp)), odd_row3(r) ? NA[pp] : NS[pp]);
-      b = mac3(b, m3(r, rep3(pp)), odd_row3(r) ? FA[pp] : FS[pp]);
-    }
-    dm[r] = k.f_scaled[r] * b - k.s_scaled[r] * a;
-  }
-  // f' - f = M^T dm: even rows give the same change to q and opp q, odd
-  // rows opposite ones
-  ch[0] = A(0);
-#pragma unroll
-  for (int pp = 0; pp < kPairs3; pp++) {
-    const int q = rep3(pp), qb = opp3(q);
-    A ev = A(0), od = A(0);
-#pragma unroll
-    for (int r = 0; r < Q; r++) {
-      if (odd_row3(r)) od = mac3(od, m3(r, q), dm[r]);
-      else ev = mac3(ev, m3(r, q), dm[r]);
-    }
-    ch[q] = ev + od;
-    ch[qb] = ev - od;
-  }
+  transform3<A>(n0, NS, NA, rho, u, k, ch);
 }
 
 // The exact-mass variant's first half of the collision (FP32 storage).  The
@@ -383,71 +395,89 @@ __device__ __forceinline__ void transform3(const A n0, const A F0, const A (&NS)
 // rounding errors of the former become relative errors of ~1e-5 of the
 // latter, and in a steady flow they repeat every step; so rho - 1, j, rho,
 // u and d - d_eq are formed in double-FP32 (the pair sums exactly, by
-// TwoSum) and d - d_eq is rounded once to FP32 for the transform.  Fbar,
-// proportional to the body force and orders of magnitude smaller, stays in
-// FP32.  rho - 1, rho and u are returned in double-FP32 for the links.
-__device__ __forceinline__ float to_f(D2 x) { return __fadd_rn(x.h, x.l); }
-__device__ __forceinline__ void exact_moments3(const float (&d)[Q], const Const3<D2> &kd, D2 &drho,
-                                               D2 &rho, D2 (&u)[3], float &n0, float &F0,
-                                               float (&NS)[kPairs3], float (&NA)[kPairs3],
-                                               float (&FS)[kPairs3], float (&FA)[kPairs3]) {
-  D2 S[kPairs3], Dd[kPairs3];
-  drho = D2(d[0], 0.0f);
+// TwoSum) and d - d_eq is rounded once to FP32 for the transform.  rho - 1,
+// rho, u and -3/2 |u|^2 are returned in double-FP32 for the links.
+// Sums of several terms run in twice the working precision without
+// normalising in between (Sum), products by lattice weights are formed once
+// per node for the axes and halved (exactly) for the diagonals, and rho's
+// reciprocal serves the three quotients: about 950 operations, straight-line
+// (the form before, one general double-FP32 operation per term, took 3 to 4
+// times as many).
+using lbm::dev::DF;
+using lbm::dev::Sum;
+struct Force3 {
+  DF a[3];  // the body acceleration as double-FP32 pairs
+};
+inline DF df_of(double x) {
+  const float h = static_cast<float>(x);
+  return DF{h, static_cast<float>(x - static_cast<double>(h))};
+}
+__device__ __forceinline__ DF df_third() {
+  constexpr float h = static_cast<float>(1.0 / 3.0);
+  return DF{h, static_cast<float>(1.0 / 3.0 - static_cast<double>(h))};
+}
+__device__ __forceinline__ DF df_ninth() {
+  constexpr float h = static_cast<float>(1.0 / 9.0);
+  return DF{h, static_cast<float>(1.0 / 9.0 - static_cast<double>(h))};
+}
+__device__ __forceinline__ void exact_moments3(const float (&d)[Q], const Force3 &force, DF &drho,
+                                               DF &rho, DF (&u)[3], DF &uu15, float &n0,
+                                               float (&NS)[kPairs3], float (&NA)[kPairs3]) {
+  using namespace lbm::dev;
+  DF S[kPairs3], D[kPairs3];
+  Sum sr(DF{d[0], 0.0f});
 #pragma unroll
   for (int pp = 0; pp < kPairs3; pp++) {
     const int q = rep3(pp), qb = opp3(q);
-    float h, l;
-    lbm::dev::two_sum(d[q], d[qb], h, l);
-    S[pp] = D2(h, l);
-    lbm::dev::two_sum(d[q], -d[qb], h, l);
-    Dd[pp] = D2(h, l);
-    drho += S[pp];
+    two_sum(d[q], d[qb], S[pp].h, S[pp].l);
+    two_sum(d[q], -d[qb], D[pp].h, D[pp].l);
+    sr.add(S[pp]);
   }
-  D2 j[3] = {D2(0.0f, 0.0f), D2(0.0f, 0.0f), D2(0.0f, 0.0f)};
+  drho = sr.value();
+  rho = df_add(DF{1.0f, 0.0f}, drho);
+  const float inv = __frcp_rn(rho.h);
 #pragma unroll
-  for (int a = 0; a < 3; a++)
+  for (int a = 0; a < 3; a++) {
+    Sum sj(D[a]);  // pair a is the axis a
 #pragma unroll
-    for (int pp = 0; pp < kPairs3; pp++) j[a] = mac3(j[a], cvel3(rep3(pp), a), Dd[pp]);
-  rho = D2(1.0f, 0.0f) + drho;
-  const D2 acc[3] = {kd.ax, kd.ay, kd.az};
+    for (int pp = 3; pp < kPairs3; pp++) {
+      const int c = cvel3(rep3(pp), a);
+      if (c != 0) sj.add(c > 0 ? D[pp] : df_neg(D[pp]));
+    }
+    DF j = sj.value();
+    if (force.a[a].h != 0.0f) j = df_add(j, df_mul(df_scale(0.5f, rho), force.a[a]));
+    u[a] = df_div_inv(j, rho, inv);
+  }
+  const DF uu = df_add(df_add(df_mul(u[0], u[0]), df_mul(u[1], u[1])), df_mul(u[2], u[2]));
+  uu15 = df_mul_f(uu, -1.5f);
+  const DF e0 = df_add(drho, df_mul(rho, uu15));
+  n0 = df_sub_f(DF{d[0], 0.0f}, df_mul(e0, df_third()));
+  const DF ea = df_mul(e0, df_ninth()), ed = df_scale(0.5f, ea);
+  const DF ra = df_scale(0.5f, rho), rd = df_scale(0.25f, rho);
+  const DF ga = df_mul(rho, df_third()), gd = df_scale(0.5f, ga);
 #pragma unroll
-  for (int a = 0; a < 3; a++) u[a] = (j[a] + D2(0.5f, 0.0f) * rho * acc[a]) / rho;
-  const D2 uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-  const float rf = rho.h, uaf = u[0].h * kd.ax.h + u[1].h * kd.ay.h + u[2].h * kd.az.h;
-  n0 = to_f(D2(d[0], 0.0f) - wq3<D2>(0) * (drho - D2(1.5) * rho * uu));
-  F0 = -3.0f * w3<float>(0) * rf * uaf;
-  // one pair per iteration, not unrolled: the double-FP32 body is long, and
-  // nine copies of it would overflow the instruction cache
-#pragma unroll 1
   for (int pp = 0; pp < kPairs3; pp++) {
     const int q = rep3(pp);
-    D2 cu(0.0f, 0.0f);
-    float caf = 0.0f;
-    const float ka[3] = {kd.ax.h, kd.ay.h, kd.az.h};
+    DF cu{0.0f, 0.0f};
+    bool first = true;
 #pragma unroll
     for (int a = 0; a < 3; a++) {
-      const int c = cvel3_rt(q, a);
-      if (c > 0) {
-        cu = cu + u[a];
-        caf += ka[a];
-      } else if (c < 0) {
-        cu = cu - u[a];
-        caf -= ka[a];
-      }
+      const int c = cvel3(q, a);
+      if (c == 0) continue;
+      const DF t = c > 0 ? u[a] : df_neg(u[a]);
+      cu = first ? t : df_add(cu, t);
+      first = false;
     }
-    const D2 wq = wq3<D2>(q);
-    NS[pp] = to_f(S[pp] - D2(2.0) * wq * (drho + rho * (D2(4.5) * cu * cu - D2(1.5) * uu)));
-    NA[pp] = to_f(Dd[pp] - D2(6.0) * wq * rho * cu);
-    const float wrf = w3<float>(q) * rf;
-    FS[pp] = 2.0f * wrf * (9.0f * cu.h * caf - 3.0f * uaf);
-    FA[pp] = 6.0f * wrf * caf;
+    const DF eq = df_add(df_mul(df_mul(cu, cu), q < 7 ? ra : rd), q < 7 ? ea : ed);
+    NS[pp] = df_sub_f(S[pp], eq);
+    NA[pp] = df_sub_f(D[pp], df_mul(q < 7 ? ga : gd, cu));
   }
 }
 
 // The exact-mass variant's extra record per warp: rho - 1, rho, u_x, u_y,
-// u_z of each boundary node in double-FP32 (pairs of rows).
+// u_z, -3/2 |u|^2 of each boundary node in double-FP32 (pairs of rows).
 struct Warp3X {
-  float v[10][33];
+  float v[12][33];
 };
 
 // Gather, collide and store one fluid node (pull layout); a boundary node
@@ -465,40 +495,50 @@ struct Warp3X {
 // node's mass in double-FP32 plus the node's carry c0 (what FP32 storage
 // dropped from its earlier values); stored rounded to nearest, the new
 // remainder is kept in c0.
-template <typename C, bool kExact = false>
-__device__ __forceinline__ void node3(const C *src, C *dst,
-                                      const Const3<C> &k, const int64_t p, const uint32_t fl,
-                                      const uint32_t lb, Warp3<C> &sh, const int lane,
-                                      float *c0 = nullptr, const uint32_t rs = 0u,
-                                      Warp3X *shx = nullptr, const Const3<D2> *kd = nullptr) {
-  const int64_t N = k.plane;
+//
+// I indexes the lattice's elements: 32 bits where all of them, link tail
+// included, fit (half the address arithmetic), else 64.
+template <typename C, bool kExact, typename I>
+__device__ __forceinline__ void node3(const C *src, C *dst, const Const3<C> &k, const uint32_t p,
+                                      const uint32_t fl, const uint32_t lb, Warp3<C> &sh,
+                                      const int lane, float *c0 = nullptr, const uint32_t rs = 0u,
+                                      Warp3X *shx = nullptr, const Force3 *force = nullptr) {
+  const I N = static_cast<I>(k.plane);
   const Coord3 c = coord3(k, p);
   C d[Q];
   {
-    // x - c_q from the wrapped coordinates, or the node's tail element
+    // x - c_q from the wrapped coordinates, or the node's next tail element
     // where x - c_q is solid (a select, so interior and boundary nodes run
     // the same instructions; on a walled axis the wrapped value is unused)
     const int xw[3] = {c.x + 1 < k.nx ? c.x + 1 : 0, c.x, c.x > 0 ? c.x - 1 : k.nx - 1};
     const int yw[3] = {c.y + 1 < k.ny ? c.y + 1 : 0, c.y, c.y > 0 ? c.y - 1 : k.ny - 1};
     const int zw[3] = {c.z + 1 < k.nz ? c.z + 1 : 0, c.z, c.z > 0 ? c.z - 1 : k.nz - 1};
-    const int64_t sx = k.nx, sxy = static_cast<int64_t>(k.nx) * k.ny;
-    const int64_t tail = 19 * N + lb;
-    lbm::dev::chain_wait();
+    uint32_t row[3][3];  // lattice nodes are below 2^31
 #pragma unroll
-    for (int q = 0; q < Q; q++) {
-      const int64_t nb = q * N + zw[cvel3(q, 2) + 1] * sxy + yw[cvel3(q, 1) + 1] * sx +
-                         xw[cvel3(q, 0) + 1];
-      const int64_t tq = tail + __popc(fl & ((1u << q) - 1u));
-      d[q] = src[(fl >> q) & 1u ? tq : nb];
+    for (int z = 0; z < 3; z++)
+#pragma unroll
+      for (int y = 0; y < 3; y++)
+        row[z][y] = static_cast<uint32_t>((zw[z] * k.ny + yw[y]) * k.nx);
+    I t = 19 * N + lb;
+    lbm::dev::chain_wait();
+    d[0] = src[p];
+#pragma unroll
+    for (int q = 1; q < Q; q++) {
+      const I nb = static_cast<I>(q) * N +
+                   (row[cvel3(q, 2) + 1][cvel3(q, 1) + 1] + static_cast<uint32_t>(xw[cvel3(q, 0) + 1]));
+      const bool link = (fl & (1u << q)) != 0u;
+      d[q] = src[link ? t : nb];
+      t += link ? 1 : 0;
     }
   }
   C o[Q];
   if constexpr (kExact) {
     static_assert(std::is_same<C, float>::value, "the exact-mass variant is FP32 storage");
-    D2 drx, rhx, ux3[3];
-    float n0, F0, NS[kPairs3], NA[kPairs3], FS[kPairs3], FA[kPairs3], ch[Q];
-    exact_moments3(d, *kd, drx, rhx, ux3, n0, F0, NS, NA, FS, FA);
-    transform3<float>(n0, F0, NS, NA, FS, FA, k, ch);
+    DF drx, rhx, ux3[3], uu15;
+    float n0, NS[kPairs3], NA[kPairs3], ch[Q];
+    exact_moments3(d, *force, drx, rhx, ux3, uu15, n0, NS, NA);
+    const float uf[3] = {ux3[0].h, ux3[1].h, ux3[2].h};
+    transform3<float>(n0, NS, NA, rhx.h, uf, k, ch);
     // f'_q = f_q + ch_q rounded to FP32 stochastically (16 random bits
     // each: the halves of the node's nine random words)
     uint32_t rw[kPairs3];
@@ -514,29 +554,29 @@ __device__ __forceinline__ void node3(const C *src, C *dst,
     // f'_0 = f_0 - sum (f'_q - f_q) plus the carry, in double-FP32 (each
     // change is the exact difference of two FP32 values); stored rounded to
     // nearest, the remainder kept
-    D2 sum(0.0f, 0.0f);
+    Sum sum(DF{d[0], 0.0f});
 #pragma unroll
     for (int q = 1; q < Q; q++) {
-      float h, l;
-      lbm::dev::two_sum(o[q], -d[q], h, l);
-      sum += D2(h, l);
+      DF dd;
+      lbm::dev::two_sum(d[q], -o[q], dd.h, dd.l);
+      sum.add(dd);
     }
-    const D2 v0 = (D2(d[0], 0.0f) - sum) + D2(*c0, 0.0f);
+    sum.add(DF{*c0, 0.0f});
     float e0;
-    lbm::dev::two_sum(v0.h, v0.l, o[0], e0);
+    lbm::dev::two_sum(sum.s, sum.e, o[0], e0);
     *c0 = e0;
 #pragma unroll
-    for (int q = 0; q < Q; q++) dst[q * N + p] = o[q];
+    for (int q = 0; q < Q; q++) dst[static_cast<I>(q) * N + p] = o[q];
     if (fl) {
 #pragma unroll
       for (int q = 1; q < Q; q++) {
         sh.v[q - 1][lane] = o[q];
         sh.v[Q - 2 + q][lane] = d[q];
       }
-      // rho - 1, rho and u as pairs of FP32 values for the links
-      const D2 nv[5] = {drx, rhx, ux3[0], ux3[1], ux3[2]};
+      // rho - 1, rho, u and -3/2 |u|^2 as pairs of FP32 values for the links
+      const DF nv[6] = {drx, rhx, ux3[0], ux3[1], ux3[2], uu15};
 #pragma unroll
-      for (int i = 0; i < 5; i++) {
+      for (int i = 0; i < 6; i++) {
         shx->v[2 * i][lane] = nv[i].h;
         shx->v[2 * i + 1][lane] = nv[i].l;
       }
@@ -555,7 +595,7 @@ __device__ __forceinline__ void node3(const C *src, C *dst,
     }
     o[0] = d[0] - sum;
 #pragma unroll
-    for (int q = 0; q < Q; q++) dst[q * N + p] = o[q];
+    for (int q = 0; q < Q; q++) dst[static_cast<I>(q) * N + p] = o[q];
     if (fl) {
 #pragma unroll
       for (int q = 1; q < Q; q++) {
@@ -577,110 +617,63 @@ __device__ __forceinline__ void node3(const C *src, C *dst,
 // warp spreads them over its lanes, one link per lane, each reading its
 // node's values from the warp's shared record -- the links of a node
 // cluster would otherwise run direction by direction on few lanes.
-// kExact: 80 registers and 6 CTAs per SM (issue-bound; 4 and 5 CTAs per SM
-// measured 2 to 4 % slower).
-template <typename C, bool kExact = false>
-__global__ void __launch_bounds__(kThreads3, kExact ? 6 : (sizeof(C) == 4 ? 8 : 2))
-step3_kernel(const C *src, C *dst, const uint32_t *__restrict__ flags,
-             const uint32_t *__restrict__ lbase, const Link3<C> *__restrict__ links,
+// Each lane finds its link's node (lane of the warp) and direction in the
+// link's entry of ldesc.
+// kExact: 96 registers and 5 CTAs per SM.
+template <typename C, bool kExact, typename I>
+__global__ void __launch_bounds__(kThreads3, kExact ? 5 : (sizeof(C) == 4 ? 8 : 2))
+step3_kernel(const C *src, C *dst, const uint32_t *__restrict__ gbase,
+             const uint16_t *__restrict__ ldesc, const Link3<C> *__restrict__ links,
              const uint2 *__restrict__ fluid, const __grid_constant__ Const3<C> k, int64_t n_fluid,
-             const lbm::LinkCoefDF *__restrict__ links_df = nullptr, float *carry = nullptr,
-             const __grid_constant__ Const3<D2> kd = Const3<D2>()) {
+             const lbm::LinkCoefDF *__restrict__ links_df, float *carry,
+             const __grid_constant__ Force3 force) {
   constexpr int kW = kThreads3 / 32;
   __shared__ Warp3<C> sh[kW];
   __shared__ Warp3X shx[kExact ? kW : 1];
-  __shared__ uint32_t sh_ex[kW][32], sh_fl[kW][32];
   // thread t of the launch runs the t-th fluid node (node order), so no
   // lane idles on a solid node
   const int64_t t0 = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   const int lane = static_cast<int>(threadIdx.x & 31u), w = static_cast<int>(threadIdx.x >> 5);
-  // the fluid-node list holds each node's index and flag word together
-  const uint2 pf = t0 < n_fluid ? fluid[t0] : make_uint2(0u, kSolid3);
-  const int64_t p = pf.x;
-  const uint32_t fl = pf.y;
-  const bool live = fl != kSolid3;
-  const uint32_t lb = live && fl ? lbase[p] : 0u;
+  const bool live = t0 < n_fluid;
+  // the fluid-node list holds each node's index and flag word together, the
+  // flag word the node's first link within its group of 32 (a warp)
+  const uint2 pf = live ? fluid[t0] : make_uint2(0u, 0u);
+  const uint32_t fl = pf.y & kFlags3;
+  const uint32_t base = t0 - lane < n_fluid ? gbase[t0 / 32] : 0u;  // the warp's first link
   // the exact-mass variant's carries: one per link, then one per fluid node
-  float *carry0 = kExact ? carry + k.n_links : nullptr;
   if (live) {
     if constexpr (kExact)
-      node3<C, true>(src, dst, k, p, fl, lb, sh[w], lane, carry0 + t0,
-                     static_cast<uint32_t>(t0) ^ k.sr_seed, &shx[w], &kd);
+      node3<C, true, I>(src, dst, k, pf.x, fl, base + (pf.y >> kRank3), sh[w], lane,
+                        carry + k.n_links + t0, static_cast<uint32_t>(t0) ^ k.sr_seed, &shx[w],
+                        &force);
     else
-      node3<C, false>(src, dst, k, p, fl, lb, sh[w], lane);
+      node3<C, false, I>(src, dst, k, pf.x, fl, base + (pf.y >> kRank3), sh[w], lane);
   }
-  const uint32_t nl = live ? static_cast<uint32_t>(__popc(fl)) : 0u;
-  const unsigned any = __ballot_sync(0xFFFFFFFFu, nl != 0u);
-  if (any == 0u) return;
-  // exclusive prefix of the lanes' link counts; link t of the warp is link
-  // base + t of the table
-  uint32_t incl = nl;
-#pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, incl, off);
-    if (lane >= off) incl += v;
-  }
-  const uint32_t excl = incl - nl, total = __shfl_sync(0xFFFFFFFFu, incl, 31);
-  const uint32_t base = __shfl_sync(0xFFFFFFFFu, lb - excl, __ffs(static_cast<int>(any)) - 1);
-  sh_ex[w][lane] = excl;
-  sh_fl[w][lane] = live ? fl : 0u;
+  const uint32_t total = __reduce_add_sync(0xFFFFFFFFu, static_cast<uint32_t>(__popc(fl)));
+  if (total == 0u) return;
   __syncwarp();
   const Warp3<C> &ws = sh[w];
+  C *tail = dst + 19 * k.plane;
   for (uint32_t t = static_cast<uint32_t>(lane); t < total; t += 32u) {
-    // the node (lane s) holding link t: the last lane whose prefix is <= t
-    int s = 0;
-#pragma unroll
-    for (int st = 16; st >= 1; st >>= 1)
-      if (sh_ex[w][s + st] <= t) s += st;
-    uint32_t m = sh_fl[w][s];
-    for (uint32_t r = t - sh_ex[w][s]; r; r--) m &= m - 1u;
-    const int j = __ffs(static_cast<int>(m)) - 1, jb = opp3_rt(j);
+    const uint32_t lj = base + t, dsc = ldesc[lj];
+    const int s = static_cast<int>(dsc >> 5), j = static_cast<int>(dsc & 31u), jb = opp3_rt(j);
     const C oj = ws.v[j - 1][s], ojb = ws.v[jb - 1][s], djb = ws.v[Q - 2 + jb][s];
     if constexpr (kExact) {
-      // Eq. EqNewBDSC in double-FP32 from the pairs of the FP64
-      // coefficients and the node's double-FP32 rho - 1, rho, u, plus the
-      // link's carry; stored rounded to nearest, the remainder kept
-      using lbm::dev::DF;
-      using lbm::dev::df_add;
-      using lbm::dev::df_mul;
-      using lbm::dev::df_mul_f;
+      // Eq. EqNewBDSC in double-FP32 with the link's carry
+      using namespace lbm::dev;
       const Warp3X &wx = shx[w];
-      const lbm::LinkCoefDF c = links_df[base + t];
-      const DF k1{c.hi[0], c.lo[0]}, k2{c.hi[1], c.lo[1]}, k3{c.hi[2], c.lo[2]},
-          al{c.hi[3], c.lo[3]};
-      const double wd = j < 7 ? 1.0 / 18 : 1.0 / 36;
-      const DF w2{static_cast<float>(wd), static_cast<float>(wd - static_cast<float>(wd))};
-      const DF drho2{wx.v[0][s], wx.v[1][s]}, rho2{wx.v[2][s], wx.v[3][s]};
-      const DF u2[3] = {{wx.v[4][s], wx.v[5][s]}, {wx.v[6][s], wx.v[7][s]}, {wx.v[8][s], wx.v[9][s]}};
-      const DF uu2 = df_add(df_add(df_mul(u2[0], u2[0]), df_mul(u2[1], u2[1])), df_mul(u2[2], u2[2]));
-      const DF r = df_add(df_add(k1, k2), k3);
-      DF c0, c2;
-      if (k.diffuse_mode == 0) {
-        c0 = al;
-        c2 = df_mul(df_add(DF{1.0f, 0.0f}, DF{-r.h, -r.l}), w2);
-      } else {
-        c0 = df_add(al, df_mul(df_add(r, DF{-1.0f, 0.0f}), w2));
-        c2 = DF{0.0f, 0.0f};
-      }
+      const DF drho{wx.v[0][s], wx.v[1][s]}, rho{wx.v[2][s], wx.v[3][s]};
       DF cu{0.0f, 0.0f};
 #pragma unroll
       for (int a = 0; a < 3; a++) {
-        const float ca = static_cast<float>(cvel3_rt(j, a));
-        cu = df_add(cu, DF{ca * u2[a].h, ca * u2[a].l});
+        const DF t1 = df_scale(static_cast<float>(cvel3_rt(j, a)),
+                               DF{wx.v[4 + 2 * a][s], wx.v[5 + 2 * a][s]});
+        cu = a == 0 ? t1 : df_add(cu, t1);
       }
-      const DF pj = df_add(df_add(df_mul_f(cu, 3.0f), df_mul_f(df_mul(cu, cu), 4.5f)),
-                           df_mul_f(uu2, -1.5f));
-      DF v = df_add(df_mul_f(k1, djb), df_mul_f(k2, oj));
-      v = df_add(v, df_mul_f(k3, ojb));
-      v = df_add(v, c0);
-      v = df_add(v, df_mul(al, drho2));
-      v = df_add(v, df_mul(c2, df_add(drho2, df_mul(rho2, pj))));
-      v = df_add(v, DF{carry[base + t], 0.0f});
-      const float tv = __fadd_rn(v.h, v.l);
-      carry[base + t] = __fadd_rn(__fadd_rn(v.h, -tv), v.l);
-      dst[19 * k.plane + base + t] = tv;
+      tail[lj] = link_value_exact(links_df[lj], k.diffuse_mode, djb, oj, ojb, drho, rho, cu,
+                                  DF{wx.v[10][s], wx.v[11][s]}, carry + lj);
     } else {
-      const Link3<C> cl = links[base + t];
+      const Link3<C> cl = links[lj];
       const C drho = ws.v[36][s], rho = ws.v[37][s], ux = ws.v[38][s], uy = ws.v[39][s],
               uz = ws.v[40][s];
       const C uu = ux * ux + uy * uy + uz * uz;
@@ -696,8 +689,8 @@ step3_kernel(const C *src, C *dst, const uint32_t *__restrict__ flags,
       }
       const C cu = C(cvel3_rt(j, 0)) * ux + C(cvel3_rt(j, 1)) * uy + C(cvel3_rt(j, 2)) * uz;
       const C pj = C(3) * cu + C(4.5) * cu * cu - C(1.5) * uu;
-      dst[19 * k.plane + base + t] = cl.k1 * djb + cl.k2 * oj + cl.k3 * ojb + c0 +
-                                     cl.alpha * drho + c2 * (drho + rho * pj);
+      tail[lj] = cl.k1 * djb + cl.k2 * oj + cl.k3 * ojb + c0 + cl.alpha * drho +
+                 c2 * (drho + rho * pj);
     }
   }
 }
@@ -707,9 +700,8 @@ step3_kernel(const C *src, C *dst, const uint32_t *__restrict__ flags,
 template <typename C>
 __global__ void __launch_bounds__(kResThreads3)
 residual3_kernel(const C *__restrict__ cur, const C *__restrict__ prev,
-                 const uint32_t *__restrict__ flags, const uint32_t *__restrict__ lbase,
-                 const uint2 *__restrict__ fluid, const Const3<C> k, int64_t n_fluid,
-                 double *__restrict__ partials) {
+                 const uint32_t *__restrict__ gbase, const uint2 *__restrict__ fluid,
+                 const Const3<C> k, int64_t n_fluid, double *__restrict__ partials) {
   // per node: rho and j of both states in the storage's arithmetic type,
   // the node's mass deviation summed in FP64; sums over nodes in FP64
   double acc[4] = {0.0, 0.0, 0.0, 0.0};
@@ -718,11 +710,11 @@ residual3_kernel(const C *__restrict__ cur, const C *__restrict__ prev,
        t += G) {
     const uint2 pf = fluid[t];
     const int64_t p = pf.x;
-    const uint32_t fl = pf.y;
+    const uint32_t fl = pf.y & kFlags3;
     const Coord3 c = coord3(k, p);
     C r1 = C(0), r0 = C(0), j1[3] = {C(0), C(0), C(0)}, j0[3] = {C(0), C(0), C(0)};
     double dm = 0.0;
-    const uint32_t lb = fl ? lbase[p] : 0u;
+    const uint32_t lb = gbase[t / 32] + (pf.y >> kRank3);
 #pragma unroll
     for (int q = 0; q < Q; q++) {
       const int64_t s = pull_slot3(k, q, c, fl, lb, k.plane);
@@ -862,7 +854,6 @@ __global__ void import3_kernel(const double *__restrict__ in, const uint32_t *__
 struct Const3Both {
   Const3<double> d;
   Const3<float> f;
-  Const3<D2> x;  // the same as double-FP32 pairs (the exact-mass variant's body force)
   Const3<double> &get(double *) { return d; }
   Const3<float> &get(float *) { return f; }
   const Const3<double> &get(double *) const { return d; }
@@ -888,7 +879,9 @@ struct lbm3d {
   int cur = 0;
   uint32_t *flags = nullptr;
   uint32_t *lbase = nullptr;
-  uint2 *fluid = nullptr;  // the fluid nodes in node order: index, flag word
+  uint2 *fluid = nullptr;  // the fluid nodes in node order: index, flag word (kFlags3)
+  uint32_t *gbase = nullptr;   // per 32 of them: the first link of the first
+  uint16_t *ldesc = nullptr;   // per link: its node's place among the 32 << 5 | direction
   // the exact-mass variant (FP32): link coefficients as FP32 pairs and the
   // carries (one per link, then one per fluid node)
   int exact = 0;
@@ -897,6 +890,7 @@ struct lbm3d {
   float *carry = nullptr;
   void *links = nullptr;
   Const3Both kc;
+  lbm3::Force3 force{};  // the exact-mass variant's body force
   double *partials = nullptr, *result = nullptr;
   std::vector<double> link_r, link_l;
   std::string err;
@@ -916,7 +910,8 @@ void release3(lbm3d_t *h) {
   if (!h) return;
   cudaStreamSynchronize(h->stream);
   for (void *p : {h->f[0], h->f[1], static_cast<void *>(h->flags), static_cast<void *>(h->lbase),
-                  static_cast<void *>(h->fluid), static_cast<void *>(h->links_df),
+                  static_cast<void *>(h->fluid), static_cast<void *>(h->gbase),
+                  static_cast<void *>(h->ldesc), static_cast<void *>(h->links_df),
                   static_cast<void *>(h->carry),
                   h->links, static_cast<void *>(h->partials),
                   static_cast<void *>(h->result)})
@@ -1079,13 +1074,31 @@ int lbm3d_create(const lbm3d_domain_t *dom, const uint8_t *solid, size_t n_links
   if (e == cudaSuccess) e = cudaMemcpy(h->flags, flags.data(), n * 4, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(h->lbase, lbase.data(), n * 4, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) {
-    std::vector<uint2> fluid;
-    fluid.reserve(static_cast<size_t>(n_fluid));
-    for (int64_t pn = 0; pn < n; pn++)
-      if (flags[pn] != kSolid3) fluid.push_back(make_uint2(static_cast<uint32_t>(pn), flags[pn]));
+    std::vector<uint2> fluid(static_cast<size_t>(n_fluid));
+    std::vector<uint32_t> gbase(static_cast<size_t>((n_fluid + 31) / 32));
+    std::vector<uint16_t> ldesc(std::max<size_t>(1, n_links));
+    uint32_t i = 0, l = 0;  // fluid nodes and links so far
+    for (int64_t pn = 0; pn < n; pn++) {
+      const uint32_t fl = flags[pn];
+      if (fl == kSolid3) continue;
+      const uint32_t at = i % 32;
+      if (at == 0) gbase[i / 32] = l;
+      // (at most 31 x 18 links precede it in its group)
+      fluid[i] = make_uint2(static_cast<uint32_t>(pn), fl | (l - gbase[i / 32]) << kRank3);
+      i++;
+      for (uint32_t m = fl; m; m &= m - 1u)
+        ldesc[l++] = static_cast<uint16_t>(at << 5 | static_cast<uint32_t>(__builtin_ctz(m)));
+    }
     e = alloc(reinterpret_cast<void **>(&h->fluid), std::max<size_t>(1, fluid.size()) * 8);
+    if (e == cudaSuccess)
+      e = alloc(reinterpret_cast<void **>(&h->gbase), std::max<size_t>(1, gbase.size()) * 4);
+    if (e == cudaSuccess) e = alloc(reinterpret_cast<void **>(&h->ldesc), ldesc.size() * 2);
     if (e == cudaSuccess && !fluid.empty())
       e = cudaMemcpy(h->fluid, fluid.data(), fluid.size() * 8, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess && !gbase.empty())
+      e = cudaMemcpy(h->gbase, gbase.data(), gbase.size() * 4, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess)
+      e = cudaMemcpy(h->ldesc, ldesc.data(), ldesc.size() * 2, cudaMemcpyHostToDevice);
   }
   if (e == cudaSuccess)
     e = dispatch3(h->precision, [&](auto tag) {
@@ -1096,8 +1109,7 @@ int lbm3d_create(const lbm3d_domain_t *dom, const uint8_t *solid, size_t n_links
         lk[slot[k]] = Link3<C>{static_cast<C>(cf[0]), static_cast<C>(cf[1]), static_cast<C>(cf[2]),
                                static_cast<C>(cf[3])};
       }
-      // the case's constants in each arithmetic type (the FP32 exact-mass
-      // variant forms its moments in double-FP32)
+      // the case's constants in each arithmetic type
       auto fill = [&](auto &kc) {
         using A = std::remove_reference_t<decltype(kc.ax)>;
         for (int a = 0; a < Q; a++) {
@@ -1114,6 +1126,8 @@ int lbm3d_create(const lbm3d_domain_t *dom, const uint8_t *solid, size_t n_links
         kc.px = per[0];
         kc.py = per[1];
         kc.pz = per[2];
+        kc.by_nx = DivBy3(static_cast<uint32_t>(nx));
+        kc.by_ny = DivBy3(static_cast<uint32_t>(ny));
         kc.diffuse_mode = p.diffuse_mode;
         kc.plane = h->plane;
         kc.n_links = h->n_links;
@@ -1121,7 +1135,6 @@ int lbm3d_create(const lbm3d_domain_t *dom, const uint8_t *solid, size_t n_links
       };
       fill(h->kc.f);
       fill(h->kc.d);
-      fill(h->kc.x);
       return cudaMemcpy(h->links, lk.data(), lk.size() * sizeof(Link3<C>), cudaMemcpyHostToDevice);
     });
   // the exact-mass variant (FP32): where mass_mode asks for it, or by
@@ -1131,8 +1144,10 @@ int lbm3d_create(const lbm3d_domain_t *dom, const uint8_t *solid, size_t n_links
   h->exact = p.precision == LBM_FP32 && p.mass_mode >= 0 &&
              (p.mass_mode > 0 || moving || n_links == 0);
   if (e == cudaSuccess && h->exact) {
+    const double acc[3] = {dom->ax, dom->ay, dom->az};
+    for (int a = 0; a < 3; a++) h->force.a[a] = df_of(acc[a]);
     std::vector<lbm::LinkCoefDF> ldf(std::max<size_t>(1, n_links));
-    for (size_t k = 0; k < n_links; k++) ldf[slot[k]] = lbm::link_coef_df(&coef[8 * k]);
+    for (size_t k = 0; k < n_links; k++) ldf[slot[k]] = lbm::link_coef_df(&coef[8 * k], wq[k], p.diffuse_mode);
     e = alloc(reinterpret_cast<void **>(&h->links_df), ldf.size() * sizeof(lbm::LinkCoefDF));
     if (e == cudaSuccess)
       e = cudaMemcpy(h->links_df, ldf.data(), ldf.size() * sizeof(lbm::LinkCoefDF),
@@ -1160,23 +1175,21 @@ int lbm3d_step(lbm3d_t *h, int64_t n) {
     cudaError_t e = dispatch3(h->precision, [&](auto tag) {
       using C = std::remove_pointer_t<decltype(tag)>;
       if (h->n_fluid == 0) return cudaSuccess;
-      const unsigned blocks = static_cast<unsigned>((h->n_fluid + kThreads3 - 1) / kThreads3);
+      const dim3 blocks(static_cast<unsigned>((h->n_fluid + kThreads3 - 1) / kThreads3));
+      Const3<C> kc = h->kc.get(tag);
+      kc.sr_seed = lbm::dev::step_seed(h->steps);
+      auto go = [&](auto *kernel) {
+        return lbm::launch_chained(kernel, blocks, kThreads3, 0, h->stream,
+                                   static_cast<const C *>(h->f[src]), static_cast<C *>(h->f[dst]),
+                                   h->gbase, h->ldesc, static_cast<const Link3<C> *>(h->links),
+                                   h->fluid, kc, h->n_fluid, h->links_df, h->carry, h->force);
+      };
+      const bool small = 19 * h->plane + h->n_links < (int64_t(1) << 32);
       if constexpr (std::is_same<C, float>::value) {
-        if (h->exact) {
-          Const3<C> kx = h->kc.get(tag);
-          kx.sr_seed = lbm::dev::step_seed(h->steps);
-          return lbm::launch_chained(
-              step3_kernel<C, true>, dim3(blocks), kThreads3, 0, h->stream, static_cast<const C *>(h->f[src]),
-              static_cast<C *>(h->f[dst]), h->flags, h->lbase,
-              static_cast<const Link3<C> *>(h->links), h->fluid, kx, h->n_fluid, h->links_df,
-              h->carry, h->kc.x);
-        }
+        if (h->exact)
+          return small ? go(step3_kernel<C, true, uint32_t>) : go(step3_kernel<C, true, int64_t>);
       }
-      return lbm::launch_chained(
-          step3_kernel<C, false>, dim3(blocks), kThreads3, 0, h->stream, static_cast<const C *>(h->f[src]),
-          static_cast<C *>(h->f[dst]), h->flags, h->lbase, static_cast<const Link3<C> *>(h->links),
-          h->fluid, h->kc.get(tag), h->n_fluid, static_cast<const lbm::LinkCoefDF *>(nullptr),
-          static_cast<float *>(nullptr), Const3<D2>());
+      return small ? go(step3_kernel<C, false, uint32_t>) : go(step3_kernel<C, false, int64_t>);
     });
     if (e != cudaSuccess) return fail3(h, LBM_ECUDA, std::string("step: ") + cudaGetErrorString(e));
     h->cur = dst;
@@ -1192,8 +1205,8 @@ int lbm3d_residual(lbm3d_t *h, double *residual, double *mass) {
   cudaError_t e = dispatch3(h->precision, [&](auto tag) {
     using C = std::remove_pointer_t<decltype(tag)>;
     residual3_kernel<C><<<kResBlocks3, kResThreads3, 0, h->stream>>>(
-        static_cast<const C *>(h->f[h->cur]), static_cast<const C *>(h->f[1 - h->cur]), h->flags,
-        h->lbase, h->fluid, h->kc.get(tag), h->n_fluid, h->partials);
+        static_cast<const C *>(h->f[h->cur]), static_cast<const C *>(h->f[1 - h->cur]), h->gbase,
+        h->fluid, h->kc.get(tag), h->n_fluid, h->partials);
     residual3_final<<<1, 1024, 0, h->stream>>>(h->partials, h->result);
     return cudaGetLastError();
   });

@@ -761,12 +761,14 @@ int lbm_create(const lbm_domain_t *dom, const uint8_t *solid, size_t n_links,
   std::vector<lbm::LinkCoefDF> ldf;
   if (h->exact) {
     ldf.resize(n_links_sz);
-    for (size_t l = 0; l < n_links_sz; l++) ldf[l] = lbm::link_coef_df(&hc.coef[4 * l]);
+    for (size_t l = 0; l < n_links_sz; l++)
+      ldf[l] = lbm::link_coef_df(&hc.coef[4 * l], (lds[l] & 15) < 5 ? 1.0 / 9 : 1.0 / 36,
+                                 p.diffuse_mode);
   }
   if (h->exact) {
     // one allocation: the per-link carries, then the per-node ones
     const size_t nl = std::max<size_t>(1, n_links_sz);
-    if (e == cudaSuccess) e = alloc(reinterpret_cast<void **>(&h->links64), nl * 32);
+    if (e == cudaSuccess) e = alloc(reinterpret_cast<void **>(&h->links64), nl * sizeof(lbm::LinkCoefDF));
     if (e == cudaSuccess) e = alloc(reinterpret_cast<void **>(&h->carry), carry_bytes(h));
     if (e == cudaSuccess) h->carry0 = h->carry + nl;
     if (e == cudaSuccess && n_links_sz)

@@ -677,10 +677,10 @@ int lbm_batch_create(const lbm_case_t *cases, int32_t n_cases, int32_t precision
   std::vector<uint16_t> lds(static_cast<size_t>(std::max<int64_t>(1, links)), 0u);
   std::vector<int32_t> rowstart(static_cast<size_t>(rows), 0), index(static_cast<size_t>(dense), -1);
   std::vector<unsigned char> lhost(std::max<int64_t>(1, links) * 4 * ces, 0);
-  std::vector<double> l64;  // FP64 link records (filled if some case runs the exact variant)
+  std::vector<lbm::LinkCoefDF> l64;  // filled if some case runs the exact variant
   bool any_exact = false;
   for (int c = 0; c < n_cases; c++) any_exact |= lbm::exact_mass(hc[c]);
-  if (any_exact) l64.assign(static_cast<size_t>(std::max<int64_t>(1, links)) * 4, 0.0);
+  if (any_exact) l64.assign(static_cast<size_t>(std::max<int64_t>(1, links)), lbm::LinkCoefDF{});
   std::vector<unsigned char> chost;
   std::vector<int32_t> xchunks;
   bool any_interval = false;
@@ -722,7 +722,9 @@ int lbm_batch_create(const lbm_case_t *cases, int32_t n_cases, int32_t precision
     b->chunk_count.push_back(static_cast<int32_t>(padded / lbm::kChunk));
     b->case_exact.push_back(lbm::exact_mass(h) ? 1 : 0);
     if (lbm::exact_mass(h)) {
-      std::copy(h.coef.begin(), h.coef.begin() + 4 * h.n_links, l64.begin() + 4 * loff);
+      for (int64_t q = 0; q < h.n_links; q++)
+        l64[loff + q] = lbm::link_coef_df(&h.coef[4 * q], (kd[q] & 15) < 5 ? 1.0 / 9 : 1.0 / 36,
+                                          h.params.diffuse_mode);
       for (int64_t q = noff / lbm::kChunk; q < (noff + padded) / lbm::kChunk; q++)
         xchunks.push_back(static_cast<int32_t>(q));
     }
@@ -782,17 +784,12 @@ int lbm_batch_create(const lbm_case_t *cases, int32_t n_cases, int32_t precision
   if (e == cudaSuccess) e = alloc(&b->links, lhost.size());
   b->n_links_total = links;
   if (any_exact) {
-    if (e == cudaSuccess) e = alloc(reinterpret_cast<void **>(&b->links64), l64.size() * 8);
-    if (e == cudaSuccess)
-      e = alloc(reinterpret_cast<void **>(&b->carry), (l64.size() / 4 + nodes) * 4);
-    if (e == cudaSuccess) b->carry0 = b->carry + l64.size() / 4;
-    if (e == cudaSuccess) e = cudaMemset(b->carry, 0, (l64.size() / 4 + nodes) * 4);
-    if (e == cudaSuccess) {
-      std::vector<lbm::LinkCoefDF> ldf(l64.size() / 4);
-      for (size_t l = 0; l < ldf.size(); l++) ldf[l] = lbm::link_coef_df(&l64[4 * l]);
-      e = cudaMemcpy(b->links64, ldf.data(), ldf.size() * sizeof(lbm::LinkCoefDF),
-                     cudaMemcpyHostToDevice);
-    }
+    const size_t lb = l64.size() * sizeof(lbm::LinkCoefDF), cb = (l64.size() + nodes) * 4;
+    if (e == cudaSuccess) e = alloc(reinterpret_cast<void **>(&b->links64), lb);
+    if (e == cudaSuccess) e = alloc(reinterpret_cast<void **>(&b->carry), cb);
+    if (e == cudaSuccess) b->carry0 = b->carry + l64.size();
+    if (e == cudaSuccess) e = cudaMemset(b->carry, 0, cb);
+    if (e == cudaSuccess) e = cudaMemcpy(b->links64, l64.data(), lb, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = alloc(reinterpret_cast<void **>(&b->exact_chunks), xchunks.size() * 4);
     if (e == cudaSuccess)
       e = cudaMemcpy(b->exact_chunks, xchunks.data(), xchunks.size() * 4, cudaMemcpyHostToDevice);

@@ -224,25 +224,61 @@ __device__ __forceinline__ DF df_norm(float s, float e) {
   two_sum(s, e, h, l);
   return DF{h, l};
 }
+// h + l of s + e where |e| is at most about |s| (what the operations below
+// leave): Dekker's FastTwoSum, the same h and l as TwoSum in half the
+// operations.
+__device__ __forceinline__ DF df_quick(float s, float e) {
+  const float h = __fadd_rn(s, e);
+  return DF{h, __fsub_rn(e, __fsub_rn(h, s))};
+}
+__device__ __forceinline__ DF df_neg(DF a) { return DF{-a.h, -a.l}; }
 __device__ __forceinline__ DF df_add(DF a, DF b) {
   float s, e;
   two_sum(a.h, b.h, s, e);
-  return df_norm(s, __fadd_rn(e, __fadd_rn(a.l, b.l)));
+  return df_quick(s, __fadd_rn(e, __fadd_rn(a.l, b.l)));
+}
+__device__ __forceinline__ DF df_sub(DF a, DF b) { return df_add(a, df_neg(b)); }
+// a - b rounded once to FP32
+__device__ __forceinline__ float df_sub_f(DF a, DF b) {
+  float s, e;
+  two_sum(a.h, -b.h, s, e);
+  return __fadd_rn(s, __fadd_rn(e, __fsub_rn(a.l, b.l)));
 }
 __device__ __forceinline__ DF df_mul_f(DF a, float b) {
   const float p = __fmul_rn(a.h, b);
-  return df_norm(p, __fmaf_rn(a.l, b, __fmaf_rn(a.h, b, -p)));
+  return df_quick(p, __fmaf_rn(a.l, b, __fmaf_rn(a.h, b, -p)));
 }
 __device__ __forceinline__ DF df_mul(DF a, DF b) {
   const float p = __fmul_rn(a.h, b.h);
   const float e = __fmaf_rn(a.h, b.h, -p);
-  return df_norm(p, __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, e)));
+  return df_quick(p, __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, e)));
+}
+// c a for c a power of two (or -1, 0, 1): exact
+__device__ __forceinline__ DF df_scale(float c, DF a) { return DF{c * a.h, c * a.l}; }
+// a / b, given inv = 1 / b.h rounded: the quotient's head, then the exact
+// remainder's
+__device__ __forceinline__ DF df_div_inv(DF a, DF b, float inv) {
+  const float q1 = __fmul_rn(a.h, inv);
+  const DF r = df_sub(a, df_mul_f(b, q1));
+  return df_quick(q1, __fmul_rn(r.h, inv));
 }
 __device__ __forceinline__ DF df_div(DF a, DF b) {
   const float q1 = __fdiv_rn(a.h, b.h);
-  const DF r = df_add(a, df_mul_f(b, -q1));  // a - q1 b
-  return df_norm(q1, __fdiv_rn(r.h, b.h));
+  const DF r = df_sub(a, df_mul_f(b, q1));
+  return df_quick(q1, __fdiv_rn(r.h, b.h));
 }
+// A running sum in twice the working precision (Sum2 over double-FP32
+// terms): s + e.
+struct Sum {
+  float s, e;
+  __device__ __forceinline__ explicit Sum(DF a) : s(a.h), e(a.l) {}
+  __device__ __forceinline__ void add(DF a) {
+    float t;
+    two_sum(s, a.h, s, t);
+    e = __fadd_rn(e, __fadd_rn(t, a.l));
+  }
+  __device__ __forceinline__ DF value() const { return df_norm(s, e); }
+};
 
 // The collision of Eq. MomentPost as the change ch_i = f'_i - f_i of each
 // population, with the node's rho - 1, rho, u and |u|^2 (Eq. FluidMacr),
@@ -444,12 +480,38 @@ __device__ __forceinline__ void collide(const C (&d)[9], const StepConst<C> &k, 
 // up, step after step, to the exact ones, so the mass a moving wall
 // exchanges with the fluid does not drift by a rounding that repeats.
 // The links of a warp's nodes are consecutive in the link table; the warp
-// spreads them over its lanes, one link per lane at a time, each reading its node's
-// values from the warp's shared record.  node = the node's index i; lane
+// spreads them over its lanes, one link per lane at a time, each finding its
+// node's column in the warp's shared record and its direction in the link's
+// entry of g.ldesc.  node = the node's index i; lane
 // i mod 32 of the warp runs node i, and the lanes of nodes below g.n_fluid
 // (a prefix of the warp) take part -- named explicitly, since the lanes
 // need not have reconverged after the collision's data-dependent branches.
 constexpr int kExactMaxWarps = 8;  // CTAs of up to 256 threads
+
+// One link's value (Eq. EqNewBDSC) in double-FP32, from its coefficients,
+// f_jb, f'_j, f'_jb and the node's rho - 1, rho, c_j . u and -3/2 |u|^2, plus
+// the link's carry; returns it rounded to nearest and keeps the remainder.
+// The terms are summed in twice the working precision without normalising
+// in between, and what depends on the link alone (c2) is in its record: on a
+// warp with links this chain of operations is the step's longest.
+__device__ __forceinline__ float link_value_exact(const LinkCoefDF &c, const int diffuse_mode,
+                                                  const float djb, const float oj,
+                                                  const float ojb, const DF drho, const DF rho,
+                                                  const DF cu, const DF uu, float *carry) {
+  const DF al{c.hi[3], c.lo[3]}, c2{c.hi[4], c.lo[4]};
+  // 3 c.u + 4.5 (c.u)^2 - 1.5 u.u
+  const DF pj = df_add(df_mul(cu, df_add(df_mul_f(cu, 4.5f), DF{3.0f, 0.0f})), uu);
+  Sum v(df_mul_f(DF{c.hi[0], c.lo[0]}, djb));
+  v.add(df_mul_f(DF{c.hi[1], c.lo[1]}, oj));
+  v.add(df_mul_f(DF{c.hi[2], c.lo[2]}, ojb));
+  v.add(al);
+  v.add(df_mul(al, drho));
+  v.add(diffuse_mode == 0 ? df_mul(c2, df_add(drho, df_mul(rho, pj))) : c2);
+  v.add(DF{*carry, 0.0f});
+  const float tv = __fadd_rn(v.s, v.e);
+  *carry = __fadd_rn(__fsub_rn(v.s, tv), v.e);
+  return tv;
+}
 
 // D2Q9 velocities (two bits each: c + 1, direction j in bits 2j, 2j + 1)
 // and opposite directions (four bits each: opp(j) in bits 4 (j - 1) ..
@@ -468,8 +530,7 @@ __device__ __forceinline__ void link_epilogue_exact(const float *src, float *dst
                                                     const StepConst<float> &k,
                                                     const uint32_t node) {
   __shared__ float xs_o[kExactMaxWarps][8][33];   // f'_1 .. f'_8
-  __shared__ float xs_n[kExactMaxWarps][10][33];  // drho, rho, ux, uy, |u|^2 (DF)
-  __shared__ uint32_t xs_ex[kExactMaxWarps][32], xs_fl[kExactMaxWarps][32];
+  __shared__ float xs_n[kExactMaxWarps][10][33];  // drho, rho, ux, uy, -3/2 |u|^2 (DF)
   const int lane = static_cast<int>(threadIdx.x & 31u), w = static_cast<int>(threadIdx.x >> 5);
   const uint32_t first = node - static_cast<uint32_t>(lane);
   const int nact = g.n_fluid - first >= 32u ? 32 : static_cast<int>(g.n_fluid - first);
@@ -482,75 +543,38 @@ __device__ __forceinline__ void link_epilogue_exact(const float *src, float *dst
     const DF drho2 = df_norm(c_.dr_hi, c_.dr_lo);
     const DF rho2 = df_add(DF{1.0f, 0.0f}, drho2);
     const DF half_rho{0.5f * rho2.h, 0.5f * rho2.l};
-    const DF ux2 = df_div(df_add(df_norm(c_.jx_hi, c_.jx_lo), df_mul_f(half_rho, k.ax)), rho2);
-    const DF uy2 = df_div(df_add(df_norm(c_.jy_hi, c_.jy_lo), df_mul_f(half_rho, k.ay)), rho2);
-    const DF uu2 = df_add(df_mul(ux2, ux2), df_mul(uy2, uy2));
+    const float inv = __frcp_rn(rho2.h);
+    const DF ux2 =
+        df_div_inv(df_add(df_norm(c_.jx_hi, c_.jx_lo), df_mul_f(half_rho, k.ax)), rho2, inv);
+    const DF uy2 =
+        df_div_inv(df_add(df_norm(c_.jy_hi, c_.jy_lo), df_mul_f(half_rho, k.ay)), rho2, inv);
+    const DF uu2 = df_mul_f(df_add(df_mul(ux2, ux2), df_mul(uy2, uy2)), -1.5f);
 #pragma unroll
     for (int q = 1; q < 9; q++) xs_o[w][q - 1][lane] = c_.o[q];
     const float nv[10] = {drho2.h, drho2.l, rho2.h, rho2.l, ux2.h, ux2.l, uy2.h, uy2.l, uu2.h, uu2.l};
 #pragma unroll
     for (int q = 0; q < 10; q++) xs_n[w][q][lane] = nv[q];
   }
-  // exclusive prefix of the lanes' link counts: link t of the warp is
-  // link base + t of the table
-  uint32_t incl = nl;
-#pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    const uint32_t v = __shfl_up_sync(am, incl, off);
-    if (lane >= off) incl += v;
-  }
-  const uint32_t excl = incl - nl, total = __shfl_sync(am, incl, nact - 1);
-  const uint32_t base = __shfl_sync(am, li - excl, __ffs(static_cast<int>(anyl)) - 1);
-  xs_ex[w][lane] = excl;
-  xs_fl[w][lane] = fl;
+  // the warp's links are links base .. base + total - 1 of the table (its
+  // first lane with links holds the first of them)
+  const uint32_t total = __reduce_add_sync(am, nl);
+  const uint32_t base = __shfl_sync(am, li, __ffs(static_cast<int>(anyl)) - 1);
   __syncwarp(am);
   const uint32_t tail = 9u * g.plane;
-  constexpr float kW9h = static_cast<float>(1.0 / 9);
-  constexpr float kW36h = static_cast<float>(1.0 / 36);
-  const float kW9l = static_cast<float>(1.0 / 9 - static_cast<double>(kW9h));
-  const float kW36l = static_cast<float>(1.0 / 36 - static_cast<double>(kW36h));
   // the nact lanes of the warp take the links in turn
   for (uint32_t t = static_cast<uint32_t>(lane); t < total; t += static_cast<uint32_t>(nact)) {
-    // the node (lane s) holding link t: the last active lane whose prefix is <= t
-    int s = 0;
-#pragma unroll
-    for (int st = 16; st >= 1; st >>= 1)
-      if (s + st < nact && xs_ex[w][s + st] <= t) s += st;
-    uint32_t m = xs_fl[w][s];
-    for (uint32_t r = t - xs_ex[w][s]; r; r--) m &= m - 1u;
-    const int j = __ffs(static_cast<int>(m));  // flag bit j - 1: direction j
+    const uint32_t lj = base + t, dsc = g.ldesc[lj];
+    const int s = static_cast<int>((dsc >> 4) & 31u), j = static_cast<int>(dsc & 15u);
     const int jb = opp2(j), cx = vel_x2(j), cy = vel_y2(j);
-    const uint32_t lj = base + t;
     const LinkCoefDF c = g.links64[lj];
-    const DF k1{c.hi[0], c.lo[0]}, k2{c.hi[1], c.lo[1]}, k3{c.hi[2], c.lo[2]},
-        al{c.hi[3], c.lo[3]};
-    const DF w2 = j < 5 ? DF{kW9h, kW9l} : DF{kW36h, kW36l};
     const DF drho2{xs_n[w][0][s], xs_n[w][1][s]}, rho2{xs_n[w][2][s], xs_n[w][3][s]};
     const DF ux2{xs_n[w][4][s], xs_n[w][5][s]}, uy2{xs_n[w][6][s], xs_n[w][7][s]};
     const DF uu2{xs_n[w][8][s], xs_n[w][9][s]};
-    const DF r = df_add(df_add(k1, k2), k3);
-    DF c0, c2;
-    if (k.diffuse_mode == 0) {
-      c0 = al;
-      c2 = df_mul(df_add(DF{1.0f, 0.0f}, DF{-r.h, -r.l}), w2);
-    } else {
-      c0 = df_add(al, df_mul(df_add(r, DF{-1.0f, 0.0f}), w2));
-      c2 = DF{0.0f, 0.0f};
-    }
     // c_j . u: the components are -1, 0 or 1
-    const DF cu = df_add(DF{cx * ux2.h, cx * ux2.l}, DF{cy * uy2.h, cy * uy2.l});
-    const DF pj = df_add(df_add(df_mul_f(cu, 3.0f), df_mul_f(df_mul(cu, cu), 4.5f)),
-                         df_mul_f(uu2, -1.5f));
-    const float djb = src[g.jbslot[lj]];
-    DF v = df_add(df_mul_f(k1, djb), df_mul_f(k2, xs_o[w][j - 1][s]));
-    v = df_add(v, df_mul_f(k3, xs_o[w][jb - 1][s]));
-    v = df_add(v, c0);
-    v = df_add(v, df_mul(al, drho2));
-    v = df_add(v, df_mul(c2, df_add(drho2, df_mul(rho2, pj))));
-    v = df_add(v, DF{g.carry[lj], 0.0f});
-    const float tv = __fadd_rn(v.h, v.l);
-    g.carry[lj] = __fadd_rn(__fadd_rn(v.h, -tv), v.l);
-    dst[tail + lj] = tv;
+    const DF cu = df_add(df_scale(static_cast<float>(cx), ux2), df_scale(static_cast<float>(cy), uy2));
+    dst[tail + lj] =
+        link_value_exact(c, k.diffuse_mode, src[g.jbslot[lj]], xs_o[w][j - 1][s],
+                         xs_o[w][jb - 1][s], drho2, rho2, cu, uu2, &g.carry[lj]);
   }
 }
 
@@ -628,9 +652,10 @@ __device__ __forceinline__ void link_epilogue_pull(const T *src, T *dst,
 
 // Eq. EqNewBDSC for the links of the one-node FP32 / FP64 step, spread
 // over the warp as in pair_links_warp: the links of the warp's 32 nodes
-// are consecutive in the table; each lane takes one link at a time and
-// reads its node's values (f'_1..f'_8, drho, rho, u, |u|^2) from the
-// warp's shared record.  The value is link_epilogue_pull's, rounded to
+// are consecutive in the table; each lane takes one link at a time, finds
+// its node's column (x mod 32) and its direction in the link's entry of
+// g.ldesc, and reads the node's values (f'_1..f'_8, drho, rho, u, |u|^2)
+// from the warp's shared record.  The value is link_epilogue_pull's, rounded to
 // storage the same way.  The lanes of nodes below g.n_fluid take part (a
 // prefix of the warp: lane i mod 32 runs node i).  kWarps: warps per CTA.
 template <typename T, typename C, int kWarps>
@@ -642,7 +667,6 @@ __device__ __forceinline__ void node_links_warp(const T *src, T *dst,
                                                 const uint32_t node) {
   static_assert(!Stor<T>::kScaled && !kStochastic<T>, "FP32 / FP64 storage");
   __shared__ C nw_v[kWarps][13][33];
-  __shared__ uint32_t nw_ex[kWarps][32], nw_fl[kWarps][32];
   const int lane = static_cast<int>(threadIdx.x & 31u), w = static_cast<int>(threadIdx.x >> 5);
   const uint32_t first = node - static_cast<uint32_t>(lane);
   const int nact = g.n_fluid - first >= 32u ? 32 : static_cast<int>(g.n_fluid - first);
@@ -660,27 +684,14 @@ __device__ __forceinline__ void node_links_warp(const T *src, T *dst,
     nw_v[w][11][lane] = c_.uy;
     nw_v[w][12][lane] = c_.uu;
   }
-  uint32_t incl = nl;
-#pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    const uint32_t v = __shfl_up_sync(am, incl, off);
-    if (lane >= off) incl += v;
-  }
-  const uint32_t excl = incl - nl, total = __shfl_sync(am, incl, nact - 1);
-  const uint32_t base = __shfl_sync(am, li - excl, __ffs(static_cast<int>(anyl)) - 1);
-  nw_ex[w][lane] = excl;
-  nw_fl[w][lane] = fl;
+  const uint32_t total = __reduce_add_sync(am, nl);
+  const uint32_t base = __shfl_sync(am, li, __ffs(static_cast<int>(anyl)) - 1);
   __syncwarp(am);
   const uint32_t tail = 9u * g.plane;
   for (uint32_t t = static_cast<uint32_t>(lane); t < total; t += static_cast<uint32_t>(nact)) {
-    int s = 0;
-#pragma unroll
-    for (int st = 16; st >= 1; st >>= 1)
-      if (s + st < nact && nw_ex[w][s + st] <= t) s += st;
-    uint32_t m = nw_fl[w][s];
-    for (uint32_t r = t - nw_ex[w][s]; r; r--) m &= m - 1u;
-    const int j = __ffs(static_cast<int>(m)), jb = opp2(j);
-    const uint32_t lj = base + t;
+    const uint32_t lj = base + t, dsc = g.ldesc[lj];
+    const int s = static_cast<int>((dsc >> 4) & 31u), j = static_cast<int>(dsc & 15u);
+    const int jb = opp2(j);
     const LinkCoef<C> c = links[lj];
     const C wj = j < 5 ? C(1.0 / 9) : C(1.0 / 36);
     const C r = c.k1 + c.k2 + c.k3;

@@ -57,16 +57,20 @@ struct alignas(sizeof(C) * 4) LinkCoef {
 };
 
 // The FP64 coefficients k1, k2, k3, alpha of a link as pairs of FP32 values
-// (hi + lo, lo the FP32 rounding of what hi leaves): the exact-mass variant
-// evaluates its links in double-FP32 arithmetic.
-struct alignas(16) LinkCoefDF {
-  float hi[4], lo[4];
+// (hi + lo, lo the FP32 rounding of what hi leaves), and a fifth pair, c2 of
+// LinkCoef's form (diffuse_mode 0: (1 - r) w_i) or c0 - alpha (diffuse_mode
+// 1: (r - 1) w_i): the exact-mass variant evaluates its links in double-FP32
+// arithmetic.
+struct alignas(8) LinkCoefDF {
+  float hi[5], lo[5];
 };
-inline LinkCoefDF link_coef_df(const double *c) {
+inline LinkCoefDF link_coef_df(const double *c, double weight, int diffuse_mode) {
   LinkCoefDF r;
-  for (int i = 0; i < 4; i++) {
-    r.hi[i] = static_cast<float>(c[i]);
-    r.lo[i] = static_cast<float>(c[i] - static_cast<double>(r.hi[i]));
+  const double m = (1.0 - (c[0] + c[1] + c[2])) * weight;
+  const double v[5] = {c[0], c[1], c[2], c[3], diffuse_mode == 0 ? m : -m};
+  for (int i = 0; i < 5; i++) {
+    r.hi[i] = static_cast<float>(v[i]);
+    r.lo[i] = static_cast<float>(v[i] - static_cast<double>(r.hi[i]));
   }
   return r;
 }
@@ -199,7 +203,7 @@ struct PullGeom {
   uint32_t plane = 0;               // P
   uint32_t n_fluid = 0;
   uint32_t pf_dist = 0;             // step kernel: CTAs ahead whose data it prefetches to L2
-  // the exact-mass variant (FP32 storage): FP64 link coefficients and, per
+  // the exact-mass variant (FP32 storage): double-FP32 link coefficients and, per
   // link and per node (rest population), the remainder of its values that
   // FP32 storage has not yet taken
   const LinkCoefDF *links64 = nullptr;
@@ -291,8 +295,9 @@ std::vector<uint32_t> link_jb_slots(const CompactCase &cc, int ny, int periodic_
 
 // For every link (node x, direction j) of a compacted case, in link-table
 // order: (x mod 64) << 4 | j.  A warp of the paired 16-bit step runs the 64
-// nodes of one 64-aligned block (x mod 64 is the node's place in it), so
-// each lane finds its link's node and direction from this one entry.
+// nodes of one 64-aligned block (x mod 64 is the node's place in it), a warp
+// of the one-node steps the 32 of a 32-aligned block (x mod 32), so each
+// lane finds its link's node and direction from this one entry.
 std::vector<uint16_t> link_descriptors(const CompactCase &cc, int64_t n_links);
 
 // Kernel constants of one case in arithmetic type C.
