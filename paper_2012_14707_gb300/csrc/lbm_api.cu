@@ -31,6 +31,7 @@ struct lbm_handle {
   int2 *grp = nullptr;    // per group of lbm::kGroup nodes: first row, first link
   uint32_t *jbslot = nullptr;  // per link: slot of f_jb(x, t) (lbm::link_jb_slots)
   uint16_t *ldesc = nullptr;   // per link: (x mod 64) << 4 | j (lbm::link_descriptors)
+  bool narrow = false;  // the step runs in one-warp CTAs (lbm::narrow_ctas)
   uint32_t pf_dist = 0;        // L2 prefetch distance of the step kernel, in CTAs
   int32_t *rowstart = nullptr;
   int32_t *index = nullptr;  // y * nx + x -> compacted index or -1
@@ -230,7 +231,7 @@ cudaError_t do_step(lbm_handle_t *h) {
     return lbm::launch_step_pull<T, C>(static_cast<const T *>(h->f[src]),
                                        static_cast<T *>(h->f[dst]), pull_geom(h), h->n_fluid,
                                        static_cast<const lbm::LinkCoef<C> *>(h->links),
-                                       step_const<C>(h), h->stream);
+                                       step_const<C>(h), h->narrow, h->stream);
   });
   if (e == cudaSuccess) {
     h->cur = dst;
@@ -706,7 +707,9 @@ int lbm_create(const lbm_domain_t *dom, const uint8_t *solid, size_t n_links,
   h->n_fluid = hc.n_fluid;
   h->n_links = hc.n_links;
   cudaGetDevice(&h->device);
-  // half the step kernel's resident CTAs (see lbm::step_kernel_pull)
+  h->narrow = lbm::narrow_ctas(p.precision, h->n_fluid);
+  // half the step kernel's resident CTAs (see lbm::step_kernel_pull; one-warp
+  // CTAs are all resident at once)
   int resident = 0;
   switch (p.precision) {
     case LBM_FP64: resident = lbm::pull_resident_ctas<double, double>(); break;
@@ -714,7 +717,7 @@ int lbm_create(const lbm_domain_t *dom, const uint8_t *solid, size_t n_links,
     case LBM_BF16: resident = lbm::pull_resident_ctas<__nv_bfloat16, float>(); break;
     default: resident = lbm::pull_resident_ctas<__half, float>(); break;
   }
-  h->pf_dist = static_cast<uint32_t>(resident / 2);
+  h->pf_dist = h->narrow ? 0u : static_cast<uint32_t>(resident / 2);
 
   const size_t es = elem_size(p.precision);
   // nine planes, then the link tail (rounded up to whole 128-byte lines)

@@ -194,72 +194,79 @@ batch_exact_kernel(const float *src, float *dst,
                   StepGate{j, active + c, counter});
 }
 
-// One CTA per case: residual of the case (FP64 sums in a fixed order); a
-// case whose residual fell below tol, or whose state is no longer finite,
-// is retired with the step count at which that happened (negative when
-// unstable).  A case with residual_mode 1 takes the interval residual: its
-// velocity against the snapshot of the previous check (snap, two values per
-// node-arena entry), divided by the K steps since, and the snapshot is
-// replaced.  init: only write the snapshots of those cases (the start of
-// the first interval), retire nothing.
+// The batched residual's first pass: CTA b sums part first_part + b, up to
+// kPartNodes nodes of one case (FP64 sums in a fixed order), into
+// partials[3 part ..]: squared change, squared velocity, non-finite nodes.  A
+// case with residual_mode 1 takes the interval residual: its velocity
+// against the snapshot of the previous check (snap, two values per
+// node-arena entry), which is replaced.  init: only write the snapshots of
+// those cases (the start of the first interval).
+// (One CTA per case, as before, left the GPU to the few largest cases: 0.9
+// ms a check on 32 cases of up to 114 k nodes, as much as 45 steps.)
+constexpr int kPartNodes = 2048;
+struct BatchPart {
+  int32_t case_, first;  // the case and its first node in this part
+};
 template <typename T, typename C>
 __global__ void __launch_bounds__(kBatchResidualThreads)
-batch_residual_kernel(const T *__restrict__ cur, const T *__restrict__ prev,
-                      const uint2 *__restrict__ node, const int2 *__restrict__ grp,
-                      const int32_t *__restrict__ rowstart,
-                      const BatchCase<C> *__restrict__ cases,
-                      int32_t *__restrict__ active, double tol, const int64_t *__restrict__ counter,
-                      int64_t K, int64_t *__restrict__ steps_done, double *__restrict__ res_out,
-                      int32_t *__restrict__ n_active, C *__restrict__ snap, const int init) {
-  const int c = blockIdx.x;
+batch_residual_partials(const T *__restrict__ cur, const T *__restrict__ prev,
+                        const PullGeom *__restrict__ geoms,
+                        const BatchCase<C> *__restrict__ cases,
+                        const BatchPart *__restrict__ parts, const int32_t first_part,
+                        const int32_t *__restrict__ active, C *__restrict__ snap,
+                        double *__restrict__ partials, const int init) {
+  const int32_t part = first_part + static_cast<int32_t>(blockIdx.x);
+  const int c = parts[part].case_;
   if (!active[c]) return;
   const BatchCase<C> &bc = cases[c];
-  const StepConst<C> k = bc.k;
+  const StepConst<C> &k = bc.k;
   const bool interval = k.residual_mode == 1 && snap;
   if (init && !interval) return;
   const T *a_base = cur + bc.f_off;
   const T *b_base = prev + bc.f_off;
   C *sn = interval ? snap + 2 * bc.node_off : nullptr;
   NodeMap map;
-  map.pull = case_geom(bc, node, grp, rowstart, static_cast<const uint32_t *>(nullptr));
+  map.pull = geoms[c];
+  const C ax = k.ax, ay = k.ay, inv_sc = k.inv_sc;
+  const uint32_t plane = static_cast<uint32_t>(k.plane);
+  const int64_t end = min(bc.n_fluid, static_cast<int64_t>(parts[part].first) + kPartNodes);
   double num = 0.0, den = 0.0, bad = 0.0;
-  {
-    for (int64_t i = threadIdx.x; i < bc.n_fluid; i += blockDim.x) {
-      uint32_t s[9];
-      map.slots(static_cast<uint32_t>(i), static_cast<uint32_t>(k.plane), s);
-      C a[9], b[9];
-      bool sat = false;
+  for (int64_t i = parts[part].first + static_cast<int64_t>(threadIdx.x); i < end;
+       i += kBatchResidualThreads) {
+    uint32_t s[9];
+    map.slots(static_cast<uint32_t>(i), plane, s);
+    C a[9], b[9];
+    bool sat = false;
 #pragma unroll
-      for (int q = 0; q < 9; q++) {
-        a[q] = Stor<T>::ld(a_base[s[q]], k.inv_sc);
-        b[q] = interval ? C(0) : Stor<T>::ld(b_base[s[q]], k.inv_sc);
-        if constexpr (kStochastic<T>)
-          sat |= fabsf(Stor<T>::ld_raw(a_base[s[q]])) >= Stor<T>::kMaxRaw ||
-                 (!interval && fabsf(Stor<T>::ld_raw(b_base[s[q]])) >= Stor<T>::kMaxRaw);
-      }
-      C n1, d1, m1;
-      if (interval) {
-        const C r = C(1) + (((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7])) + a[8]);
-        const C jx = a[1] - a[3] + (a[5] - a[6]) + (a[8] - a[7]);
-        const C jy = a[2] - a[4] + (a[5] + a[6]) - (a[7] + a[8]);
-        const C ux = (jx + C(0.5) * r * k.ax) / r, uy = (jy + C(0.5) * r * k.ay) / r;
-        const C dx = ux - sn[2 * i], dy = uy - sn[2 * i + 1];
-        sn[2 * i] = ux;
-        sn[2 * i + 1] = uy;
-        n1 = dx * dx + dy * dy;
-        d1 = ux * ux + uy * uy;
-        m1 = r - C(1);
-      } else {
-        residual_terms<C>(a, b, k.ax, k.ay, n1, d1, m1);
-      }
-      // a saturated 16-bit value counts as non-finite
-      if (sat || !(isfinite(n1) && isfinite(d1) && isfinite(m1))) {
-        bad += 1.0;
-        continue;
-      }
-      num += static_cast<double>(n1);
-      den += static_cast<double>(d1);
+    for (int q = 0; q < 9; q++) {
+      a[q] = Stor<T>::ld(a_base[s[q]], inv_sc);
+      b[q] = interval ? C(0) : Stor<T>::ld(b_base[s[q]], inv_sc);
+      if constexpr (kStochastic<T>)
+        sat |= fabsf(Stor<T>::ld_raw(a_base[s[q]])) >= Stor<T>::kMaxRaw ||
+               (!interval && fabsf(Stor<T>::ld_raw(b_base[s[q]])) >= Stor<T>::kMaxRaw);
     }
+    C n1, d1, m1;
+    if (interval) {
+      const C r = C(1) + (((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7])) + a[8]);
+      const C jx = a[1] - a[3] + (a[5] - a[6]) + (a[8] - a[7]);
+      const C jy = a[2] - a[4] + (a[5] + a[6]) - (a[7] + a[8]);
+      const C ux = (jx + C(0.5) * r * ax) / r, uy = (jy + C(0.5) * r * ay) / r;
+      const C dx = ux - sn[2 * i], dy = uy - sn[2 * i + 1];
+      sn[2 * i] = ux;
+      sn[2 * i + 1] = uy;
+      n1 = dx * dx + dy * dy;
+      d1 = ux * ux + uy * uy;
+      m1 = r - C(1);
+    } else {
+      residual_terms<C>(a, b, ax, ay, n1, d1, m1);
+    }
+    // a saturated 16-bit value counts as non-finite
+    if (sat || !(isfinite(n1) && isfinite(d1) && isfinite(m1))) {
+      bad += 1.0;
+      continue;
+    }
+    num += static_cast<double>(n1);
+    den += static_cast<double>(d1);
   }
   if (init) return;
   __shared__ double sh[kBatchResidualThreads / 32][3];
@@ -273,14 +280,39 @@ batch_residual_kernel(const T *__restrict__ cur, const T *__restrict__ prev,
     sh[w][2] = bad;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (threadIdx.x < 3) {
+    double t = 0.0;
+    for (int i = 0; i < kBatchResidualThreads / 32; i++) t += sh[i][threadIdx.x];
+    partials[3 * static_cast<int64_t>(part) + threadIdx.x] = t;
+  }
+}
+
+// The second pass, one CTA: each warp takes cases in turn, adds a case's
+// parts in a fixed order, and retires a case whose residual fell below tol,
+// or whose state is no longer finite, with the step count at which that
+// happened (negative when unstable); the interval residual is divided by the
+// K steps since the previous check.  Then the step counter advances.
+constexpr int kBatchFinalThreads = 1024;
+template <typename C>
+__global__ void __launch_bounds__(kBatchFinalThreads)
+batch_residual_final(const double *__restrict__ partials, const int32_t *__restrict__ part_first,
+                     const BatchCase<C> *__restrict__ cases, const int n_cases,
+                     int32_t *__restrict__ active, double tol, int64_t *__restrict__ counter,
+                     int64_t K, int64_t *__restrict__ steps_done, double *__restrict__ res_out,
+                     int32_t *__restrict__ n_active, const int has_snap) {
+  const int lane = threadIdx.x & 31;
+  const int64_t now = *counter + K;
+  for (int c = static_cast<int>(threadIdx.x >> 5); c < n_cases; c += kBatchFinalThreads / 32) {
+    if (!active[c]) continue;
     double s[3] = {0.0, 0.0, 0.0};
-    for (int i = 0; i < kBatchResidualThreads / 32; i++)
-      for (int q = 0; q < 3; q++) s[q] += sh[i][q];
+    for (int32_t p = part_first[c] + lane; p < part_first[c + 1]; p += 32)
+      for (int q = 0; q < 3; q++) s[q] += partials[3 * static_cast<int64_t>(p) + q];
+    for (int q = 0; q < 3; q++) s[q] = warp_sum(s[q]);
+    if (lane != 0) continue;
+    const bool interval = cases[c].k.residual_mode == 1 && has_snap;
     const double res = (s[1] > 0.0 ? sqrt(s[0] / s[1]) : (s[0] > 0.0 ? INFINITY : 0.0)) /
                        (interval ? static_cast<double>(K) : 1.0);
     res_out[c] = res;
-    const int64_t now = *counter + K;
     if (s[2] > 0.0 || isnan(res)) {
       active[c] = 0;
       steps_done[c] = -now;
@@ -291,9 +323,9 @@ batch_residual_kernel(const T *__restrict__ cur, const T *__restrict__ prev,
       atomicSub(n_active, 1);
     }
   }
+  __syncthreads();
+  if (threadIdx.x == 0) *counter = now;
 }
-
-__global__ void batch_advance(int64_t *counter, int64_t K) { *counter += K; }
 
 template <typename T, typename C, int THREADS>
 cudaError_t launch_batch_step(const T *src, T *dst, const uint2 *node, const int2 *grp,
@@ -302,7 +334,8 @@ cudaError_t launch_batch_step(const T *src, T *dst, const uint2 *node, const int
                               const int32_t *active, const int32_t *work, int32_t n_work,
                               uint32_t pf_dist, const int64_t *counter, uint32_t j,
                               const PullGeom *geoms, const int32_t *exact_chunks,
-                              int32_t n_exact_chunks, cudaStream_t s) {
+                              int32_t n_exact_chunks, cudaStream_t s, cudaStream_t side,
+                              cudaEvent_t fork, cudaEvent_t join) {
   if constexpr (kStochastic<T>) {
     if constexpr (THREADS <= kChunk / 2) {
       if (n_work > 0)
@@ -319,18 +352,34 @@ cudaError_t launch_batch_step(const T *src, T *dst, const uint2 *node, const int
   }
   const int64_t blocks = static_cast<int64_t>(n_work) * (kChunk / THREADS);
   cudaError_t e = cudaSuccess;
-  if (blocks > 0)
-    e = launch_chained(batch_step_kernel<T, C, THREADS>, dim3(static_cast<unsigned>(blocks)), THREADS, 0, s,
-                       src, dst, node, grp, ccase, rowstart, jbslot,
-                       static_cast<const LinkCoef<C> *>(links),
-                       static_cast<const BatchCase<C> *>(cases), active, work,
-                       static_cast<uint32_t>(blocks), pf_dist, counter, j, geoms);
+  // Exact-mass cases beside others, while a step is captured: their launch
+  // goes to the side stream, forked from and joined to this one, and the two
+  // become parallel nodes of the graph.  32 uneven cases of up to 512 x 256
+  // nodes (0.72 M plain, 0.18 M exact-mass fluid nodes): 21.6 us a step
+  // against 23.6 in a row as a chain (12.7 and 9.5 alone); one launch for
+  // both kinds took 22.8 (the plain step at the exact one's registers).
+  const bool beside = side && blocks > 0 && n_exact_chunks > 0;
+  if (beside) {
+    e = cudaEventRecord(fork, s);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(side, fork, 0);
+  }
   if constexpr (std::is_same<T, float>::value) {
     if (e == cudaSuccess && n_exact_chunks > 0)
-      e = launch_chained(batch_exact_kernel, dim3(static_cast<unsigned>(n_exact_chunks)), kChunk, 0, s, src,
-                         dst, ccase, static_cast<const LinkCoef<float> *>(links),
-                         static_cast<const BatchCase<float> *>(cases), active, exact_chunks,
-                         counter, j, geoms);
+      e = launch_kernel(!beside, batch_exact_kernel, dim3(static_cast<unsigned>(n_exact_chunks)),
+                        kChunk, 0, beside ? side : s, src, dst, ccase,
+                        static_cast<const LinkCoef<float> *>(links),
+                        static_cast<const BatchCase<float> *>(cases), active, exact_chunks, counter,
+                        j, geoms);
+  }
+  if (e == cudaSuccess && blocks > 0)
+    e = launch_kernel(!beside, batch_step_kernel<T, C, THREADS>,
+                      dim3(static_cast<unsigned>(blocks)), THREADS, 0, s, src, dst, node, grp,
+                      ccase, rowstart, jbslot, static_cast<const LinkCoef<C> *>(links),
+                      static_cast<const BatchCase<C> *>(cases), active, work,
+                      static_cast<uint32_t>(blocks), pf_dist, counter, j, geoms);
+  if (beside) {
+    if (e == cudaSuccess) e = cudaEventRecord(join, side);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(s, join, 0);
   }
   return e;
 }
@@ -404,6 +453,18 @@ struct lbm_batch {
   int32_t n_work = 0;
   int32_t n_listed = 0;  // active cases when the lists were last built
   void *snap = nullptr;  // interval-residual snapshots (2 values per node-arena entry), or null
+  // the batched residual's parts (device; part_first: per case, n_cases + 1)
+  // and their sums
+  lbm::BatchPart *parts = nullptr;
+  int32_t *part_first = nullptr;
+  std::vector<int32_t> h_part_first;
+  double *partials = nullptr;
+  // one case's FP64 fields on the device (the largest case's size), on their
+  // way from or to the caller
+  double *stage = nullptr;
+  // the exact-mass cases' steps beside the others' in the captured graph
+  cudaStream_t side = nullptr;
+  cudaEvent_t fork = nullptr, join = nullptr;
   int threads = 0;
   uint32_t pf_dist = 0;  // L2 prefetch distance of the step kernel (CTAs), for `threads`
   int32_t *active = nullptr;
@@ -456,8 +517,9 @@ lbm::NodeMap case_map(const lbm_batch_t *b, int c) {
 }
 
 // One step launch; j = the step's position after the last advance of the
-// device step counter (seeds the random bits).
-cudaError_t step_once(lbm_batch_t *b, int threads, uint32_t pf_dist, int src, uint32_t j) {
+// device step counter (seeds the random bits).  capturing: into the graph.
+cudaError_t step_once(lbm_batch_t *b, int threads, uint32_t pf_dist, int src, uint32_t j,
+                      bool capturing = false) {
   const int dst = 1 - src;
   return dispatch_b(b->precision, [&](auto tT, auto tC) {
     using T = std::remove_pointer_t<decltype(tT)>;
@@ -467,7 +529,8 @@ cudaError_t step_once(lbm_batch_t *b, int threads, uint32_t pf_dist, int src, ui
       return lbm::launch_batch_step<T, C, TH>(
           static_cast<const T *>(b->f[src]), static_cast<T *>(b->f[dst]), b->node, b->grp,
           b->ccase, b->rowstart, b->jbslot, b->links, b->cases, b->active, b->work, b->n_work,
-          pf_dist, b->counter, j, b->geoms, b->exact_chunks, b->n_exact_chunks, b->stream);
+          pf_dist, b->counter, j, b->geoms, b->exact_chunks, b->n_exact_chunks, b->stream,
+          capturing ? b->side : nullptr, b->fork, b->join);
     };
     if (threads == 64) return go(std::integral_constant<int, 64>());
     if (threads == 128) return go(std::integral_constant<int, 128>());
@@ -503,19 +566,27 @@ cudaError_t build_lists(lbm_batch_t *b, const int32_t *active_host) {
   return e;
 }
 
-// Snapshots of the interval residual from the current state (lattice 0,
-// every active case with residual_mode 1): the start of an interval.
-cudaError_t init_snapshots(lbm_batch_t *b) {
-  if (!b->snap) return cudaSuccess;
+// The residual's first pass over the parts of case c (all cases: c < 0).
+cudaError_t residual_parts(lbm_batch_t *b, int c, int init) {
+  const int32_t p0 = c < 0 ? 0 : b->h_part_first[c];
+  const int32_t p1 = c < 0 ? b->h_part_first[b->n_cases] : b->h_part_first[c + 1];
   return dispatch_b(b->precision, [&](auto tT, auto tC) {
     using T = std::remove_pointer_t<decltype(tT)>;
     using C = std::remove_pointer_t<decltype(tC)>;
-    lbm::batch_residual_kernel<T, C><<<b->n_cases, lbm::kBatchResidualThreads, 0, b->stream>>>(
-        static_cast<const T *>(b->f[0]), static_cast<const T *>(b->f[1]), b->node, b->grp,
-        b->rowstart, static_cast<const lbm::BatchCase<C> *>(b->cases), b->active, 0.0, b->counter,
-        1, b->steps_done, b->res, b->n_active, static_cast<C *>(b->snap), 1);
+    lbm::batch_residual_partials<T, C>
+        <<<static_cast<unsigned>(p1 - p0), lbm::kBatchResidualThreads, 0, b->stream>>>(
+            static_cast<const T *>(b->f[0]), static_cast<const T *>(b->f[1]), b->geoms,
+            static_cast<const lbm::BatchCase<C> *>(b->cases), b->parts, p0, b->active,
+            static_cast<C *>(b->snap), b->partials, init);
     return cudaGetLastError();
   });
+}
+
+// Snapshots of the interval residual from the current state (lattice 0,
+// case c or, c < 0, every active case with residual_mode 1): the start of an
+// interval.
+cudaError_t init_snapshots(lbm_batch_t *b, int c) {
+  return b->snap ? residual_parts(b, c, 1) : cudaSuccess;
 }
 
 int bfail(lbm_batch_t *b, int code, const std::string &m) {
@@ -533,9 +604,14 @@ void batch_release(lbm_batch_t *b) {
                   static_cast<void *>(b->counter), static_cast<void *>(b->n_active),
                   static_cast<void *>(b->links64), static_cast<void *>(b->carry),
                   static_cast<void *>(b->exact_chunks), static_cast<void *>(b->geoms), b->snap,
+                  static_cast<void *>(b->parts), static_cast<void *>(b->part_first),
+                  static_cast<void *>(b->partials), static_cast<void *>(b->stage),
                   static_cast<void *>(b->work)})
     if (p) cudaFree(p);
   if (b->h_n_active) cudaFreeHost(b->h_n_active);
+  if (b->fork) cudaEventDestroy(b->fork);
+  if (b->join) cudaEventDestroy(b->join);
+  if (b->side) cudaStreamDestroy(b->side);
   if (b->own_stream) cudaStreamDestroy(b->stream);
   delete b;
 }
@@ -801,6 +877,35 @@ int lbm_batch_create(const lbm_case_t *cases, int32_t n_cases, int32_t precision
   if (e == cudaSuccess) e = alloc(reinterpret_cast<void **>(&b->res), n_cases * 8);
   if (e == cudaSuccess) e = alloc(reinterpret_cast<void **>(&b->counter), 8);
   if (e == cudaSuccess) e = alloc(reinterpret_cast<void **>(&b->n_active), 4);
+  {
+    std::vector<lbm::BatchPart> parts;
+    for (int32_t c = 0; c < n_cases; c++) {
+      b->h_part_first.push_back(static_cast<int32_t>(parts.size()));
+      for (int64_t i = 0; i < std::max<int64_t>(1, b->n_fluid[c]); i += lbm::kPartNodes)
+        parts.push_back({c, static_cast<int32_t>(i)});
+    }
+    b->h_part_first.push_back(static_cast<int32_t>(parts.size()));
+    const size_t pb = parts.size() * sizeof(parts[0]), fb = b->h_part_first.size() * 4;
+    if (e == cudaSuccess) e = alloc(reinterpret_cast<void **>(&b->parts), pb);
+    if (e == cudaSuccess) e = alloc(reinterpret_cast<void **>(&b->part_first), fb);
+    if (e == cudaSuccess)
+      e = alloc(reinterpret_cast<void **>(&b->partials), parts.size() * 3 * sizeof(double));
+    if (e == cudaSuccess) e = cudaMemcpy(b->parts, parts.data(), pb, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess)
+      e = cudaMemcpy(b->part_first, b->h_part_first.data(), fb, cudaMemcpyHostToDevice);
+  }
+  {
+    int64_t most = 1;
+    for (int32_t c = 0; c < n_cases; c++)
+      most = std::max(most, static_cast<int64_t>(b->nx[c]) * b->ny[c]);
+    if (e == cudaSuccess)
+      e = alloc(reinterpret_cast<void **>(&b->stage), static_cast<size_t>(most) * 3 * sizeof(double));
+  }
+  if (e == cudaSuccess && any_exact) {
+    e = cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->join, cudaEventDisableTiming);
+  }
   if (e == cudaSuccess && any_interval)
     e = alloc(&b->snap, static_cast<size_t>(nodes) * 2 * (precision == LBM_FP64 ? 8 : 4));
   if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void **>(&b->h_n_active), 4);
@@ -882,7 +987,7 @@ int lbm_batch_reset(lbm_batch_t *b) {
     e = cudaMemcpyAsync(b->steps_done, zeros.data(), n * 8, cudaMemcpyHostToDevice, b->stream);
   if (e == cudaSuccess) e = cudaMemcpyAsync(b->counter, &zero, 8, cudaMemcpyHostToDevice, b->stream);
   if (e == cudaSuccess) e = cudaMemcpyAsync(b->n_active, &n, 4, cudaMemcpyHostToDevice, b->stream);
-  if (e == cudaSuccess) e = init_snapshots(b);
+  if (e == cudaSuccess) e = init_snapshots(b, -1);
   if (e == cudaSuccess && b->n_listed != b->n_cases) e = build_lists(b, nullptr);
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
   if (e != cudaSuccess) return bfail(b, LBM_ECUDA, std::string("lbm_batch_reset: ") + cudaGetErrorString(e));
@@ -909,22 +1014,17 @@ int lbm_batch_run_to(lbm_batch_t *b, double tol, int64_t max_steps, int32_t chec
     cudaGraph_t g = nullptr;
     cudaError_t ec = cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal);
     for (int s = 0; s < check_every && ec == cudaSuccess; s++)
-      ec = step_once(b, b->threads, b->pf_dist, s & 1, static_cast<uint32_t>(s));
+      ec = step_once(b, b->threads, b->pf_dist, s & 1, static_cast<uint32_t>(s), true);
+    if (ec == cudaSuccess) ec = residual_parts(b, -1, 0);
     if (ec == cudaSuccess)
-      ec = dispatch_b(b->precision, [&](auto tT, auto tC) {
-        using T = std::remove_pointer_t<decltype(tT)>;
+      ec = dispatch_b(b->precision, [&](auto, auto tC) {
         using C = std::remove_pointer_t<decltype(tC)>;
-        lbm::batch_residual_kernel<T, C><<<b->n_cases, lbm::kBatchResidualThreads, 0, b->stream>>>(
-            static_cast<const T *>(b->f[0]), static_cast<const T *>(b->f[1]), b->node, b->grp,
-            b->rowstart, static_cast<const lbm::BatchCase<C> *>(b->cases), b->active, tol,
-            b->counter, check_every, b->steps_done, b->res, b->n_active, static_cast<C *>(b->snap),
-            0);
+        lbm::batch_residual_final<C><<<1, lbm::kBatchFinalThreads, 0, b->stream>>>(
+            b->partials, b->part_first, static_cast<const lbm::BatchCase<C> *>(b->cases),
+            b->n_cases, b->active, tol, b->counter, check_every, b->steps_done, b->res,
+            b->n_active, b->snap ? 1 : 0);
         return cudaGetLastError();
       });
-    if (ec == cudaSuccess) {
-      lbm::batch_advance<<<1, 1, 0, b->stream>>>(b->counter, check_every);
-      ec = cudaGetLastError();
-    }
     if (ec == cudaSuccess)
       ec = cudaMemcpyAsync(b->h_n_active, b->n_active, 4, cudaMemcpyDeviceToHost, b->stream);
     cudaError_t e2 = cudaStreamEndCapture(b->stream, &g);
@@ -976,21 +1076,19 @@ int lbm_batch_fields(lbm_batch_t *b, int32_t c, double *rho, double *ux, double 
   if (!b) return LBM_EINVAL;
   if (c < 0 || c >= b->n_cases) return bfail(b, LBM_EINVAL, "case index out of range");
   const int64_t n = static_cast<int64_t>(b->nx[c]) * b->ny[c];
-  double *d = nullptr;
-  cudaError_t e = cudaMalloc(&d, 3 * n * sizeof(double));
-  if (e != cudaSuccess) return bfail(b, LBM_ENOMEM, cudaGetErrorString(e));
+  double *d = b->stage;
   const int64_t plane = b->plane[c];
-  e = dispatch_b(b->precision, [&](auto tT, auto tC) {
+  cudaError_t e = dispatch_b(b->precision, [&](auto tT, auto tC) {
     using T = std::remove_pointer_t<decltype(tT)>;
     return lbm::launch_fields<T>(static_cast<const T *>(b->f[b->cur]) + b->f_off[c], case_map(b, c),
-                                 plane, b->ax[c], b->ay[c], b->scale[c], d, d + n, d + 2 * n,
-                                 b->stream);
+                                 plane, b->ax[c], b->ay[c], b->scale[c], rho ? d : nullptr,
+                                 ux ? d + n : nullptr, uy ? d + 2 * n : nullptr, b->stream);
   });
+  double *out[3] = {rho, ux, uy};
+  for (int q = 0; q < 3; q++)
+    if (e == cudaSuccess && out[q])
+      e = cudaMemcpyAsync(out[q], d + q * n, n * 8, cudaMemcpyDeviceToHost, b->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
-  if (e == cudaSuccess && rho) e = cudaMemcpy(rho, d, n * 8, cudaMemcpyDeviceToHost);
-  if (e == cudaSuccess && ux) e = cudaMemcpy(ux, d + n, n * 8, cudaMemcpyDeviceToHost);
-  if (e == cudaSuccess && uy) e = cudaMemcpy(uy, d + 2 * n, n * 8, cudaMemcpyDeviceToHost);
-  cudaFree(d);
   if (e != cudaSuccess) return bfail(b, LBM_ECUDA, cudaGetErrorString(e));
   return LBM_OK;
 }
@@ -1001,12 +1099,11 @@ int lbm_batch_set_fields(lbm_batch_t *b, int32_t c, const double *rho, const dou
   if (c < 0 || c >= b->n_cases) return bfail(b, LBM_EINVAL, "case index out of range");
   if (b->cur != 0) return bfail(b, LBM_EINVAL, "batch state is mid-graph; call lbm_batch_reset");
   const int64_t n = static_cast<int64_t>(b->nx[c]) * b->ny[c];
-  double *d = nullptr;
-  cudaError_t e = cudaMalloc(&d, 3 * n * sizeof(double));
-  if (e != cudaSuccess) return bfail(b, LBM_ENOMEM, cudaGetErrorString(e));
-  e = cudaMemcpy(d, rho, n * 8, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(d + n, ux, n * 8, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(d + 2 * n, uy, n * 8, cudaMemcpyHostToDevice);
+  double *d = b->stage;
+  const double *in[3] = {rho, ux, uy};
+  cudaError_t e = cudaSuccess;
+  for (int q = 0; q < 3 && e == cudaSuccess; q++)
+    e = cudaMemcpyAsync(d + q * n, in[q], n * 8, cudaMemcpyHostToDevice, b->stream);
   const int64_t plane = b->plane[c];
   if (e == cudaSuccess)
     e = dispatch_b(b->precision, [&](auto tT, auto tC) {
@@ -1016,9 +1113,9 @@ int lbm_batch_set_fields(lbm_batch_t *b, int32_t c, const double *rho, const dou
                                        static_cast<T *>(b->f[0]) + b->f_off[c],
                                        static_cast<T *>(b->f[1]) + b->f_off[c], b->stream);
     });
-  if (e == cudaSuccess) e = init_snapshots(b);
+  if (e == cudaSuccess) e = init_snapshots(b, c);
+  // (the caller's arrays may be pinned, and then still on their way)
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
-  cudaFree(d);
   if (e != cudaSuccess) return bfail(b, LBM_ECUDA, cudaGetErrorString(e));
   return LBM_OK;
 }

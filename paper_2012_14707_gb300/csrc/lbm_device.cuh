@@ -183,31 +183,21 @@ __device__ __forceinline__ void sum2(const float (&a)[N], float &s, float &e) {
 }
 
 // a + b rounded to FP32 stochastically: the FP32 sum s (round to nearest)
-// or its neighbour on the side of the exact remainder e = a + b - s
-// (TwoSum, Knuth), taken with probability |e| / (spacing there), so the
-// result is a + b on average.  u16: 16 random bits.
+// or its neighbour s2 on the side of the exact remainder e = a + b - s
+// (TwoSum, Knuth), taken with probability |e| / |s2 - s|, so the result is a
+// + b on average.  u16: 16 random bits, as a fraction of |s2 - s| (1.u16
+// times the gap less the gap: no integer conversion).  e = 0 (and with it s
+// = 0) keeps s: no fraction is below zero, and a gap that is no number
+// compares false.
 __device__ __forceinline__ float add_stochastic(float a, float b, uint32_t u16) {
   const float s = a + b;
   const float bb = s - a;
   const float e = (a - (s - bb)) + (b - bb);
-  if (e == 0.0f || s == 0.0f) return s;
   const int bits = __float_as_int(s);
   const float s2 = __int_as_float(((e > 0.0f) == (s > 0.0f)) ? bits + 1 : bits - 1);
-  return static_cast<float>(u16) * 0x1p-16f * fabsf(s2 - s) < fabsf(e) ? s2 : s;
-}
-
-// x rounded to FP32 stochastically: the nearest FP32 value s or its
-// neighbour on the side of the remainder e = x - s (exact in FP64), taken
-// with probability |e| / (spacing there), so the result is x on average.
-// u16: 16 random bits.
-__device__ __forceinline__ float round_stochastic(double x, uint32_t u16) {
-  const float s = __double2float_rn(x);
-  const double e = x - static_cast<double>(s);
-  if (e == 0.0 || s == 0.0f) return s;
-  const int bits = __float_as_int(s);
-  const float s2 = __int_as_float(((e > 0.0) == (s > 0.0f)) ? bits + 1 : bits - 1);
-  return static_cast<double>(u16) * 0x1p-16 * fabs(static_cast<double>(s2) - s) < fabs(e) ? s2
-                                                                                          : s;
+  const float gap = fabsf(s2 - s);
+  const float f = __int_as_float(static_cast<int>(0x3F800000u | (u16 << 7)));
+  return __fmaf_rn(f, gap, -gap) < fabsf(e) ? s2 : s;
 }
 
 // Double-FP32 values h + l with |l| <= ulp(h) / 2 (Dekker's double-length
@@ -367,8 +357,7 @@ __device__ __forceinline__ void collision_change(const C (&d)[9], const StepCons
 // mass with the fluid at a rate set by the velocity next to it, so every
 // rounding that leans the same way step after step shows up in the mass.
 // Hence: rho - 1 and j are summed in twice the working precision (sum2),
-// rho and u rounded once each (u by the correctly rounded division, no
-// approximate reciprocal) for the equilibrium, and kept for the links'
+// rho and u rounded once each for the equilibrium, and kept for the links'
 // FP64 values; f'_1..f'_8 are rounded to FP32 stochastically
 // (add_stochastic, random bits from rs); f'_0 closes the node's mass in
 // twice the working precision plus the node's carry c0 (what FP32 storage
@@ -386,16 +375,21 @@ __device__ __forceinline__ void collide(const C (&d)[9], const StepConst<C> &k, 
   T(&t)[9] = r.t;
   C ch[9];
   if constexpr (kExact) {
-    // rho - 1 and j in twice the working precision; rho and u rounded once
-    // each (u by the correctly rounded division, no approximate reciprocal)
+    // rho - 1 and j in twice the working precision; rho and u rounded once each
     sum2(d, r.dr_hi, r.dr_lo);
     const float jxs[6] = {d[1], -d[3], d[5], -d[6], -d[7], d[8]};
     const float jys[6] = {d[2], -d[4], d[5], d[6], -d[7], -d[8]};
     sum2(jxs, r.jx_hi, r.jx_lo);
     sum2(jys, r.jy_hi, r.jy_lo);
-    const float rho = 1.0f + (r.dr_hi + r.dr_lo);
-    const C given[3] = {rho, __fdiv_rn(r.jx_hi + (r.jx_lo + 0.5f * rho * k.ax), rho),
-                        __fdiv_rn(r.jy_hi + (r.jy_lo + 0.5f * rho * k.ay), rho)};
+    const float rho = 1.0f + (r.dr_hi + r.dr_lo), inv = __frcp_rn(rho);
+    // u: the reciprocal's product and one correction from the exact remainder
+    // (the correctly rounded quotient, but for rare last-place ties)
+    auto over_rho = [&](float v) {
+      const float q = __fmul_rn(v, inv);
+      return __fmaf_rn(__fmaf_rn(-q, rho, v), inv, q);
+    };
+    const C given[3] = {rho, over_rho(r.jx_hi + (r.jx_lo + 0.5f * rho * k.ax)),
+                        over_rho(r.jy_hi + (r.jy_lo + 0.5f * rho * k.ay))};
     collision_change<kS, true>(d, k, ch, r.drho, r.rho, r.ux, r.uy, r.uu, given);
   } else {
     collision_change<kS, false>(d, k, ch, r.drho, r.rho, r.ux, r.uy, r.uu);
@@ -1017,6 +1011,59 @@ static __device__ __noinline__ void step_node_exact(const float *src, float *dst
                                              const StepConst<float> &k, const uint32_t i,
                                              const StepGate &gate) {
   step_node_pull<float, float, true>(src, dst, g, links, k, i, gate);
+}
+
+// rho and u = (j + rho a / 2) / rho in FP64 from rho - 1 and j, as FP64 or
+// double-FP32 values (the components of j and of a given one after the
+// other).  FP32 and 16-bit storage: the sums in twice the working precision
+// and the quotient in double-FP32, about 48 significant bits of values that
+// are FP32 to begin with, converted at the end -- this GPU's FP64 units are
+// so few that FP64 sums and divisions per node took several times as long as
+// the memory they read (8.4 M nodes, FP32: fields 711 us, now 150).
+template <int D>
+__device__ __forceinline__ void macro_fields(DF drho, const DF (&j)[D], const DF (&a)[D],
+                                             double &rho, double (&u)[D]) {
+  const DF r = df_add(DF{1.0f, 0.0f}, drho);
+  const float inv = __frcp_rn(r.h);
+  rho = 1.0 + (static_cast<double>(drho.h) + static_cast<double>(drho.l));
+#pragma unroll
+  for (int c = 0; c < D; c++) {
+    const DF v = df_div_inv(df_add(j[c], df_mul(df_scale(0.5f, r), a[c])), r, inv);
+    u[c] = static_cast<double>(v.h) + static_cast<double>(v.l);
+  }
+}
+template <int D>
+__device__ __forceinline__ void macro_fields(double drho, const double (&j)[D],
+                                             const double (&a)[D], double &rho, double (&u)[D]) {
+  rho = 1.0 + drho;
+  for (int c = 0; c < D; c++) u[c] = (j[c] + 0.5 * rho * a[c]) / rho;
+}
+// x in the arithmetic of macro_fields
+template <typename C>
+struct Wide {
+  using type = DF;
+  static __host__ __device__ DF of(double x) {
+    const float h = static_cast<float>(x);
+    return DF{h, static_cast<float>(x - static_cast<double>(h))};
+  }
+};
+template <>
+struct Wide<double> {
+  using type = double;
+  static __host__ __device__ double of(double x) { return x; }
+};
+// Sum of n values: FP64, or FP32 values in twice the working precision.
+template <int N>
+__device__ __forceinline__ double wide_sum(const double (&a)[N]) {
+  double s = a[0];
+  for (int i = 1; i < N; i++) s += a[i];
+  return s;
+}
+template <int N>
+__device__ __forceinline__ DF wide_sum(const float (&a)[N]) {
+  float s, e;
+  sum2(a, s, e);
+  return df_norm(s, e);
 }
 
 // Eq. FluidMacr from deviations: returns rho - 1 (kept exact for the mass sum).

@@ -364,8 +364,8 @@ void parallel_for(int64_t n, F &&f, int64_t min_per_thread = 1 << 14) {
 // its CTAs, and read what no step writes, while this one's last CTAs still
 // run; it waits at dev::chain_wait() for this one's results.
 template <typename... P, typename... A>
-cudaError_t launch_chained(void (*f)(P...), dim3 grid, unsigned threads, size_t smem,
-                           cudaStream_t s, A &&...args) {
+cudaError_t launch_kernel(bool chained, void (*f)(P...), dim3 grid, unsigned threads, size_t smem,
+                          cudaStream_t s, A &&...args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3(threads);
@@ -375,8 +375,13 @@ cudaError_t launch_chained(void (*f)(P...), dim3 grid, unsigned threads, size_t 
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = chained ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, f, P(args)...);
+}
+template <typename... P, typename... A>
+cudaError_t launch_chained(void (*f)(P...), dim3 grid, unsigned threads, size_t smem,
+                           cudaStream_t s, A &&...args) {
+  return launch_kernel(true, f, grid, threads, smem, s, args...);
 }
 
 // Validation and layout of one case (lbm_api.cu).
@@ -437,9 +442,13 @@ struct PairOcc {
 // CTAs of step_kernel_pull<T, C> resident at once on the current device.
 template <typename T, typename C>
 int pull_resident_ctas();
+// Whether a lattice's step runs in CTAs of one warp: FP64, with at most
+// kPullThreads fluid nodes per SM.
+bool narrow_ctas(int precision, int64_t n_fluid);
 template <typename T, typename C>
 cudaError_t launch_step_pull(const T *src, T *dst, const PullGeom &g, int64_t n_fluid,
-                             const LinkCoef<C> *links, const StepConst<C> &k, cudaStream_t s);
+                             const LinkCoef<C> *links, const StepConst<C> &k, bool narrow,
+                             cudaStream_t s);
 
 // Residual and mass of the states in cur and prev (the lattices of two
 // consecutive steps), nodes in the layout of map.

@@ -27,7 +27,11 @@ namespace {
 using namespace dev;
 
 // One time step of a single case (pull layout): thread t of CTA b runs
-// fluid node b * kPullThreads + t.
+// fluid node b * THREADS + t.  THREADS is kPullThreads, or in FP64 one warp
+// where the lattice has at most a CTA's nodes for every SM (narrow_ctas): it
+// then spreads over up to four times as many SMs, whose few FP64 units the
+// four warps of a CTA would queue for (4 x 32 nodes: 6.7 -> 5.6 us a step).
+// FP32 and 16-bit steps of 128 to 34 k nodes ran no faster in one-warp CTAs.
 //
 // Each node waits out two dependent memory latencies (its node word, then
 // the gathers it addresses), which 64 warps per SM do not hide.  So every
@@ -40,20 +44,21 @@ using namespace dev;
 //
 // kExact: the exact-mass variant of FP32 storage (cases with moving walls;
 // see collide and link_epilogue_pull), with 64 registers per thread.
-template <typename T, typename C, bool kExact>
-__global__ void __launch_bounds__(kPullThreads, kExact ? 8 : PullOcc<T>::min_blocks)
+template <typename T, typename C, bool kExact, int THREADS>
+__global__ void __launch_bounds__(THREADS,
+                                  (kExact ? 8 : PullOcc<T>::min_blocks) * kPullThreads / THREADS)
 step_kernel_pull(const T *src, T *dst, __grid_constant__ const PullGeom g,
                  const uint32_t n_fluid, const LinkCoef<C> *__restrict__ links,
                  __grid_constant__ const StepConst<C> k) {
   {
-    constexpr uint32_t kNodeLines = kPullThreads * sizeof(uint2) / 128;
-    constexpr uint32_t kPlaneLines = kPullThreads * sizeof(T) / 128;
+    constexpr uint32_t kNodeLines = THREADS * sizeof(uint2) / 128;
+    constexpr uint32_t kPlaneLines = (THREADS * sizeof(T) + 127) / 128;
     constexpr uint32_t kPerLine = 128 / sizeof(T);
-    const uint32_t base = (blockIdx.x + g.pf_dist) * kPullThreads;
+    const uint32_t base = (blockIdx.x + g.pf_dist) * THREADS;
     const uint32_t t = threadIdx.x;
     // whole warps: the others skip the block without diverging
     constexpr uint32_t kPfThreads = (kNodeLines + 9 * kPlaneLines + 1 + 31) / 32 * 32;
-    static_assert(kPfThreads <= kPullThreads, "one prefetch per thread");
+    static_assert(kPfThreads <= THREADS, "one prefetch per thread");
     if (t < kPfThreads && g.pf_dist && base < n_fluid) {
       if (t < kNodeLines) {
         if (base + t * 16 < n_fluid)
@@ -67,12 +72,12 @@ step_kernel_pull(const T *src, T *dst, __grid_constant__ const PullGeom g,
       }
     }
   }
-  const uint32_t i = blockIdx.x * kPullThreads + threadIdx.x;
+  const uint32_t i = blockIdx.x * THREADS + threadIdx.x;
   if (i >= n_fluid) return;
   if constexpr (kExact)
     step_node_exact(src, dst, g, links, k, i, StepGate{k.sr_seed});
   else
-    step_node_pull<T, C, false, kPullThreads / 32>(src, dst, g, links, k, i, StepGate{k.sr_seed});
+    step_node_pull<T, C, false, THREADS / 32>(src, dst, g, links, k, i, StepGate{k.sr_seed});
 }
 
 // One time step of a single case in 16-bit storage: thread t of CTA b runs
@@ -261,16 +266,21 @@ residual_interval_compact(const T *__restrict__ cur, const NodeMap map, int64_t 
 }
 
 // Pass 2: one block of kFinalThreads sums the partials in a fixed order
-// (thread t first adds blocks t, t + kFinalThreads, ...).
+// (thread t first adds blocks t, t + kFinalThreads, ...).  Pass 1 has a thread
+// per node up to kResidualBlocks blocks; a smaller lattice launches the
+// blocks that have nodes (the others' sums were zeros, so nothing changes).
 constexpr int kFinalThreads = 1024;
-static_assert(kResidualBlocks % kFinalThreads == 0, "whole rounds of partials");
+int residual_blocks(int64_t n_fluid) {
+  const int64_t b = (n_fluid + kResidualThreads - 1) / kResidualThreads;
+  return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(kResidualBlocks, b)));
+}
 __global__ void __launch_bounds__(kFinalThreads)
-residual_final(const double *__restrict__ partials, double *__restrict__ out) {
+residual_final(const double *__restrict__ partials, const int blocks, double *__restrict__ out) {
   __shared__ double sh[kFinalThreads / 32][kPartialStride];
   double v[kPartialStride];
   for (int c = 0; c < kPartialStride; c++) {
     double t = 0.0;
-    for (int b = threadIdx.x; b < kResidualBlocks; b += kFinalThreads)
+    for (int b = threadIdx.x; b < blocks; b += kFinalThreads)
       t += partials[b * kPartialStride + c];
     v[c] = warp_sum(t);
   }
@@ -286,26 +296,31 @@ residual_final(const double *__restrict__ partials, double *__restrict__ out) {
 }
 
 template <typename T>
-__global__ void fields_kernel(const T *__restrict__ f, const NodeMap map, int64_t plane, double ax,
-                              double ay, double inv_scale, double *rho, double *ux, double *uy) {
+__global__ void fields_kernel(const T *__restrict__ f, const NodeMap map, int64_t plane,
+                              const typename Wide<typename Stor<T>::C>::type ax,
+                              const typename Wide<typename Stor<T>::C>::type ay, double inv_scale,
+                              double *rho, double *ux, double *uy) {
   using C = typename Stor<T>::C;
   const int64_t n = static_cast<int64_t>(map.nx) * map.ny;
   for (int64_t p = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; p < n;
        p += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const int64_t y = p / map.nx, x = p - y * map.nx;
-    const int64_t node = map.at(static_cast<int>(x), static_cast<int>(y));
-    double r = 0.0, u = 0.0, v = 0.0;
+    const int64_t node = map.index[p];
+    double r = 0.0, u[2] = {0.0, 0.0};
     if (node >= 0) {
       uint32_t s[9];
       map.slots(static_cast<uint32_t>(node), static_cast<uint32_t>(plane), s);
-      double a[9];
-      for (int i = 0; i < 9; i++)
-        a[i] = static_cast<double>(Stor<T>::ld(f[s[i]], static_cast<C>(inv_scale)));
-      node_velocity(a, ax, ay, r, u, v);
+      C a[9];
+#pragma unroll
+      for (int i = 0; i < 9; i++) a[i] = Stor<T>::ld(f[s[i]], static_cast<C>(inv_scale));
+      const C jx[6] = {a[1], -a[3], a[5], -a[6], -a[7], a[8]};
+      const C jy[6] = {a[2], -a[4], a[5], a[6], -a[7], -a[8]};
+      using W = typename Wide<C>::type;
+      const W j[2] = {wide_sum(jx), wide_sum(jy)}, acc[2] = {ax, ay};
+      macro_fields<2>(wide_sum(a), j, acc, r, u);
     }
     if (rho) rho[p] = r;
-    if (ux) ux[p] = u;
-    if (uy) uy[p] = v;
+    if (ux) ux[p] = u[0];
+    if (uy) uy[p] = u[1];
   }
 }
 
@@ -442,32 +457,42 @@ int pull_resident_ctas() {
   if constexpr (kStochastic<T>)
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, step_kernel_pair<T>, kPairThreads, 0);
   else
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, step_kernel_pull<T, C, false>,
-                                                      kPullThreads, 0);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+        &per, step_kernel_pull<T, C, false, kPullThreads>, kPullThreads, 0);
   return e == cudaSuccess ? sms * per : 0;
+}
+
+bool narrow_ctas(int precision, int64_t n_fluid) {
+  int dev = 0, sms = 0;
+  if (precision != LBM_FP64 || cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return false;
+  return n_fluid <= static_cast<int64_t>(sms) * kPullThreads;
 }
 
 template <typename T, typename C>
 cudaError_t launch_step_pull(const T *src, T *dst, const PullGeom &g, int64_t n_fluid,
-                             const LinkCoef<C> *links, const StepConst<C> &k, cudaStream_t s) {
+                             const LinkCoef<C> *links, const StepConst<C> &k, bool narrow,
+                             cudaStream_t s) {
   if (n_fluid <= 0) return cudaSuccess;
+  auto go = [&](auto *kernel, int64_t threads, int64_t nodes) {
+    return launch_chained(kernel, dim3(static_cast<unsigned>((n_fluid + nodes - 1) / nodes)),
+                          static_cast<unsigned>(threads), 0, s, src, dst, g,
+                          static_cast<uint32_t>(n_fluid), links, k);
+  };
   if constexpr (kStochastic<T>) {
-    const int64_t pairs = (n_fluid + 1) / 2;
-    return launch_chained(step_kernel_pair<T>,
-                          dim3(static_cast<unsigned>((pairs + kPairThreads - 1) / kPairThreads)),
-                          kPairThreads, 0, s, src, dst, g, static_cast<uint32_t>(n_fluid), links, k);
+    return go(step_kernel_pair<T>, kPairThreads, 2 * kPairThreads);
   } else {
-    const int64_t blocks = (n_fluid + kPullThreads - 1) / kPullThreads;
     if constexpr (std::is_same<T, float>::value) {
       if (k.exact) {
         if (!g.links64 || !g.carry || !g.carry0) return cudaErrorInvalidValue;
-        return launch_chained(step_kernel_pull<T, C, true>, dim3(static_cast<unsigned>(blocks)),
-                              kPullThreads, 0, s, src, dst, g, static_cast<uint32_t>(n_fluid), links,
-                              k);
+        return go(step_kernel_pull<T, C, true, kPullThreads>, kPullThreads, kPullThreads);
       }
     }
-    return launch_chained(step_kernel_pull<T, C, false>, dim3(static_cast<unsigned>(blocks)),
-                          kPullThreads, 0, s, src, dst, g, static_cast<uint32_t>(n_fluid), links, k);
+    if constexpr (std::is_same<T, double>::value) {
+      if (narrow) return go(step_kernel_pull<T, C, false, 32>, 32, 32);
+    }
+    return go(step_kernel_pull<T, C, false, kPullThreads>, kPullThreads, kPullThreads);
   }
 }
 
@@ -475,9 +500,10 @@ template <typename T>
 cudaError_t launch_residual_compact(const T *cur, const T *prev, const NodeMap &map,
                                     int64_t n_fluid, int64_t plane, double ax, double ay,
                                     double scale, double *partials, double *result, cudaStream_t s) {
-  residual_partials_compact<T><<<kResidualBlocks, kResidualThreads, 0, s>>>(
+  const int blocks = residual_blocks(n_fluid);
+  residual_partials_compact<T><<<blocks, kResidualThreads, 0, s>>>(
       cur, prev, map, n_fluid, plane, ax, ay, 1.0 / scale, partials);
-  residual_final<<<1, kFinalThreads, 0, s>>>(partials, result);
+  residual_final<<<1, kFinalThreads, 0, s>>>(partials, blocks, result);
   return cudaGetLastError();
 }
 
@@ -485,10 +511,11 @@ template <typename T>
 cudaError_t launch_residual_interval(const T *cur, const NodeMap &map, int64_t n_fluid,
                                      int64_t plane, double ax, double ay, double scale, void *snap,
                                      double *partials, double *result, cudaStream_t s) {
-  residual_interval_compact<T><<<kResidualBlocks, kResidualThreads, 0, s>>>(
+  const int blocks = residual_blocks(n_fluid);
+  residual_interval_compact<T><<<blocks, kResidualThreads, 0, s>>>(
       cur, map, n_fluid, plane, ax, ay, 1.0 / scale, static_cast<typename Stor<T>::C *>(snap),
       partials);
-  residual_final<<<1, kFinalThreads, 0, s>>>(partials, result);
+  residual_final<<<1, kFinalThreads, 0, s>>>(partials, blocks, result);
   return cudaGetLastError();
 }
 
@@ -496,7 +523,9 @@ template <typename T>
 cudaError_t launch_fields(const T *f, const NodeMap &map, int64_t plane, double ax, double ay,
                           double scale, double *rho, double *ux, double *uy, cudaStream_t s) {
   const int64_t n = static_cast<int64_t>(map.nx) * map.ny;
-  fields_kernel<T><<<grid_for(n, 256), 256, 0, s>>>(f, map, plane, ax, ay, 1.0 / scale, rho, ux, uy);
+  using W = Wide<typename Stor<T>::C>;
+  fields_kernel<T><<<grid_for(n, 256), 256, 0, s>>>(f, map, plane, W::of(ax), W::of(ay),
+                                                    1.0 / scale, rho, ux, uy);
   return cudaGetLastError();
 }
 
@@ -528,9 +557,9 @@ cudaError_t launch_import_f(const double *in, const NodeMap &map, int64_t plane,
 }
 
 #define LBM_INSTANTIATE(T, C)                                                                      \
-  template int pull_resident_ctas<T, C>();                                                         \
+  template int pull_resident_ctas<T, C>();                                                           \
   template cudaError_t launch_step_pull<T, C>(const T *, T *, const PullGeom &, int64_t,          \
-                                              const LinkCoef<C> *, const StepConst<C> &,           \
+                                              const LinkCoef<C> *, const StepConst<C> &, bool,     \
                                               cudaStream_t);                                       \
   template cudaError_t launch_residual_compact<T>(const T *, const T *, const NodeMap &, int64_t,  \
                                                   int64_t, double, double, double, double *,       \
