@@ -65,6 +65,13 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t phase, volatil
   return false;
 }
 
+// The same for a warp that waits as one: the answer is warp-uniform, so the
+// loops around it are, and their counters and descriptors.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, uint32_t phase,
+                                               volatile int *gave_up) {
+  return __all_sync(0xFFFFFFFFu, mbar_wait(bar, phase, gave_up));
+}
+
 // Shared-memory matrix descriptor without swizzle; lbo, sbo in bytes.
 // K-major operand: lbo between core matrices along K, sbo between groups of
 // 8 rows.  MN-major operand: sbo between core matrices along M (N), lbo
@@ -76,6 +83,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t phase, volatil
 __device__ __forceinline__ uint32_t desc_lo(uint32_t addr, uint32_t lbo) {
   return ((addr >> 4) & 0x3FFFu) | (((lbo >> 4) & 0x3FFFu) << 16);
 }
+constexpr uint32_t kSwizzle128 = 2u << 29;  // layout type, high word
 __device__ __forceinline__ uint32_t desc_hi(uint32_t sbo) {
   return ((sbo >> 4) & 0x3FFFu) | (1u << 14);
 }
@@ -228,7 +236,9 @@ struct TileShape {
   static constexpr int kW = 8 * MT, kH = 16;
   static constexpr int kWp = kW + 2 * kHalo, kHp = kH + 2 * kHalo;
   static constexpr int kPix = kWp * kHp;
-  static constexpr uint32_t kSlab = (kPix | 1) * 16;
+  // 64 channels of the tile: a row of 128 bytes per pixel, in whole swizzle
+  // patterns of 1024 bytes
+  static constexpr uint32_t kChunk = (kPix * 128 + 1023) / 1024 * 1024;
 };
 
 template <int KS, int MT>
@@ -243,11 +253,10 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_halo_tc(const __grid_con
   __shared__ int gave_up;
   const int warp = __shfl_sync(0xFFFFFFFFu, static_cast<int>(threadIdx.x >> 5), 0);
   const int lane = threadIdx.x & 31;
-  const uint32_t a_bytes = static_cast<uint32_t>(a.p8) * S::kSlab;
+  const uint32_t stride_a = static_cast<uint32_t>((a.p8 + 7) / 8) * S::kChunk;
   const uint32_t b_bytes = static_cast<uint32_t>(a.NT) * 128u;  // 64 channels
-  const uint32_t base_a = smem_addr(dyn);
-  const uint32_t base_b = base_a + static_cast<uint32_t>(a.stages_a) * ((a_bytes + 127u) & ~127u);
-  const uint32_t stride_a = (a_bytes + 127u) & ~127u;
+  const uint32_t base_a = (smem_addr(dyn) + 1023u) & ~1023u;
+  const uint32_t base_b = base_a + static_cast<uint32_t>(a.stages_a) * stride_a;
   if (threadIdx.x == 0) {
     for (int i = 0; i < a.stages_a; i++) {
       mbar_init(&full_a[i], kLoadThreads);
@@ -296,10 +305,10 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_halo_tc(const __grid_con
             }
             const int tap = t0 + b / chunks, c8 = (b % chunks) * 8;
             const uint32_t bytes = static_cast<uint32_t>(min(8, k8 - c8)) * a.NT * 16u;
+            const int64_t at = static_cast<int64_t>(tap * a.k8 + p * a.p8 + c8) * a.NT * 16;
             mbar_expect(&full_b[st], bytes);
-            bulk_copy(base_b + st * b_bytes,
-                      src + static_cast<int64_t>(tap * a.k8 + p * a.p8 + c8) * a.NT * 16, bytes,
-                      &full_b[st]);
+            bulk_copy(base_b + (a.resident ? static_cast<uint32_t>(at) : st * b_bytes), src + at,
+                      bytes, &full_b[st]);
             issued++;
             if (++st == a.stages_b) {
               st = 0;
@@ -323,15 +332,14 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_halo_tc(const __grid_con
     const uint32_t leader = elect_leader();
     const uint32_t idesc = umma_idesc(a.NT, false);
     const uint32_t lbo_b = static_cast<uint32_t>(a.NT) * 16u;
-    const uint32_t ahi = desc_hi(S::kWp * 16u), bhi = desc_hi(128u);
-    constexpr uint32_t kStepA = 2 * S::kSlab / 16;  // 16 channels on
+    const uint32_t ahi = desc_hi(S::kWp * 128u) | kSwizzle128, bhi = desc_hi(128u);
     const uint32_t step_b = 2 * lbo_b / 16;
     int sa = 0, sb = 0, it = 0;
     uint32_t pa = 0, pb = 0;
     bool ok = true;
     for (int t = blockIdx.x; ok && t < a.tiles; t += gridDim.x, it++) {
       const int acc = it & 1;
-      if (it >= 2 && !mbar_wait(&empty_d[acc], ((it >> 1) & 1) ^ 1u, &gave_up)) {
+      if (it >= 2 && !mbar_wait_warp(&empty_d[acc], ((it >> 1) & 1) ^ 1u, &gave_up)) {
         ok = false;
         break;
       }
@@ -341,27 +349,29 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_halo_tc(const __grid_con
         sb = 0;
         pb = 0;
       }
-      uint32_t accumulate = 0;
+      uint32_t accumulate = 0, b_at = 0;
       // the MMAs of one tap of a tile in shared memory
       auto do_tap = [&](uint32_t alo, int k8) {
 #pragma unroll 1
-        for (int c8 = 0; c8 < k8; c8 += 8) {
+        for (int c8 = 0; c8 < k8; c8 += 8, alo += S::kChunk / 16 - 8u) {
           if (wait_b) {
-            if (!mbar_wait(&full_b[sb], pb, &gave_up)) {
+            if (!mbar_wait_warp(&full_b[sb], pb, &gave_up)) {
               ok = false;
               return;
             }
             fence_after();
           }
-          uint32_t blo = desc_lo(base_b + sb * b_bytes, lbo_b);
+          // resident blocks lie end to end, a ring's at its stride
+          uint32_t blo = desc_lo(base_b, lbo_b) + (a.resident ? b_at : sb * (b_bytes / 16));
           const int k16 = min(4, (k8 - c8) >> 1);
+          b_at += static_cast<uint32_t>(k16) * step_b;
 #pragma unroll 1
           for (int k = 0; k < k16; k++) {
 #pragma unroll
             for (int m = 0; m < MT; m++)
-              mma_bf16(leader, d0 + m * a.NT, alo + m * 8u, ahi, blo, bhi, idesc, accumulate);
+              mma_bf16(leader, d0 + m * a.NT, alo + m * 64u, ahi, blo, bhi, idesc, accumulate);
             accumulate = 1;
-            alo += kStepA;
+            alo += 2;  // 16 channels on
             blo += step_b;
           }
           if (!a.resident) mma_commit(leader, &empty_b[sb]);
@@ -372,13 +382,13 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_halo_tc(const __grid_con
         }
       };
       auto next_tile = [&](uint32_t *ta) {
-        if (!mbar_wait(&full_a[sa], pa, &gave_up)) {
+        if (!mbar_wait_warp(&full_a[sa], pa, &gave_up)) {
           ok = false;
           return;
         }
         fence_async_proxy();  // the landed copies, for the MMAs
         fence_after();
-        *ta = desc_lo(base_a + sa * stride_a, S::kSlab);
+        *ta = desc_lo(base_a + sa * stride_a, 16u);
       };
       auto free_tile = [&]() {
         mma_commit(leader, &empty_a[sa]);
@@ -397,10 +407,10 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_halo_tc(const __grid_con
         for (int tap = 0; tap < KS * KS; tap++) {
           do_tap(ta, a.k8);
           if (!ok) break;
-          ta++;
+          ta += 8;
           if (++dx == KS) {
             dx = 0;
-            ta += S::kWp - KS;
+            ta += (S::kWp - KS) * 8;
           }
         }
         if (!ok) break;
@@ -410,7 +420,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_halo_tc(const __grid_con
           for (int p = 0; ok && p < a.parts; p++) {
             next_tile(&ta);
             if (!ok) break;
-            do_tap(ta + (tap / KS) * S::kWp + (tap % KS), min(a.p8, a.k8 - p * a.p8));
+            do_tap(ta + ((tap / KS) * S::kWp + (tap % KS)) * 8, min(a.p8, a.k8 - p * a.p8));
             if (ok) free_tile();
           }
         if (!ok) break;
@@ -422,7 +432,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_halo_tc(const __grid_con
       if (lane == 0) atomicExch(a.err, 1);
       int never = 0;
       mma_commit(leader, &drained);  // the MMAs in flight end before the memory is given back
-      mbar_wait(&drained, 0, &never);
+      mbar_wait_warp(&drained, 0, &never);
     }
   } else if (warp < 10) {
     // epilogue: lane = pixel of a block; the two groups of four warps take a
@@ -531,54 +541,36 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_halo_tc(const __grid_con
           break;
         }
         const int k8 = min(a.p8, a.k8 - p * a.p8);
-        // (a copy instruction whose 16-byte pieces scatter over slabs takes about
-        // 36 cycles whatever the order of the arithmetic: batches of pixels were
-        // no faster)
-        constexpr int kBatch = 1;
         int y = y0, x = x0;
-        uint32_t dst = base_a + sa * stride_a + pix0 * 16 + g8 * S::kSlab;
+        const uint32_t dst = base_a + sa * stride_a;
         const int Wa = a.W >> a.x.up, rows = n * (a.H >> a.x.up);
         const int first = (n * a.H + i0) * a.W + j0, c0 = p * a.p8 + g8;
         const bool plain = !a.x.up && a.x.n8 == a.x.n8a;  // one source at full resolution
-        for (int pix = pix0; pix < S::kPix; pix += kBatch * pstep) {
-          const __nv_bfloat16 *pa8[kBatch], *pb8[kBatch];
-          bool in[kBatch];
-#pragma unroll
-          for (int q = 0; q < kBatch; q++) {
-            const int i = i0 + y, j = j0 + x;
-            in[q] = static_cast<unsigned>(i) < static_cast<unsigned>(a.H) &&
-                    static_cast<unsigned>(j) < static_cast<unsigned>(a.W);
-            const int here = first + y * a.W + x;
-            pa8[q] = a.x.xa;
-            pb8[q] = a.x.xa;
-            if (in[q]) {
-              pa8[q] += static_cast<int64_t>(
-                            plain ? here : (rows + (i >> a.x.up)) * Wa + (j >> a.x.up)) *
-                            a.x.sa +
-                        c0 * 8;
-              if (!plain)
-                pb8[q] = a.x.xb + static_cast<int64_t>(here) * a.x.sb + (c0 - a.x.n8a) * 8;
-            }
-            y += dy;
-            x += dx;
-            if (x >= S::kWp) {
-              x -= S::kWp;
-              y++;
-            }
+        for (int pix = pix0; pix < S::kPix; pix += pstep) {
+          const int i = i0 + y, j = j0 + x;
+          const bool in = static_cast<unsigned>(i) < static_cast<unsigned>(a.H) &&
+                          static_cast<unsigned>(j) < static_cast<unsigned>(a.W);
+          const int here = first + y * a.W + x;
+          const __nv_bfloat16 *pa8 = a.x.xa, *pb8 = a.x.xa;
+          if (in) {
+            pa8 += static_cast<int64_t>(plain ? here
+                                              : (rows + (i >> a.x.up)) * Wa + (j >> a.x.up)) *
+                       a.x.sa +
+                   c0 * 8;
+            if (!plain) pb8 = a.x.xb + static_cast<int64_t>(here) * a.x.sb + (c0 - a.x.n8a) * 8;
           }
-          uint32_t d = dst;
-          for (int s8 = 0; s8 + g8 < k8; s8 += lanes) {
-            const bool slab = c0 + s8 < a.x.n8, from_a = c0 + s8 < a.x.n8a;
-#pragma unroll
-            for (int q = 0; q < kBatch; q++) {
-              const bool valid = in[q] && slab;
-              if (pix + q * pstep < S::kPix)
-                cp_async16(d + q * pstep * 16,
-                           valid ? (from_a ? pa8[q] : pb8[q]) + s8 * 8 : a.x.xa, valid);
-            }
-            d += lanes * S::kSlab;
+          for (int s8 = g8; s8 < k8; s8 += lanes) {
+            const int c8 = p * a.p8 + s8;
+            const bool valid = in && c8 < a.x.n8;
+            cp_async16(dst + (s8 >> 3) * S::kChunk + pix * 128 + (((s8 ^ pix) & 7) << 4),
+                       valid ? (c8 < a.x.n8a ? pa8 : pb8) + (s8 - g8) * 8 : a.x.xa, valid);
           }
-          dst += kBatch * pstep * 16;
+          y += dy;
+          x += dx;
+          if (x >= S::kWp) {
+            x -= S::kWp;
+            y++;
+          }
         }
         cp_async_arrive(&full_a[sa]);
         if (++sa == a.stages_a) {
@@ -697,7 +689,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc(const __grid_constant_
     int st = 0;
     uint32_t ph = 0, acc = 0;
     for (int t = t0; t < t1; t++) {
-      if (!mbar_wait(&full[st], ph, &gave_up)) {
+      if (!mbar_wait_warp(&full[st], ph, &gave_up)) {
         ok = false;
         break;
       }
@@ -734,7 +726,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc(const __grid_constant_
       gave_up = 1;
       if (lane == 0) atomicExch(a.err, 1);
       int never = 0;
-      mbar_wait(&done, 0, &never);
+      mbar_wait_warp(&done, 0, &never);
     }
     __syncwarp();
   } else {
@@ -988,30 +980,34 @@ cudaError_t conv_launch(ConvDev d, int sms, cudaStream_t s) {
   // input channels a tile takes at once: all, if one tile of them fits beside
   // three weight blocks
   const int b_bytes = d.NT * 128;
-  const int fit = (kSmemMax - 3 * b_bytes) / static_cast<int>(S::kSlab) / 8 * 8;
+  const int fit = (kSmemMax - 1024 - 3 * b_bytes) / static_cast<int>(S::kChunk) * 8;
   d.parts = d.k8 <= fit ? 1 : (d.k8 + fit - 1) / fit;
   d.p8 = d.parts == 1 ? d.k8 : fit;
   const int last = d.k8 - (d.parts - 1) * d.p8;
   d.lanes_log2 = 1;  // both are even
-  while (d.lanes_log2 < 5 && (d.p8 >> d.lanes_log2) % 2 == 0 && (last >> d.lanes_log2) % 2 == 0)
+  while (d.lanes_log2 < 3 && (d.p8 >> d.lanes_log2) % 2 == 0 && (last >> d.lanes_log2) % 2 == 0)
     d.lanes_log2++;
-  const int sa_bytes = (d.p8 * static_cast<int>(S::kSlab) + 127) / 128 * 128;
+  const int sa_bytes = (d.p8 + 7) / 8 * static_cast<int>(S::kChunk);
   d.unit_taps = d.parts == 1 ? KS * KS : 1;
   const int blocks =
       KS * KS * ((d.parts - 1) * ((d.p8 + 7) / 8) + (last + 7) / 8);
   // all weights in shared memory where one image tile (two if there are
   // more) still fits beside them, else a ring of at least three blocks
   const int want_a = std::min(per * (d.parts == 1 ? 1 : d.parts * KS * KS), 2);
-  d.resident = blocks <= kMaxStagesB && blocks * b_bytes + want_a * sa_bytes <= kSmemMax;
+  // (their blocks end to end; parts of the channels never are)
+  const int all_b = KS * KS * d.k8 * d.NT * 16;
+  d.resident = d.parts == 1 && blocks <= kMaxStagesB &&
+               all_b + want_a * sa_bytes <= kSmemMax - 1024;
   d.stages_a = want_a;
-  if (!d.resident && want_a * sa_bytes + 3 * b_bytes > kSmemMax) d.stages_a = 1;
+  if (!d.resident && want_a * sa_bytes + 3 * b_bytes > kSmemMax - 1024) d.stages_a = 1;
   d.stages_b = d.resident ? blocks
-                          : std::min({blocks, 8, (kSmemMax - d.stages_a * sa_bytes) / b_bytes});
+                          : std::min({blocks, 8, (kSmemMax - 1024 - d.stages_a * sa_bytes) / b_bytes});
   if (d.stages_b < 1) return cudaErrorInvalidValue;
   d.tmem_cols = pow2_cols(2 * MT * d.NT);
   // where the CTA takes more than half of tensor memory: more than half of
   // shared memory too, so that no other CTA waits beside it
-  const int smem = std::max(d.stages_a * sa_bytes + d.stages_b * b_bytes,
+  const int smem = std::max(1024 + d.stages_a * sa_bytes +
+                                (d.resident ? all_b : d.stages_b * b_bytes),
                             d.tmem_cols > 256 ? 120 * 1024 : 0);
   return launch_chained(conv_halo_tc<KS, MT>, dim3(gx, n_blocks), kConvThreads, smem, s, d);
 }
@@ -1101,8 +1097,9 @@ cudaError_t launch_conv_tc(const ConvCall &c, int sms, int *err, cudaStream_t s)
   // fit beside three weight blocks, or would leave SMs without a tile
   const int tiles2 = c.N * ((c.W + 15) / 16) * ((c.H + 15) / 16);
   const int n_blocks = (pad16(c.co) + d.NT - 1) / d.NT;
-  const int a2 = d.k8 * static_cast<int>(c.ks == 3 ? TileShape<3, 2>::kSlab : TileShape<1, 2>::kSlab);
-  const bool two = a2 + 3 * d.NT * 128 <= kSmemMax && tiles2 * n_blocks >= sms;
+  const int a2 = (d.k8 + 7) / 8 *
+                 static_cast<int>(c.ks == 3 ? TileShape<3, 2>::kChunk : TileShape<1, 2>::kChunk);
+  const bool two = a2 + 3 * d.NT * 128 <= kSmemMax - 1024 && tiles2 * n_blocks >= sms;
   if (c.ks == 3) return two ? conv_launch<3, 2>(d, sms, s) : conv_launch<3, 1>(d, sms, s);
   return two ? conv_launch<1, 2>(d, sms, s) : conv_launch<1, 1>(d, sms, s);
 }
