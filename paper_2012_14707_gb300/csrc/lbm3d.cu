@@ -21,10 +21,11 @@
 // step t.  Per node: a flag word (bit q: x - c_q solid; kSolid3 for solid
 // nodes) and the index of its first link (links sorted by node, then
 // direction); the step runs one thread per fluid node from a list of the
-// fluid nodes (index and flag word).  The collision works in moment space with the D3Q19 basis
-// built here from its defining polynomials (d'Humieres et al. 2002):
-// m - m_eq = M (d - d_eq), M Fbar, then f' - f = M^T diag(1/|M_k|^2) (m' -
-// m) (the basis is orthogonal), and the rest population closes the mass.
+// fluid nodes (index, flag word and the node's first link).  The collision
+// works in moment space with the D3Q19 basis built here from its defining
+// polynomials (d'Humieres et al. 2002): m - m_eq = M (d - d_eq), M Fbar,
+// then f' - f = M^T diag(1/|M_k|^2) (m' - m) (the basis is orthogonal), and
+// the rest population closes the mass.
 #include <cmath>
 #include <cstdio>
 #include <cstring>

@@ -11,12 +11,13 @@
 // arena; a CTA looks up its case's constants in a descriptor table and runs
 // the single-case kernel's per-node update (step_node_pull), so a case in a
 // batch follows exactly the arithmetic of the case run alone.  Every K
-// steps a batched reduction (one CTA per case, fixed order) computes each
-// case's residual and retires converged cases on the device; retired
-// cases' CTAs return immediately.  K steps plus the reduction are captured
-// once in a CUDA graph that the host replays, reading back only the number
-// of active cases.  The CTA width and the L2 prefetch are picked by timing
-// the candidates on the batch itself (autotuner), cached per size class and
+// steps a batched reduction (fixed parts of a case's nodes, one CTA each,
+// then one CTA per case, summed in a fixed order) computes each case's
+// residual and retires converged cases on the device; retired cases' CTAs
+// return immediately.  K steps plus the reduction are captured once in a
+// CUDA graph that the host replays, reading back only the number of active
+// cases.  The CTA width and the L2 prefetch are picked by timing the
+// candidates on the batch itself (autotuner), cached per size class and
 // precision.
 #include <algorithm>
 #include <chrono>

@@ -2,18 +2,26 @@
 // cores: forward and backward-data (conv_halo_tc) and the weight gradient
 // (wgrad_tc), with the packing of their weights.
 //
-// Shared-memory layout of an image tile (both kernels): the tile's pixels
-// with the halo its taps reach, as "slabs" of 8 channels -- slab c8 holds
-// 16 bytes (8 BF16 channels) per pixel, pixels row by row.  In the tensor
-// cores' canonical layout without swizzle a core matrix is 8 rows of 16
-// contiguous bytes, rows 16 bytes apart: 8 neighbouring pixels of a slab are
-// one core matrix, whatever pixel it starts at.  So a tap's shifted operand
-// is the same tile with another start address, and each input element is
-// copied to shared memory once per tile instead of once per tap.  Read with
-// the channels as K (K-major) the tile is the forward operand, with the
-// pixels as K (MN-major) it is the weight gradient's.  A slab's length is an
-// odd number of 16-byte units, so the copies of a pixel's slabs fall in
-// different banks.
+// An image tile -- its pixels with the halo its taps reach -- is copied to
+// shared memory once, and a tap's shifted operand is the same tile at another
+// start address.  (Gathered per tap, nine times, the operands cost four
+// times what the MMAs did: forward pass 256x256 x 8 images 3.23 ms, now 0.41;
+// gradients 18.1 ms, now 1.49.)  Two layouts allow that:
+// * conv_halo_tc: a 128-byte row of 64 channels per pixel, in the 128-byte
+//   swizzle, which goes by address: row r's 16-byte unit u lies at unit u ^ (r
+//   mod 8).  Channels are K (K-major).
+// * wgrad_tc: "slabs" of 8 channels, 16 bytes per pixel, no swizzle: 8
+//   neighbouring pixels of a slab are one core matrix, whatever pixel it
+//   starts at.  Pixels are K (MN-major), so nothing is transposed.  A slab's
+//   length is an odd number of 16-byte units, so the copies of a pixel's
+//   slabs fall in different banks.
+//
+// What bounds them: an MMA of M = 128, K = 16 takes 54 cycles up to N = 64
+// and 64 at N = 128 (measured, either layout), so the layers of 32 and 64
+// output channels, 60 % of the network's flops, reach a quarter and a half of
+// the tensor peak at best; issuing the MMAs from one warp costs 70 to 100
+// cycles each around that.  The channel order of the sums (taps outermost) is
+// kept over all shapes, so results do not depend on them.
 //
 // Every wait is bounded; one that runs out sets *err, and the CTA's roles
 // give up in turn after waiting for the copies they started.
@@ -183,7 +191,7 @@ __device__ __forceinline__ void bulk_copy(uint32_t dst, const void *src, uint32_
       : "memory");
 }
 
-// Both sources of a convolution's input, in slabs.
+// Both sources of a convolution's input, in slabs (groups of 8 channels).
 struct InputDev {
   const __nv_bfloat16 *xa, *xb;
   int sa, sb;        // pixel strides (elements)

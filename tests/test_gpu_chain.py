@@ -61,3 +61,31 @@ def test_chained_steps_are_the_single_steps_3d(name, precision):
         got.append(s.get_f())
         s.close()
     assert np.array_equal(got[0], got[1])
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+def test_captured_steps_replay(precision):
+    """Two steps captured in a caller's CUDA graph and replayed three times
+    are six steps."""
+    import torch
+
+    lbm_build.build()
+    torch.cuda.set_device(0)
+    c = CASES2["cylinders_300x150"]()
+    f = cases.random_populations(c.nx, c.ny, 3)
+    st = torch.cuda.Stream()
+    s = lbm.Solver(c, precision=precision, stream=st.cuda_stream)
+    s.set_f(f)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=st):
+        s.step(2)
+    for _ in range(3):
+        g.replay()
+    torch.cuda.synchronize()
+    got = s.get_f()
+    s.close()
+    s = lbm.Solver(c, precision=precision)
+    s.set_f(f)
+    s.step(6)
+    assert np.array_equal(got, s.get_f())
+    s.close()
