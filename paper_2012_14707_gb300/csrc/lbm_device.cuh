@@ -862,7 +862,15 @@ __device__ __forceinline__ float link_value_rt(const LinkCoef<float> &c, const i
 // the random bits of its node and direction, as a node doing its own links
 // would.  The lanes whose pair is complete take part (a prefix of the
 // warp; a lone last node runs the one-node step instead).
+// The record holds a lane's two nodes side by side, one 8-byte store a row:
+// a float at a time the stores had two-way bank conflicts and ran once per
+// node (8192x4096, BF16: 274 us a step against 267.5).
 constexpr int kPairMaxWarps = 4;  // CTAs of up to 128 threads
+// The lanes of the warp of pair i0 that hold a complete pair.
+__device__ __forceinline__ unsigned pair_lanes(const PullGeom &g, const uint32_t i0) {
+  const uint32_t pairs = (g.n_fluid - (i0 - 2u * (threadIdx.x & 31u))) / 2u;
+  return pairs >= 32u ? 0xFFFFFFFFu : (1u << pairs) - 1u;
+}
 template <typename T>
 __device__ __forceinline__ void pair_links_warp(const T *src, T *dst,
                                                 const PullGeom &g,
@@ -873,38 +881,24 @@ __device__ __forceinline__ void pair_links_warp(const T *src, T *dst,
                                                 const F2 (&o)[9], const F2 drho_s, const F2 rho_s,
                                                 const F2 ux, const F2 uy, const F2 uu,
                                                 const uint32_t h0, const uint32_t h1) {
-  __shared__ float pw_v[kPairMaxWarps][13][65];
-  __shared__ uint32_t pw_h[kPairMaxWarps][64];
+  __shared__ float2 pw_v[kPairMaxWarps][13][33];
+  __shared__ uint2 pw_h[kPairMaxWarps][32];
   const int lane = static_cast<int>(threadIdx.x & 31u), w = static_cast<int>(threadIdx.x >> 5);
-  const uint32_t first = i0 - 2u * static_cast<uint32_t>(lane);
-  const uint32_t pairs = (g.n_fluid - first) / 2u;
-  const int nact = pairs >= 32u ? 32 : static_cast<int>(pairs);
-  const unsigned am = nact == 32 ? 0xFFFFFFFFu : ((1u << nact) - 1u);
+  const unsigned am = pair_lanes(g, i0);
+  const int nact = __popc(am);
   __syncwarp(am);
   const uint32_t nl = static_cast<uint32_t>(__popc(fl0)) + static_cast<uint32_t>(__popc(fl1));
   const unsigned anyl = __ballot_sync(am, nl != 0u);
   if (anyl == 0u) return;
-  if (fl0) {
-    const int n = 2 * lane;
+  if (nl) {
 #pragma unroll
-    for (int q = 1; q < 9; q++) pw_v[w][q - 1][n] = o[q].v.x;
-    pw_v[w][8][n] = drho_s.v.x;
-    pw_v[w][9][n] = rho_s.v.x;
-    pw_v[w][10][n] = ux.v.x;
-    pw_v[w][11][n] = uy.v.x;
-    pw_v[w][12][n] = uu.v.x;
-    pw_h[w][n] = h0;
-  }
-  if (fl1) {
-    const int n = 2 * lane + 1;
-#pragma unroll
-    for (int q = 1; q < 9; q++) pw_v[w][q - 1][n] = o[q].v.y;
-    pw_v[w][8][n] = drho_s.v.y;
-    pw_v[w][9][n] = rho_s.v.y;
-    pw_v[w][10][n] = ux.v.y;
-    pw_v[w][11][n] = uy.v.y;
-    pw_v[w][12][n] = uu.v.y;
-    pw_h[w][n] = h1;
+    for (int q = 1; q < 9; q++) pw_v[w][q - 1][lane] = o[q].v;
+    pw_v[w][8][lane] = drho_s.v;
+    pw_v[w][9][lane] = rho_s.v;
+    pw_v[w][10][lane] = ux.v;
+    pw_v[w][11][lane] = uy.v;
+    pw_v[w][12][lane] = uu.v;
+    pw_h[w][lane] = make_uint2(h0, h1);
   }
   // the warp's links are links base .. base + total - 1 of the table (its
   // first lane with links holds the first of them)
@@ -917,12 +911,12 @@ __device__ __forceinline__ void pair_links_warp(const T *src, T *dst,
     const uint32_t lj = base + t;
     const uint32_t dsc = g.ldesc[lj];
     const int n = static_cast<int>(dsc >> 4), j = static_cast<int>(dsc & 15u), jb = opp2(j);
-    const float v = link_value_rt<T>(links[lj], j, Stor<T>::ld_raw(src[g.jbslot[lj]]),
-                                     pw_v[w][j - 1][n], pw_v[w][jb - 1][n], pw_v[w][8][n],
-                                     pw_v[w][9][n], pw_v[w][10][n], pw_v[w][11][n],
-                                     pw_v[w][12][n], k);
+    const auto rec = [&](int row) { return reinterpret_cast<const float *>(pw_v[w][row])[n]; };
+    const float v = link_value_rt<T>(links[lj], j, Stor<T>::ld_raw(src[g.jbslot[lj]]), rec(j - 1),
+                                     rec(jb - 1), rec(8), rec(9), rec(10), rec(11), rec(12), k);
+    const uint32_t h = reinterpret_cast<const uint32_t *>(pw_h[w])[n];
     dst[tail + lj] =
-        Stor<T>::bits(Stor<T>::st_rs2(v, 0.0f, fmix32(pw_h[w][n] ^ (0x27D4EB2Fu * j))) >> 16);
+        Stor<T>::bits(Stor<T>::st_rs2(v, 0.0f, fmix32(h ^ (0x27D4EB2Fu * j))) >> 16);
   }
 }
 
@@ -945,11 +939,18 @@ __device__ __forceinline__ void step_pair_pull(const T *src, T *dst,
   {
     uint32_t s0[9], s1[9];
     pull_slots(nw0, gr, i0, P, g.n_fluid, g.ny, g.periodic_y, g.rowstart, s0);
-    pull_slots(nw1, gr, i0 + 1u, P, g.n_fluid, g.ny, g.periodic_y, g.rowstart, s1);
+    // node i0's gathers fly while node i0 + 1's slots are formed: 8192x4096
+    // (BF16) took 267.5 us a step with the wait after both, 264.5 here; with
+    // the wait before both 264.3, but 2048x1024 (FP16) 20.1 instead of 19.6
+    // and 1024x512 8.3 instead of 8.15, as less then overlaps the step before
     if (!gate.open()) return;
+    pull_slots(nw1, gr, i0 + 1u, P, g.n_fluid, g.ny, g.periodic_y, g.rowstart, s1);
 #pragma unroll
-    for (int q = 0; q < 9; q++)
+    for (int q = 1; q < 9; q++)
       d[q] = F2(make_float2(Stor<T>::ld_raw(src[s0[q]]), Stor<T>::ld_raw(src[s1[q]])));
+    const uint32_t own = *reinterpret_cast<const uint32_t *>(src + i0);
+    d[0] = F2(make_float2(Stor<T>::ld_raw(Stor<T>::bits(own & 0xFFFFu)),
+                          Stor<T>::ld_raw(Stor<T>::bits(own >> 16))));
     if (fl0) {
       asm volatile("prefetch.global.L1 [%0];" ::"l"(links + li0));
       asm volatile("prefetch.global.L1 [%0];" ::"l"(g.jbslot + li0));
