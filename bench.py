@@ -465,13 +465,13 @@ ACCURACY = {
 
 ACCURACY_3D = {
     "fp32": {"velocity_target": 1e-5,
-             "velocity": "met (1.7e-6 to 3.6e-6 with the plain step on the 20^3 sphere array over "
-                         "4000 steps; 2e-8 to 4e-8 with the exact-mass step)",
+             "velocity": "met (4e-8 on the 20^3 sphere array over 4000 steps, 2e-8 on the "
+                         "moving-lid channel)",
              "mass_target": 1e-10,
-             "mass": "the plain step this line times (walls at rest) misses it at static curved "
-                     "walls after 2000 steps (4.6e-10 on the 20^3 sphere array; 1.2e-9 after 4000); "
-                     "met with mass_mode=1 (2.4e-11 after 2000 steps, at 3.7x the step time) and by "
-                     "default where walls move (5.2e-11 after 2000 steps on the moving-lid channel)"},
+             "mass": "the plain step this line times (walls at rest) meets it on the 20^3 sphere "
+                     "array up to 2000 steps (4.9e-11; 1.25e-10 after 4000); met with mass_mode=1 "
+                     "(3.1e-11 after 4000 steps, at 1.8x the step time) and by default where walls "
+                     "move (4.0e-11 after 2000 steps on the moving-lid channel)"},
     "fp64": {"populations": "within 1e-13 of the oracle, element by element"},
 }
 

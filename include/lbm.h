@@ -117,7 +117,7 @@ typedef struct {
                            next value: the stored mass then follows the exact trajectory
                            instead of drifting by roundings that repeat every step.  It costs
                            4 B per link and 8 B per fluid node of extra traffic per step and
-                           about 2.5x the plain step's time. */
+                           about 2.3x the plain step's time. */
   int32_t residual_mode; /* 0 (default): lbm_residual's residual is the one-step change
                             ||u^n - u^(n-1)|| / ||u^n||.  1: the interval change
                             ||u^n - u^m|| / ((n - m) ||u^n||), u^m the velocity field at the
@@ -409,7 +409,7 @@ int lbm_load(lbm_handle_t *h, const char *path);
  *     exact-mass step where a wall moves or the lattice has no boundary
  *     links (d - d_eq in double-FP32, stochastic rounding of f'_1..f'_18 to
  *     FP32, double-FP32 link values, per-link and per-node carries; about
- *     3.7x the plain step's time).  The lattice
+ *     1.8x the plain step's time).  The lattice
  *     is dense (every node has slots).  Calls synchronise the handle's
  *     stream, except lbm3d_step.
  * ------------------------------------------------------------------------- */
