@@ -309,7 +309,10 @@ int lbm_batch_run_to(lbm_batch_t *b, double tol, int64_t max_steps, int32_t chec
  * lbm_batch_reset and before lbm_batch_run_to. */
 int lbm_batch_set_fields(lbm_batch_t *b, int32_t c, const double *rho, const double *ux,
                          const double *uy);
-/* Density and velocity of case c (host arrays of nx*ny doubles, may be NULL). */
+/* Density and velocity of case c (host arrays of nx*ny doubles, may be NULL).
+ * Several threads may read, or set, the fields of one batch's cases at once:
+ * the calls take turns on the batch's staging memory.  The other calls of a
+ * batch are for one thread at a time, with none of these in progress. */
 int lbm_batch_fields(lbm_batch_t *b, int32_t c, double *rho, double *ux, double *uy);
 /* Sizes of the batch (outputs may be NULL): lattice nodes and fluid nodes
  * of all cases, the step kernel's CTA width and its CTAs per step. */

@@ -461,8 +461,10 @@ struct lbm_batch {
   std::vector<int32_t> h_part_first;
   double *partials = nullptr;
   // one case's FP64 fields on the device (the largest case's size), on their
-  // way from or to the caller
+  // way from or to the caller; a call holds stage_use while they are there,
+  // so threads that read or set different cases take turns
   double *stage = nullptr;
+  std::mutex stage_use;
   // the exact-mass cases' steps beside the others' in the captured graph
   cudaStream_t side = nullptr;
   cudaEvent_t fork = nullptr, join = nullptr;
@@ -1075,6 +1077,7 @@ int lbm_batch_run_to(lbm_batch_t *b, double tol, int64_t max_steps, int32_t chec
 
 int lbm_batch_fields(lbm_batch_t *b, int32_t c, double *rho, double *ux, double *uy) {
   if (!b) return LBM_EINVAL;
+  const std::lock_guard<std::mutex> own(b->stage_use);
   if (c < 0 || c >= b->n_cases) return bfail(b, LBM_EINVAL, "case index out of range");
   const int64_t n = static_cast<int64_t>(b->nx[c]) * b->ny[c];
   double *d = b->stage;
@@ -1096,7 +1099,9 @@ int lbm_batch_fields(lbm_batch_t *b, int32_t c, double *rho, double *ux, double 
 
 int lbm_batch_set_fields(lbm_batch_t *b, int32_t c, const double *rho, const double *ux,
                          const double *uy) {
-  if (!b || !rho || !ux || !uy) return b ? bfail(b, LBM_EINVAL, "null field") : LBM_EINVAL;
+  if (!b) return LBM_EINVAL;
+  const std::lock_guard<std::mutex> own(b->stage_use);
+  if (!rho || !ux || !uy) return bfail(b, LBM_EINVAL, "null field");
   if (c < 0 || c >= b->n_cases) return bfail(b, LBM_EINVAL, "case index out of range");
   if (b->cur != 0) return bfail(b, LBM_EINVAL, "batch state is mid-graph; call lbm_batch_reset");
   const int64_t n = static_cast<int64_t>(b->nx[c]) * b->ny[c];
