@@ -409,6 +409,10 @@ using lbm::dev::Sum;
 struct Force3 {
   DF a[3];  // the body acceleration as double-FP32 pairs
 };
+inline DF df_of(double x) {
+  const float h = static_cast<float>(x);
+  return DF{h, static_cast<float>(x - static_cast<double>(h))};
+}
 __device__ __forceinline__ DF df_third() {
   constexpr float h = static_cast<float>(1.0 / 3.0);
   return DF{h, static_cast<float>(1.0 / 3.0 - static_cast<double>(h))};
@@ -800,14 +804,13 @@ __global__ void export3_kernel(const C *__restrict__ f, const uint32_t *__restri
 
 // Eq. FluidMacr at every node (solid nodes 0): rho, ux, uy, uz arrays of
 // nx*ny*nz doubles.
-template <typename C>
-struct Accel3 {
-  typename lbm::dev::Wide<C>::type x, y, z;
+struct HalfAccel3 {
+  double a[3];
 };
 template <typename C>
 __global__ void fields3_kernel(const C *__restrict__ f, const uint32_t *__restrict__ flags,
                                const uint32_t *__restrict__ lbase, const Const3<C> k,
-                               const Accel3<C> acc, int64_t n_nodes, double *__restrict__ out) {
+                               const HalfAccel3 half, int64_t n_nodes, double *__restrict__ out) {
   for (int64_t p = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; p < n_nodes;
        p += static_cast<int64_t>(gridDim.x) * blockDim.x) {
     const uint32_t fl = flags[p];
@@ -818,19 +821,15 @@ __global__ void fields3_kernel(const C *__restrict__ f, const uint32_t *__restri
       C d[Q];
 #pragma unroll
       for (int q = 0; q < Q; q++) d[q] = f[pull_slot3(k, q, c, fl, lb, k.plane)];
-      using W = typename lbm::dev::Wide<C>::type;
-      W j[3];
+      C j[3][10];
 #pragma unroll
       for (int e = 0; e < 3; e++) {
-        C m[10];
         int at = 0;
 #pragma unroll
         for (int q = 1; q < Q; q++)
-          if (cvel3(q, e) != 0) m[at++] = cvel3(q, e) > 0 ? d[q] : -d[q];
-        j[e] = lbm::dev::wide_sum(m);
+          if (cvel3(q, e) != 0) j[e][at++] = cvel3(q, e) > 0 ? d[q] : -d[q];
       }
-      const W a[3] = {acc.x, acc.y, acc.z};
-      lbm::dev::macro_fields<3>(lbm::dev::wide_sum(d), j, a, r, u);
+      lbm::dev::node_fields(d, j, half.a, r, u);
     }
     out[p] = r;
     out[n_nodes + p] = u[0];
@@ -1150,7 +1149,7 @@ int lbm3d_create(const lbm3d_domain_t *dom, const uint8_t *solid, size_t n_links
              (p.mass_mode > 0 || moving || n_links == 0);
   if (e == cudaSuccess && h->exact) {
     const double acc[3] = {dom->ax, dom->ay, dom->az};
-    for (int a = 0; a < 3; a++) h->force.a[a] = lbm::dev::Wide<float>::of(acc[a]);
+    for (int a = 0; a < 3; a++) h->force.a[a] = df_of(acc[a]);
     std::vector<lbm::LinkCoefDF> ldf(std::max<size_t>(1, n_links));
     for (size_t k = 0; k < n_links; k++) ldf[slot[k]] = lbm::link_coef_df(&coef[8 * k], wq[k], p.diffuse_mode);
     e = alloc(reinterpret_cast<void **>(&h->links_df), ldf.size() * sizeof(lbm::LinkCoefDF));
@@ -1280,10 +1279,9 @@ int lbm3d_fields(lbm3d_t *h, double *rho, double *ux, double *uy, double *uz) {
   if (e == cudaSuccess)
     e = dispatch3(h->precision, [&](auto tag) {
       using C = std::remove_pointer_t<decltype(tag)>;
-      using W = lbm::dev::Wide<C>;
       fields3_kernel<C><<<grid_for3(h->n_nodes, 256), 256, 0, h->stream>>>(
           static_cast<const C *>(h->f[h->cur]), h->flags, h->lbase, h->kc.get(tag),
-          Accel3<C>{W::of(h->ax), W::of(h->ay), W::of(h->az)}, h->n_nodes, d);
+          HalfAccel3{{0.5 * h->ax, 0.5 * h->ay, 0.5 * h->az}}, h->n_nodes, d);
       return cudaGetLastError();
     });
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);

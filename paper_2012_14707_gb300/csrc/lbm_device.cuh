@@ -182,6 +182,21 @@ __device__ __forceinline__ void sum2(const float (&a)[N], float &s, float &e) {
   }
 }
 
+// The same with the errors' sum and its errors kept apart: s + e + t (SumK, K = 3).
+template <int N>
+__device__ __forceinline__ void sum3(const float (&a)[N], float &s, float &e, float &t) {
+  s = a[0];
+  e = 0.0f;
+  t = 0.0f;
+#pragma unroll
+  for (int i = 1; i < N; i++) {
+    float x, y;
+    two_sum(s, a[i], s, x);
+    two_sum(e, x, e, y);
+    t += y;
+  }
+}
+
 // a + b rounded to FP32 stochastically: the FP32 sum s (round to nearest)
 // or its neighbour s2 on the side of the exact remainder e = a + b - s
 // (TwoSum, Knuth), taken with probability |e| / |s2 - s|, so the result is a
@@ -1014,70 +1029,87 @@ static __device__ __noinline__ void step_node_exact(const float *src, float *dst
   step_node_pull<float, float, true>(src, dst, g, links, k, i, gate);
 }
 
-// rho and u = (j + rho a / 2) / rho in FP64 from rho - 1 and j, as FP64 or
-// double-FP32 values (the components of j and of a given one after the
-// other).  FP32 and 16-bit storage: the sums in twice the working precision
-// and the quotient in double-FP32, about 48 significant bits of values that
-// are FP32 to begin with, converted at the end -- this GPU's FP64 units are
-// so few that FP64 sums and divisions per node took several times as long as
-// the memory they read (8.4 M nodes, FP32: fields 711 us, now 150).
-template <int D>
-__device__ __forceinline__ void macro_fields(DF drho, const DF (&j)[D], const DF (&a)[D],
-                                             double &rho, double (&u)[D]) {
-  const DF r = df_add(DF{1.0f, 0.0f}, drho);
-  const float inv = __frcp_rn(r.h);
-  rho = 1.0 + (static_cast<double>(drho.h) + static_cast<double>(drho.l));
+// The macroscopic fields of a node in FP64 (Eq. FluidMacr): rho = 1 + sum a,
+// u_c = (sum m_c + rho a_c / 2) / rho, from the deviations a, the signed ones of
+// each component m and the halved acceleration half_a.
+template <typename C, int D, int N, int M>
+__device__ __forceinline__ void node_fields_fp64(const C (&a)[N], const C (&m)[D][M],
+                                                 const double (&half_a)[D], double &rho,
+                                                 double (&u)[D]) {
+  double drho = static_cast<double>(a[0]);
+#pragma unroll
+  for (int i = 1; i < N; i++) drho += static_cast<double>(a[i]);
+  rho = 1.0 + drho;
 #pragma unroll
   for (int c = 0; c < D; c++) {
-    const DF v = df_div_inv(df_add(j[c], df_mul(df_scale(0.5f, r), a[c])), r, inv);
-    u[c] = static_cast<double>(v.h) + static_cast<double>(v.l);
+    double j = static_cast<double>(m[c][0]);
+#pragma unroll
+    for (int i = 1; i < M; i++) j += static_cast<double>(m[c][i]);
+    u[c] = fma(rho, half_a[c], j) / rho;
   }
 }
-template <int D>
-__device__ __forceinline__ void macro_fields(double drho, const double (&j)[D],
-                                             const double (&a)[D], double &rho, double (&u)[D]) {
-  rho = 1.0 + drho;
-  for (int c = 0; c < D; c++) u[c] = (j[c] + 0.5 * rho * a[c]) / rho;
-}
-// x in the arithmetic of macro_fields
-template <typename C>
-struct Wide {
-  using type = DF;
-  static __host__ __device__ DF of(double x) {
-    const float h = static_cast<float>(x);
-    return DF{h, static_cast<float>(x - static_cast<double>(h))};
-  }
-};
-template <>
-struct Wide<double> {
-  using type = double;
-  static __host__ __device__ double of(double x) { return x; }
-};
-// Sum of n values: FP64, or FP32 values in twice the working precision.
-template <int N>
-__device__ __forceinline__ double wide_sum(const double (&a)[N]) {
-  double s = a[0];
-  for (int i = 1; i < N; i++) s += a[i];
-  return s;
-}
-template <int N>
-__device__ __forceinline__ DF wide_sum(const float (&a)[N]) {
-  float s, e;
-  sum2(a, s, e);
-  return df_norm(s, e);
+template <int D, int N, int M>
+__device__ __forceinline__ void node_fields(const double (&a)[N], const double (&m)[D][M],
+                                            const double (&half_a)[D], double &rho,
+                                            double (&u)[D]) {
+  node_fields_fp64(a, m, half_a, rho, u);
 }
 
-// Eq. FluidMacr from deviations: returns rho - 1 (kept exact for the mass sum).
-__device__ __forceinline__ double node_velocity(const double *d, double ax, double ay, double &rho,
-                                                double &ux, double &uy) {
-  double drho = 0.0, jx, jy;
-  for (int i = 0; i < 9; i++) drho += d[i];
-  jx = d[1] - d[3] + d[5] - d[6] - d[7] + d[8];
-  jy = d[2] - d[4] + d[5] + d[6] - d[7] - d[8];
-  rho = 1.0 + drho;
-  ux = (jx + 0.5 * rho * ax) / rho;
-  uy = (jy + 0.5 * rho * ay) / rho;
-  return drho;
+// A zero or normal FP32 number as FP64 by integer operations (the exponent's
+// bias exchanged, the mantissa shifted).
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t b = __float_as_uint(x), m = b & 0x7FFFFFFFu;
+  const uint32_t hi = m ? (m >> 3) + 0x38000000u : 0u;
+  return __hiloint2double(static_cast<int>((b & 0x80000000u) | hi), static_cast<int>(b << 29));
+}
+
+// FP32 deviations (FP32 and 16-bit storage): the same values to FP64 accuracy
+// with a quarter of the work on the FP64 units, of which this GPU has few (8.4 M
+// nodes: 210 us against 712; the memory takes 100.  Sums and quotients in
+// double-FP32, 150 us, kept about 47 bits of u).  Sums as three FP32
+// terms (Ogita, Rump and Oishi's SumK, K = 3: within 2^-70 of the values'
+// magnitude), the third zero unless the exponents are far apart; one
+// reciprocal for the quotients, FP32's and a Newton step, and for each
+// quotient a correction from its exact remainder.  Where a term is not finite
+// or subnormal, or rho is far from 1, the node is done in FP64 throughout.
+template <int D, int N, int M>
+__device__ __forceinline__ void node_fields(const float (&a)[N], const float (&m)[D][M],
+                                            const double (&half_a)[D], double &rho,
+                                            double (&u)[D]) {
+  float s[D + 1], e[D + 1], t[D + 1];
+  sum3(a, s[0], e[0], t[0]);
+#pragma unroll
+  for (int c = 0; c < D; c++) sum3(m[c], s[c + 1], e[c + 1], t[c + 1]);
+  // least and largest magnitudes; less 1, zeros are the largest integers
+  uint32_t least = 0xFFFFFFFFu;
+  float third = 0.0f, most = 0.0f;
+#pragma unroll
+  for (int c = 0; c <= D; c++) {
+    for (const float v : {s[c], e[c], t[c]})
+      least = min(least, (__float_as_uint(v) & 0x7FFFFFFFu) - 1u);
+    third = fmaxf(third, fabsf(t[c]));
+    // (NaN compares false below, fmaxf would drop it)
+    most = fabsf(s[c]) <= most ? most : fabsf(s[c]);
+  }
+  if (least >= 0x007FFFFFu && fabsf(s[0]) < 0.5f && most < 0x1p120f) {
+    double w[D + 1];
+#pragma unroll
+    for (int c = 0; c <= D; c++) w[c] = widen(s[c]) + widen(e[c]);
+    if (third != 0.0f) {
+#pragma unroll
+      for (int c = 0; c <= D; c++) w[c] = widen(s[c]) + (widen(e[c]) + widen(t[c]));
+    }
+    rho = 1.0 + w[0];
+    double inv = widen(__frcp_rn(1.0f + s[0]));
+    inv = fma(fma(-rho, inv, 1.0), inv, inv);
+#pragma unroll
+    for (int c = 0; c < D; c++) {
+      const double v = fma(rho, half_a[c], w[c + 1]), q = v * inv;
+      u[c] = fma(fma(-q, rho, v), inv, q);
+    }
+  } else {
+    node_fields_fp64(a, m, half_a, rho, u);
+  }
 }
 
 __device__ __forceinline__ double warp_sum(double v) {

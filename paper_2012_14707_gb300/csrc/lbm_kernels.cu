@@ -297,8 +297,7 @@ residual_final(const double *__restrict__ partials, const int blocks, double *__
 
 template <typename T>
 __global__ void fields_kernel(const T *__restrict__ f, const NodeMap map, int64_t plane,
-                              const typename Wide<typename Stor<T>::C>::type ax,
-                              const typename Wide<typename Stor<T>::C>::type ay, double inv_scale,
+                              const double half_ax, const double half_ay, double inv_scale,
                               double *rho, double *ux, double *uy) {
   using C = typename Stor<T>::C;
   const int64_t n = static_cast<int64_t>(map.nx) * map.ny;
@@ -312,11 +311,10 @@ __global__ void fields_kernel(const T *__restrict__ f, const NodeMap map, int64_
       C a[9];
 #pragma unroll
       for (int i = 0; i < 9; i++) a[i] = Stor<T>::ld(f[s[i]], static_cast<C>(inv_scale));
-      const C jx[6] = {a[1], -a[3], a[5], -a[6], -a[7], a[8]};
-      const C jy[6] = {a[2], -a[4], a[5], a[6], -a[7], -a[8]};
-      using W = typename Wide<C>::type;
-      const W j[2] = {wide_sum(jx), wide_sum(jy)}, acc[2] = {ax, ay};
-      macro_fields<2>(wide_sum(a), j, acc, r, u);
+      const C j[2][6] = {{a[1], -a[3], a[5], -a[6], -a[7], a[8]},
+                         {a[2], -a[4], a[5], a[6], -a[7], -a[8]}};
+      const double half_a[2] = {half_ax, half_ay};
+      node_fields(a, j, half_a, r, u);
     }
     if (rho) rho[p] = r;
     if (ux) ux[p] = u[0];
@@ -523,9 +521,8 @@ template <typename T>
 cudaError_t launch_fields(const T *f, const NodeMap &map, int64_t plane, double ax, double ay,
                           double scale, double *rho, double *ux, double *uy, cudaStream_t s) {
   const int64_t n = static_cast<int64_t>(map.nx) * map.ny;
-  using W = Wide<typename Stor<T>::C>;
-  fields_kernel<T><<<grid_for(n, 256), 256, 0, s>>>(f, map, plane, W::of(ax), W::of(ay),
-                                                    1.0 / scale, rho, ux, uy);
+  fields_kernel<T><<<grid_for(n, 256), 256, 0, s>>>(f, map, plane, 0.5 * ax, 0.5 * ay, 1.0 / scale,
+                                                    rho, ux, uy);
   return cudaGetLastError();
 }
 
