@@ -52,12 +52,12 @@ __device__ __forceinline__ void mbar_expect(uint64_t *bar, uint32_t bytes) {
                : "memory");
 }
 // Waits for the phase with parity `phase`; false if it did not come within
-// kWaitLimit tries or the CTA gave up.  try_wait suspends the warp (for up to
+// kWaitLimit tries or the CTA gave up.  For a role that one lane runs.  try_wait suspends the warp (for up to
 // about the hint, a microsecond): warps polling with test_wait took so many
 // issue slots that the roles with work to do ran several times slower (a
 // 32-channel 256x256 layer 90 us).
 constexpr int kWaitLimit = 1 << 20;
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t phase, volatile int *gave_up) {
+__device__ __forceinline__ bool mbar_wait_lane(uint64_t *bar, uint32_t phase, volatile int *gave_up) {
   const uint32_t a = smem_addr(bar);
   for (int it = 0; it < kWaitLimit; it++) {
     uint32_t done;
@@ -74,10 +74,11 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t phase, volatil
 }
 
 // The same for a warp that waits as one: the answer is warp-uniform, so the
-// loops around it are, and their counters and descriptors.
+// loops around it are, and their counters and descriptors -- and no lane
+// leaves alone ahead of a tcgen05 instruction that the whole warp executes.
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, uint32_t phase,
                                                volatile int *gave_up) {
-  return __all_sync(0xFFFFFFFFu, mbar_wait(bar, phase, gave_up));
+  return __all_sync(0xFFFFFFFFu, mbar_wait_lane(bar, phase, gave_up));
 }
 
 // Shared-memory matrix descriptor without swizzle; lbo, sbo in bytes.
@@ -307,7 +308,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_halo_tc(const __grid_con
           const int t0 = u / a.parts * a.unit_taps, p = u % a.parts;
           const int k8 = min(a.p8, a.k8 - p * a.p8), chunks = (k8 + 7) / 8;
           for (int b = 0; b < a.unit_taps * chunks; b++) {
-            if (issued >= a.stages_b && !mbar_wait(&empty_b[st], ph ^ 1u, &gave_up)) {
+            if (issued >= a.stages_b && !mbar_wait_lane(&empty_b[st], ph ^ 1u, &gave_up)) {
               ok = false;
               break;
             }
@@ -332,7 +333,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_halo_tc(const __grid_con
         // the copies in flight land before the CTA ends
         int never = 0;
         for (int i = max(0, issued - a.stages_b); i < issued; i++)
-          mbar_wait(&full_b[i % a.stages_b], (i / a.stages_b) & 1, &never);
+          mbar_wait_lane(&full_b[i % a.stages_b], (i / a.stages_b) & 1, &never);
       }
     }
   } else if (warp == 1) {
@@ -459,12 +460,11 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_halo_tc(const __grid_con
       const int i = ty * S::kH + py, j = tx * S::kW + m * 8 + px;
       const bool in = i < a.H && j < a.W;
       const int64_t pix = in ? static_cast<int64_t>((n * a.H + i) * a.W + j) : 0;
-      if (!mbar_wait(&full_d[acc], (it >> 1) & 1, &gave_up)) {
+      if (!mbar_wait_warp(&full_d[acc], (it >> 1) & 1, &gave_up)) {
         gave_up = 1;
-        atomicExch(a.err, 1);
+        if (lane == 0) atomicExch(a.err, 1);
         break;
       }
-      __syncwarp();
       fence_after();
       const uint32_t col = tmem + (static_cast<uint32_t>(q * 32) << 16) +
                            static_cast<uint32_t>((acc * MT + m) * a.NT);
@@ -544,7 +544,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_halo_tc(const __grid_con
       const int units = a.parts * (KS * KS / a.unit_taps);
       for (int u = 0; u < units; u++, it++) {
         const int p = u % a.parts;
-        if (it >= a.stages_a && !mbar_wait(&empty_a[sa], pa ^ 1u, &gave_up)) {
+        if (it >= a.stages_a && !mbar_wait_warp(&empty_a[sa], pa ^ 1u, &gave_up)) {
           ok = false;
           break;
         }
@@ -590,7 +590,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_halo_tc(const __grid_con
     cp_async_wait_all();
     if (!ok) {
       gave_up = 1;
-      atomicExch(a.err, 1);
+      if (lane == 0) atomicExch(a.err, 1);
     }
   }
   __syncwarp();
@@ -758,7 +758,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc(const __grid_constant_
     int st = 0, it = 0;
     uint32_t ph = 0;
     for (int t = t0; t < t1; t++, it++) {
-      if (it >= a.stages && !mbar_wait(&empty[st], ph ^ 1u, &gave_up)) {
+      if (it >= a.stages && !mbar_wait_warp(&empty[st], ph ^ 1u, &gave_up)) {
         ok = false;
         break;
       }
@@ -834,15 +834,14 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc(const __grid_constant_
     cp_async_wait_all();
     if (!ok) {
       gave_up = 1;
-      atomicExch(a.err, 1);
+      if (lane == 0) atomicExch(a.err, 1);
     }
     // the sums of this split: lane = input channel (and horizontal tap)
-    const bool have = ok && warp < 4 && mbar_wait(&done, 0, &gave_up);
+    const bool have = ok && warp < 4 && mbar_wait_warp(&done, 0, &gave_up);
     if (!have && warp < 4) {
       gave_up = 1;
-      atomicExch(a.err, 1);
+      if (lane == 0) atomicExch(a.err, 1);
     }
-    __syncwarp();
     if (have) {
       fence_after();
       const bool empty_split = t1 <= t0;
