@@ -308,6 +308,10 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_halo_tc(const __grid_con
           const int t0 = u / a.parts * a.unit_taps, p = u % a.parts;
           const int k8 = min(a.p8, a.k8 - p * a.p8), chunks = (k8 + 7) / 8;
           for (int b = 0; b < a.unit_taps * chunks; b++) {
+            // the ring's first blocks are copied while the kernel before
+            // runs; the bounded wait for a free block starts after it, when
+            // the MMAs do
+            if (issued == a.stages_b) chain_wait();
             if (issued >= a.stages_b && !mbar_wait_lane(&empty_b[st], ph ^ 1u, &gave_up)) {
               ok = false;
               break;

@@ -44,3 +44,14 @@ def test_lane_waits_only_where_one_lane_runs():
             single = any(b.endswith("if (lane == 0)") for b in blocks)
             assert inside or single, (name, blocks[-3:])
     assert found
+
+
+def test_ring_of_weights_waits_after_the_kernel_before():
+    """The weights are copied without waiting for the stream's earlier kernel,
+    but a wait for the MMAs to free a block has a limit, and no MMA runs before
+    that kernel ends: it may take longer than the limit."""
+    text = re.sub(r"//[^\n]*", "", open(SRC).read())
+    kernel = text.split("conv_halo_tc(const __grid_constant__ ConvDev a) {")[1]
+    role = kernel.split("if (warp == 0) {")[1].split("} else if (warp == 1)")[0]
+    before = role.split("&empty_b[st]")[0]
+    assert re.search(r"if \(issued == a\.stages_b\) chain_wait\(\);", before)
