@@ -145,6 +145,39 @@ __device__ __forceinline__ void fence_before() {
 __device__ __forceinline__ void fence_after() {
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
 }
+// p = v (set) or p += v in FP32, rounded to nearest, without waiting for it
+__device__ __forceinline__ void add_or_set(float *p, const float (&v)[4], bool set) {
+  if (set)
+    *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
+  else
+    asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};\n" ::"l"(p),
+                 "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3])
+                 : "memory");
+}
+__device__ __forceinline__ void add_or_set(float *p, float v, bool set) {
+  if (set)
+    *p = v;
+  else
+    asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;\n" ::"l"(p), "f"(v) : "memory");
+}
+// v[r] (of each of 4 neighbouring lanes: the lane's r-th quarter) becomes the
+// lane's own quarter of the r-th of them: the four then write a row together
+__device__ __forceinline__ void transpose4(float (&v)[4][4], int lane) {
+#pragma unroll
+  for (int x = 1; x < 4; x *= 2) {
+    const bool up = lane & x;
+#pragma unroll
+    for (int r = 0; r < 4; r++) {
+      if (r & x) continue;
+#pragma unroll
+      for (int s = 0; s < 4; s++) {
+        const float got = __shfl_xor_sync(0xFFFFFFFFu, up ? v[r][s] : v[r + x][s], x);
+        if (up) v[r][s] = got;
+        else v[r + x][s] = got;
+      }
+    }
+  }
+}
 // 16 columns of this warp's 32 lanes of D
 __device__ __forceinline__ void tmem_ld16(uint32_t addr, uint32_t (&r)[16]) {
   asm volatile(
@@ -615,11 +648,22 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_halo_tc(const __grid_con
 // split of the tiles; the splits' sums go to `partials` and wgrad_reduce adds
 // them in order (the same gradient every time).  The bias gradient is one
 // more accumulator, whose X is all ones.
+// The accumulators hold FP32, but the tensor cores truncate as they add: a sum
+// is biased towards zero by half a unit in the last place of its size per
+// MMA.  So an accumulator runs over kWgChain tiles (512 pixels, 32 MMAs) at
+// most; then eight warps read it and add it, rounding to nearest, to the
+// split's sums in memory, tap by tap, while the next chain's MMAs follow.
+// Relative error of the gradients of positive operands (base 32 and 64,
+// 256x256 x 8) for chains without limit, of 6, 4 and 3 tiles: 7.6e-6 and
+// 2.2e-5, 6.9e-7 and 7.5e-7, 3.6e-7 and 3.7e-7, 2.6e-7; gradients of the
+// 256x256 x 8 network 1414, 1484, 1542, 1602 us.
 // kRep (few input channels): M = 3 x channels, the three horizontal taps of
 // a row at once -- the tile is stored three times, shifted, and one
 // accumulator per vertical tap remains.
-constexpr int kWgLoaders = 256;  // of which the first 128 also read the sums back
-constexpr int kWgThreads = kWgLoaders + 32;
+constexpr int kWgLoaders = 256;
+constexpr int kWgDrain = 256;  // threads that read the sums back
+constexpr int kWgChain = 4;    // tiles an accumulator runs over, at most
+constexpr int kWgThreads = kWgLoaders + 32 + kWgDrain;
 constexpr int kWgStages = 3;
 
 struct WgradDev {
@@ -651,7 +695,8 @@ template <int KS, bool kRep>
 __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc(const __grid_constant__ WgradDev a) {
   using S = WgShape<KS, kRep>;
   extern __shared__ __align__(128) unsigned char dyn[];
-  __shared__ uint64_t full[kWgStages], empty[kWgStages], done;
+  __shared__ uint64_t full[kWgStages], empty[kWgStages];
+  __shared__ uint64_t done, drained[10];  // a chain's sums; read back, per tap (9: the bias)
   __shared__ uint32_t tmem_slot;
   __shared__ int gave_up;
   const int warp = __shfl_sync(0xFFFFFFFFu, static_cast<int>(threadIdx.x >> 5), 0);
@@ -671,12 +716,17 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc(const __grid_constant_
   // this split's tiles
   const int t0 = static_cast<int>(static_cast<int64_t>(a.tiles) * blockIdx.y / a.splits);
   const int t1 = static_cast<int>(static_cast<int64_t>(a.tiles) * (blockIdx.y + 1) / a.splits);
+  // ... in as few chains as kWgChain allows, all about as long
+  const int fewest = (t1 - t0 + kWgChain - 1) / kWgChain;
+  const int per_chain = (t1 - t0 + fewest - 1) / fewest;
   if (tid == 0) {
     for (int i = 0; i < kWgStages; i++) {
       mbar_init(&full[i], kWgLoaders);
       mbar_init(&empty[i], 1);
     }
     mbar_init(&done, 1);
+    for (int i = 0; i < 9; i++) mbar_init(&drained[i], kWgDrain);
+    mbar_init(&drained[9], 32);
     gave_up = 0;
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
@@ -698,8 +748,8 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc(const __grid_constant_
     const uint32_t ones_lo = desc_lo(ones, 128u), ones_hi = desc_hi(256u);
     const uint32_t bias_d = tmem + a.group_taps * a.NT;
     bool ok = true;
-    int st = 0;
-    uint32_t ph = 0, acc = 0;
+    int st = 0, chain = 0, left = 0;  // chains committed, tiles left of this one
+    uint32_t ph = 0;
     for (int t = t0; t < t1; t++) {
       if (!mbar_wait_warp(&full[st], ph, &gave_up)) {
         ok = false;
@@ -711,37 +761,67 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc(const __grid_constant_
       // 16 pixels (two rows of the tile) per MMA
       uint32_t xlo = desc_lo(sx, S::kWp * 16u);
       uint32_t glo = desc_lo(sx + S::kBytesX, 128u);
+      if (left == 0 && chain > 0) {
+        // a further chain's first tile goes tap by tap (the bias last), each
+        // as soon as the sums of the chain before have been read
 #pragma unroll 1
-      for (int k = 0; k < 8; k++) {
-        // taps tap0 .. tap0 + ntap - 1 (vertical taps where kRep)
-#pragma unroll
-        for (int tap = 0; tap < (kRep ? KS : KS * KS); tap++) {
-          const int j = tap - tap0;
-          if (j >= 0 && j < ntap)
-            mma_bf16(leader, tmem + j * a.NT,
-                     xlo + (kRep ? tap * S::kWp : (tap / KS) * S::kWp + tap % KS), ahi, glo, bhi,
-                     idesc, acc);
+        for (int j = 0; j < ntap + (with_bias ? 1 : 0); j++) {
+          const bool bias = j == ntap;
+          if (!mbar_wait_warp(&drained[bias ? 9 : j], (chain - 1) & 1, &gave_up)) {
+            ok = false;
+            break;
+          }
+          fence_after();
+          const int tap = tap0 + j;
+          const uint32_t d = bias ? bias_d : tmem + j * a.NT;
+          const uint32_t alo = bias ? ones_lo
+                                    : xlo + (kRep ? tap * S::kWp : (tap / KS) * S::kWp + tap % KS);
+#pragma unroll 1
+          for (int k = 0; k < 8; k++)
+            mma_bf16(leader, d, alo + (bias ? 0 : k * 2 * S::kWp), bias ? ones_hi : ahi,
+                     glo + 16 * k, bhi, idesc, k);
         }
-        if (with_bias) mma_bf16(leader, bias_d, ones_lo, ones_hi, glo, bhi, idesc, acc);
-        acc = 1;
-        xlo += 2 * S::kWp;
-        glo += 16;
+        if (!ok) break;
+      } else {
+#pragma unroll 1
+        for (int k = 0; k < 8; k++) {
+          // taps tap0 .. tap0 + ntap - 1 (vertical taps where kRep)
+          const uint32_t acc = left != 0 || k != 0;
+#pragma unroll
+          for (int tap = 0; tap < (kRep ? KS : KS * KS); tap++) {
+            const int j = tap - tap0;
+            if (j >= 0 && j < ntap)
+              mma_bf16(leader, tmem + j * a.NT,
+                       xlo + (kRep ? tap * S::kWp : (tap / KS) * S::kWp + tap % KS), ahi, glo, bhi,
+                       idesc, acc);
+          }
+          if (with_bias) mma_bf16(leader, bias_d, ones_lo, ones_hi, glo, bhi, idesc, acc);
+          xlo += 2 * S::kWp;
+          glo += 16;
+        }
       }
+      if (left == 0) left = min(per_chain, t1 - t);
       mma_commit(leader, &empty[st]);
       if (++st == a.stages) {
         st = 0;
         ph ^= 1u;
       }
+      if (--left == 0) {
+        mma_commit(leader, &done);
+        chain++;
+      }
     }
-    mma_commit(leader, &done);
     if (!ok) {
       gave_up = 1;
       if (lane == 0) atomicExch(a.err, 1);
+      // the MMAs in flight end before the memory is given back
       int never = 0;
-      mbar_wait_warp(&done, 0, &never);
+      if (chain > 0) mbar_wait_warp(&done, (chain - 1) & 1, &never);
+      mma_commit(leader, &done);
+      mbar_wait_warp(&done, chain & 1, &never);
     }
     __syncwarp();
-  } else {
+  } else if (warp < 8) {
     // loads: this block's input slabs, then the gradient's
     const int n8x = min(16, a.x.n8 - mb * 16);
     constexpr int kPix = S::kHp * (8 + 2 * S::kHalo);
@@ -840,60 +920,89 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc(const __grid_constant_
       gave_up = 1;
       if (lane == 0) atomicExch(a.err, 1);
     }
-    // the sums of this split: lane = input channel (and horizontal tap)
-    const bool have = ok && warp < 4 && mbar_wait_warp(&done, 0, &gave_up);
-    if (!have && warp < 4) {
-      gave_up = 1;
-      if (lane == 0) atomicExch(a.err, 1);
-    }
-    if (have) {
+  } else {
+    // the sums of each chain: lane = input channel (and horizontal tap), a
+    // tap's blocks of 16 outputs in turn for the two groups of four warps
+    const int q = warp & 3, row = q * 32 + lane, half = (warp - 9) >> 2;
+    // row -> (dx, channel as the kernels see it) -> channel of the layer
+    const int rows = min(16, a.x.n8 - mb * 16) * 8;
+    const int dxr = kRep ? row / rows : 0;
+    const int cp = kRep ? row - dxr * rows : row;
+    const int ck = mb * 128 + cp;  // padded channel
+    const int ca8 = a.x.n8a * 8;
+    const int c = ck < ca8 ? (ck < a.ca ? ck : -1)
+                           : (a.ca + ck - ca8 < a.ci ? a.ca + ck - ca8 : -1);
+    const bool valid = cp < rows && c >= 0 && (!kRep || dxr < KS);
+    // the row's place among a tap's (a row of taps') sums, or -1; and those of
+    // the four rows that four neighbouring lanes write together
+    const int at = valid ? (dxr * a.ci + c) * a.co : -1;
+    int at4[4];
+#pragma unroll
+    for (int r = 0; r < 4; r++) at4[r] = __shfl_sync(0xFFFFFFFFu, at, (lane & ~3) + r);
+    float *out = a.partials + static_cast<int64_t>(blockIdx.y) * a.len;
+    const bool v4 = a.co % 4 == 0;
+    for (int ch = 0; ch * per_chain < t1 - t0; ch++) {
+      if (!mbar_wait_warp(&done, ch & 1, &gave_up)) {
+        gave_up = 1;
+        if (lane == 0) atomicExch(a.err, 1);
+        break;
+      }
       fence_after();
-      const bool empty_split = t1 <= t0;
-      const int row = warp * 32 + lane;
-      // row -> (dx, channel as the kernels see it) -> channel of the layer
-      const int rows = n8x * 8;
-      const int dxr = kRep ? row / rows : 0;
-      const int cp = kRep ? row - dxr * rows : row;
-      const int ck = mb * 128 + cp;  // padded channel
-      const int ca8 = a.x.n8a * 8;
-      const int c = ck < ca8 ? (ck < a.ca ? ck : -1)
-                             : (a.ca + ck - ca8 < a.ci ? a.ca + ck - ca8 : -1);
-      const bool valid = cp < rows && c >= 0 && (!kRep || dxr < KS);
-      float *out = a.partials + static_cast<int64_t>(blockIdx.y) * a.len;
-      const bool v4 = a.co % 4 == 0;
-      for (int j = 0; j < ntap + (with_bias ? 1 : 0); j++) {
-        const bool bias = j == ntap;
-        const int col = bias ? a.group_taps : j;
-        const int tap = kRep ? (tap0 + j) * KS + dxr : tap0 + j;
-        float *dst = bias ? out + static_cast<int64_t>(KS * KS) * a.ci * a.co
-                          : out + (static_cast<int64_t>(tap) * a.ci + c) * a.co;
-        const bool write = bias ? row == 0 : valid;
-        for (int cc = 0; cc < a.NT; cc += 16) {
-          uint32_t v[16];
-          tmem_ld16(tmem + (static_cast<uint32_t>(warp * 32) << 16) +
-                        static_cast<uint32_t>(col * a.NT + cc),
-                    v);
+      for (int j = 0; j < ntap; j++) {
+        float *dst = out + static_cast<int64_t>(tap0 + j) * (kRep ? KS : 1) * a.ci * a.co + o0;
+        for (int cc = 16 * ((half + j * (a.NT / 16)) & 1); cc < a.NT; cc += 64) {
+          float v[2][4][4];
+          const bool two = cc + 32 < a.NT;
+          const uint32_t at0 = tmem + (static_cast<uint32_t>(q * 32) << 16) +
+                               static_cast<uint32_t>(j * a.NT + cc);
+          tmem_ld16(at0, reinterpret_cast<uint32_t (&)[16]>(v[0]));
+          if (two) tmem_ld16(at0 + 32, reinterpret_cast<uint32_t (&)[16]>(v[1]));
           tmem_wait_ld();
-          if (!write) continue;
-          const int o = o0 + cc;
+          if (cc + 64 >= a.NT) {
+            fence_before();
+            mbar_arrive(&drained[j]);
+          }
 #pragma unroll
-          for (int e = 0; e < 16; e += 4) {
-            float f[4];
-#pragma unroll
-            for (int s = 0; s < 4; s++) f[s] = empty_split ? 0.f : __uint_as_float(v[e + s]);
+          for (int h = 0; h < 2; h++) {
+            if (h == 1 && !two) break;
             if (v4) {
-              if (o + e < a.co)
-                *reinterpret_cast<float4 *>(dst + o + e) = make_float4(f[0], f[1], f[2], f[3]);
+              transpose4(v[h], lane);
+              const int o = cc + 32 * h + 4 * (lane & 3);
+#pragma unroll
+              for (int r = 0; r < 4; r++)
+                if (at4[r] >= 0 && o0 + o < a.co) add_or_set(dst + at4[r] + o, v[h][r], ch == 0);
             } else {
 #pragma unroll
-              for (int s = 0; s < 4; s++)
-                if (o + e + s < a.co) dst[o + e + s] = f[s];
+              for (int e = 0; e < 16; e++)
+                if (at >= 0 && o0 + cc + 32 * h + e < a.co)
+                  add_or_set(dst + at + cc + 32 * h + e, v[h][e / 4][e % 4], ch == 0);
             }
           }
+          __syncwarp();
         }
+        // (a half without a block of this tap)
+        if (16 * ((half + j * (a.NT / 16)) & 1) >= a.NT) mbar_arrive(&drained[j]);
+      }
+      if (with_bias && warp == 12) {  // every row holds it
+        for (int cc = 0; cc < a.NT; cc += 16) {
+          uint32_t v[16];
+          tmem_ld16(tmem + static_cast<uint32_t>(a.group_taps * a.NT + cc), v);
+          tmem_wait_ld();
+          float mine = 0.f;
+#pragma unroll
+          for (int e = 0; e < 16; e++)
+            if (lane == e) mine = __uint_as_float(v[e]);
+          if (lane < 16 && o0 + cc + lane < a.co)
+            add_or_set(out + static_cast<int64_t>(KS * KS) * a.ci * a.co + o0 + cc + lane, mine,
+                       ch == 0);
+          __syncwarp();
+        }
+        fence_before();
+        mbar_arrive(&drained[9]);
       }
     }
   }
+  __syncwarp();
   fence_before();
   __syncthreads();
   fence_after();
