@@ -329,16 +329,8 @@ __device__ __forceinline__ void transform3(const A n0, const A (&NS)[kPairs3],
   }
 }
 
-// v / r by r's reciprocal and one correction from the exact remainder (the
-// correctly rounded quotient, but for rare last-place ties): three divisions
-// by the same density cost one.
 __device__ __forceinline__ float recip3(float r) { return __frcp_rn(r); }
 __device__ __forceinline__ double recip3(double r) { return 1.0 / r; }
-template <typename A>
-__device__ __forceinline__ A quotient3(A v, A r, A inv) {
-  const A q = v * inv;
-  return fma(fma(-q, r, v), inv, q);
-}
 
 // The collision change f' - f of one node from its deviations d (Eq.
 // FluidMacr, Eq. LBEequi, Eq. LBEforce, Eq. MomentPost through M^-1), in
@@ -366,9 +358,9 @@ __device__ __forceinline__ void collide3(const A (&d)[Q], const Const3<A> &k, A 
     for (int pp = 0; pp < kPairs3; pp++) j[a] = mac3(j[a], cvel3(rep3(pp), a), D[pp]);
   rho = A(1) + drho;
   const A inv = recip3(rho), half = A(0.5) * rho;
-  u[0] = quotient3(fma(half, k.ax, j[0]), rho, inv);
-  u[1] = quotient3(fma(half, k.ay, j[1]), rho, inv);
-  u[2] = quotient3(fma(half, k.az, j[2]), rho, inv);
+  u[0] = lbm::dev::quotient(fma(half, k.ax, j[0]), rho, inv);
+  u[1] = lbm::dev::quotient(fma(half, k.ay, j[1]), rho, inv);
+  u[2] = lbm::dev::quotient(fma(half, k.az, j[2]), rho, inv);
   const A ux = u[0], uy = u[1], uz = u[2];
   const A uu = ux * ux + uy * uy + uz * uz;
   // d - d_eq (Eq. LBEequi), as pair sums and differences; the rest

@@ -260,17 +260,20 @@ __device__ __forceinline__ DF df_mul(DF a, DF b) {
 }
 // c a for c a power of two (or -1, 0, 1): exact
 __device__ __forceinline__ DF df_scale(float c, DF a) { return DF{c * a.h, c * a.l}; }
+// v / r by r's rounded reciprocal inv and a correction from the exact
+// remainder: the correctly rounded quotient (Markstein's division), so several
+// divisions by one density cost one.
+template <typename A>
+__device__ __forceinline__ A quotient(A v, A r, A inv) {
+  const A q = v * inv;
+  return fma(fma(-q, r, v), inv, q);
+}
 // a / b, given inv = 1 / b.h rounded: the quotient's head, then the exact
 // remainder's
 __device__ __forceinline__ DF df_div_inv(DF a, DF b, float inv) {
-  const float q1 = __fmul_rn(a.h, inv);
+  const float q1 = quotient(a.h, b.h, inv);
   const DF r = df_sub(a, df_mul_f(b, q1));
-  return df_quick(q1, __fmul_rn(r.h, inv));
-}
-__device__ __forceinline__ DF df_div(DF a, DF b) {
-  const float q1 = __fdiv_rn(a.h, b.h);
-  const DF r = df_sub(a, df_mul_f(b, q1));
-  return df_quick(q1, __fdiv_rn(r.h, b.h));
+  return df_quick(q1, quotient(r.h, b.h, inv));
 }
 // A running sum in twice the working precision (Sum2 over double-FP32
 // terms): s + e.
@@ -397,14 +400,8 @@ __device__ __forceinline__ void collide(const C (&d)[9], const StepConst<C> &k, 
     sum2(jxs, r.jx_hi, r.jx_lo);
     sum2(jys, r.jy_hi, r.jy_lo);
     const float rho = 1.0f + (r.dr_hi + r.dr_lo), inv = __frcp_rn(rho);
-    // u: the reciprocal's product and one correction from the exact remainder
-    // (the correctly rounded quotient, but for rare last-place ties)
-    auto over_rho = [&](float v) {
-      const float q = __fmul_rn(v, inv);
-      return __fmaf_rn(__fmaf_rn(-q, rho, v), inv, q);
-    };
-    const C given[3] = {rho, over_rho(r.jx_hi + (r.jx_lo + 0.5f * rho * k.ax)),
-                        over_rho(r.jy_hi + (r.jy_lo + 0.5f * rho * k.ay))};
+    const C given[3] = {rho, quotient(r.jx_hi + (r.jx_lo + 0.5f * rho * k.ax), rho, inv),
+                        quotient(r.jy_hi + (r.jy_lo + 0.5f * rho * k.ay), rho, inv)};
     collision_change<kS, true>(d, k, ch, r.drho, r.rho, r.ux, r.uy, r.uu, given);
   } else {
     collision_change<kS, false>(d, k, ch, r.drho, r.rho, r.ux, r.uy, r.uu);
