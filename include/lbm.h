@@ -164,7 +164,12 @@ int lbm_create(const lbm_domain_t *dom, const uint8_t *solid, size_t n_links,
                double Kn, const lbm_params_t *params, lbm_handle_t **out);
 
 /* Advance n >= 0 time steps (collision, streaming, boundary links: Sec. 2,
- * Eq. EqNewBDSC).  Asynchronous on the handle's stream. */
+ * Eq. EqNewBDSC).  Asynchronous on the handle's stream.  The launches can be
+ * captured in a CUDA graph; the handle advances (lattice and step count) once,
+ * at capture, and does not count replays.  So that replays continue one
+ * another, capture an even number of steps; and of FP64 or plain FP32 steps
+ * only, since the random bits of 16-bit and exact-mass steps are drawn per
+ * step of the handle and would be the same in every replay. */
 int lbm_step(lbm_handle_t *h, int64_t n);
 
 /*

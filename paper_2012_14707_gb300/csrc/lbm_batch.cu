@@ -12,9 +12,9 @@
 // the single-case kernel's per-node update (step_node_pull), so a case in a
 // batch follows exactly the arithmetic of the case run alone.  Every K
 // steps a batched reduction (fixed parts of a case's nodes, one CTA each,
-// then one CTA per case, summed in a fixed order) computes each case's
-// residual and retires converged cases on the device; retired cases' CTAs
-// return immediately.  K steps plus the reduction are captured once in a
+// then one CTA in which a warp per case adds the parts in a fixed order)
+// computes each case's residual and retires converged cases on the device;
+// retired cases' CTAs return immediately.  K steps plus the reduction are captured once in a
 // CUDA graph that the host replays, reading back only the number of active
 // cases.  The CTA width and the L2 prefetch are picked by timing the
 // candidates on the batch itself (autotuner), cached per size class and
@@ -434,7 +434,7 @@ struct lbm_batch {
   int32_t *index = nullptr;
   void *links = nullptr;
   void *cases = nullptr;
-  // FP32 cases with moving walls: FP64 link records and per-link carry
+  // FP32 cases with moving walls: double-FP32 link records and per-link carry
   // (the exact-mass variant), over the whole link arena; null if no case
   // needs them
   lbm::LinkCoefDF *links64 = nullptr;

@@ -156,7 +156,7 @@ struct Collided {
   T t[9];
   C drho, rho, ux, uy, uu;
   // the exact-mass variant (FP32 storage): rho - 1 and j in twice the
-  // working precision (hi + lo), for the FP64 link values
+  // working precision (hi + lo), for the double-FP32 link values
   float dr_hi, dr_lo, jx_hi, jx_lo, jy_hi, jy_lo;
 };
 
@@ -375,13 +375,13 @@ __device__ __forceinline__ void collision_change(const C (&d)[9], const StepCons
 // mass with the fluid at a rate set by the velocity next to it, so every
 // rounding that leans the same way step after step shows up in the mass.
 // Hence: rho - 1 and j are summed in twice the working precision (sum2),
-// rho and u rounded once each for the equilibrium, and kept for the links'
-// FP64 values; f'_1..f'_8 are rounded to FP32 stochastically
+// rho and u rounded once each for the equilibrium, and the sums kept for the
+// links' double-FP32 values; f'_1..f'_8 are rounded to FP32 stochastically
 // (add_stochastic, random bits from rs); f'_0 closes the node's mass in
 // twice the working precision plus the node's carry c0 (what FP32 storage
 // dropped from its earlier values), is stored rounded to nearest, and the
-// new remainder is kept in c0.  Only boundary nodes do FP64 arithmetic
-// (this GPU has few FP64 units).
+// new remainder is kept in c0.  Nothing of it is FP64 arithmetic (this GPU
+// has few FP64 units).
 // 16-bit storage rounds f'_0..f'_8 stochastically with random bits from rs,
 // the node's random word (fmix32 of the node index and the step seed).
 template <typename T, typename C, bool kExact = false>
@@ -813,35 +813,10 @@ __device__ __forceinline__ void step_node_pull(const T *src, T *dst,
 // the folded form of LinkCoef, in the storage's units, from the node's
 // post-collision values oj = f'_j, ojb = f'_jb, its pre-collision f_jb,
 // drho, rho (storage units where scaled) and u.
+// (The velocity components and the weight come from packed tables: j is
+// known only at run time.)
 template <typename T>
-__device__ __forceinline__ float link_value(const LinkCoef<float> &c, const int j, const float djb,
-                                            const float oj, const float ojb, const float drho,
-                                            const float rho, const float ux, const float uy,
-                                            const float uu, const StepConst<float> &k) {
-  constexpr bool kS = Stor<T>::kScaled;
-  constexpr int cx_tab[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1};
-  constexpr int cy_tab[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
-  constexpr float w_tab[9] = {4.0f / 9, 1.0f / 9, 1.0f / 9, 1.0f / 9, 1.0f / 9,
-                              1.0f / 36, 1.0f / 36, 1.0f / 36, 1.0f / 36};
-  const float r = c.k1 + c.k2 + c.k3;
-  float c0, c2;
-  if (k.diffuse_mode == 0) {
-    c0 = c.alpha;
-    c2 = (1.0f - r) * w_tab[j];
-  } else {
-    c0 = c.alpha + (r - 1.0f) * w_tab[j];
-    c2 = 0.0f;
-  }
-  const float cu = float(cx_tab[j]) * ux + float(cy_tab[j]) * uy;
-  const float pj = 3.0f * cu + 4.5f * cu * cu - 1.5f * uu;
-  return c.k1 * djb + c.k2 * oj + c.k3 * ojb + (kS ? c0 * k.sc : c0) + c.alpha * drho +
-         c2 * (drho + rho * pj);
-}
-
-// link_value for a direction j known only at run time (the same
-// arithmetic; the velocity components and weight come from packed tables).
-template <typename T>
-__device__ __forceinline__ float link_value_rt(const LinkCoef<float> &c, const int j,
+__device__ __forceinline__ float link_value(const LinkCoef<float> &c, const int j,
                                                const float djb, const float oj, const float ojb,
                                                const float drho, const float rho, const float ux,
                                                const float uy, const float uu,
@@ -924,7 +899,7 @@ __device__ __forceinline__ void pair_links_warp(const T *src, T *dst,
     const uint32_t dsc = g.ldesc[lj];
     const int n = static_cast<int>(dsc >> 4), j = static_cast<int>(dsc & 15u), jb = opp2(j);
     const auto rec = [&](int row) { return reinterpret_cast<const float *>(pw_v[w][row])[n]; };
-    const float v = link_value_rt<T>(links[lj], j, Stor<T>::ld_raw(src[g.jbslot[lj]]), rec(j - 1),
+    const float v = link_value<T>(links[lj], j, Stor<T>::ld_raw(src[g.jbslot[lj]]), rec(j - 1),
                                      rec(jb - 1), rec(8), rec(9), rec(10), rec(11), rec(12), k);
     const uint32_t h = reinterpret_cast<const uint32_t *>(pw_h[w])[n];
     dst[tail + lj] =

@@ -5,8 +5,8 @@
 // solver, which then runs to the same residual as from rest.
 //
 // Layout: activations NHWC, weights [kh][kw][ci][co] (the layout of the
-// FP64 reference in the tests).  Storage type A of activations and
-// activation gradients: BF16 (training) or FP32 (gradient checks); every
+// FP64 reference in the tests).  Activations and activation gradients are
+// stored in BF16 (training) or FP32 (gradient checks); every
 // product is accumulated in FP32; master weights, weight gradients and Adam
 // moments are FP32.
 //
@@ -31,7 +31,6 @@
 #include <cstdint>
 #include <cstring>
 #include <string>
-#include <type_traits>
 #include <vector>
 
 #include <cuda_bf16.h>
@@ -45,19 +44,6 @@ namespace lbm {
 namespace net {
 namespace {
 
-template <typename A>
-__device__ __forceinline__ float to_f(A v);
-template <>
-__device__ __forceinline__ float to_f<float>(float v) {
-  return v;
-}
-template <typename A>
-__device__ __forceinline__ A from_f(float v);
-template <>
-__device__ __forceinline__ float from_f<float>(float v) {
-  return v;
-}
-
 constexpr int TP = 16;  // pixel tile edge
 constexpr int TC = 16;  // channel tile (input slice and output block)
 
@@ -65,10 +51,11 @@ constexpr int TC = 16;  // channel tile (input slice and output block)
 // over a channel range; `relu` applies max(., 0).  xs: channel stride of x
 // (x may be a slice of a wider tensor: element (n,i,j,c) at
 // ((n*H + i)*W + j)*xs + c).  Grid: (ceil(W/16)*ceil(H/16), ceil(Co/16), N).
-template <typename A, int KS>
+template <int KS>
 __global__ void __launch_bounds__(TP * TP)
-conv_fwd(const A *__restrict__ x, int xs, const A *__restrict__ w, const float *__restrict__ b,
-         A *__restrict__ y, int ys, int H, int W, int Ci, int Co, int relu) {
+conv_fwd(const float *__restrict__ x, int xs, const float *__restrict__ w,
+         const float *__restrict__ b, float *__restrict__ y, int ys, int H, int W, int Ci, int Co,
+         int relu) {
   constexpr int HALO = KS / 2;
   constexpr int T = TP + 2 * HALO;
   __shared__ float sx[T][T][TC + 1];  // +1: conflict-free strided reads
@@ -89,13 +76,13 @@ conv_fwd(const A *__restrict__ x, int xs, const A *__restrict__ w, const float *
       const int gi = ti * TP + pi - HALO, gj = tj * TP + pj - HALO;
       float v = 0.f;
       if (gi >= 0 && gi < H && gj >= 0 && gj < W && c0 + c < Ci)
-        v = to_f<A>(x[((static_cast<int64_t>(n) * H + gi) * W + gj) * xs + c0 + c]);
+        v = x[((static_cast<int64_t>(n) * H + gi) * W + gj) * xs + c0 + c];
       sx[pi][pj][c] = v;
     }
     for (int e = threadIdx.x; e < KS * KS * TC * TC; e += TP * TP) {
       const int o = e % TC, c = (e / TC) % TC, d = e / (TC * TC);
       float v = 0.f;
-      if (c0 + c < Ci && o0 + o < Co) v = to_f<A>(w[(static_cast<int64_t>(d) * Ci + c0 + c) * Co + o0 + o]);
+      if (c0 + c < Ci && o0 + o < Co) v = w[(static_cast<int64_t>(d) * Ci + c0 + c) * Co + o0 + o];
       sw[d / KS][d % KS][c][o] = v;
     }
     __syncthreads();
@@ -112,13 +99,13 @@ conv_fwd(const A *__restrict__ x, int xs, const A *__restrict__ w, const float *
     __syncthreads();
   }
   if (i < H && j < W) {
-    A *yp = y + ((static_cast<int64_t>(n) * H + i) * W + j) * ys;
+    float *yp = y + ((static_cast<int64_t>(n) * H + i) * W + j) * ys;
 #pragma unroll
     for (int q = 0; q < TC; q++) {
       if (o0 + q < Co) {
         float v = acc[q] + (b ? b[o0 + q] : 0.f);
         if (relu) v = fmaxf(v, 0.f);
-        yp[o0 + q] = from_f<A>(v);
+        yp[o0 + q] = v;
       }
     }
   }
@@ -127,10 +114,11 @@ conv_fwd(const A *__restrict__ x, int xs, const A *__restrict__ w, const float *
 // dW[dy][dx][c][o] += sum over a pixel chunk of x[p + d - HALO][c] gz[p][o];
 // db[o] += sum gz[p][o] (blockIdx.y == 0 tiles only).  Grid:
 // (ceil(Ci/16) * ceil(Co/16), chunks); 256 threads = 16 (c) x 16 (o).
-template <typename A, int KS>
+template <int KS>
 __global__ void __launch_bounds__(256)
-conv_bwd_weight(const A *__restrict__ x, int xs, const A *__restrict__ gz, int N, int H, int W,
-                int Ci, int Co, int pix_per_chunk, float *__restrict__ dw, float *__restrict__ db) {
+conv_bwd_weight(const float *__restrict__ x, int xs, const float *__restrict__ gz, int N, int H,
+                int W, int Ci, int Co, int pix_per_chunk, float *__restrict__ dw,
+                float *__restrict__ db) {
   constexpr int HALO = KS / 2;
   const int tiles_o = (Co + TC - 1) / TC;
   const int c0 = (blockIdx.x / tiles_o) * TC, o0 = (blockIdx.x % tiles_o) * TC;
@@ -149,7 +137,7 @@ conv_bwd_weight(const A *__restrict__ x, int xs, const A *__restrict__ gz, int N
     for (int e = threadIdx.x; e < 32 * TC; e += 256) {
       const int pp = e / TC, oo = e % TC;
       const int64_t p = pb + pp;
-      sg[pp][oo] = (p < p1 && o0 + oo < Co) ? to_f<A>(gz[p * Co + o0 + oo]) : 0.f;
+      sg[pp][oo] = (p < p1 && o0 + oo < Co) ? gz[p * Co + o0 + oo] : 0.f;
     }
     for (int e = threadIdx.x; e < 32 * KS * KS * TC; e += 256) {
       const int cc = e % TC, d = (e / TC) % (KS * KS), pp = e / (TC * KS * KS);
@@ -160,7 +148,7 @@ conv_bwd_weight(const A *__restrict__ x, int xs, const A *__restrict__ gz, int N
         const int rem = static_cast<int>(p - n * H * W);
         const int i = rem / W + d / KS - HALO, j = rem % W + d % KS - HALO;
         if (i >= 0 && i < H && j >= 0 && j < W)
-          v = to_f<A>(x[((n * H + i) * W + j) * xs + c0 + cc]);
+          v = x[((n * H + i) * W + j) * xs + c0 + cc];
       }
       sxv[pp][d][cc] = v;
     }
@@ -183,45 +171,42 @@ conv_bwd_weight(const A *__restrict__ x, int xs, const A *__restrict__ gz, int N
 }
 
 // wt[d'][o][c] = w[KS*KS-1-d'][c][o]: the weights of the adjoint convolution.
-template <typename A>
-__global__ void flip_weights(const float *__restrict__ w, A *__restrict__ wt, int KS2, int Ci, int Co) {
+__global__ void flip_weights(const float *__restrict__ w, float *__restrict__ wt, int KS2, int Ci,
+                             int Co) {
   const int64_t n = static_cast<int64_t>(KS2) * Ci * Co;
   for (int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; e < n;
        e += static_cast<int64_t>(gridDim.x) * blockDim.x) {
     const int c = static_cast<int>(e % Ci), o = static_cast<int>((e / Ci) % Co),
               d = static_cast<int>(e / (static_cast<int64_t>(Ci) * Co));
-    wt[e] = from_f<A>(w[(static_cast<int64_t>(KS2 - 1 - d) * Ci + c) * Co + o]);
+    wt[e] = w[(static_cast<int64_t>(KS2 - 1 - d) * Ci + c) * Co + o];
   }
 }
 
-template <typename A>
-__global__ void to_storage(const float *__restrict__ s, A *__restrict__ d, int64_t n) {
+__global__ void to_storage(const float *__restrict__ s, float *__restrict__ d, int64_t n) {
   for (int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; e < n;
        e += static_cast<int64_t>(gridDim.x) * blockDim.x)
-    d[e] = from_f<A>(s[e]);
+    d[e] = s[e];
 }
 
-template <typename A>
-__global__ void to_float(const A *__restrict__ s, int ss, float *__restrict__ d, int C, int64_t npix) {
+__global__ void to_float(const float *__restrict__ s, int ss, float *__restrict__ d, int C,
+                         int64_t npix) {
   for (int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; e < npix * C;
        e += static_cast<int64_t>(gridDim.x) * blockDim.x) {
     const int64_t p = e / C;
-    d[e] = to_f<A>(s[p * ss + e % C]);
+    d[e] = s[p * ss + e % C];
   }
 }
 
 // g[p][c] *= (h[p][c] > 0)  (ReLU backward; h is the layer output)
-template <typename A>
-__global__ void relu_mask(A *__restrict__ g, const A *__restrict__ h, int64_t n) {
+__global__ void relu_mask(float *__restrict__ g, const float *__restrict__ h, int64_t n) {
   for (int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; e < n;
        e += static_cast<int64_t>(gridDim.x) * blockDim.x)
-    if (!(to_f<A>(h[e]) > 0.f)) g[e] = from_f<A>(0.f);
+    if (!(h[e] > 0.f)) g[e] = 0.f;
 }
 
 // 2x2 average pooling, y has H/2 x W/2 pixels; x channel stride xs.
-template <typename A>
-__global__ void pool2_fwd(const A *__restrict__ x, int xs, A *__restrict__ y, int N, int H, int W,
-                          int C) {
+__global__ void pool2_fwd(const float *__restrict__ x, int xs, float *__restrict__ y, int N, int H,
+                          int W, int C) {
   const int h2 = H / 2, w2 = W / 2;
   const int64_t n_out = static_cast<int64_t>(N) * h2 * w2 * C;
   for (int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; e < n_out;
@@ -233,15 +218,14 @@ __global__ void pool2_fwd(const A *__restrict__ x, int xs, A *__restrict__ y, in
     float s = 0.f;
     for (int a = 0; a < 2; a++)
       for (int bb = 0; bb < 2; bb++)
-        s += to_f<A>(x[((n * H + 2 * i + a) * W + 2 * j + bb) * xs + c]);
-    y[e] = from_f<A>(0.25f * s);
+        s += x[((n * H + 2 * i + a) * W + 2 * j + bb) * xs + c];
+    y[e] = 0.25f * s;
   }
 }
 
 // gx[.] (+)= gy / 4 spread over each 2x2 block; gx channel stride xs
-template <typename A>
-__global__ void pool2_bwd(const A *__restrict__ gy, A *__restrict__ gx, int xs, int N, int H, int W,
-                          int C, int accumulate) {
+__global__ void pool2_bwd(const float *__restrict__ gy, float *__restrict__ gx, int xs, int N,
+                          int H, int W, int C, int accumulate) {
   const int64_t n_in = static_cast<int64_t>(N) * H * W * C;
   for (int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; e < n_in;
        e += static_cast<int64_t>(gridDim.x) * blockDim.x) {
@@ -249,17 +233,16 @@ __global__ void pool2_bwd(const A *__restrict__ gy, A *__restrict__ gx, int xs, 
     const int64_t p = e / C;
     const int j = static_cast<int>(p % W), i = static_cast<int>((p / W) % H);
     const int64_t n = p / (static_cast<int64_t>(W) * H);
-    float v = 0.25f * to_f<A>(gy[((n * (H / 2) + i / 2) * (W / 2) + j / 2) * C + c]);
-    A *dst = gx + p * xs + c;
-    if (accumulate) v += to_f<A>(*dst);
-    *dst = from_f<A>(v);
+    float v = 0.25f * gy[((n * (H / 2) + i / 2) * (W / 2) + j / 2) * C + c];
+    float *dst = gx + p * xs + c;
+    if (accumulate) v += *dst;
+    *dst = v;
   }
 }
 
 // y (channel stride ys, first C channels) = nearest 2x upsampling of x
-template <typename A>
-__global__ void up2_fwd(const A *__restrict__ x, A *__restrict__ y, int ys, int N, int H, int W,
-                        int C) {
+__global__ void up2_fwd(const float *__restrict__ x, float *__restrict__ y, int ys, int N, int H,
+                        int W, int C) {
   const int64_t n_out = static_cast<int64_t>(N) * H * W * C;  // H, W: output size
   for (int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; e < n_out;
        e += static_cast<int64_t>(gridDim.x) * blockDim.x) {
@@ -272,9 +255,8 @@ __global__ void up2_fwd(const A *__restrict__ x, A *__restrict__ y, int ys, int 
 }
 
 // gx (H/2 x W/2, C channels) = sum of gy over each 2x2 block; gy channel stride gs
-template <typename A>
-__global__ void up2_bwd(const A *__restrict__ gy, int gs, A *__restrict__ gx, int N, int H, int W,
-                        int C) {
+__global__ void up2_bwd(const float *__restrict__ gy, int gs, float *__restrict__ gx, int N, int H,
+                        int W, int C) {
   const int h2 = H / 2, w2 = W / 2;
   const int64_t n_out = static_cast<int64_t>(N) * h2 * w2 * C;
   for (int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; e < n_out;
@@ -285,35 +267,33 @@ __global__ void up2_bwd(const A *__restrict__ gy, int gs, A *__restrict__ gx, in
     const int64_t n = p / (static_cast<int64_t>(w2) * h2);
     float s = 0.f;
     for (int a = 0; a < 2; a++)
-      for (int bb = 0; bb < 2; bb++) s += to_f<A>(gy[((n * H + 2 * i + a) * W + 2 * j + bb) * gs + c]);
-    gx[e] = from_f<A>(s);
+      for (int bb = 0; bb < 2; bb++) s += gy[((n * H + 2 * i + a) * W + 2 * j + bb) * gs + c];
+    gx[e] = s;
   }
 }
 
 // copy C channels between tensors with channel strides (and offsets applied by the caller)
-template <typename A>
-__global__ void copy_channels(const A *__restrict__ s, int ss, A *__restrict__ d, int ds, int C,
-                              int64_t npix, int accumulate) {
+__global__ void copy_channels(const float *__restrict__ s, int ss, float *__restrict__ d, int ds,
+                              int C, int64_t npix, int accumulate) {
   for (int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; e < npix * C;
        e += static_cast<int64_t>(gridDim.x) * blockDim.x) {
     const int64_t p = e / C;
     const int c = static_cast<int>(e % C);
-    float v = to_f<A>(s[p * ss + c]);
-    if (accumulate) v += to_f<A>(d[p * ds + c]);
-    d[p * ds + c] = from_f<A>(v);
+    float v = s[p * ss + c];
+    if (accumulate) v += d[p * ds + c];
+    d[p * ds + c] = v;
   }
 }
 
 // MSE: loss partials and gy = 2 (y - t) / n
-template <typename A>
-__global__ void mse_kernel(const A *__restrict__ y, const float *__restrict__ t, A *__restrict__ gy,
-                           int64_t n, double *__restrict__ loss) {
+__global__ void mse_kernel(const float *__restrict__ y, const float *__restrict__ t,
+                           float *__restrict__ gy, int64_t n, double *__restrict__ loss) {
   double s = 0.0;
   for (int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; e < n;
        e += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const float d = to_f<A>(y[e]) - t[e];
+    const float d = y[e] - t[e];
     s += static_cast<double>(d) * d;
-    gy[e] = from_f<A>(2.f * d / static_cast<float>(n));
+    gy[e] = 2.f * d / static_cast<float>(n);
   }
   for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
   if ((threadIdx.x & 31) == 0) atomicAdd(loss, s);
@@ -618,9 +598,9 @@ void launch_conv(lbm_net_t *n, const float *x, int xs, const float *w, const flo
   using namespace lbm::net;
   dim3 grid(((W + TP - 1) / TP) * ((H + TP - 1) / TP), (Co + TC - 1) / TC, N);
   if (ks == 3)
-    conv_fwd<float, 3><<<grid, TP * TP, 0, n->stream>>>(x, xs, w, b, y, ys, H, W, Ci, Co, relu);
+    conv_fwd<3><<<grid, TP * TP, 0, n->stream>>>(x, xs, w, b, y, ys, H, W, Ci, Co, relu);
   else
-    conv_fwd<float, 1><<<grid, TP * TP, 0, n->stream>>>(x, xs, w, b, y, ys, H, W, Ci, Co, relu);
+    conv_fwd<1><<<grid, TP * TP, 0, n->stream>>>(x, xs, w, b, y, ys, H, W, Ci, Co, relu);
 }
 
 void launch_wgrad(const lbm_net_t *n, const float *x, int xs, const float *gz, int N, int H, int W,
@@ -631,33 +611,32 @@ void launch_wgrad(const lbm_net_t *n, const float *x, int xs, const float *gz, i
   const int per = static_cast<int>((npix + chunks - 1) / chunks);
   dim3 grid(((Ci + TC - 1) / TC) * ((Co + TC - 1) / TC), chunks);
   if (ks == 3)
-    conv_bwd_weight<float, 3><<<grid, 256, 0, n->stream>>>(x, xs, gz, N, H, W, Ci, Co, per, dw, db);
+    conv_bwd_weight<3><<<grid, 256, 0, n->stream>>>(x, xs, gz, N, H, W, Ci, Co, per, dw, db);
   else
-    conv_bwd_weight<float, 1><<<grid, 256, 0, n->stream>>>(x, xs, gz, N, H, W, Ci, Co, per, dw, db);
+    conv_bwd_weight<1><<<grid, 256, 0, n->stream>>>(x, xs, gz, N, H, W, Ci, Co, per, dw, db);
 }
 
 // FP32 mode: forward (and, if t != nullptr, loss + backward into n->grads)
 cudaError_t run_fp32(lbm_net_t *n, const float *x_in, int N, const float *t, float *y_out) {
   using namespace lbm::net;
-  using A = float;
   Plan p = make_plan(n);
   const int L = n->levels;
-  auto buf = [&](int i) { return static_cast<A *>(n->bufs[i]); };
-  auto gbuf = [&](int i) { return static_cast<A *>(n->bufs[p.elems.size() + i]); };
+  auto buf = [&](int i) { return static_cast<float *>(n->bufs[i]); };
+  auto gbuf = [&](int i) { return static_cast<float *>(n->bufs[p.elems.size() + i]); };
   const int64_t HW = static_cast<int64_t>(n->H) * n->W;
   cudaStream_t s = n->stream;
-  to_storage<A><<<grid1(HW * N * n->c_in), 256, 0, s>>>(x_in, buf(p.x_in), HW * N * n->c_in);
+  to_storage<<<grid1(HW * N * n->c_in), 256, 0, s>>>(x_in, buf(p.x_in), HW * N * n->c_in);
   int li = 0;
   auto W_of = [&](int k) { return n->params + n->layers[k].w_off; };
   auto B_of = [&](int k) { return n->params + n->layers[k].b_off; };
   // encoder
-  const A *h = buf(p.x_in);
+  const float *h = buf(p.x_in);
   int hc = n->c_in;
   for (int l = 0; l < L; l++) {
     const int H = n->H >> l, Wd = n->W >> l, ch = n->base << l;
     if (l > 0) {
-      pool2_fwd<A><<<grid1(static_cast<int64_t>(N) * H * Wd * hc), 256, 0, s>>>(h, hc, buf(p.pool[l]), N,
-                                                                                  H * 2, Wd * 2, hc);
+      pool2_fwd<<<grid1(static_cast<int64_t>(N) * H * Wd * hc), 256, 0, s>>>(h, hc, buf(p.pool[l]), N,
+                                                                             H * 2, Wd * 2, hc);
       h = buf(p.pool[l]);
     }
     launch_conv(n, h, hc, W_of(li), B_of(li), buf(p.ea[l]), ch, N, H, Wd, hc, ch, 3, 1);
@@ -671,9 +650,9 @@ cudaError_t run_fp32(lbm_net_t *n, const float *x_in, int N, const float *t, flo
   for (int l = L - 2; l >= 0; l--) {
     const int H = n->H >> l, Wd = n->W >> l, ch = n->base << l;
     const int cu = hc, ct = hc + ch;
-    A *cat = buf(p.cat[l]);
-    up2_fwd<A><<<grid1(static_cast<int64_t>(N) * H * Wd * cu), 256, 0, s>>>(h, cat, ct, N, H, Wd, cu);
-    copy_channels<A><<<grid1(static_cast<int64_t>(N) * H * Wd * ch), 256, 0, s>>>(
+    float *cat = buf(p.cat[l]);
+    up2_fwd<<<grid1(static_cast<int64_t>(N) * H * Wd * cu), 256, 0, s>>>(h, cat, ct, N, H, Wd, cu);
+    copy_channels<<<grid1(static_cast<int64_t>(N) * H * Wd * ch), 256, 0, s>>>(
         buf(p.eb[l]), ch, cat + cu, ct, ch, static_cast<int64_t>(N) * H * Wd, 0);
     launch_conv(n, cat, ct, W_of(li), B_of(li), buf(p.da[l]), ch, N, H, Wd, ct, ch, 3, 1);
     li++;
@@ -686,20 +665,21 @@ cudaError_t run_fp32(lbm_net_t *n, const float *x_in, int N, const float *t, flo
   launch_conv(n, h, hc, W_of(head), B_of(head), buf(p.y), n->c_out, N, n->H, n->W, hc, n->c_out, 1,
                  0);
   if (y_out)
-    to_float<A><<<grid1(HW * N * n->c_out), 256, 0, s>>>(buf(p.y), n->c_out, y_out, n->c_out, HW * N);
+    to_float<<<grid1(HW * N * n->c_out), 256, 0, s>>>(buf(p.y), n->c_out, y_out, n->c_out, HW * N);
   if (!t) return cudaGetLastError();
 
   // loss and backward
-  mse_kernel<A><<<grid1(HW * N * n->c_out), 256, 0, s>>>(buf(p.y), t, gbuf(p.y), HW * N * n->c_out,
+  mse_kernel<<<grid1(HW * N * n->c_out), 256, 0, s>>>(buf(p.y), t, gbuf(p.y), HW * N * n->c_out,
                                                         &n->status->loss);
   cudaMemsetAsync(n->grads, 0, n->n_params * sizeof(float), s);
-  A *wt = n->wt;
-  auto conv_back = [&](int k, const A *x, int xs, A *gz, A *gx, int gxs, int H, int Wd, bool need_gx) {
+  float *wt = n->wt;
+  auto conv_back = [&](int k, const float *x, int xs, float *gz, float *gx, int gxs, int H, int Wd,
+                       bool need_gx) {
     const Layer &ly = n->layers[k];
     launch_wgrad(n, x, xs, gz, N, H, Wd, ly.ci, ly.co, ly.ks, n->grads + ly.w_off,
                     n->grads + ly.b_off);
     if (need_gx) {
-      flip_weights<A><<<grid1(static_cast<int64_t>(ly.ks * ly.ks) * ly.ci * ly.co), 256, 0, s>>>(
+      flip_weights<<<grid1(static_cast<int64_t>(ly.ks * ly.ks) * ly.ci * ly.co), 256, 0, s>>>(
           n->params + ly.w_off, wt, ly.ks * ly.ks, ly.ci, ly.co);
       launch_conv(n, gz, ly.co, wt, nullptr, gx, gxs, N, H, Wd, ly.co, ly.ci, ly.ks, 0);
     }
@@ -718,18 +698,18 @@ cudaError_t run_fp32(lbm_net_t *n, const float *x_in, int N, const float *t, flo
     const int cu = ch * 2, ct = cu + ch;
     const int kb = head - 1 - 2 * l, ka = kb - 1;
     // through d_l b
-    relu_mask<A><<<grid1(static_cast<int64_t>(N) * H * Wd * ch), 256, 0, s>>>(
+    relu_mask<<<grid1(static_cast<int64_t>(N) * H * Wd * ch), 256, 0, s>>>(
         gbuf(gh_idx), buf(p.db[l]), static_cast<int64_t>(N) * H * Wd * ch);
     conv_back(kb, buf(p.da[l]), ch, gbuf(gh_idx), gbuf(p.da[l]), ch, H, Wd, true);
-    relu_mask<A><<<grid1(static_cast<int64_t>(N) * H * Wd * ch), 256, 0, s>>>(
+    relu_mask<<<grid1(static_cast<int64_t>(N) * H * Wd * ch), 256, 0, s>>>(
         gbuf(p.da[l]), buf(p.da[l]), static_cast<int64_t>(N) * H * Wd * ch);
     conv_back(ka, buf(p.cat[l]), ct, gbuf(p.da[l]), gbuf(p.cat[l]), ct, H, Wd, true);
     // split the concat gradient: skip part into the encoder level-l output grad,
     // upsampled part into the grad of the level-(l+1) output
-    copy_channels<A><<<grid1(static_cast<int64_t>(N) * H * Wd * ch), 256, 0, s>>>(
+    copy_channels<<<grid1(static_cast<int64_t>(N) * H * Wd * ch), 256, 0, s>>>(
         gbuf(p.cat[l]) + cu, ct, gbuf(p.eb[l]), ch, ch, static_cast<int64_t>(N) * H * Wd, 0);
     const int up_idx = (l + 1 <= L - 2) ? p.db[l + 1] : p.eb[L - 1];
-    up2_bwd<A><<<grid1(static_cast<int64_t>(N) * (H / 2) * (Wd / 2) * cu), 256, 0, s>>>(
+    up2_bwd<<<grid1(static_cast<int64_t>(N) * (H / 2) * (Wd / 2) * cu), 256, 0, s>>>(
         gbuf(p.cat[l]), ct, gbuf(up_idx), N, H, Wd, cu);
     gh_idx = up_idx;
   }
@@ -739,15 +719,15 @@ cudaError_t run_fp32(lbm_net_t *n, const float *x_in, int N, const float *t, flo
     const int H = n->H >> l, Wd = n->W >> l, ch = n->base << l;
     const int ka = 2 * l, kb = 2 * l + 1;
     const int cin = l == 0 ? n->c_in : (n->base << (l - 1));
-    relu_mask<A><<<grid1(static_cast<int64_t>(N) * H * Wd * ch), 256, 0, s>>>(
+    relu_mask<<<grid1(static_cast<int64_t>(N) * H * Wd * ch), 256, 0, s>>>(
         gbuf(p.eb[l]), buf(p.eb[l]), static_cast<int64_t>(N) * H * Wd * ch);
     conv_back(kb, buf(p.ea[l]), ch, gbuf(p.eb[l]), gbuf(p.ea[l]), ch, H, Wd, true);
-    relu_mask<A><<<grid1(static_cast<int64_t>(N) * H * Wd * ch), 256, 0, s>>>(
+    relu_mask<<<grid1(static_cast<int64_t>(N) * H * Wd * ch), 256, 0, s>>>(
         gbuf(p.ea[l]), buf(p.ea[l]), static_cast<int64_t>(N) * H * Wd * ch);
-    const A *xin = l == 0 ? buf(p.x_in) : buf(p.pool[l]);
+    const float *xin = l == 0 ? buf(p.x_in) : buf(p.pool[l]);
     conv_back(ka, xin, cin, gbuf(p.ea[l]), l == 0 ? nullptr : gbuf(p.pool[l]), cin, H, Wd, l > 0);
     if (l > 0)
-      pool2_bwd<A><<<grid1(static_cast<int64_t>(N) * H * 2 * Wd * 2 * cin), 256, 0, s>>>(
+      pool2_bwd<<<grid1(static_cast<int64_t>(N) * H * 2 * Wd * 2 * cin), 256, 0, s>>>(
           gbuf(p.pool[l]), gbuf(p.eb[l - 1]), cin, N, H * 2, Wd * 2, cin, 1);
   }
   return cudaGetLastError();

@@ -249,7 +249,7 @@ struct InputDev {
 constexpr int kLoadThreads = 256;
 constexpr int kConvThreads = 320 + kLoadThreads;
 constexpr int kMaxStagesB = 54;   // 9 taps x 6 chunks of 64: every weight block resident
-constexpr int kMaxStagesA = 3;
+constexpr int kMaxStagesA = 2;
 constexpr int kSmemMax = 232448 - 2048;  // dynamic shared memory a CTA may use (static below)
 
 struct ConvDev {
