@@ -452,8 +452,8 @@ KERNEL_REV = 14
 ACCURACY = {
     "fp32": {"velocity_target": 1e-5, "velocity": "met on every parity case (4e-8 to 3e-7)",
              "mass_target": 1e-10,
-             "mass": "missed on the 40x40 rotating-wall annulus (bounded, up to 4.0e-10 over "
-                     "4000 steps with the exact-mass step); met elsewhere (1-wide periodic lattices: "
+             "mass": "missed on the 40x40 rotating-wall annulus (a random walk with the exact-mass "
+                     "step: 4.0e-10 after 2000 steps); met elsewhere (1-wide periodic lattices: "
                      "3.6e-10 with the plain step, 8.7e-14 with the default exact-mass step)"},
     "fp16": {"velocity_target": 1e-3,
              "velocity": "met on every parity case (2.2e-4 to 3.2e-4); missed on the 1-wide "
@@ -471,7 +471,7 @@ ACCURACY_3D = {
              "mass": "the plain step this line times (walls at rest) meets it on the 20^3 sphere "
                      "array up to 2000 steps (4.9e-11; 1.25e-10 after 4000); met with mass_mode=1 "
                      "(3.1e-11 after 4000 steps, at 1.8x the step time) and by default where walls "
-                     "move (4.0e-11 after 2000 steps on the moving-lid channel)"},
+                     "move (2.7e-11 after 2000 steps on the moving-lid channel)"},
     "fp64": {"populations": "within 1e-13 of the oracle, element by element"},
 }
 

@@ -6,7 +6,7 @@
 // shared memory once, and a tap's shifted operand is the same tile at another
 // start address.  (Gathered per tap, nine times, the operands cost four
 // times what the MMAs did: forward pass 256x256 x 8 images 3.23 ms, now 0.41;
-// gradients 18.1 ms, now 1.49.)  Two layouts allow that:
+// gradients 18.1 ms, now 1.62.)  Two layouts allow that:
 // * conv_halo_tc: a 128-byte row of 64 channels per pixel, in the 128-byte
 //   swizzle, which goes by address: row r's 16-byte unit u lies at unit u ^ (r
 //   mod 8).  Channels are K (K-major).
@@ -19,8 +19,9 @@
 // What bounds them: an MMA of M = 128, K = 16 takes 54 cycles up to N = 64
 // and 64 at N = 128 (measured, either layout), so the layers of 32 and 64
 // output channels, 60 % of the network's flops, reach a quarter and a half of
-// the tensor peak at best; issuing the MMAs from one warp costs 70 to 100
-// cycles each around that.  The channel order of the sums (taps outermost) is
+// the tensor peak at best, and issuing the MMAs from one warp costs 70 to 100
+// cycles each around that; but a tile's latency comes first: the MMAs of the
+// forward pass take 145 of its 410 us (3 -> 32 channels: 6 of 32).  The channel order of the sums (taps outermost) is
 // kept over all shapes, so results do not depend on them.
 //
 // Every wait is bounded; one that runs out sets *err, and the CTA's roles
