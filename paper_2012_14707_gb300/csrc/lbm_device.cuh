@@ -1052,18 +1052,18 @@ __device__ __forceinline__ void node_fields(const float (&a)[N], const float (&m
   sum3(a, s[0], e[0], t[0]);
 #pragma unroll
   for (int c = 0; c < D; c++) sum3(m[c], s[c + 1], e[c + 1], t[c + 1]);
-  // least and largest magnitudes; less 1, zeros are the largest integers
+  // zeros are the largest integers after subtracting 1, subnormals the least
   uint32_t least = 0xFFFFFFFFu;
-  float third = 0.0f, most = 0.0f;
+  float third = 0.0f;
+  bool ordinary = fabsf(s[0]) < 0.5f;
 #pragma unroll
   for (int c = 0; c <= D; c++) {
     for (const float v : {s[c], e[c], t[c]})
       least = min(least, (__float_as_uint(v) & 0x7FFFFFFFu) - 1u);
     third = fmaxf(third, fabsf(t[c]));
-    // (NaN compares false below, fmaxf would drop it)
-    most = fabsf(s[c]) <= most ? most : fabsf(s[c]);
+    ordinary = ordinary && fabsf(s[c]) < 0x1p120f;  // (false for NaN)
   }
-  if (least >= 0x007FFFFFu && fabsf(s[0]) < 0.5f && most < 0x1p120f) {
+  if (ordinary && least >= 0x007FFFFFu) {
     double w[D + 1];
 #pragma unroll
     for (int c = 0; c <= D; c++) w[c] = widen(s[c]) + widen(e[c]);
