@@ -21,8 +21,9 @@
 // output channels, 60 % of the network's flops, reach a quarter and a half of
 // the tensor peak at best, and issuing the MMAs from one warp costs 70 to 100
 // cycles each around that; but a tile's latency comes first: the MMAs of the
-// forward pass take 145 of its 410 us (3 -> 32 channels: 6 of 32).  The channel order of the sums (taps outermost) is
-// kept over all shapes, so results do not depend on them.
+// forward pass take 145 of its 410 us (3 -> 32 channels: 6 of 32).  The channel
+// order of the sums (taps outermost) is kept over all shapes, so results do
+// not depend on them.
 //
 // Every wait is bounded; one that runs out sets *err, and the CTA's roles
 // give up in turn after waiting for the copies they started.
@@ -53,12 +54,13 @@ __device__ __forceinline__ void mbar_expect(uint64_t *bar, uint32_t bytes) {
                : "memory");
 }
 // Waits for the phase with parity `phase`; false if it did not come within
-// kWaitLimit tries or the CTA gave up.  For a role that one lane runs.  try_wait suspends the warp (for up to
-// about the hint, a microsecond): warps polling with test_wait took so many
-// issue slots that the roles with work to do ran several times slower (a
-// 32-channel 256x256 layer 90 us).
+// kWaitLimit tries or the CTA gave up.  For a role that one lane runs.
+// try_wait suspends the warp (for up to about the hint, a microsecond): warps
+// polling with test_wait took so many issue slots that the roles with work to
+// do ran several times slower (a 32-channel 256x256 layer 90 us).
 constexpr int kWaitLimit = 1 << 20;
-__device__ __forceinline__ bool mbar_wait_lane(uint64_t *bar, uint32_t phase, volatile int *gave_up) {
+__device__ __forceinline__ bool mbar_wait_lane(uint64_t *bar, uint32_t phase,
+                                               volatile int *gave_up) {
   const uint32_t a = smem_addr(bar);
   for (int it = 0; it < kWaitLimit; it++) {
     uint32_t done;
